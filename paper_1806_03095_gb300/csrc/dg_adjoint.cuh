@@ -38,13 +38,13 @@ constexpr int adj_cell_elems() {
 template <typename T, int N, int QC, int QV, bool PAIR>
 constexpr int adj_cells_per_cta() {
   constexpr int per_cell = adj_cell_elems<N, QC, QV, PAIR>() * (int)sizeof(T) + 16;
-  constexpr int cb = (112 * 1024 - table_elems<N, QC, QV>() * (int)sizeof(T)) / per_cell;
+  constexpr int cb = (112 * 1024 - table_elems<T, N, QC, QV>() * (int)sizeof(T)) / per_cell;
   return cb < 1 ? 1 : (cb > 4 ? 4 : cb);
 }
 
 template <typename T, int N, int QC, int QV, int CB, bool PAIR>
 constexpr size_t adj_smem_bytes() {
-  return (table_elems<N, QC, QV>() + (size_t)CB * adj_cell_elems<N, QC, QV, PAIR>() + CB) * sizeof(T) +
+  return (table_elems<T, N, QC, QV>() + (size_t)CB * adj_cell_elems<N, QC, QV, PAIR>() + CB) * sizeof(T) +
          2 * CB * sizeof(int) + 64;
 }
 
@@ -502,7 +502,7 @@ __global__ void __launch_bounds__(NT) dg_adj_kernel(const KParams kp, const doub
   extern __shared__ __align__(16) unsigned char smem_raw[];
   T* sm = reinterpret_cast<T*>(smem_raw);
   T* stab = sm;
-  T* su = stab + table_elems<N, QC, QV>();
+  T* su = stab + table_elems<T, N, QC, QV>();
   T* sy = su + CB * 5 * N3;
   T* sg = sy + CB * 5 * N3;
   T* snu = sg + CB * 5 * N3;

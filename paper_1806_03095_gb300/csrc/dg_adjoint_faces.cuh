@@ -306,13 +306,13 @@ __device__ void adj_face_pair_terms(const double* __restrict__ U, const T* __res
 template <typename T, int N, int QC, int QV>
 constexpr int adj_faces_per_cta() {
   constexpr int per_face = AdjPairSizes<N, QC, QV>::PER_FACE * (int)sizeof(T) + 16;
-  constexpr int cb = (112 * 1024 - table_elems<N, QC, QV>() * (int)sizeof(T)) / per_face;
+  constexpr int cb = (112 * 1024 - table_elems<T, N, QC, QV>() * (int)sizeof(T)) / per_face;
   return cb < 1 ? 1 : (cb > 8 ? 8 : cb);
 }
 
 template <typename T, int N, int QC, int QV, int CB>
 constexpr size_t adj_face_smem_bytes() {
-  return ((size_t)table_elems<N, QC, QV>() + (size_t)CB * AdjPairSizes<N, QC, QV>::PER_FACE + CB) * sizeof(T) +
+  return ((size_t)table_elems<T, N, QC, QV>() + (size_t)CB * AdjPairSizes<N, QC, QV>::PER_FACE + CB) * sizeof(T) +
          2 * CB * sizeof(int) + 64;
 }
 
@@ -323,7 +323,7 @@ __global__ void __launch_bounds__(NT) dg_adj_face_kernel(const KParams kp, const
   using S = AdjPairSizes<N, QC, QV>;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   T* stab = reinterpret_cast<T*>(smem_raw);
-  T* lay = stab + table_elems<N, QC, QV>();
+  T* lay = stab + table_elems<T, N, QC, QV>();
   T* ar = lay + CB * S::LAYERS;
   T* lcm = ar + CB * S::ARENA;
   T* lcp = lcm + CB * 5 * S::N2;

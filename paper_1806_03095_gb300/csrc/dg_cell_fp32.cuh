@@ -43,7 +43,7 @@ struct TaskCellSizes {
 
 template <int N, int QC, int QV, int CPB>
 constexpr size_t task_cell_smem_bytes() {
-  return ((size_t)table_elems<N, QC, QV>() + 4 + (size_t)CPB * TaskCellSizes<N, QC, QV>::PER_CELL) * sizeof(float) +
+  return ((size_t)table_elems<float, N, QC, QV>() + 4 + (size_t)CPB * TaskCellSizes<N, QC, QV>::PER_CELL) * sizeof(float) +
          64;
 }
 
@@ -91,7 +91,7 @@ __global__ void __launch_bounds__(NTH) dg_cell_task_kernel(const KParams kp, con
   constexpr int N2 = N * N, N3 = N * N * N, PC2 = S::PC2, PV2 = S::PV2, PC3 = S::PC3, PV3 = S::PV3;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   float* stab = reinterpret_cast<float*>(smem_raw);
-  float* scell = stab + ((table_elems<N, QC, QV>() + 3) & ~3);
+  float* scell = stab + ((table_elems<float, N, QC, QV>() + 3) & ~3);
   const int e0 = blockIdx.x * CPB;
   const int nb = min(CPB, kp.Nc - e0);
   if (nb <= 0) return;

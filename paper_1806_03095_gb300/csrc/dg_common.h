@@ -25,6 +25,10 @@ struct TableLayout {
   int wc, wv, wm;   // 1D Gauss weights on [0,1]
   int dl0, dl1;     // dl0[i] = l_i'(0), dl1[i] = l_i'(1)
   int total;
+  // FP64 form only, after the `total` doubles: the even-odd operators as scaled integers ({t, 0} and one
+  // {high, low} pair per entry, dg_fixed.cuh), 8 bytes each
+  int fx[EO_NOPS];
+  int total64;
 };
 
 constexpr TableLayout make_layout(int N, int QC, int QV) {
@@ -45,6 +49,12 @@ constexpr TableLayout make_layout(int N, int QC, int QV) {
   L.dl0 = o; o += N;
   L.dl1 = o; o += N;
   L.total = (o + 3) & ~3;
+  o = L.total;
+  for (int k = 0; k < EO_NOPS; ++k) {
+    L.fx[k] = o;
+    o += eo_size(dims[k][0], dims[k][1]) + 1;
+  }
+  L.total64 = (o + 3) & ~3;
   return L;
 }
 

@@ -200,7 +200,7 @@ struct TaskFaceSizes {
 
 template <int N, int QC, int QV, int FPB>
 constexpr size_t task_face_smem_bytes() {
-  return ((size_t)table_elems<N, QC, QV>() + (size_t)FPB * TaskFaceSizes<N, QC, QV>::PER_FACE + 3 * FPB) *
+  return ((size_t)table_elems<float, N, QC, QV>() + (size_t)FPB * TaskFaceSizes<N, QC, QV>::PER_FACE + 3 * FPB) *
              sizeof(float) + 64;
 }
 
@@ -418,7 +418,7 @@ __global__ void __launch_bounds__(NTH) dg_face_task_kernel(const KParams kp, flo
   using S = TaskFaceSizes<N, QC, QV>;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   float* stab = reinterpret_cast<float*>(smem_raw);
-  float* sface = stab + ((table_elems<N, QC, QV>() + 3) & ~3);
+  float* sface = stab + ((table_elems<float, N, QC, QV>() + 3) & ~3);
   float* stau = sface + FPB * S::PER_FACE;
   int* eo = reinterpret_cast<int*>(stau + FPB);
   int* en = eo + FPB;

@@ -21,6 +21,7 @@
 #include <cstdint>
 
 #include "dg_common.h"
+#include "dg_fixed.cuh"
 
 namespace dgcns {
 
@@ -65,9 +66,25 @@ __device__ __forceinline__ void batched_pass(int rank, int stride, int n, Ld ld,
 // ---------------------------------------------------------------------------
 // Shared-memory tables
 // ---------------------------------------------------------------------------
+// A 1D operator: the even-odd entries; in FP64 with the same entries as scaled integers.
+struct EoFp64 {
+  const double* p;
+  const int2* f;
+};
+template <typename T>
+struct EoOf {
+  using type = const T*;
+};
+template <>
+struct EoOf<double> {
+  using type = EoFp64;
+};
+template <typename T>
+using Eo = typename EoOf<T>::type;
+
 template <typename T>
 struct Tab {
-  const T *eSc, *eScT, *eDc, *eDcT, *eSv, *eSvT, *eDv, *eDvT, *eSmi, *eSmiT, *eSm, *eDm;
+  Eo<T> eSc, eScT, eDc, eDcT, eSv, eSvT, eDv, eDvT, eSmi, eSmiT, eSm, eDm;
   const T *wc, *wv, *wm, *dl0, *dl1;
 };
 
@@ -95,25 +112,28 @@ int upload_const_tables(const double* t64, const float* t32, cudaStream_t st) {
 }
 }  // namespace
 
+// 8- or 4-byte elements of the tables a kernel of type T keeps in shared memory.
+template <typename T, int N, int QC, int QV>
+constexpr int table_elems() {
+  return sizeof(T) == 8 ? make_layout(N, QC, QV).total64 : make_layout(N, QC, QV).total;
+}
+
 template <typename T, int N, int QC, int QV>
 __device__ __forceinline__ Tab<T> load_tables(const T* __restrict__ g, T* s) {
   constexpr TableLayout L = make_layout(N, QC, QV);
-  for (int i = threadIdx.x; i < L.total; i += blockDim.x) s[i] = g[i];
-  // FP32: operators from constant memory (6 % faster, measured); FP64: from shared memory (the constant
-  // operands made both FP64 kernels 2-3 % slower, measured)
-  const T* c = s;
-  if constexpr (sizeof(T) == 4) c = c_tab<T, N, QC, QV>;
+  for (int i = threadIdx.x; i < table_elems<T, N, QC, QV>(); i += blockDim.x) s[i] = g[i];
   Tab<T> t;
-  t.eSc = c + L.eo[EO_SC]; t.eScT = c + L.eo[EO_SCT]; t.eDc = c + L.eo[EO_DC]; t.eDcT = c + L.eo[EO_DCT];
-  t.eSv = c + L.eo[EO_SV]; t.eSvT = c + L.eo[EO_SVT]; t.eDv = c + L.eo[EO_DV]; t.eDvT = c + L.eo[EO_DVT];
-  t.eSmi = c + L.eo[EO_SMI]; t.eSmiT = c + L.eo[EO_SMIT]; t.eSm = c + L.eo[EO_SM]; t.eDm = c + L.eo[EO_DM];
+  auto op = [&](int k) -> Eo<T> {
+    if constexpr (sizeof(T) == 8)
+      return EoFp64{s + L.eo[k], reinterpret_cast<const int2*>(s + L.fx[k])};
+    else  // FP32: operators from constant memory (6 % faster than from shared memory, measured)
+      return c_tab<T, N, QC, QV> + L.eo[k];
+  };
+  t.eSc = op(EO_SC); t.eScT = op(EO_SCT); t.eDc = op(EO_DC); t.eDcT = op(EO_DCT);
+  t.eSv = op(EO_SV); t.eSvT = op(EO_SVT); t.eDv = op(EO_DV); t.eDvT = op(EO_DVT);
+  t.eSmi = op(EO_SMI); t.eSmiT = op(EO_SMIT); t.eSm = op(EO_SM); t.eDm = op(EO_DM);
   t.wc = s + L.wc; t.wv = s + L.wv; t.wm = s + L.wm; t.dl0 = s + L.dl0; t.dl1 = s + L.dl1;
   return t;
-}
-
-template <int N, int QC, int QV>
-constexpr int table_elems() {
-  return make_layout(N, QC, QV).total;
 }
 
 // 16-byte vector loads/stores of K contiguous values (K * sizeof(T) a multiple of 16, p 16-byte aligned).
@@ -150,6 +170,100 @@ __device__ __forceinline__ void vec_store(T* p, const T* x) {
   }
 }
 
+// One line through an operator O (DOUT x DIN) in even-odd form, symmetry SYM = +1 or -1, in registers.
+template <typename T, int DIN, int DOUT, int SYM>
+__device__ __forceinline__ void eo_apply(const T* __restrict__ E, const T (&x)[DIN], T (&y)[DOUT]) {
+  constexpr int IH = DIN / 2, OH = (DOUT + 1) / 2;
+  const T* __restrict__ A = E;
+  const T* __restrict__ B = E + OH * IH;
+  const T* __restrict__ C = E + 2 * OH * IH;
+  T xe[IH > 0 ? IH : 1], xo[IH > 0 ? IH : 1];
+#pragma unroll
+  for (int i = 0; i < IH; ++i) {
+    xe[i] = x[i] + x[DIN - 1 - i];
+    xo[i] = x[i] - x[DIN - 1 - i];
+  }
+  const T xm = (DIN & 1) ? x[IH] : T(0);
+#pragma unroll
+  for (int q = 0; q < OH; ++q) {
+    // the centre output of an odd-length result: a symmetric operator (SYM > 0) has no odd part there and an
+    // antisymmetric one no even part (exactly, for the symmetric point sets; the tables hold rounding-level
+    // values), so only the other half is formed
+    const bool centre = (DOUT & 1) && q == OH - 1;
+    const bool need_e = !(centre && SYM < 0), need_o = !(centre && SYM > 0);
+    T e = (DIN & 1) && need_e ? C[q] * xm : T(0);
+    T o = T(0);
+#pragma unroll
+    for (int i = 0; i < IH; ++i) {
+      if (need_e) e += A[q * IH + i] * xe[i];
+      if (need_o) o += B[q * IH + i] * xo[i];
+    }
+    if (centre) {
+      y[q] = SYM > 0 ? e : o;
+    } else {
+      y[q] = e + o;
+      y[DOUT - 1 - q] = SYM > 0 ? e - o : o - e;
+    }
+  }
+}
+
+// The same line in the kernel's precision: FP64 in integer arithmetic (dg_fixed.cuh) unless the line holds
+// values outside its range, FP32 as it is.
+template <typename T, int DIN, int DOUT, int SYM>
+__device__ __forceinline__ void line_apply(Eo<T> E, const T (&x)[DIN], T (&y)[DOUT]) {
+  if constexpr (sizeof(T) == 8) {
+    if (!fx_line<DIN, DOUT, SYM>(E.f, x, y)) eo_apply<T, DIN, DOUT, SYM>(E.p, x, y);
+  } else {
+    eo_apply<T, DIN, DOUT, SYM>(E, x, y);
+  }
+}
+
+// The FP64 sweep over `nlines` lines of contiguous arrays, as one function per (DIN, DOUT, SYM, ACC) and not
+// inlined: an integer line is 200 to 400 instructions, and the three axes of a sweep, the two sides of a face and
+// all the kernels of a translation unit share it (inlined, the k = 3 operator kernels were 3 times as long and a
+// cell's phases did not fit the instruction cache).  n0: the number of values below the swept axis, i.e. the
+// stride of a line; line l = (outer, inner) starts at outer n0 DIN + inner.
+template <int DIN, int DOUT, int SYM, bool ACC>
+__device__ __noinline__ void fx_sweep(const double* in, double* out, EoFp64 E, int nlines, int n0, int rank, int stride) {
+  const uint32_t magic = n0 > 1 ? (uint32_t)((0x100000000ull + n0 - 1) / n0) : 0u;  // l / n0 for l n0 < 2^32
+#pragma unroll 1
+  for (int l = rank; l < nlines; l += stride) {
+    const int outer = n0 > 1 ? (int)__umulhi((uint32_t)l, magic) : l;
+    const int inner = l - outer * n0;
+    const double* ip = in + (size_t)(outer * n0 * DIN + inner);
+    double* op = out + (size_t)(outer * n0 * DOUT + inner);
+    double x[DIN], y[DOUT];
+    bool loaded = false;
+    if constexpr (DIN % 2 == 0) {
+      // a line along x is contiguous: 16-byte accesses avoid the bank conflicts of threads reading DIN-value
+      // lines at a DIN-value stride
+      if (n0 == 1 && (reinterpret_cast<uintptr_t>(ip) & 15) == 0) {
+        vec_load<double, DIN>(ip, x);
+        loaded = true;
+      }
+    }
+    if (!loaded) {
+#pragma unroll
+      for (int i = 0; i < DIN; ++i) x[i] = ip[i * n0];
+    }
+    line_apply<double, DIN, DOUT, SYM>(E, x, y);
+    if constexpr (DOUT % 2 == 0) {
+      if (n0 == 1 && (reinterpret_cast<uintptr_t>(op) & 15) == 0) {
+        if (ACC) {
+          double z[DOUT];
+          vec_load<double, DOUT>(op, z);
+#pragma unroll
+          for (int q = 0; q < DOUT; ++q) y[q] += z[q];
+        }
+        vec_store<double, DOUT>(op, y);
+        continue;
+      }
+    }
+#pragma unroll
+    for (int q = 0; q < DOUT; ++q) op[q * n0] = ACC ? op[q * n0] + y[q] : y[q];
+  }
+}
+
 // ---------------------------------------------------------------------------
 // 1D sweep with even-odd decomposition: apply the operator O (DOUT x DIN, in
 // the even-odd form above, symmetry SYM = +1 or -1) along axis AX of nblk
@@ -158,8 +272,7 @@ __device__ __forceinline__ void vec_store(T* p, const T* x) {
 // registers, the operator broadcast from shared memory.  ACC adds into out.
 // ---------------------------------------------------------------------------
 template <typename T, int AX, int D0, int D1, int D2, int DOUT, int SYM, bool ACC, class G = CtaGroup>
-__device__ __forceinline__ void sweep(const T* __restrict__ in, T* __restrict__ out, const T* __restrict__ E,
-                                      int nblk, G grp = G()) {
+__device__ __forceinline__ void sweep(const T* __restrict__ in, T* __restrict__ out, Eo<T> E, int nblk, G grp = G()) {
   constexpr int DIN = AX == 0 ? D0 : (AX == 1 ? D1 : D2);
   constexpr int IH = DIN / 2, OH = (DOUT + 1) / 2;
   constexpr int O0 = AX == 0 ? DOUT : D0;
@@ -167,16 +280,18 @@ __device__ __forceinline__ void sweep(const T* __restrict__ in, T* __restrict__ 
   constexpr int O2 = AX == 2 ? DOUT : D2;
   constexpr int ISZ = D0 * D1 * D2, OSZ = O0 * O1 * O2;
   constexpr int NL = ISZ / DIN;
+  if constexpr (sizeof(T) == 8) {
+    constexpr int n0 = AX == 0 ? 1 : (AX == 1 ? D0 : D0 * D1);
+    fx_sweep<DIN, DOUT, SYM, ACC>(in, out, E, nblk * NL, n0, grp.rank(), grp.size());
+    return;
+  }
   constexpr int IST = AX == 0 ? 1 : (AX == 1 ? D0 : D0 * D1);
   constexpr int OST = AX == 0 ? 1 : (AX == 1 ? O0 : O0 * O1);
   for (int l = grp.rank(); l < nblk * NL; l += grp.size()) {
     // the operator table is loop-invariant; where it is large (high degrees) its loads stay inside the
     // loop (the pointer passes through an empty asm), so that it is not hoisted into registers and spilled
-    const T* Ep = E;
-    if constexpr (2 * OH * IH > 48) asm volatile("" : "+l"(Ep));
-    const T* __restrict__ A = Ep;
-    const T* __restrict__ B = Ep + OH * IH;
-    const T* __restrict__ C = Ep + 2 * OH * IH;
+    Eo<T> Ep = E;
+    if constexpr (sizeof(T) == 4 && 2 * OH * IH > 48) asm volatile("" : "+l"(Ep));
     const int blk = l / NL, r = l - blk * NL;
     int ib, ob;
     if (AX == 0) {
@@ -203,35 +318,8 @@ __device__ __forceinline__ void sweep(const T* __restrict__ in, T* __restrict__ 
 #pragma unroll
       for (int i = 0; i < DIN; ++i) x[i] = ip[i * IST];
     }
-    T xe[IH], xo[IH];
-#pragma unroll
-    for (int i = 0; i < IH; ++i) {
-      xe[i] = x[i] + x[DIN - 1 - i];
-      xo[i] = x[i] - x[DIN - 1 - i];
-    }
-    const T xm = (DIN & 1) ? x[IH] : T(0);
     T y[DOUT];
-#pragma unroll
-    for (int q = 0; q < OH; ++q) {
-      // the centre output of an odd-length result: a symmetric operator (SYM > 0) has no odd part there and an
-      // antisymmetric one no even part (exactly, for the symmetric point sets; the tables hold rounding-level
-      // values), so only the other half is formed
-      const bool centre = (DOUT & 1) && q == OH - 1;
-      const bool need_e = !(centre && SYM < 0), need_o = !(centre && SYM > 0);
-      T e = (DIN & 1) && need_e ? C[q] * xm : T(0);
-      T o = T(0);
-#pragma unroll
-      for (int i = 0; i < IH; ++i) {
-        if (need_e) e += A[q * IH + i] * xe[i];
-        if (need_o) o += B[q * IH + i] * xo[i];
-      }
-      if (centre) {
-        y[q] = SYM > 0 ? e : o;
-      } else {
-        y[q] = e + o;
-        y[DOUT - 1 - q] = SYM > 0 ? e - o : o - e;
-      }
-    }
+    line_apply<T, DIN, DOUT, SYM>(Ep, x, y);
     if (VOUT && (reinterpret_cast<uintptr_t>(op) & 15) == 0) {
       if (ACC) {
         T z[DOUT];
@@ -428,7 +516,7 @@ constexpr int fill_face_tmp() { return 6 * N * N + 3 * N * Q + 12 * Q * Q; }
 
 // out[e][10][Q^3]: J^{-1} and |det J| at the Gauss points (Q per direction), matrices eS: N->Q, eD: Q->Q
 template <typename T, int N, int Q, int CB, class G>
-__device__ void fill_cell_geo(const T* X, T* buf, const T* eS, const T* eD, T* out, int nb, G grp) {
+__device__ void fill_cell_geo(const T* X, T* buf, Eo<T> eS, Eo<T> eD, T* out, int nb, G grp) {
   constexpr int P = Q * Q * Q;
   T* A = buf;
   T* B = A + CB * 3 * N * N * Q;
@@ -467,7 +555,7 @@ __device__ void fill_cell_geo(const T* X, T* buf, const T* eS, const T* eD, T* o
 
 // out[e][13][Q^2] on face (d, s): J^{-1} (9), unit outward normal (3), dA (1); dl = l_i' at the face
 template <typename T, int N, int Q, int CB, int d, class G>
-__device__ void fill_face_geo(const T* X, int s, T* buf, const T* eS, const T* eD, const T* dl, T* out, int nb,
+__device__ void fill_face_geo(const T* X, int s, T* buf, Eo<T> eS, Eo<T> eD, const T* dl, T* out, int nb,
                               G grp) {
   constexpr int P = Q * Q, N2 = N * N, N3 = N * N * N;
   constexpr int t1 = d == 0 ? 1 : 0, t2 = d == 2 ? 1 : 2;
@@ -526,7 +614,7 @@ __device__ void fill_face_geo(const T* X, int s, T* buf, const T* eS, const T* e
 
 // out[e][N^3]: |det J| at the k+1 mass points (interpolation eSm, collocation eDm)
 template <typename T, int N, int CB, class G>
-__device__ void fill_mass_geo(const T* X, T* buf, const T* eSm, const T* eDm, T* out, int nb, G grp) {
+__device__ void fill_mass_geo(const T* X, T* buf, Eo<T> eSm, Eo<T> eDm, T* out, int nb, G grp) {
   constexpr int N3 = N * N * N;
   T* A = buf;
   T* B = A + CB * 3 * N3;

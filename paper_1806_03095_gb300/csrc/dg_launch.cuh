@@ -44,7 +44,7 @@ constexpr int cells_per_cta() {
   using S = Sizes<N, QC, QV>;
   constexpr int arena = S::CELL_ARENA > S::FACE_ARENA ? S::CELL_ARENA : S::FACE_ARENA;
   constexpr int per_cell = (3 * 5 * S::N3 + arena) * (int)sizeof(T) + 8;
-  constexpr int cb = (112 * 1024 - table_elems<N, QC, QV>() * (int)sizeof(T)) / per_cell;
+  constexpr int cb = (112 * 1024 - table_elems<T, N, QC, QV>() * (int)sizeof(T)) / per_cell;
   // FP64 at k >= 3 without element-centric faces: 2 cells per CTA (4 CTAs per SM hide more latency than
   // 4 cells in 2 CTAs: the face-centric cell + stage kernel at k = 3 is 2.5 % faster, measured; the fused
   // kernel is 9 % slower with 2 cells, so it keeps the larger batch)
@@ -90,7 +90,7 @@ constexpr size_t op_geo_elems() {
 template <typename T, int N, int QC, int QV, int CB, bool CELL, bool FACE, bool MASS, int GEO>
 constexpr size_t op_smem_bytes() {
   using S = Sizes<N, QC, QV>;
-  const size_t elems = table_elems<N, QC, QV>() + (size_t)CB * 5 * S::N3 * (FACE ? 3 : 2) +
+  const size_t elems = table_elems<T, N, QC, QV>() + (size_t)CB * 5 * S::N3 * (FACE ? 3 : 2) +
                        op_arena_elems<N, QC, QV, CB, CELL, FACE, MASS, GEO>() +
                        op_geo_elems<N, QC, QV, CB, FACE, GEO>() + 2 * CB;
   return elems * sizeof(T) + 2 * CB * sizeof(int) + 64;
@@ -131,7 +131,7 @@ __global__ void __launch_bounds__(op_threads<T>()) dg_op_kernel(const KParams kp
   extern __shared__ __align__(16) unsigned char smem_raw[];
   T* sm = reinterpret_cast<T*>(smem_raw);
   T* stab = sm;
-  T* su = stab + table_elems<N, QC, QV>();
+  T* su = stab + table_elems<T, N, QC, QV>();
   if constexpr (op_gws<T, N, QC, QV, CB, CELL, FACE, MASS, GEO>())  // this CTA's slice of the global workspace
     su = static_cast<T*>(kp.gws) + (size_t)blockIdx.x * op_work_elems<T, N, QC, QV, CB, CELL, FACE, MASS, GEO>();
   T* sr = su + CB * 5 * N3;
@@ -277,7 +277,7 @@ __global__ void __launch_bounds__(NT) dg_diag_kernel(const KParams kp, const dou
   extern __shared__ __align__(16) unsigned char smem_raw[];
   double* sm = reinterpret_cast<double*>(smem_raw);
   double* stab = sm;
-  double* su = stab + table_elems<N, QC, QV>();
+  double* su = stab + table_elems<double, N, QC, QV>();
   double* sl = su + CB * 5 * N3;
   double* V0 = sl + CB * 5 * N3;   // values at the Gauss points
   double* V1 = V0 + CB * 5 * P;    // temporaries / one gradient direction
@@ -425,7 +425,7 @@ __global__ void __launch_bounds__(NT) dg_diag_kernel(const KParams kp, const dou
 template <int N, int QC, int QV, int CB, int GEO>
 constexpr size_t diag_smem_bytes() {
   constexpr int N3 = N * N * N, P = QC * QC * QC;
-  return (table_elems<N, QC, QV>() + 2 * CB * 5 * N3 + 4 * CB * 5 * P + NT * NACC + (GEO ? 9 * CB * P : 0)) *
+  return (table_elems<double, N, QC, QV>() + 2 * CB * 5 * N3 + 4 * CB * 5 * P + NT * NACC + (GEO ? 9 * CB * P : 0)) *
              sizeof(double) + 64;
 }
 
@@ -460,7 +460,7 @@ __device__ __forceinline__ double inv3(const double J[3][3], double Ji[9]) {
 
 // Cell points of one point set (Q points per direction, matrices eS: N->Q, eD: Q->Q collocation).
 template <int N, int Q>
-__device__ void geom_cell(const double* X, double* buf, const double* eS, const double* eD, const double* w1,
+__device__ void geom_cell(const double* X, double* buf, Eo<double> eS, Eo<double> eD, const double* w1,
                           double* g, double* vol) {
   constexpr int P = Q * Q * Q;
   double* A = buf;            // [3][P]
@@ -498,7 +498,7 @@ __device__ void geom_cell(const double* X, double* buf, const double* eS, const 
 
 // Face points of face (d, s) for one point set; returns the face area (Gauss sum) via *area.
 template <int N, int Q, int d>
-__device__ void geom_face(const double* X, double* buf, const double* eS, const double* eD, const double* w1,
+__device__ void geom_face(const double* X, double* buf, Eo<double> eS, Eo<double> eD, const double* w1,
                           const double* dl, int s, double* g, double* area) {
   constexpr int P = Q * Q, N2 = N * N, N3 = N * N * N;
   constexpr int t1 = d == 0 ? 1 : 0, t2 = d == 2 ? 1 : 2;
@@ -568,7 +568,7 @@ __global__ void __launch_bounds__(NT) dg_geom_kernel(const KParams kp, const dou
   extern __shared__ __align__(16) unsigned char smem_raw[];
   double* sm = reinterpret_cast<double*>(smem_raw);
   double* stab = sm;
-  double* X = stab + table_elems<N, QC, QV>();
+  double* X = stab + table_elems<double, N, QC, QV>();
   double* buf = X + 3 * N3;
   double* red = buf + geom_buf_elems<N, QC, QV>();  // [0] volume, [1] interior area, [2] boundary area, [3] face tmp
   const Tab<double> tb = load_tables<double, N, QC, QV>(static_cast<const double*>(kp.tables), stab);
@@ -638,7 +638,7 @@ int geom_launch(const KParams& kp, const double* xyz, double* gcc, double* gcv, 
     return -2;
   } else {
   auto k = dg_geom_kernel<N, QC, QV>;
-  constexpr size_t smem = (table_elems<N, QC, QV>() + 3 * N * N * N + geom_buf_elems<N, QC, QV>() + 8) * sizeof(double);
+  constexpr size_t smem = (table_elems<double, N, QC, QV>() + 3 * N * N * N + geom_buf_elems<N, QC, QV>() + 8) * sizeof(double);
   if (smem > 227 * 1024) return -2;
   static bool attr[kMaxDevices] = {};
   if (smem_attr_once(k, smem, attr)) return -1;
@@ -659,7 +659,7 @@ __global__ void __launch_bounds__(NT) dg_ekgrad_kernel(const KParams kp, const d
   extern __shared__ __align__(16) unsigned char smem_raw[];
   double* sm = reinterpret_cast<double*>(smem_raw);
   double* stab = sm;
-  double* su = stab + table_elems<N, QC, QV>();
+  double* su = stab + table_elems<double, N, QC, QV>();
   double* V0 = su + CB * 5 * N3;
   double* V1 = V0 + CB * 5 * P;
   double* V2 = V1 + CB * 5 * P;
@@ -707,7 +707,7 @@ __global__ void __launch_bounds__(NT) dg_ekgrad_kernel(const KParams kp, const d
 template <int N, int QC, int QV, int GEO>
 int ekgrad_launch_geo(const KParams& kp, const double* U, double* G, double inv_volume, cudaStream_t st) {
   constexpr int CB = QC * QC * QC > 300 ? 1 : 2;
-  constexpr size_t smem = (table_elems<N, QC, QV>() + CB * 5 * N * N * N + 3 * CB * 5 * QC * QC * QC) * sizeof(double) + 64;
+  constexpr size_t smem = (table_elems<double, N, QC, QV>() + CB * 5 * N * N * N + 3 * CB * 5 * QC * QC * QC) * sizeof(double) + 64;
   if (smem > 227 * 1024) return -2;
   auto k = dg_ekgrad_kernel<N, QC, QV, CB, GEO>;
   static bool attr[kMaxDevices] = {};
@@ -731,7 +731,7 @@ int launch_op(const KParams& kp, const double* U, const void* Rin, void* Rout, v
               cudaStream_t st) {
   auto k = dg_op_kernel<T, N, QC, QV, CB, CELL, FACE, MASS, GEO>;
   constexpr bool GWS = op_gws<T, N, QC, QV, CB, CELL, FACE, MASS, GEO>();
-  constexpr size_t smem = GWS ? table_elems<N, QC, QV>() * sizeof(T) + 64
+  constexpr size_t smem = GWS ? table_elems<T, N, QC, QV>() * sizeof(T) + 64
                               : op_smem_bytes<T, N, QC, QV, CB, CELL, FACE, MASS, GEO>();
   if (smem > 227 * 1024) return -2;
   static bool attr[kMaxDevices] = {};
@@ -789,7 +789,7 @@ constexpr int warp_slice_elems() {
 
 template <typename T, int N, int QC, int QV, int WPC, bool CELL, bool FACE, bool MASS, int GEO>
 constexpr size_t warp_smem_bytes() {
-  return ((size_t)table_elems<N, QC, QV>() +
+  return ((size_t)table_elems<T, N, QC, QV>() +
           (size_t)WPC * warp_slice_elems<T, N, QC, QV, CELL, FACE, MASS, GEO>()) * sizeof(T) + 64;
 }
 
@@ -808,7 +808,7 @@ __global__ void __launch_bounds__(WPC * 32) dg_op_warp_kernel(const KParams kp, 
   const int e0 = blockIdx.x * WPC + w;
   if (e0 >= kp.Nc) return;  // only warp barriers below
   const WarpGroup grp;
-  T* su = stab + table_elems<N, QC, QV>() + w * SL;
+  T* su = stab + table_elems<T, N, QC, QV>() + w * SL;
   T* sr = su + 5 * N3;
   T* sn = sr + 5 * N3;
   T* ar = sn + (FACE ? 5 * N3 : 0);
@@ -1058,7 +1058,7 @@ template <typename T, int N, int QC, int QV, int CB, int GEO>
 constexpr size_t face_smem_bytes() {
   using S = Sizes<N, QC, QV>;
   const size_t geo = GEO == GEO_FLY ? (size_t)CB * (2 * 3 * S::N3 + S::FLY_OUT) : 0;
-  const size_t elems = table_elems<N, QC, QV>() + (size_t)CB * PairSizes<N, QC, QV>::LAYERS +
+  const size_t elems = table_elems<T, N, QC, QV>() + (size_t)CB * PairSizes<N, QC, QV>::LAYERS +
                        (size_t)CB * 5 * S::N2 + face_arena_elems<T, N, QC, QV, CB, GEO>() + geo + CB;
   return elems * sizeof(T) + 3 * CB * sizeof(int) + 64;
 }
@@ -1071,7 +1071,7 @@ constexpr int faces_per_cta() {
                                                                                     : PairSizes<N, QC, QV>::ARENA;
   constexpr int geo = GEO == GEO_FLY ? 2 * 3 * S::N3 + S::FLY_OUT : 0;
   constexpr int per_face = (PairSizes<N, QC, QV>::LAYERS + 5 * S::N2 + arena + geo) * (int)sizeof(T) + 16;
-  constexpr int cb = (112 * 1024 - table_elems<N, QC, QV>() * (int)sizeof(T)) / per_face;
+  constexpr int cb = (112 * 1024 - table_elems<T, N, QC, QV>() * (int)sizeof(T)) / per_face;
   constexpr int cap = sizeof(T) == 4 ? 8 : DGCNS_FP64_FACE_CAP;
   return cb < 1 ? 1 : (cb > cap ? cap : cb);
 }
@@ -1091,7 +1091,7 @@ __global__ void __launch_bounds__(face_threads<T, GEO>()) dg_face_kernel(const K
   constexpr int N3 = S::N3;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   T* stab = reinterpret_cast<T*>(smem_raw);
-  T* lay = stab + table_elems<N, QC, QV>();
+  T* lay = stab + table_elems<T, N, QC, QV>();
   T* lc = lay + CB * PairSizes<N, QC, QV>::LAYERS;
   T* fa = lc + CB * 5 * S::N2;
   T* sx = fa + face_arena_elems<T, N, QC, QV, CB, GEO>();  // GEO_FLY only
@@ -1202,7 +1202,7 @@ constexpr int face_warp_slice_elems() {
 
 template <typename T, int N, int QC, int QV, int WPC, int GEO>
 constexpr size_t face_warp_smem_bytes() {
-  return ((size_t)table_elems<N, QC, QV>() + (size_t)WPC * face_warp_slice_elems<T, N, QC, QV, GEO>()) * sizeof(T) +
+  return ((size_t)table_elems<T, N, QC, QV>() + (size_t)WPC * face_warp_slice_elems<T, N, QC, QV, GEO>()) * sizeof(T) +
          64;
 }
 
@@ -1239,7 +1239,7 @@ __global__ void __launch_bounds__(WPC * 32) dg_face_warp_kernel(const KParams kp
     }
   }
   const WarpGroup grp;
-  T* lay = stab + table_elems<N, QC, QV>() + w * SL;
+  T* lay = stab + table_elems<T, N, QC, QV>() + w * SL;
   T* lc = lay + PairSizes<N, QC, QV>::LAYERS;
   T* fa = lc + 5 * S::N2;
   T* sx = fa + face_arena_elems<T, N, QC, QV, 1, GEO>();  // GEO_FLY only

@@ -63,7 +63,7 @@ constexpr bool mass_tma_ok() {
 
 template <typename T, int N, int QC, int QV, bool STAGE>
 constexpr int mass_tma_table_elems() {
-  return (int)(((table_elems<N, QC, QV>() * sizeof(T) + 15) / 16) * 16 / sizeof(T));
+  return (int)(((table_elems<T, N, QC, QV>() * sizeof(T) + 15) / 16) * 16 / sizeof(T));
 }
 
 // Pipeline depth: FP32 needs more bytes in flight per SM (its sweeps are short); FP64 is ALU-bound.
@@ -90,34 +90,6 @@ constexpr int mass_tma_cells() {
 
 constexpr int kMassThreads = 256;
 
-// One 1D line through a square even-odd operator table (the layout of the sweep tables: even part
-// OH x IH, odd part OH x IH, centre column when DIN is odd), input and output in registers.
-template <typename T, int DIN, int DOUT>
-__device__ __forceinline__ void eo_line(const T* __restrict__ E, const T (&x)[DIN], T (&y)[DOUT]) {
-  constexpr int IH = DIN / 2, OH = (DOUT + 1) / 2;
-  const T* A = E;
-  const T* B = E + OH * IH;
-  const T* C = E + 2 * OH * IH;
-  T xe[IH > 0 ? IH : 1], xo[IH > 0 ? IH : 1];
-#pragma unroll
-  for (int i = 0; i < IH; ++i) {
-    xe[i] = x[i] + x[DIN - 1 - i];
-    xo[i] = x[i] - x[DIN - 1 - i];
-  }
-#pragma unroll
-  for (int q = 0; q < OH; ++q) {
-    T e = (DIN & 1) ? C[q] * x[IH] : T(0);
-    T o = T(0);
-#pragma unroll
-    for (int i = 0; i < IH; ++i) {
-      e += A[q * IH + i] * xe[i];
-      o += B[q * IH + i] * xo[i];
-    }
-    y[q] = e + o;
-    if (!((DOUT & 1) && q == OH - 1)) y[DOUT - 1 - q] = e - o;
-  }
-}
-
 // M^{-1} of a batch (Sec. 2.3, M_e^{-1} = S^{-1} diag(1/(|J| w)) S^{-T}, the three 1D factors of each
 // commuting): S^{-T} along x, y; then per z-line, in registers, S^{-T} along z, the scaling and S^{-1}
 // along z; then S^{-1} along y, x, the last sweep writing to `out` (global memory or shared).  Five
@@ -139,7 +111,7 @@ __device__ void mass_apply(const T* in, T* Abuf, T* Bbuf, T* out, const Tab<T>& 
     T x[N], y[N], z[N];
 #pragma unroll
     for (int i = 0; i < N; ++i) x[i] = ip[i * N2];
-    eo_line<T, N, N>(tb.eSmiT, x, y);
+    line_apply<T, N, N, 1>(tb.eSmiT, x, y);
     const T wxy = tb.wm[r % N] * tb.wm[r / N];
 #pragma unroll
     for (int q = 0; q < N; ++q) {
@@ -150,7 +122,7 @@ __device__ void mass_apply(const T* in, T* Abuf, T* Bbuf, T* out, const Tab<T>& 
         w *= static_cast<const T*>(kp.gm)[(size_t)(e0 + blk / 5) * N3 + r + q * N2];
       y[q] *= sg / w;
     }
-    eo_line<T, N, N>(tb.eSmi, y, z);
+    line_apply<T, N, N, 1>(tb.eSmi, y, z);
     T* op = Abuf + blk * N3 + r;
 #pragma unroll
     for (int i = 0; i < N; ++i) op[i * N2] = z[i];
@@ -357,7 +329,7 @@ __global__ void __launch_bounds__(kMassRegThreads) dg_mass_reg_kernel(const KPar
   constexpr int N3 = N * N * N, V4 = N3 / 4, RS = N3 + 4, NB = kMassRegThreads;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   float* stab = reinterpret_cast<float*>(smem_raw);
-  float* sb = stab + ((table_elems<N, QC, QV>() + 3) & ~3);  // [NB][RS]
+  float* sb = stab + ((table_elems<float, N, QC, QV>() + 3) & ~3);  // [NB][RS]
   const long long nblocks = (long long)kp.Nc * 5;
   const long long b0 = (long long)blockIdx.x * NB;
   if (b0 >= nblocks) return;
@@ -434,7 +406,7 @@ template <int N, int QC, int QV, bool STAGE>
 int launch_mass_reg(const KParams& kp, const void* Rin, void* Rout, void* dU, const double* U, double* Uout,
                     cudaStream_t st) {
   constexpr size_t smem =
-      ((size_t)((table_elems<N, QC, QV>() + 3) & ~3) + (size_t)kMassRegThreads * (N * N * N + 4)) * sizeof(float) + 64;
+      ((size_t)((table_elems<float, N, QC, QV>() + 3) & ~3) + (size_t)kMassRegThreads * (N * N * N + 4)) * sizeof(float) + 64;
   static_assert(smem <= 227 * 1024, "register mass kernel shared memory");
   auto k = dg_mass_reg_kernel<N, QC, QV, STAGE>;
   static bool attr[kMaxDevices] = {};

@@ -13,6 +13,7 @@
 #include <vector>
 
 #include "dg_common.h"
+#include "dg_fixed.cuh"
 #include "dg_launchers.h"
 #include "dgcns.h"
 
@@ -179,6 +180,34 @@ void put_eo(std::vector<double>& t, int off, const std::vector<double>& O, int d
   }
 }
 
+// The even-odd operator at t + off (oh x ih halves, as put_eo leaves it) as integers at t + fx, for fx_line:
+// {t, 0}, then {high, low} of round(entry 2^t) with the largest t for which (row sum) 2^t <= 2^61.
+void put_fixed(std::vector<double>& t, int off, int fx, int dout, int din) {
+  const int oh = (dout + 1) / 2, ih = din / 2;
+  const double *A = &t[off], *B = A + oh * ih, *C = B + oh * ih;
+  double R = 0.0;
+  for (int q = 0; q < oh; ++q) {
+    double e = std::fabs(C[q]), o = 0.0;
+    for (int i = 0; i < ih; ++i) {
+      e += std::fabs(A[q * ih + i]);
+      o += std::fabs(B[q * ih + i]);
+    }
+    R = std::max(R, std::max(e, o));
+  }
+  int sc = 0;
+  std::frexp(R, &sc);  // R < 2^sc
+  auto put = [&](int at, int32_t a, int32_t b) {
+    const int32_t v[2] = {a, b};
+    std::memcpy(&t[at], v, sizeof v);
+  };
+  put(fx, 61 - sc, 0);
+  for (int i = 0; i < eo_size(dout, din); ++i) {
+    int32_t h, l;
+    fx_split((int64_t)std::llrint(std::ldexp(A[i], 61 - sc)), h, l);
+    put(fx + 1 + i, h, l);
+  }
+}
+
 std::vector<double> transpose(const std::vector<double>& O, int rows, int cols) {
   std::vector<double> T((size_t)rows * cols);
   for (int r = 0; r < rows; ++r)
@@ -189,7 +218,7 @@ std::vector<double> transpose(const std::vector<double>& O, int rows, int cols) 
 std::vector<double> build_tables(int k, int QC, int QV) {
   const int N = k + 1;
   const TableLayout L = make_layout(N, QC, QV);
-  std::vector<double> t(L.total, 0.0);
+  std::vector<double> t(L.total64, 0.0);
   std::vector<double> nodes = lgl(k);
   symmetrize(nodes);
   std::vector<double> xc, wc, xv, wv, xm, wm, V, D, Vg, Dg;
@@ -226,6 +255,9 @@ std::vector<double> build_tables(int k, int QC, int QV) {
     t[L.dl0 + i] = D[i];
     t[L.dl1 + i] = D[N + i];
   }
+  const int dims[EO_NOPS][2] = {{QC, N}, {N, QC}, {QC, QC}, {QC, QC}, {QV, N}, {N, QV},
+                                {QV, QV}, {QV, QV}, {N, N},   {N, N},   {N, N},  {N, N}};
+  for (int q = 0; q < EO_NOPS; ++q) put_fixed(t, L.eo[q], L.fx[q], dims[q][0], dims[q][1]);
   return t;
 }
 
@@ -642,7 +674,7 @@ int dg_cns_create(const dgcns_mesh* mesh, const dgcns_params* prm, void* stream,
   // tables
   std::vector<double> t64 = build_tables(k, prm->nq_conv, prm->nq_visc);
   if (t64.empty()) return bad(DGCNS_ERR_INVALID_ARG, "singular mass interpolation matrix");
-  std::vector<float> t32(t64.begin(), t64.end());
+  std::vector<float> t32(t64.begin(), t64.begin() + make_layout(k + 1, prm->nq_conv, prm->nq_visc).total);
   // penalty per cell (Eq. TauIP_Element): nu (k+1)^2 (A_interior/2 + A_boundary)/V; affine box
   double h[3];
   for (int d = 0; d < 3; ++d) h[d] = (mesh->hi[d] - mesh->lo[d]) / mesh->n[d];
