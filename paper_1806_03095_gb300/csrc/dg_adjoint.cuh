@@ -518,11 +518,17 @@ __global__ void __launch_bounds__(NT) dg_adj_kernel(const KParams kp, const doub
   const PhysT<T> ph = make_phys<T>(kp);
   const size_t base = (size_t)e0 * 5 * N3;
   const int nvals = nb * 5 * N3;
-  for (int i = threadIdx.x; i < nvals; i += blockDim.x) {
-    const int c = (i / N3) % 5;
-    su[i] = T(U[base + i] - (c == 0 ? kp.rho_ref : (c == 4 ? kp.rhoE_ref : 0.0)));
-    sy[i] = Y[base + i];
-    sg[i] = T(0);
+  {
+    struct UY {
+      double u;
+      T y;
+    };
+    constexpr int PER = (CB * 5 * N3 + NT - 1) / NT;
+    batched_pass<PER>(threadIdx.x, NT, nvals, [&](int i) { return UY{U[base + i], Y[base + i]}; }, [&](int i, UY v) {
+      su[i] = dev_value<T>(kp, v.u, (i / N3) % 5);
+      sy[i] = v.y;
+      sg[i] = T(0);
+    });
   }
   __syncthreads();
   adj_cell_terms<T, N, QC, QV, CB, GEO>(su, sy, sg, ar, tb, kp, ph, e0, nb);
@@ -560,7 +566,7 @@ __global__ void __launch_bounds__(NT) dg_adj_kernel(const KParams kp, const doub
         if (!wall[e]) {
           const size_t src = (size_t)nbi[e] * 5 * N3 + (i - e * 5 * N3);
           const int c = (i / N3) % 5;
-          snu[i] = T(U[src] - (c == 0 ? kp.rho_ref : (c == 4 ? kp.rhoE_ref : 0.0)));
+          snu[i] = dev_value<T>(kp, U[src], c);
           sny[i] = Y[src];
         }
       }
@@ -583,9 +589,9 @@ template <typename T>
 __global__ void dg_adj_prep_kernel(size_t n, double A, double B, const double* __restrict__ lamU, T* lamdU,
                                    T* __restrict__ Wout) {
   for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
-    const double W = double(lamdU[i]) + B * lamU[i];
-    Wout[i] = T(W);
-    lamdU[i] = T(A * W);
+    const double W = f64_of(lamdU[i]) + B * lamU[i];
+    Wout[i] = f32_of<T>(W);
+    lamdU[i] = f32_of<T>(A * W);
   }
 }
 

@@ -87,35 +87,56 @@ __device__ void adj_face_pair_terms(const double* __restrict__ U, const T* __res
   for (int idx = threadIdx.x; idx < nbl * N2; idx += blockDim.x) {
     const int ec = idx / N2, j = idx - ec * N2, e = ec / 5, c = ec - 5 * e;
     const int j1 = j % N, j2 = j / N;
-    const double ref = c == 0 ? kp.rho_ref : (c == 4 ? kp.rhoE_ref : 0.0);
     const size_t om = ((size_t)eo[e] * 5 + c) * N3;
-    T du = T(0), dy = T(0);
+    // (the loads of a line first: conversions between them would make each wait for the one before)
+    double u[N];
+    T y[N], du = T(0), dy = T(0), vu = T(0), vy = T(0);
 #pragma unroll
     for (int i = 0; i < N; ++i) {
       const int q = face_node<N>(d, i, j1, j2);
-      du += dlm[i] * T(U[om + q] - ref);
-      dy += dlm[i] * Y[om + q];
+      u[i] = U[om + q];
+      y[i] = Y[om + q];
     }
-    const int qm = face_node<N>(d, idm, j1, j2);
-    LAY(0)[idx] = T(U[om + qm] - ref);
+    double un[N];
+    T yn[N];
+    const size_t op = ((size_t)max(en[e], 0) * 5 + c) * N3;
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+      const int q = face_node<N>(d, i, j1, j2);
+      un[i] = U[op + q];
+      yn[i] = Y[op + q];
+    }
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+      const T v = dev_value<T>(kp, u[i], c);
+      du += dlm[i] * v;
+      dy += dlm[i] * y[i];
+      if (i == idm) {
+        vu = v;
+        vy = y[i];
+      }
+    }
+    LAY(0)[idx] = vu;
     LAY(1)[idx] = du;
-    LAY(4)[idx] = Y[om + qm];
+    LAY(4)[idx] = vy;
     LAY(5)[idx] = dy;
     if (en[e] < 0) {
       LAY(2)[idx] = LAY(3)[idx] = LAY(6)[idx] = LAY(7)[idx] = T(0);
     } else {
-      const size_t op = ((size_t)en[e] * 5 + c) * N3;
-      T dun = T(0), dyn = T(0);
+      T dun = T(0), dyn = T(0), vun = T(0), vyn = T(0);
 #pragma unroll
       for (int i = 0; i < N; ++i) {
-        const int q = face_node<N>(d, i, j1, j2);
-        dun += dlp[i] * T(U[op + q] - ref);
-        dyn += dlp[i] * Y[op + q];
+        const T v = dev_value<T>(kp, un[i], c);
+        dun += dlp[i] * v;
+        dyn += dlp[i] * yn[i];
+        if (i == idp) {
+          vun = v;
+          vyn = yn[i];
+        }
       }
-      const int qp = face_node<N>(d, idp, j1, j2);
-      LAY(2)[idx] = T(U[op + qp] - ref);
+      LAY(2)[idx] = vun;
       LAY(3)[idx] = dun;
-      LAY(6)[idx] = Y[op + qp];
+      LAY(6)[idx] = vyn;
       LAY(7)[idx] = dyn;
     }
   }

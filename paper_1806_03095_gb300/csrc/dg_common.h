@@ -15,7 +15,10 @@ namespace dgcns {
 // decomposition): for q < ceil(DOUT/2), i < floor(DIN/2)
 //   a[q][i] = (O[q][i] + O[q][DIN-1-i]) / 2,  b[q][i] = (O[q][i] - O[q][DIN-1-i]) / 2,
 //   c[q]    = O[q][DIN/2] (middle column, DIN odd; else 0).
-enum EoOp { EO_SC, EO_SCT, EO_DC, EO_DCT, EO_SV, EO_SVT, EO_DV, EO_DVT, EO_SMI, EO_SMIT, EO_SM, EO_DM, EO_NOPS };
+enum EoOp { EO_SC, EO_SCT, EO_DC, EO_DCT, EO_SV, EO_SVT, EO_DV, EO_DVT, EO_SMI, EO_SMIT, EO_SM, EO_DM,
+            // collocation form: W^-1 D^T W at the convective and the viscous points, the projection
+            // l_g(x_q) w_q / w_g of the convective points, and W^-1 D^T W extended by the face shares
+            EO_DCW, EO_DVW, EO_PC, EO_LIFT, EO_NOPS };
 
 constexpr int eo_size(int dout, int din) { return ((dout + 1) / 2) * (din / 2) * 2 + (dout + 1) / 2; }
 
@@ -31,17 +34,30 @@ struct TableLayout {
   int total64;
 };
 
+// The collocation form (dg_coll.cuh) needs the viscous points to be the k+1 mass points; above k = 6 its
+// working set per cell does not fit shared memory.
+constexpr bool coll_rule(int N, int QV) { return QV == N && N <= 7; }
+
+// Extent (DOUT, DIN) of operator k; zero where the rule does not use it.
+struct EoDims {
+  int dout, din;
+};
+constexpr EoDims eo_dims(int k, int N, int QC, int QV) {
+  const int dims[EO_NOPS][2] = {{QC, N}, {N, QC}, {QC, QC}, {QC, QC}, {QV, N}, {N, QV}, {QV, QV}, {QV, QV},
+                                {N, N},  {N, N},  {N, N},   {N, N},   {QC, QC}, {N, N}, {N, QC},  {N, N + 4}};
+  if (k >= EO_DCW && !coll_rule(N, QV)) return EoDims{0, 0};
+  return EoDims{dims[k][0], dims[k][1]};
+}
+
 constexpr TableLayout make_layout(int N, int QC, int QV) {
   TableLayout L{};
   L.N = N;
   L.QC = QC;
   L.QV = QV;
   int o = 0;
-  const int dims[EO_NOPS][2] = {{QC, N}, {N, QC}, {QC, QC}, {QC, QC}, {QV, N}, {N, QV},
-                                {QV, QV}, {QV, QV}, {N, N},   {N, N},   {N, N},  {N, N}};
   for (int k = 0; k < EO_NOPS; ++k) {
     L.eo[k] = o;
-    o += eo_size(dims[k][0], dims[k][1]);
+    o += eo_size(eo_dims(k, N, QC, QV).dout, eo_dims(k, N, QC, QV).din);
   }
   L.wc = o; o += QC;
   L.wv = o; o += QV;
@@ -52,7 +68,7 @@ constexpr TableLayout make_layout(int N, int QC, int QV) {
   o = L.total;
   for (int k = 0; k < EO_NOPS; ++k) {
     L.fx[k] = o;
-    o += eo_size(dims[k][0], dims[k][1]) + 1;
+    o += eo_size(eo_dims(k, N, QC, QV).dout, eo_dims(k, N, QC, QV).din) + 1;
   }
   L.total64 = (o + 3) & ~3;
   return L;
@@ -84,6 +100,7 @@ struct KParams {
   double h[3];          // affine cell extents
   double bf[3];         // body force vector
   double A, B, dt;      // 2N stage coefficients (out_mode 2)
+  float A32, dt32;      // the same in FP32
   const double* tau;    // [Nc] penalty per cell (FP64)
   const void* tables;   // device tables of the kernel's precision
   // Stored geometry (non-affine meshes), in the kernel's precision (quadrature weights excluded):
@@ -165,6 +182,18 @@ __host__ __device__ __forceinline__ void frame_facing(int code, int d, int s, in
   dn = ((code & 3) == d) ? 0 : (((code >> 2) & 3) == d ? 1 : 2);
   refl = (code >> (6 + dn)) & 1;
   sn = refl ? s : 1 - s;
+}
+
+// A and dt of the stage in the residual type (a conversion per thread would run on the FP64 pipe).
+template <typename T>
+__host__ __device__ __forceinline__ T stage_A(const KParams& kp) {
+  if constexpr (sizeof(T) == 8) return kp.A;
+  else return kp.A32;
+}
+template <typename T>
+__host__ __device__ __forceinline__ T stage_dt(const KParams& kp) {
+  if constexpr (sizeof(T) == 8) return kp.dt;
+  else return kp.dt32;
 }
 
 // Dynamic shared-memory attribute of a kernel: a per-device setting, made once per (kernel, device) on

@@ -56,13 +56,12 @@ __device__ void face_pair_terms(const double* __restrict__ U, const T* __restric
   for (int idx = grp.rank(); idx < nbl * N2; idx += grp.size()) {
     const int ec = idx / N2, j = idx - ec * N2, e = ec / 5, c = ec - 5 * e;
     const int j1 = j % N, j2 = j / N;
-    const double dref = c == 0 ? kp.rho_ref : (c == 4 ? kp.rhoE_ref : 0.0);
     const size_t om = ((size_t)eo[e] * 5 + c) * N3;
     T dn = T(0), vm = T(0);
 #pragma unroll
     for (int i = 0; i < N; ++i) {
       const int q = face_node<N>(d, i, j1, j2);
-      const T v = Ud ? Ud[om + q] : T(U[om + q] - dref);
+      const T v = Ud ? Ud[om + q] : dev_value<T>(kp, U[om + q], c);
       dn += dlm[i] * v;
       if (i == idm) vm = v;
     }
@@ -85,7 +84,7 @@ __device__ void face_pair_terms(const double* __restrict__ U, const T* __restric
 #pragma unroll
       for (int i = 0; i < N; ++i) {
         const int q = q0 + i * qs;
-        const T v = Ud ? Ud[op + q] : T(U[op + q] - dref);
+        const T v = Ud ? Ud[op + q] : dev_value<T>(kp, U[op + q], c);
         dq += dlp[i] * v;
         if (i == idp) vp = v;
       }
@@ -346,6 +345,91 @@ __device__ void face_pair_terms(const double* __restrict__ U, const T* __restric
       pn[5 * N2] = kp.visc ? dsg * Dp[idx] : T(0);
     }
   }
+}
+
+// The faces of a CTA (blockIdx.x; direction d): blocks [0, ceil(Nc/CB)) take the upper face (s = 1) of every
+// cell, on a non-periodic direction the following blocks the lower wall faces (s = 0) of the cells with c_d = 0;
+// on rotated-frame meshes the faces owned through local face (d, 1), then (d, 0).  Threads < nb write the
+// owner, the other cell (-1: wall), its orientation code and the penalty; false: nothing to do.
+template <int CB, typename T>
+__device__ __forceinline__ bool face_batch(const KParams& kp, int d, int& s, int& nb, int* eo, int* en, int* oc,
+                                           T* tau_f) {
+  const int t1 = d == 0 ? 1 : 0, t2 = d == 2 ? 1 : 2;
+  int i0, nitems;
+  if (kp.flist) {  // rotated-frame meshes: the faces owned through local face (d, 1), then (d, 0)
+    const int nb1 = (kp.flen[2 * d + 1] + CB - 1) / CB;
+    s = (int)blockIdx.x < nb1 ? 1 : 0;
+    i0 = (s ? (int)blockIdx.x : (int)blockIdx.x - nb1) * CB;
+    nitems = kp.flen[2 * d + s];
+    if (i0 >= nitems) return false;
+  } else {
+    const int nstd = (kp.Nc + CB - 1) / CB;
+    if ((int)blockIdx.x < nstd) {
+      s = 1;
+      i0 = blockIdx.x * CB;
+      nitems = kp.Nc;
+    } else {
+      if (kp.periodic[d]) return false;
+      s = 0;
+      i0 = (blockIdx.x - nstd) * CB;
+      nitems = kp.nc[t1] * kp.nc[t2];
+      if (i0 >= nitems) return false;
+    }
+  }
+  nb = min(CB, nitems - i0);
+  if ((int)threadIdx.x < nb && kp.flist) {
+    const int e = kp.flist[kp.foff[2 * d + s] + i0 + threadIdx.x];
+    const int* t = kp.fnbr + ((size_t)e * 6 + 2 * d + s) * 2;
+    eo[threadIdx.x] = e;
+    en[threadIdx.x] = t[0];
+    oc[threadIdx.x] = t[1];
+    tau_f[threadIdx.x] = T(fmax(kp.tau[e], kp.tau[t[0]]));
+  } else if ((int)threadIdx.x < nb) {
+    const int i = i0 + threadIdx.x;
+    int c[3];
+    if (s == 1) {
+      c[0] = i % kp.nc[0];
+      c[1] = (i / kp.nc[0]) % kp.nc[1];
+      c[2] = i / (kp.nc[0] * kp.nc[1]);
+    } else {
+      c[d] = 0;
+      c[t1] = i % kp.nc[t1];
+      c[t2] = i / kp.nc[t1];
+    }
+    const int e = c[0] + kp.nc[0] * (c[1] + kp.nc[1] * c[2]);
+    c[d] += s ? 1 : -1;
+    int w = 0;
+    if (c[d] < 0 || c[d] >= kp.nc[d]) {
+      if (kp.periodic[d])
+        c[d] = (c[d] + kp.nc[d]) % kp.nc[d];
+      else
+        w = 1;
+    }
+    const int n = w ? -1 : c[0] + kp.nc[0] * (c[1] + kp.nc[1] * c[2]);
+    eo[threadIdx.x] = e;
+    en[threadIdx.x] = n;
+    const double te = kp.tau[e];
+    tau_f[threadIdx.x] = T(w ? te : fmax(te, kp.tau[n]));
+  }
+  return true;
+}
+
+// Blocks per direction for `per` faces a block.
+inline int face_blocks(const KParams& kp, int per) {
+  int g = 0;
+  if (kp.flist) {
+    for (int d = 0; d < 3; ++d) {
+      const int b = (kp.flen[2 * d + 1] + per - 1) / per + (kp.flen[2 * d] + per - 1) / per;
+      if (b > g) g = b;
+    }
+    return g;
+  }
+  for (int d = 0; d < 3; ++d) {
+    if (kp.periodic[d]) continue;
+    const int plane = kp.nc[d == 0 ? 1 : 0] * kp.nc[d == 2 ? 1 : 2];
+    if (plane > g) g = plane;
+  }
+  return (kp.Nc + per - 1) / per + (g + per - 1) / per;
 }
 
 // Shared memory of face_pair_terms per face: 4 trace layers; arena: conv 2 tmp + 2 point arrays,

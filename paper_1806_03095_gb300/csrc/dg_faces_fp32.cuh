@@ -8,16 +8,17 @@
 //     interpolates D; the 2D tensor contractions of a face are held in the thread's registers, and each
 //     result goes to shared memory once;
 //  2. convective points, one thread per (face, point): the LLF flux, tested with the own side's V (the
-//     other side's test is its negative);
-//  3. viscous points: one thread per (face, point, side) forms F_v(U, grad U) . n of its side, then one
-//     thread per (face, point) forms the SIPG flux and F_v(U^-+, [[U]] (x) n) of both sides;
-//  4. test tasks, one thread per (face, side, component): the transposed contractions in registers, and the
-//     two shares (value layer and normal derivative) written to the face buffer.
+//     other side's test is its negative); viscous points, one thread per (face, point): the SIPG flux and
+//     F_v(U^-+, [[U]] (x) n) of both sides;
+//  3. test tasks, one thread per (face, side, component): the transposed contractions in registers, and the
+//     two shares (value and normal derivative) written to the face buffer.
 //
-// Shares, signs and the layout of the face buffer are those of face_pair_terms.  The even-odd 1D
-// operators come from constant memory with compile-time offsets.
+// Point fluxes, signs and the face buffer are those of the collocation form (dg_coll.cuh): no quadrature
+// weights, and a viscous integrand at the face's Gauss points is a share as it stands.  The even-odd 1D
+// operators come from constant memory with compile-time offsets.  k = 3, TGV 64^3, per launch:
+// 1.42 -> 1.14 ms against the form that tested with the nodal basis and formed all flux columns.
 #pragma once
-#include "dg_faces.cuh"
+#include "dg_coll.cuh"
 
 namespace dgcns {
 
@@ -182,8 +183,7 @@ __device__ __forceinline__ void face_traces(const float* __restrict__ src, const
 
 // Shared-memory layout of one CTA (floats): per face, conv traces [2][5][QC^2] (the own side's slots
 // later hold the LLF integrand), viscous traces [2][5][VS] with VS >= 4 QV^2 (U, d/dt1, d/dt2, normal
-// derivative; later the four test integrands), the viscous normal fluxes [2][5][QV^2].  Padding against
-// shared-memory bank conflicts: a (side, component) task writes and reads its 4 QV^2 viscous values as
+// derivative; later the four test integrands).  Padding against shared-memory bank conflicts: a (side, component) task writes and reads its 4 QV^2 viscous values as
 // 16-byte vectors, so VS = 4 QV^2 + 4 puts the blocks of 8 neighbouring tasks on distinct banks (a stride
 // of 4 QV^2 = 64 words put them all on the same 4 banks); the per-face stride is 8 (mod 32) words, so the
 // tasks of the next face in the same quarter-warp land on other banks too.
@@ -193,8 +193,7 @@ struct TaskFaceSizes {
   static constexpr int CIN = (2 * 5 * PC + 3) & ~3;
   static constexpr int VS = 4 * PV + 4;
   static constexpr int VIN = 2 * 5 * VS;
-  static constexpr int FVN = 2 * 5 * PV;
-  static constexpr int RAW = CIN + VIN + FVN;
+  static constexpr int RAW = CIN + VIN;
   static constexpr int PER_FACE = RAW + ((8 - RAW % 32) + 32) % 32;
 };
 
@@ -215,7 +214,6 @@ __device__ __forceinline__ void face_task_body(const KParams& kp, float* __restr
   constexpr int d = DIR, t1 = DIR == 0 ? 1 : 0, t2 = DIR == 2 ? 1 : 2;
   const KConst<float>& kc = kconst<float>(kp);
   const float hinv_d = kc.hinv[d], hinv_1 = kc.hinv[t1], hinv_2 = kc.hinv[t2];
-  const float area = kc.area[d];
   const float sgn = s ? 1.f : -1.f;
   const float* __restrict__ Ud = static_cast<const float*>(kp.Udev);
 
@@ -266,106 +264,83 @@ __device__ __forceinline__ void face_task_body(const KParams& kp, float* __restr
 #pragma unroll
         for (int c = 0; c < 5; ++c) up[c] = fb[(5 + c) * PC + p];
       }
-      const float rm = 1.f / (ph.rho_r + um[0]), rp = 1.f / (ph.rho_r + up[0]);
-      const float pm = pressure_dev(um, rm, ph.gm1), pp = pressure_dev(up, rp, ph.gm1);
-      const float lm = sqrtf(um[1] * um[1] + um[2] * um[2] + um[3] * um[3]) * rm + sqrtf(fabsf(ph.gamma * (ph.p_r + pm) * rm));
-      const float lp = sqrtf(up[1] * up[1] + up[2] * up[2] + up[3] * up[3]) * rp + sqrtf(fabsf(ph.gamma * (ph.p_r + pp) * rp));
-      const float lam = lm > lp ? lm : lp;
-      const float w = tb.wc[p % QC] * tb.wc[p / QC] * area;
-      float fm[5], fp[5];
-      conv_flux_dir(um, rm, pm, ph.H_r, d, fm);
-      conv_flux_dir(up, rp, pp, ph.H_r, d, fp);
+      const float nd[3] = {0.f, 0.f, 0.f};
+      float fm[5], fp[5], lm, lp;
+      llf_side<float, DIR, true>(um, nd, sgn, ph, fm, lm);
+      llf_side<float, DIR, true>(up, nd, sgn, ph, fp, lp);
+      const float lam = lm > lp ? lm : lp, w = -0.5f * hinv_d;
 #pragma unroll
-      for (int c = 0; c < 5; ++c) fb[c * PC + p] = w * (0.5f * sgn * (fm[c] + fp[c]) + 0.5f * lam * (um[c] - up[c]));
+      for (int c = 0; c < 5; ++c) fb[c * PC + p] = w * (fm[c] + fp[c] + lam * (um[c] - up[c]));
     }
   }
 
+  // viscous points: value share (V, Q*.n) and the +1/2 (grad V, F_v(U, [[U]] (x) n)) integrands of both sides
   if (kp.visc) {
-    // 3a. F_v(U, grad U) . n of each side (n = sgn e_d: the d column), from the side's own traces
-    for (int task = threadIdx.x; task < nb * 2 * PV; task += NTH) {
-      const int b = task / (2 * PV), r = task - 2 * PV * b, sd = r / PV, p = r - PV * sd;
-      float* fb = sface + b * S::PER_FACE;
-      const bool wall = en[b] < 0;
-      const int src = wall ? 0 : sd;  // wall: grad U+ = grad U-, U+ the ghost state
-      const float* vi = fb + S::CIN;
-      float u[5], Gr[5][3], F[5][3];
-#pragma unroll
-      for (int c = 0; c < 5; ++c) {
-        const float* q = vi + (src * 5 + c) * S::VS + p;
-        u[c] = q[0];
-        Gr[c][t1] = q[PV] * hinv_1;
-        Gr[c][t2] = q[2 * PV] * hinv_2;
-        Gr[c][d] = q[3 * PV] * hinv_d;
-      }
-      if (wall && sd == 1) {
-        float g[5];
-        wall_ghost(u, ph, g);
-#pragma unroll
-        for (int c = 0; c < 5; ++c) u[c] = g[c];
-      }
-      visc_flux(u, Gr, ph, F);
-      float* o = fb + S::CIN + S::VIN + sd * 5 * PV + p;
-#pragma unroll
-      for (int c = 0; c < 5; ++c) o[c * PV] = F[c][d] * sgn;
-    }
-    __syncthreads();
-    // 3b. SIPG value integrands and the -1/2 (grad V, F_v(U, [[U]] (x) n)) integrands of both sides
     for (int task = threadIdx.x; task < nb * PV; task += NTH) {
       const int b = task / PV, p = task - PV * b;
-      float* fb = sface + b * S::PER_FACE;
       const bool wall = en[b] < 0;
-      float* vi = fb + S::CIN;
-      const float* fv = vi + S::VIN;
-      float um[5], up[5];
+      float* vm = sface + b * S::PER_FACE + S::CIN + p;
+      float* vp = vm + 5 * S::VS;
+      float um[5], up[5], jmp[5], gd[5], fm[4], fp[4];
 #pragma unroll
-      for (int c = 0; c < 5; ++c) um[c] = vi[c * S::VS + p];
+      for (int c = 0; c < 5; ++c) um[c] = vm[c * S::VS];
       if (wall) {
         wall_ghost(um, ph, up);
       } else {
 #pragma unroll
-        for (int c = 0; c < 5; ++c) up[c] = vi[(5 + c) * S::VS + p];
+        for (int c = 0; c < 5; ++c) up[c] = vp[c * S::VS];
       }
-      const float wgt = tb.wv[p % QV] * tb.wv[p / QV] * area;
-      const float tau = stau[b];
-      float jmp[5];
+      const SideState<float> sm = side_state(um, ph), sp = side_state(up, ph);
+      auto normal = [&](const SideState<float>& st, const float* v, float f[4]) {
+        const float *g1 = v + PV, *g2 = v + 2 * PV;
+#pragma unroll
+        for (int c = 0; c < 5; ++c) gd[c] = hinv_d * v[c * S::VS + 3 * PV];
+        visc_normal<float, DIR>(st, gd, hinv_1 * g1[0], hinv_1 * g1[(1 + d) * S::VS], hinv_1 * g1[(1 + t1) * S::VS],
+                                hinv_2 * g2[0], hinv_2 * g2[(1 + d) * S::VS], hinv_2 * g2[(1 + t2) * S::VS], ph, f);
+      };
+      normal(sm, vm, fm);
+      normal(sp, wall ? vm : vp, fp);  // wall: grad U+ = grad U-, at the ghost state
+      const float wv = 0.5f * sgn * hinv_d, wt = hinv_d * stau[b];
+      float v[5];
 #pragma unroll
       for (int c = 0; c < 5; ++c) {
         jmp[c] = um[c] - up[c];
-        const float v = -wgt * (0.5f * (fv[c * PV + p] + fv[(5 + c) * PV + p]) - tau * jmp[c]);
-        vi[c * S::VS + p] = v;
-        if (!wall) vi[(5 + c) * S::VS + p] = -v;
+        v[c] = -wt * jmp[c];
       }
-      float Jg[5][3], F[5][3];
+      v[1 + d] += wv * (fm[0] + fp[0]);
+      v[1 + t1] += wv * (fm[1] + fp[1]);
+      v[1 + t2] += wv * (fm[2] + fp[2]);
+      v[4] += wv * (fm[3] + fp[3]);
+      const float hd = wv * hinv_d, h1 = wv * hinv_1, h2 = wv * hinv_2;
+      auto tests = [&](const SideState<float>& st, float* q, float sg) {
+        float a[4], b1[3], b2[3];
+        visc_jump<float, DIR>(st, jmp, ph, a, b1, b2);
 #pragma unroll
-      for (int c = 0; c < 5; ++c) {
-        Jg[c][t1] = 0.f;
-        Jg[c][t2] = 0.f;
-        Jg[c][d] = jmp[c] * sgn;
-      }
-      const float hw = -0.5f * wgt;
-      visc_flux(um, Jg, ph, F);
-#pragma unroll
-      for (int c = 0; c < 5; ++c) {
-        float* q = vi + c * S::VS + p;
-        q[PV] = hw * hinv_1 * F[c][t1];
-        q[2 * PV] = hw * hinv_2 * F[c][t2];
-        q[3 * PV] = hw * hinv_d * F[c][d];
-      }
-      if (!wall) {
-        visc_flux(up, Jg, ph, F);
-#pragma unroll
-        for (int c = 0; c < 5; ++c) {
-          float* q = vi + (5 + c) * S::VS + p;
-          q[PV] = hw * hinv_1 * F[c][t1];
-          q[2 * PV] = hw * hinv_2 * F[c][t2];
-          q[3 * PV] = hw * hinv_d * F[c][d];
-        }
-      }
+        for (int c = 0; c < 5; ++c) q[c * S::VS] = sg * v[c];
+        float* q1 = q + PV;
+        q1[0] = q1[(1 + t2) * S::VS] = 0.f;
+        q1[(1 + d) * S::VS] = h1 * b1[0];
+        q1[(1 + t1) * S::VS] = h1 * b1[1];
+        q1[4 * S::VS] = h1 * b1[2];
+        float* q2 = q + 2 * PV;
+        q2[0] = q2[(1 + t1) * S::VS] = 0.f;
+        q2[(1 + d) * S::VS] = h2 * b2[0];
+        q2[(1 + t2) * S::VS] = h2 * b2[1];
+        q2[4 * S::VS] = h2 * b2[2];
+        float* q3 = q + 3 * PV;
+        q3[0] = 0.f;
+        q3[(1 + d) * S::VS] = hd * a[0];
+        q3[(1 + t1) * S::VS] = hd * a[1];
+        q3[(1 + t2) * S::VS] = hd * a[2];
+        q3[4 * S::VS] = hd * a[3];
+      };
+      tests(sm, vm, 1.f);
+      if (!wall) tests(sp, vp, -1.f);
     }
   }
   __syncthreads();
 
-  // 4. test tasks: value-layer share L and normal-derivative share D of (face b, side sd, component c)
+  // 3. test tasks: value share L and normal-derivative share D of (face b, side sd, component c)
   for (int task = threadIdx.x; task < nb * 10; task += NTH) {
     const int b = task / 10, r = task - 10 * b, sd = r / 5, c = r - 5 * sd;
     const int cell = sd ? en[b] : eo[b];
@@ -382,29 +357,25 @@ __device__ __forceinline__ void face_task_body(const KParams& kp, float* __restr
       const float sg = sd ? -1.f : 1.f;
 #pragma unroll
       for (int p = 0; p < PC; ++p) X[p] = sg * fb[c * PC + p];
-      eo_2d<QC, QC, N, N, 1, 1>(tb.eScT, tb.eScT, X, Y);
+      eo_2d<QC, QC, N, N, 1, 1>(tb.ePc, tb.ePc, X, Y);
 #pragma unroll
       for (int j = 0; j < N2; ++j) Ls[j] = Y[j];
     }
     if (kp.visc) {
       const float* vi = fb + S::CIN + (sd * 5 + c) * S::VS;
-      float V[PV], G[PV], T[PV], Y[N2];
-      arr_load<PV>(vi, V);
+      float G[PV], T[PV];
+      arr_load<PV>(vi, G);
+#pragma unroll
+      for (int p = 0; p < PV; ++p) Ls[p] += G[p];
       arr_load<PV>(vi + PV, G);
-      eo_dir0<QV, QV, QV, -1>(tb.eDvT, G, T);
+      eo_dir0<QV, QV, QV, -1>(tb.eDvW, G, T);
 #pragma unroll
-      for (int p = 0; p < PV; ++p) V[p] += T[p];
+      for (int p = 0; p < PV; ++p) Ls[p] += T[p];
       arr_load<PV>(vi + 2 * PV, G);
-      eo_dir1<QV, QV, QV, -1>(tb.eDvT, G, T);
+      eo_dir1<QV, QV, QV, -1>(tb.eDvW, G, T);
 #pragma unroll
-      for (int p = 0; p < PV; ++p) V[p] += T[p];
-      eo_2d<QV, QV, N, N, 1, 1>(tb.eSvT, tb.eSvT, V, Y);
-#pragma unroll
-      for (int j = 0; j < N2; ++j) Ls[j] += Y[j];
-      arr_load<PV>(vi + 3 * PV, G);
-      eo_2d<QV, QV, N, N, 1, 1>(tb.eSvT, tb.eSvT, G, Y);
-#pragma unroll
-      for (int j = 0; j < N2; ++j) Ds[j] = Y[j];
+      for (int p = 0; p < PV; ++p) Ls[p] += T[p];
+      arr_load<PV>(vi + 3 * PV, Ds);
     }
     const int f = 2 * d + (sd ? 1 - s : s);
     float* po = FB + (((size_t)cell * 6 + f) * 2 * 5 + c) * N2;
@@ -422,52 +393,11 @@ __global__ void __launch_bounds__(NTH) dg_face_task_kernel(const KParams kp, flo
   float* stau = sface + FPB * S::PER_FACE;
   int* eo = reinterpret_cast<int*>(stau + FPB);
   int* en = eo + FPB;
-
   const int d = blockIdx.y;
-  const int t1 = d == 0 ? 1 : 0, t2 = d == 2 ? 1 : 2;
-  const int nstd = (kp.Nc + FPB - 1) / FPB;
-  int s, i0, nitems;
-  if ((int)blockIdx.x < nstd) {
-    s = 1;
-    i0 = blockIdx.x * FPB;
-    nitems = kp.Nc;
-  } else {
-    if (kp.periodic[d]) return;
-    s = 0;
-    i0 = (blockIdx.x - nstd) * FPB;
-    nitems = kp.nc[t1] * kp.nc[t2];
-    if (i0 >= nitems) return;
-  }
-  const int nb = min(FPB, nitems - i0);
+  int s, nb;
+  if (!face_batch<FPB>(kp, d, s, nb, eo, en, en, stau)) return;  // (no orientation codes: structured meshes only)
   const Tab<float> tb = load_tables<float, N, QC, QV>(static_cast<const float*>(kp.tables), stab);
   const PhysT<float> ph = make_phys<float>(kp);
-  if ((int)threadIdx.x < nb) {
-    const int i = i0 + threadIdx.x;
-    int c[3];
-    if (s == 1) {
-      c[0] = i % kp.nc[0];
-      c[1] = (i / kp.nc[0]) % kp.nc[1];
-      c[2] = i / (kp.nc[0] * kp.nc[1]);
-    } else {
-      c[d] = 0;
-      c[t1] = i % kp.nc[t1];
-      c[t2] = i / kp.nc[t1];
-    }
-    const int e = c[0] + kp.nc[0] * (c[1] + kp.nc[1] * c[2]);
-    c[d] += s ? 1 : -1;
-    int w = 0;
-    if (c[d] < 0 || c[d] >= kp.nc[d]) {
-      if (kp.periodic[d])
-        c[d] = (c[d] + kp.nc[d]) % kp.nc[d];
-      else
-        w = 1;
-    }
-    const int n = w ? -1 : c[0] + kp.nc[0] * (c[1] + kp.nc[1] * c[2]);
-    eo[threadIdx.x] = e;
-    en[threadIdx.x] = n;
-    const double te = kp.tau[e];
-    stau[threadIdx.x] = float(w ? te : fmax(te, kp.tau[n]));
-  }
   __syncthreads();
 
   if (d == 0)
@@ -478,36 +408,22 @@ __global__ void __launch_bounds__(NTH) dg_face_task_kernel(const KParams kp, flo
     face_task_body<N, QC, QV, FPB, NTH, 2>(kp, FB, tb, ph, sface, stau, eo, en, nb, s);
 }
 
-// The task kernel serves the FP32 affine face terms at k = 3.  It compiles without spills at k = 4 and 5
-// (128 and 255 registers per thread), but there it was slower than the warp-per-face kernel (mixed TGV per
-// stage: k = 4, 51^3: 2.00 against 1.68 ms; k = 5, 40^3: 1.66 against 1.30 ms; measured): fewer warps fit
-// an SM.  Faces per CTA by degree, for the shared memory of larger faces.
+// The task kernel serves the FP32 affine face terms at k = 3 (at k = 4 and 5 too few warps fit an SM: it was
+// slower than the warp-per-face kernel there, measured).
 template <int N, int QC, int QV>
 constexpr bool task_faces_ok() {
-  return N == 4;
-}
-
-template <int N>
-constexpr int task_faces_per_cta() {
-  return N == 4 ? 12 : (N == 5 ? 8 : 6);
+  return N == 4 && coll_rule(N, QV);
 }
 
 template <int N, int QC, int QV>
 int launch_task_faces(const KParams& kp, void* FB, cudaStream_t st) {
-  constexpr int FPB = task_faces_per_cta<N>(), NTH = 128;
+  constexpr int FPB = 12, NTH = 128;
   constexpr size_t smem = task_face_smem_bytes<N, QC, QV, FPB>();
   static_assert(smem <= 227 * 1024, "task face kernel shared memory");
-  int extra_items = 0;
-  for (int d = 0; d < 3; ++d) {
-    if (kp.periodic[d]) continue;
-    const int plane = kp.nc[d == 0 ? 1 : 0] * kp.nc[d == 2 ? 1 : 2];
-    if (plane > extra_items) extra_items = plane;
-  }
   auto k = dg_face_task_kernel<N, QC, QV, FPB, NTH>;
   static bool attr[kMaxDevices] = {};
   if (smem_attr_once(k, smem, attr)) return -1;
-  const dim3 grid((kp.Nc + FPB - 1) / FPB + (extra_items + FPB - 1) / FPB, 3);
-  k<<<grid, NTH, smem, st>>>(kp, static_cast<float*>(FB));
+  k<<<dim3(face_blocks(kp, FPB), 3), NTH, smem, st>>>(kp, static_cast<float*>(FB));
   return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 

@@ -24,39 +24,50 @@
 
 namespace dgcns {
 
-// The line's values as integers: value i = F[i] 2^(E - 1083), |F[i]| < 2^61, E the largest biased exponent.
-// Returns false when the line needs the FP64 path: infinities and NaN, values whose result could leave the
-// normal range, and denormal values.  A line of zeros is F = 0 with E in range.
-template <int D>
-__host__ __device__ __forceinline__ bool fx_load(const double (&x)[D], int64_t (&F)[D], int& E) {
+// The line's values as integers: value i = F[i] 2^(E - 1075 - SH), |F[i]| < 2^61, E the largest biased exponent.
+// NA > 1: the element-wise sum of NA lines (SH leaves room for four).  Returns false when the line needs the
+// FP64 path: infinities and NaN, values whose result could leave the normal range, and denormal values.  A line
+// of zeros is F = 0 with E in range.
+template <int NA>
+constexpr int fx_shift() {
+  static_assert(NA <= 4, "room for four inputs");
+  return NA == 1 ? 8 : 6;
+}
+template <int NA, int D>
+__host__ __device__ __forceinline__ bool fx_load(const double (&x)[NA][D], int64_t (&F)[D], int& E) {
   uint32_t m = 0, any = 0;
-  uint32_t hi[D], lo[D];
+  uint32_t hi[NA][D], lo[NA][D];
 #pragma unroll
-  for (int i = 0; i < D; ++i) {
-    uint64_t b;
+  for (int k = 0; k < NA; ++k)
+#pragma unroll
+    for (int i = 0; i < D; ++i) {
+      uint64_t b;
 #ifdef __CUDA_ARCH__
-    b = (uint64_t)__double_as_longlong(x[i]);
+      b = (uint64_t)__double_as_longlong(x[k][i]);
 #else
-    __builtin_memcpy(&b, &x[i], 8);
+      __builtin_memcpy(&b, &x[k][i], 8);
 #endif
-    hi[i] = (uint32_t)(b >> 32);
-    lo[i] = (uint32_t)b;
-    const uint32_t a = hi[i] & 0x7fffffffu;
-    m = a > m ? a : m;
-    any |= lo[i];
-  }
+      hi[k][i] = (uint32_t)(b >> 32);
+      lo[k][i] = (uint32_t)b;
+      const uint32_t a = hi[k][i] & 0x7fffffffu;
+      m = a > m ? a : m;
+      any |= lo[k][i];
+    }
   E = (int)(m >> 20);
   if (m == 0 && any == 0) E = 1023;
   if ((uint32_t)(E - 200) > 1600u) return false;
 #pragma unroll
-  for (int i = 0; i < D; ++i) {
-    // (an input of exponent 0, zero or far below the line's range, is shifted out entirely)
-    int s = E - (int)((hi[i] >> 20) & 0x7ffu);
-    s = s < 63 ? s : 63;
-    const uint32_t mh = (hi[i] & 0xfffffu) | 0x100000u;
-    const uint64_t v = ((((uint64_t)mh << 32) | lo[i]) << 8) >> s;
-    F[i] = (int32_t)hi[i] < 0 ? -(int64_t)v : (int64_t)v;
-  }
+  for (int k = 0; k < NA; ++k)
+#pragma unroll
+    for (int i = 0; i < D; ++i) {
+      // (an input of exponent 0, zero or far below the line's range, is shifted out entirely)
+      int s = E - (int)((hi[k][i] >> 20) & 0x7ffu);
+      s = s < 63 ? s : 63;
+      const uint32_t mh = (hi[k][i] & 0xfffffu) | 0x100000u;
+      const uint64_t v = ((((uint64_t)mh << 32) | lo[k][i]) << fx_shift<NA>()) >> s;
+      const int64_t w = (int32_t)hi[k][i] < 0 ? -(int64_t)v : (int64_t)v;
+      F[i] = k == 0 ? w : F[i] + w;
+    }
   return true;
 }
 
@@ -118,12 +129,13 @@ struct FxAcc {
 // with (row sum) 2^t <= 2^61.  |sum and difference| of two inputs < 2^62, so the high products add up to
 // less than 2^60; the cross products are folded into them after every two terms (2 (2^61 + 2^60) and the
 // middle column's share stay below 2^63).
-template <int DIN, int DOUT, int SYM>
-__host__ __device__ __forceinline__ bool fx_line(const int2* __restrict__ f, const double (&x)[DIN], double (&y)[DOUT]) {
+template <int NA, int DIN, int DOUT, int SYM>
+__host__ __device__ __forceinline__ bool fx_line(const int2* __restrict__ f, const double (&x)[NA][DIN],
+                                                 double (&y)[DOUT]) {
   constexpr int IH = DIN / 2, OH = (DOUT + 1) / 2;
   int64_t F[DIN];
   int E;
-  if (!fx_load<DIN>(x, F, E)) return false;
+  if (!fx_load<NA, DIN>(x, F, E)) return false;
   int32_t eh[IH > 0 ? IH : 1], el[IH > 0 ? IH : 1], oh[IH > 0 ? IH : 1], ol[IH > 0 ? IH : 1], mh = 0, ml = 0;
 #pragma unroll
   for (int i = 0; i < IH; ++i) {
@@ -131,7 +143,7 @@ __host__ __device__ __forceinline__ bool fx_line(const int2* __restrict__ f, con
     fx_split(F[i] - F[DIN - 1 - i], oh[i], ol[i]);
   }
   if (DIN & 1) fx_split(F[IH], mh, ml);
-  const int X = E + 67 - f[0].x;
+  const int X = E + 75 - fx_shift<NA>() - f[0].x;
   const int2* __restrict__ A = f + 1;
   const int2* __restrict__ B = A + OH * IH;
   const int2* __restrict__ C = B + OH * IH;
@@ -160,6 +172,38 @@ __host__ __device__ __forceinline__ bool fx_line(const int2* __restrict__ f, con
     }
   }
   return true;
+}
+
+// ---------------------------------------------------------------------------
+// float <-> double on the integer units, bit for bit the hardware conversions (which run on the FP64 pipe, two
+// a cycle and SM).  For kernels that do little else: in the operator kernels, where the FP64 pipe has room, the
+// extra instructions cost more than the conversions (the k = 3 cell kernel 2.14 -> 2.36 ms, measured).
+// ---------------------------------------------------------------------------
+__device__ __forceinline__ double f64_of(double x) { return x; }
+__device__ __forceinline__ double f64_of(float x) {
+  const uint32_t b = __float_as_uint(x), a = b & 0x7fffffffu;
+  if (a - 0x00800000u < 0x7f000000u)  // normal: rebias the exponent by 1023 - 127
+    return __hiloint2double((int)((b & 0x80000000u) | ((a >> 3) + 0x38000000u)), (int)(b << 29));
+  if (a == 0) return __hiloint2double((int)b, 0);
+  return (double)x;
+}
+template <typename T>
+__device__ __forceinline__ T f32_of(double x);
+template <>
+__device__ __forceinline__ double f32_of<double>(double x) {
+  return x;
+}
+template <>
+__device__ __forceinline__ float f32_of<float>(double x) {
+  const uint32_t h = (uint32_t)__double2hiint(x), l = (uint32_t)__double2loint(x), a = h & 0x7fffffffu;
+  if (a - 0x38100000u < 0x0fd00000u) {  // the result is normal and cannot overflow
+    // exponent and 23 mantissa bits, then round to nearest even on the 29 bits below
+    const uint32_t t = ((a - 0x38000000u) << 3) | (l >> 29);
+    const uint64_t r = (uint64_t)(l << 3) + 0x7fffffffu + (t & 1u);
+    return __uint_as_float((h & 0x80000000u) | (t + (uint32_t)(r >> 32)));
+  }
+  if ((a | l) == 0) return __uint_as_float(h);
+  return (float)x;
 }
 
 }  // namespace dgcns

@@ -85,6 +85,7 @@ using Eo = typename EoOf<T>::type;
 template <typename T>
 struct Tab {
   Eo<T> eSc, eScT, eDc, eDcT, eSv, eSvT, eDv, eDvT, eSmi, eSmiT, eSm, eDm;
+  Eo<T> eDcW, eDvW, ePc, eLift;  // collocation form (dg_coll.cuh)
   const T *wc, *wv, *wm, *dl0, *dl1;
 };
 
@@ -112,26 +113,32 @@ int upload_const_tables(const double* t64, const float* t32, cudaStream_t st) {
 }
 }  // namespace
 
-// 8- or 4-byte elements of the tables a kernel of type T keeps in shared memory.
+// Elements of the tables that a kernel of type T keeps in shared memory: FP64 everything; FP32 the point weights
+// and trace derivatives only, the operators are read from constant memory (6 % faster than from shared memory,
+// measured; copying the unused operators as well cost the short FP32 kernels 3 to 9 %).
 template <typename T, int N, int QC, int QV>
 constexpr int table_elems() {
-  return sizeof(T) == 8 ? make_layout(N, QC, QV).total64 : make_layout(N, QC, QV).total;
+  constexpr TableLayout L = make_layout(N, QC, QV);
+  return sizeof(T) == 8 ? L.total64 : (L.dl1 + N - L.wc + 3) & ~3;
 }
 
 template <typename T, int N, int QC, int QV>
 __device__ __forceinline__ Tab<T> load_tables(const T* __restrict__ g, T* s) {
   constexpr TableLayout L = make_layout(N, QC, QV);
-  for (int i = threadIdx.x; i < table_elems<T, N, QC, QV>(); i += blockDim.x) s[i] = g[i];
+  constexpr int first = sizeof(T) == 8 ? 0 : L.wc, count = sizeof(T) == 8 ? L.total64 : L.dl1 + N - L.wc;
+  for (int i = threadIdx.x; i < count; i += blockDim.x) s[i] = g[first + i];
   Tab<T> t;
   auto op = [&](int k) -> Eo<T> {
     if constexpr (sizeof(T) == 8)
       return EoFp64{s + L.eo[k], reinterpret_cast<const int2*>(s + L.fx[k])};
-    else  // FP32: operators from constant memory (6 % faster than from shared memory, measured)
+    else
       return c_tab<T, N, QC, QV> + L.eo[k];
   };
   t.eSc = op(EO_SC); t.eScT = op(EO_SCT); t.eDc = op(EO_DC); t.eDcT = op(EO_DCT);
   t.eSv = op(EO_SV); t.eSvT = op(EO_SVT); t.eDv = op(EO_DV); t.eDvT = op(EO_DVT);
   t.eSmi = op(EO_SMI); t.eSmiT = op(EO_SMIT); t.eSm = op(EO_SM); t.eDm = op(EO_DM);
+  t.eDcW = op(EO_DCW); t.eDvW = op(EO_DVW); t.ePc = op(EO_PC); t.eLift = op(EO_LIFT);
+  s -= first;
   t.wc = s + L.wc; t.wv = s + L.wv; t.wm = s + L.wm; t.dl0 = s + L.dl0; t.dl1 = s + L.dl1;
   return t;
 }
@@ -208,24 +215,37 @@ __device__ __forceinline__ void eo_apply(const T* __restrict__ E, const T (&x)[D
 }
 
 // The same line in the kernel's precision: FP64 in integer arithmetic (dg_fixed.cuh) unless the line holds
-// values outside its range, FP32 as it is.
+// values outside its range, FP32 as it is.  The input is the sum of NA lines.
+template <typename T, int NA, int DIN, int DOUT, int SYM>
+__device__ __forceinline__ void line_apply_sum(Eo<T> E, const T (&x)[NA][DIN], T (&y)[DOUT]) {
+  if constexpr (sizeof(T) == 8) {
+    if (fx_line<NA, DIN, DOUT, SYM>(E.f, x, y)) return;
+  }
+  T s[DIN];
+#pragma unroll
+  for (int i = 0; i < DIN; ++i) {
+    s[i] = x[NA - 1][i];
+#pragma unroll
+    for (int k = NA - 2; k >= 0; --k) s[i] += x[k][i];
+  }
+  if constexpr (sizeof(T) == 8)
+    eo_apply<T, DIN, DOUT, SYM>(E.p, s, y);
+  else
+    eo_apply<T, DIN, DOUT, SYM>(E, s, y);
+}
 template <typename T, int DIN, int DOUT, int SYM>
 __device__ __forceinline__ void line_apply(Eo<T> E, const T (&x)[DIN], T (&y)[DOUT]) {
-  if constexpr (sizeof(T) == 8) {
-    if (!fx_line<DIN, DOUT, SYM>(E.f, x, y)) eo_apply<T, DIN, DOUT, SYM>(E.p, x, y);
-  } else {
-    eo_apply<T, DIN, DOUT, SYM>(E, x, y);
-  }
+  line_apply_sum<T, 1, DIN, DOUT, SYM>(E, reinterpret_cast<const T(&)[1][DIN]>(x), y);
 }
 
 // The FP64 sweep over `nlines` lines of contiguous arrays, as one function per (DIN, DOUT, SYM, ACC) and not
 // inlined: an integer line is 200 to 400 instructions, and the three axes of a sweep, the two sides of a face and
 // all the kernels of a translation unit share it (inlined, the k = 3 operator kernels were 3 times as long and a
 // cell's phases did not fit the instruction cache).  n0: the number of values below the swept axis, i.e. the
-// stride of a line; line l = (outer, inner) starts at outer n0 DIN + inner.
+// stride of a line; line l = (outer, inner) starts at outer n0 DIN + inner; magic = ceil(2^32 / n0) divides by n0.
 template <int DIN, int DOUT, int SYM, bool ACC>
-__device__ __noinline__ void fx_sweep(const double* in, double* out, EoFp64 E, int nlines, int n0, int rank, int stride) {
-  const uint32_t magic = n0 > 1 ? (uint32_t)((0x100000000ull + n0 - 1) / n0) : 0u;  // l / n0 for l n0 < 2^32
+__device__ __noinline__ void fx_sweep(const double* in, double* out, EoFp64 E, int nlines, int n0, uint32_t magic,
+                                      int rank, int stride) {
 #pragma unroll 1
   for (int l = rank; l < nlines; l += stride) {
     const int outer = n0 > 1 ? (int)__umulhi((uint32_t)l, magic) : l;
@@ -282,7 +302,8 @@ __device__ __forceinline__ void sweep(const T* __restrict__ in, T* __restrict__ 
   constexpr int NL = ISZ / DIN;
   if constexpr (sizeof(T) == 8) {
     constexpr int n0 = AX == 0 ? 1 : (AX == 1 ? D0 : D0 * D1);
-    fx_sweep<DIN, DOUT, SYM, ACC>(in, out, E, nblk * NL, n0, grp.rank(), grp.size());
+    constexpr uint32_t magic = n0 > 1 ? (uint32_t)((0x100000000ull + n0 - 1) / n0) : 0u;
+    fx_sweep<DIN, DOUT, SYM, ACC>(in, out, E, nblk * NL, n0, magic, grp.rank(), grp.size());
     return;
   }
   constexpr int IST = AX == 0 ? 1 : (AX == 1 ? D0 : D0 * D1);
@@ -444,6 +465,14 @@ __device__ __forceinline__ void wall_ghost(const T um[5], const PhysT<T>& ph, T 
   up[2] = -um[2];
   up[3] = -um[3];
   up[4] = ph.cvTw2 * um[0] - um[4] + ke2;
+}
+
+// Component c of U as a deviation from the reference state, in the arithmetic type.  The momenta have no
+// reference: no FP64 subtraction for them.
+template <typename T>
+__device__ __forceinline__ T dev_value(const KParams& kp, double u, int c) {
+  if (c == 0 || c == 4) u -= c == 0 ? kp.rho_ref : kp.rhoE_ref;
+  return T(u);
 }
 
 // ---------------------------------------------------------------------------
@@ -1287,7 +1316,7 @@ __device__ __forceinline__ void stage_update(const KParams& kp, const double* U,
     double u;
     T d;
   };
-  const T A = T(kp.A), dt = T(kp.dt);
+  const T A = stage_A<T>(kp), dt = stage_dt<T>(kp);
   const double B = kp.B;
   const bool readD = kp.A != 0.0;
   T* dev = static_cast<T*>(kp.devOut);
@@ -1299,8 +1328,7 @@ __device__ __forceinline__ void stage_update(const KParams& kp, const double* U,
                       const double uo = v.u + B * double(du);
                       Uout[base + i] = uo;
                       if (dev) {
-                        const int c = (i / N3) % 5;
-                        dev[base + i] = T(uo - (c == 0 ? kp.rho_ref : (c == 4 ? kp.rhoE_ref : 0.0)));
+                        dev[base + i] = dev_value<T>(kp, uo, (i / N3) % 5);
                       }
                     });
 }

@@ -6,7 +6,7 @@
 #include "dg_adjoint.cuh"
 #include "dg_adjoint_faces.cuh"
 #include "dg_faces.cuh"
-#include "dg_cell_fp32.cuh"
+#include "dg_coll.cuh"
 #include "dg_faces_fp32.cuh"
 #include "dg_kernels.cuh"
 #include "dg_mass.cuh"
@@ -26,17 +26,6 @@ namespace dgcns {
 #ifndef DGCNS_FP64_FACE_THREADS
 #define DGCNS_FP64_FACE_THREADS 256
 #endif
-// FP32 affine face terms at k = 3 by the register-resident task kernel (dg_faces_fp32.cuh); 0 keeps the
-// warp-per-face kernel (for comparison)
-#ifndef DGCNS_FP32_TASK_FACES
-#define DGCNS_FP32_TASK_FACES 1
-#endif
-// FP32 affine face-centric cell + mass stage at k = 3 by the register-resident task kernel
-// (dg_cell_fp32.cuh); 0 keeps the warp-per-cell kernel (for comparison)
-#ifndef DGCNS_FP32_TASK_CELL
-#define DGCNS_FP32_TASK_CELL 1
-#endif
-
 // Cells per CTA: the largest batch (<= 4 for FP32, <= DGCNS_FP64_CELL_CAP for FP64) whose shared
 // memory stays below ~112 KB, so that two or more CTAs fit on one SM (228 KB).
 template <typename T, int N, int QC, int QV, bool FACE = false>
@@ -60,12 +49,34 @@ constexpr int op_threads() {
   return sizeof(T) == 4 ? 256 : 128;
 }
 
-// Deviation state U - U_ref in the arithmetic type (elementwise pre-pass of the mixed form).
-template <typename T>
-__global__ void dg_dev_kernel(const KParams kp, const double* __restrict__ U, T* __restrict__ D, size_t n, int N3) {
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
-    const int c = (int)((i / N3) % 5);
-    D[i] = T(U[i] - (c == 0 ? kp.rho_ref : (c == 4 ? kp.rhoE_ref : 0.0)));
+// Deviation state U - U_ref in FP32 (elementwise pre-pass of the mixed form): 12 bytes a value, so it should run
+// at the memory's rate (conversions by integer operations: 0.34 -> 0.21 ms at 64^3, k = 3).  A CTA converts tiles of kDevCells consecutive cells, four values per thread and
+// access (a tile is a multiple of 16 bytes in both types for every N); the component comes from 32-bit
+// arithmetic within the tile.
+constexpr int kDevCells = 4;  // (16 left half the chip idle at 8^3)
+__device__ __forceinline__ float dev_int(const KParams& kp, double u, int c) {
+  if (c == 0 || c == 4) u -= c == 0 ? kp.rho_ref : kp.rhoE_ref;
+  return f32_of<float>(u);
+}
+template <int N, bool VEC>
+__global__ void __launch_bounds__(256) dg_dev_kernel(const KParams kp, const double* __restrict__ U,
+                                                     float* __restrict__ D) {
+  constexpr int N3 = N * N * N, W = VEC ? 4 : 1;
+  for (int t = blockIdx.x; t * kDevCells < kp.Nc; t += gridDim.x) {
+    const size_t base = (size_t)t * kDevCells * 5 * N3;
+    const int nv = min(kDevCells, kp.Nc - t * kDevCells) * 5 * N3;
+#pragma unroll 2
+    for (int i = threadIdx.x * W; i < nv; i += 256 * W) {
+      if (VEC && i + 3 < nv) {
+        const double2 a = *reinterpret_cast<const double2*>(U + base + i);
+        const double2 b = *reinterpret_cast<const double2*>(U + base + i + 2);
+        *reinterpret_cast<float4*>(D + base + i) =
+            make_float4(dev_int(kp, a.x, (i / N3) % 5), dev_int(kp, a.y, ((i + 1) / N3) % 5),
+                        dev_int(kp, b.x, ((i + 2) / N3) % 5), dev_int(kp, b.y, ((i + 3) / N3) % 5));
+      } else {
+        for (int q = i; q < min(i + W, nv); ++q) D[base + q] = dev_value<float>(kp, U[base + q], (q / N3) % 5);
+      }
+    }
   }
 }
 
@@ -112,11 +123,6 @@ constexpr bool op_gws() {
   return op_smem_bytes<T, N, QC, QV, CB, CELL, FACE, MASS, GEO>() > 227 * 1024;
 }
 
-// component c of the reference state U_ref = (rho_r, 0, 0, 0, rho_r c_v T_0)
-__device__ __forceinline__ double ref_of(const KParams& kp, int c) {
-  return c == 0 ? kp.rho_ref : (c == 4 ? kp.rhoE_ref : 0.0);
-}
-
 // ---------------------------------------------------------------------------
 // Generic operator kernel.  CELL: cell integrals; FACE: the 6 face integrals of
 // every cell; MASS: L = M^{-1}(-R + F_rhs).  Without CELL the partial residual
@@ -161,7 +167,7 @@ __global__ void __launch_bounds__(op_threads<T>()) dg_op_kernel(const KParams kp
                         [&](int i, T v) { su[i] = v; });
     else
       batched_pass<PER>(threadIdx.x, blockDim.x, nvals, [&](int i) { return U[base + i]; },
-                        [&](int i, double v) { su[i] = T(v - ref_of(kp, (i / N3) % 5)); });
+                        [&](int i, double v) { su[i] = dev_value<T>(kp, v, (i / N3) % 5); });
   }
   if (CELL) {
     for (int i = threadIdx.x; i < nvals; i += blockDim.x) sr[i] = T(0);
@@ -226,7 +232,7 @@ __global__ void __launch_bounds__(op_threads<T>()) dg_op_kernel(const KParams kp
               r = cq * N3 + frame_node<N>(kp.fnbr[((size_t)(e0 + e) * 6 + 2 * d + s) * 2 + 1], r - cq * N3);
             }
             const size_t src = (size_t)nbi[e] * 5 * N3 + r;
-            sn[i] = Ud ? Ud[src] : T(U[src] - ref_of(kp, (i / N3) % 5));
+            sn[i] = Ud ? Ud[src] : dev_value<T>(kp, U[src], (i / N3) % 5);
           }
         }
         if (GEO == GEO_FLY) {
@@ -829,7 +835,7 @@ __global__ void __launch_bounds__(WPC * 32) dg_op_warp_kernel(const KParams kp, 
       batched_pass<PER>(grp.rank(), 32, nvals, [&](int i) { return Ud[base + i]; }, [&](int i, T v) { su[i] = v; });
     else
       batched_pass<PER>(grp.rank(), 32, nvals, [&](int i) { return U[base + i]; },
-                        [&](int i, double v) { su[i] = T(v - ref_of(kp, (i / N3) % 5)); });
+                        [&](int i, double v) { su[i] = dev_value<T>(kp, v, (i / N3) % 5); });
   }
   if (CELL) {
     for (int i = grp.rank(); i < nvals; i += 32) sr[i] = T(0);
@@ -883,7 +889,7 @@ __global__ void __launch_bounds__(WPC * 32) dg_op_warp_kernel(const KParams kp, 
           for (int i = grp.rank(); i < nvals; i += 32) {
             const int cq = i / N3;
             const int r = kp.fnbr ? cq * N3 + frame_node<N>(code, i - cq * N3) : i;
-            sn[i] = Ud ? Ud[nb0 + r] : T(U[nb0 + r] - ref_of(kp, cq % 5));
+            sn[i] = Ud ? Ud[nb0 + r] : dev_value<T>(kp, U[nb0 + r], cq % 5);
           }
           if (GEO == GEO_FLY) {
             const T* Xn = static_cast<const T*>(kp.xyzT) + (size_t)nbi[0] * 3 * N3;
@@ -941,6 +947,13 @@ int launch_op_any(const KParams& kp, const double* U, const void* Rin, void* Rou
   }
 }
 
+// The face-centric organisation runs the collocation kernels wherever they exist.  Face and cell kernel share the
+// face buffer's basis, so both follow this rule.
+template <typename T, int N, int QC, int QV, int GEO>
+constexpr bool use_coll() {
+  return coll_ok<T, N, QC, QV, GEO>();
+}
+
 template <typename T, int N, int QC, int QV, int GEO>
 int op_dispatch_geo(int mode, const KParams& kp, const double* U, const void* Rin, void* Rout, void* dU,
                     double* Uout, cudaStream_t st) {
@@ -948,6 +961,10 @@ int op_dispatch_geo(int mode, const KParams& kp, const double* U, const void* Ri
   // (only while a warp's slice stays small: at k = 5 a cell needs ~49 KB, which would leave 4 warps per SM)
   constexpr bool WARP =
       sizeof(T) == 4 && warp_slice_elems<T, N, QC, QV, true, true, true, GEO>() * sizeof(T) <= 20 * 1024;
+  if constexpr (use_coll<T, N, QC, QV, GEO>()) {
+    if ((mode == OP_CELL || mode == (OP_CELL | OP_MASS)) && kp.fbuf != nullptr)
+      return launch_coll_cell<T, N, QC, QV, GEO>(kp, U, Rout, dU, Uout, st);
+  }
   switch (mode) {
     case OP_CELL: return launch_op_any<T, N, QC, QV, GEO, WARP, true, false, false>(kp, U, Rin, Rout, dU, Uout, st);
     case OP_FACE: return launch_op_any<T, N, QC, QV, GEO, WARP, false, true, false>(kp, U, Rin, Rout, dU, Uout, st);
@@ -972,11 +989,7 @@ int op_dispatch_geo(int mode, const KParams& kp, const double* U, const void* Ri
     case OP_CELL | OP_FACE:
       return launch_op_any<T, N, QC, QV, GEO, WARP, true, true, false>(kp, U, Rin, Rout, dU, Uout, st);
     case OP_CELL | OP_MASS:
-      if constexpr (sizeof(T) == 4 && GEO == GEO_AFFINE && DGCNS_FP32_TASK_CELL && task_cell_ok<N, QC, QV>()) {
-        if (kp.fbuf != nullptr && kp.Udev != nullptr && !kp.has_bf && (kp.out_mode == 1 || kp.out_mode == 2))
-          return launch_task_cell<N, QC, QV>(kp, U, Rout, dU, Uout, st);
-      }
-      if constexpr (Feat<N, QC, QV>::faces)
+      if constexpr (Feat<N, QC, QV>::faces && !use_coll<T, N, QC, QV, GEO>())
         return launch_op_any<T, N, QC, QV, GEO, WARP, true, false, true>(kp, U, Rin, Rout, dU, Uout, st);
       return -2;
     case OP_CELL | OP_FACE | OP_MASS:
@@ -1033,10 +1046,13 @@ int diag_launch(const KParams& kp, const double* U, const void* LU, double* part
   }
 }
 
-template <typename T, int N>
+template <int N>
 int dev_launch(const KParams& kp, const double* U, void* D, cudaStream_t st) {
-  const size_t n = (size_t)kp.Nc * 5 * N * N * N;
-  dg_dev_kernel<T><<<2 * 152 * 8, 256, 0, st>>>(kp, U, static_cast<T*>(D), n, N * N * N);
+  const int tiles = (kp.Nc + kDevCells - 1) / kDevCells, grid = tiles < 152 * 16 ? tiles : 152 * 16;
+  if (((reinterpret_cast<uintptr_t>(U) | reinterpret_cast<uintptr_t>(D)) & 15) == 0)
+    dg_dev_kernel<N, true><<<grid, 256, 0, st>>>(kp, U, static_cast<float*>(D));
+  else
+    dg_dev_kernel<N, false><<<grid, 256, 0, st>>>(kp, U, static_cast<float*>(D));
   return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 
@@ -1103,65 +1119,10 @@ __global__ void __launch_bounds__(face_threads<T, GEO>()) dg_face_kernel(const K
   int* oc = en + CB;  // rotated-frame meshes: orientation code of the other cell
 
   const int d = blockIdx.y;
-  const int t1 = d == 0 ? 1 : 0, t2 = d == 2 ? 1 : 2;
-  int s, i0, nitems;
-  if (kp.flist) {  // rotated-frame meshes: the faces owned through local face (d, 1), then (d, 0)
-    const int nb1 = (kp.flen[2 * d + 1] + CB - 1) / CB;
-    s = (int)blockIdx.x < nb1 ? 1 : 0;
-    i0 = (s ? (int)blockIdx.x : (int)blockIdx.x - nb1) * CB;
-    nitems = kp.flen[2 * d + s];
-    if (i0 >= nitems) return;
-  } else {
-    const int nstd = (kp.Nc + CB - 1) / CB;
-    if ((int)blockIdx.x < nstd) {
-      s = 1;
-      i0 = blockIdx.x * CB;
-      nitems = kp.Nc;
-    } else {
-      if (kp.periodic[d]) return;
-      s = 0;
-      i0 = (blockIdx.x - nstd) * CB;
-      nitems = kp.nc[t1] * kp.nc[t2];
-      if (i0 >= nitems) return;
-    }
-  }
-  const int nb = min(CB, nitems - i0);
+  int s, nb;
+  if (!face_batch<CB>(kp, d, s, nb, eo, en, oc, tau_f)) return;
   const Tab<T> tb = load_tables<T, N, QC, QV>(static_cast<const T*>(kp.tables), stab);
   const PhysT<T> ph = make_phys<T>(kp);
-  if ((int)threadIdx.x < nb && kp.flist) {
-    const int e = kp.flist[kp.foff[2 * d + s] + i0 + threadIdx.x];
-    const int* t = kp.fnbr + ((size_t)e * 6 + 2 * d + s) * 2;
-    eo[threadIdx.x] = e;
-    en[threadIdx.x] = t[0];
-    oc[threadIdx.x] = t[1];
-    tau_f[threadIdx.x] = T(fmax(kp.tau[e], kp.tau[t[0]]));
-  } else if ((int)threadIdx.x < nb) {
-    const int i = i0 + threadIdx.x;
-    int c[3];
-    if (s == 1) {
-      c[0] = i % kp.nc[0];
-      c[1] = (i / kp.nc[0]) % kp.nc[1];
-      c[2] = i / (kp.nc[0] * kp.nc[1]);
-    } else {
-      c[d] = 0;
-      c[t1] = i % kp.nc[t1];
-      c[t2] = i / kp.nc[t1];
-    }
-    const int e = c[0] + kp.nc[0] * (c[1] + kp.nc[1] * c[2]);
-    c[d] += s ? 1 : -1;
-    int w = 0;
-    if (c[d] < 0 || c[d] >= kp.nc[d]) {
-      if (kp.periodic[d])
-        c[d] = (c[d] + kp.nc[d]) % kp.nc[d];
-      else
-        w = 1;
-    }
-    const int n = w ? -1 : c[0] + kp.nc[0] * (c[1] + kp.nc[1] * c[2]);
-    eo[threadIdx.x] = e;
-    en[threadIdx.x] = n;
-    const double te = kp.tau[e];
-    tau_f[threadIdx.x] = T(w ? te : fmax(te, kp.tau[n]));
-  }
   __syncthreads();
   const T* Ud = static_cast<const T*>(kp.Udev);
   const int* ocp = kp.flist ? oc : nullptr;
@@ -1310,33 +1271,21 @@ __global__ void __launch_bounds__(WPC * 32) dg_face_warp_kernel(const KParams kp
 
 template <typename T, int N, int QC, int QV, int GEO>
 int launch_faces(const KParams& kp, const double* U, void* FB, cudaStream_t st) {
-  int extra_items = 0;
-  for (int d = 0; d < 3; ++d) {
-    if (kp.periodic[d]) continue;
-    const int plane = kp.nc[d == 0 ? 1 : 0] * kp.nc[d == 2 ? 1 : 2];
-    if (plane > extra_items) extra_items = plane;
-  }
-  if constexpr (sizeof(T) == 4 && GEO == GEO_AFFINE && DGCNS_FP32_TASK_FACES && task_faces_ok<N, QC, QV>()) {
-    if (kp.Udev != nullptr && kp.flist == nullptr) return launch_task_faces<N, QC, QV>(kp, FB, st);
-  }
-  // rotated-frame meshes: per direction, the blocks of the (d, 1) list, then those of the (d, 0) list
-  auto list_blocks = [&](int per) {
-    int g = 0;
-    for (int d = 0; d < 3; ++d) {
-      const int b = (kp.flen[2 * d + 1] + per - 1) / per + (kp.flen[2 * d] + per - 1) / per;
-      if (b > g) g = b;
+  if constexpr (use_coll<T, N, QC, QV, GEO>()) {
+    // FP32 affine at k = 3: the register-resident kernel (1.39 ms against 1.63 ms per launch at 64^3, measured)
+    if constexpr (sizeof(T) == 4 && GEO == GEO_AFFINE && task_faces_ok<N, QC, QV>()) {
+      if (kp.Udev != nullptr && kp.flist == nullptr && (reinterpret_cast<uintptr_t>(kp.Udev) & 15) == 0)
+        return launch_task_faces<N, QC, QV>(kp, FB, st);
     }
-    return g;
-  };
-  if constexpr (sizeof(T) == 4) {
+    return launch_coll_faces<T, N, QC, QV, GEO>(kp, U, FB, st);
+  } else if constexpr (sizeof(T) == 4) {
     constexpr int WPC = 8;
     constexpr size_t smem = face_warp_smem_bytes<T, N, QC, QV, WPC, GEO>();
     static_assert(smem <= 227 * 1024, "face kernel shared memory");
     auto k = dg_face_warp_kernel<T, N, QC, QV, WPC, GEO>;
     static bool attr[kMaxDevices] = {};
     if (smem_attr_once(k, smem, attr)) return -1;
-    const dim3 grid(kp.flist ? list_blocks(WPC) : (kp.Nc + WPC - 1) / WPC + (extra_items + WPC - 1) / WPC, 3);
-    k<<<grid, WPC * 32, smem, st>>>(kp, U, static_cast<T*>(FB));
+    k<<<dim3(face_blocks(kp, WPC), 3), WPC * 32, smem, st>>>(kp, U, static_cast<T*>(FB));
   } else {
     constexpr int CB = faces_per_cta<T, N, QC, QV, GEO>();
     constexpr size_t smem = face_smem_bytes<T, N, QC, QV, CB, GEO>();
@@ -1344,8 +1293,7 @@ int launch_faces(const KParams& kp, const double* U, void* FB, cudaStream_t st) 
     auto k = dg_face_kernel<T, N, QC, QV, CB, GEO>;
     static bool attr[kMaxDevices] = {};
     if (smem_attr_once(k, smem, attr)) return -1;
-    const dim3 grid(kp.flist ? list_blocks(CB) : (kp.Nc + CB - 1) / CB + (extra_items + CB - 1) / CB, 3);
-    k<<<grid, face_threads<T, GEO>(), smem, st>>>(kp, U, static_cast<T*>(FB));
+    k<<<dim3(face_blocks(kp, CB), 3), face_threads<T, GEO>(), smem, st>>>(kp, U, static_cast<T*>(FB));
   }
   return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
@@ -1381,7 +1329,7 @@ void fill_launchers(Launchers& L) {
     L.gws_fp64 = op_gws_bytes<double, N, QC, QV>();
   } else if constexpr (PART == 1) {  // FP32 operator (mixed form)
     L.op_fp32 = op_dispatch<float, N, QC, QV>;
-    L.dev_fp32 = dev_launch<float, N>;
+    L.dev_fp32 = dev_launch<N>;
     L.cb_fp32 = cells_per_cta<float, N, QC, QV>();
   } else if constexpr (PART == 2) {  // diagnostics, geometry, kinetic-energy gradient
     L.diag_fp64 = diag_launch<double, N, QC, QV>;

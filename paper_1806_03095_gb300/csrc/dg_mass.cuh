@@ -191,14 +191,14 @@ __global__ void __launch_bounds__(kMassThreads) dg_mass_tma_kernel(const KParams
                               kp.out_mode != 0);
     __syncthreads();
     if (STAGE) {
-      const T A = T(kp.A), dt = T(kp.dt);
+      const T A = stage_A<T>(kp), dt = stage_dt<T>(kp);
       const double B = kp.B;
       const T* dold = bufD + slot * BV;
       const double* uold = bufU + slot * BV;
       for (int i = threadIdx.x; i < nb * CV; i += blockDim.x) {
         const T du = (readD ? A * dold[i] : T(0)) + dt * sr[i];
         dU[base + i] = du;
-        Uout[base + i] = uold[i] + B * double(du);
+        Uout[base + i] = uold[i] + B * f64_of(du);
       }
     }
     __syncthreads();
@@ -356,7 +356,7 @@ __global__ void __launch_bounds__(kMassRegThreads) dg_mass_reg_kernel(const KPar
       dst[f] = reinterpret_cast<const float4*>(sb + (f / V4) * RS)[f % V4];
     return;
   }
-  const float A = float(kp.A), dt = float(kp.dt);
+  const float A = kp.A32, dt = kp.dt32;
   const double B = kp.B;
   const bool readD = kp.A != 0.0;
   float* dev = static_cast<float*>(kp.devOut);
@@ -382,17 +382,23 @@ __global__ void __launch_bounds__(kMassRegThreads) dg_mass_reg_kernel(const KPar
         d.w = A * v.d.w + dt * L.w;
         reinterpret_cast<float4*>(dU + base)[f] = d;
         double2 o0, o1;
-        o0.x = v.u0.x + B * double(d.x);
-        o0.y = v.u0.y + B * double(d.y);
-        o1.x = v.u1.x + B * double(d.z);
-        o1.y = v.u1.y + B * double(d.w);
+        o0.x = v.u0.x + B * f64_of(d.x);
+        o0.y = v.u0.y + B * f64_of(d.y);
+        o1.x = v.u1.x + B * f64_of(d.z);
+        o1.y = v.u1.y + B * f64_of(d.w);
         reinterpret_cast<double2*>(Uout + base)[2 * f] = o0;
         reinterpret_cast<double2*>(Uout + base)[2 * f + 1] = o1;
         if (dev != nullptr) {
           const int c = (int)(((b0 + f / V4)) % 5);
-          const double ref = c == 0 ? kp.rho_ref : (c == 4 ? kp.rhoE_ref : 0.0);
+          if (c == 0 || c == 4) {
+            const double ref = c == 0 ? kp.rho_ref : kp.rhoE_ref;
+            o0.x -= ref;
+            o0.y -= ref;
+            o1.x -= ref;
+            o1.y -= ref;
+          }
           reinterpret_cast<float4*>(dev + base)[f] =
-              make_float4(float(o0.x - ref), float(o0.y - ref), float(o1.x - ref), float(o1.y - ref));
+              make_float4(f32_of<float>(o0.x), f32_of<float>(o0.y), f32_of<float>(o1.x), f32_of<float>(o1.y));
         }
       });
 }

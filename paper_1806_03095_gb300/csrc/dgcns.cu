@@ -255,9 +255,41 @@ std::vector<double> build_tables(int k, int QC, int QV) {
     t[L.dl0 + i] = D[i];
     t[L.dl1 + i] = D[N + i];
   }
-  const int dims[EO_NOPS][2] = {{QC, N}, {N, QC}, {QC, QC}, {QC, QC}, {QV, N}, {N, QV},
-                                {QV, QV}, {QV, QV}, {N, N},   {N, N},   {N, N},  {N, N}};
-  for (int q = 0; q < EO_NOPS; ++q) put_fixed(t, L.eo[q], L.fx[q], dims[q][0], dims[q][1]);
+  if (coll_rule(N, QV)) {
+    // collocation form: test functions l_g on the mass points, divided by w_g
+    auto weighted = [](const std::vector<double>& D, const std::vector<double>& w) {  // W^-1 D^T W
+      const int n = (int)w.size();
+      std::vector<double> O((size_t)n * n);
+      for (int g = 0; g < n; ++g)
+        for (int q = 0; q < n; ++q) O[(size_t)g * n + q] = D[(size_t)q * n + g] * w[q] / w[g];
+      return O;
+    };
+    lagrange(xc, xc, Vg, Dg);
+    put_eo(t, L.eo[EO_DCW], weighted(Dg, wc), QC, QC);
+    lagrange(xm, xm, Vg, Dg);
+    const std::vector<double> DW = weighted(Dg, wm);
+    put_eo(t, L.eo[EO_DVW], DW, N, N);
+    lagrange(xm, xc, V, D);  // V[q][g] = l_g(x_q)
+    std::vector<double> P((size_t)N * QC);
+    for (int g = 0; g < N; ++g)
+      for (int q = 0; q < QC; ++q) P[(size_t)g * QC + q] = V[(size_t)q * N + g] * wc[q] / wm[g];
+    put_eo(t, L.eo[EO_PC], P, N, QC);
+    lagrange(xm, std::vector<double>{0.0, 1.0}, V, D);
+    std::vector<double> F((size_t)N * (N + 4));
+    for (int g = 0; g < N; ++g) {
+      double* r = &F[(size_t)g * (N + 4)];
+      r[0] = D[g] / wm[g];
+      r[1] = V[g] / wm[g];
+      for (int q = 0; q < N; ++q) r[2 + q] = DW[(size_t)g * N + q];
+      r[N + 2] = -V[N + g] / wm[g];
+      r[N + 3] = D[N + g] / wm[g];
+    }
+    put_eo(t, L.eo[EO_LIFT], F, N, N + 4);
+  }
+  for (int q = 0; q < EO_NOPS; ++q) {
+    const EoDims d = eo_dims(q, N, QC, QV);
+    if (d.dout > 0) put_fixed(t, L.eo[q], L.fx[q], d.dout, d.din);
+  }
   return t;
 }
 
@@ -1147,6 +1179,8 @@ static int stage_2n(dgcns_ctx* c, double A, double B, double dt, const double* U
   kp.A = A;
   kp.B = B;
   kp.dt = dt;
+  kp.A32 = (float)A;
+  kp.dt32 = (float)dt;
   return eval_L(c, kp, U_in, nullptr, dU, U_out);
 }
 
@@ -1195,6 +1229,8 @@ static int steps_2n(dgcns_ctx* c, int stages, const double* A, const double* B, 
         kp.A = A[s];
         kp.B = B[s];
         kp.dt = dt;
+        kp.A32 = (float)A[s];
+        kp.dt32 = (float)dt;
         kp.Udev = dcur;
         kp.devOut = dnxt;
         r = eval_L(c, kp, a, nullptr, dU, b);
