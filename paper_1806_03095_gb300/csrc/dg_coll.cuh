@@ -24,6 +24,7 @@
 // Bound by: FP64 faces the FP64 pipe (64 % busy, 6,450 instructions a face); FP64 cells latency and
 // instruction fetch (ALU 46 %, FP64 34 %, issue 43 %).
 #pragma once
+#include "dg_chain.cuh"
 #include "dg_faces.cuh"
 #include "dg_kernels.cuh"
 
@@ -57,91 +58,150 @@ __device__ __forceinline__ double sqrt_of(double a) {
 }
 
 // ---------------------------------------------------------------------------
-// Sweeps.  Lines of DIN values at stride n0 of contiguous arrays -> DOUT values; line l = (outer, inner)
-// with inner < n0 starts at outer n0 DIN + inner.  NIN: the input is the sum of NIN arrays ks apart (and of
-// `extra` when EX).  OG > 0: OG consecutive outers form a block, blocks IBS apart in the input.  OBS > 0:
-// outers are OBS apart in the output (an in-place sweep that keeps its block stride).
+// Sweeps.  nblk blocks of (D2, D1, D0) values (D0 fastest), the planes of D1 x D0 values IPS apart; the operator
+// acts along axis AX, the output's planes are OPS apart.  NIN: the input is the sum of NIN arrays ks apart (and
+// of `extra` when EX).  IBS > 0: blocks IBS apart in the input; OBS > 0: in the output (an in-place sweep that
+// keeps its block stride).
+//
+// FP32 planes whose rows are 8 values (k = 5: QC = 8) are padded so that the lines along y of 32 lanes (D0 neighbours, then the
+// next plane) fall on distinct banks, and lines along x are read as 16- or 8-byte vectors: with dense planes at k = 3, 43 % of the
+// cell kernel's shared-memory wavefronts were conflicts and that pipe was 82 % busy.  FP64 planes are dense (the
+// padding would cost a resident CTA; its kernels keep that pipe 30 % busy).
 // ---------------------------------------------------------------------------
-template <typename T, int DIN, int DOUT, int SYM, int NIN, bool EX, int OG, int IBS, int OBS>
-__device__ __forceinline__ void lines_body(const T* in, int ks, const T* extra, T* out, Eo<T> E, int nlines, int n0,
-                                           uint32_t magic, int rank, int stride) {
-  for (int l = rank; l < nlines; l += stride) {
-    int outer;
-    if constexpr (sizeof(T) == 8)
-      outer = n0 > 1 ? (int)__umulhi((uint32_t)l, magic) : l;
+template <typename T>
+constexpr int plane_stride(int d0, int d1) {
+  if (sizeof(T) == 8) return d0 * d1;
+  if (d0 % 8 != 0) return d0 * d1;
+  int best = d0 * d1, bestc = 99;
+  for (int s = d0 * d1; s <= d0 * d1 + 12; s += 4) {
+    int cnt[32] = {}, c = 0;
+    for (int l = 0; l < 32; ++l) {
+      const int k = (l % d0 + l / d0 * s) % 32;
+      if (++cnt[k] > c) c = cnt[k];
+    }
+    if (c < bestc) {
+      bestc = c;
+      best = s;
+    }
+  }
+  return best;
+}
+
+// K consecutive values with the widest aligned vectors the extent allows (arrays start on 16 bytes).
+template <typename T, int K, bool LD>
+__device__ __forceinline__ void line_io(T* p, T (&x)[K]) {
+  if constexpr ((K * sizeof(T)) % 16 == 0) {
+    if constexpr (LD)
+      vec_load<T, K>(p, x);
     else
-      outer = l / n0;
-    const int inner = l - outer * n0;
-    const int ib = (OG > 0 ? (outer / (OG > 0 ? OG : 1)) * IBS + (outer % (OG > 0 ? OG : 1)) * n0 * DIN : outer * n0 * DIN) + inner;
-    const int ob = (OBS > 0 ? outer * OBS : outer * n0 * DOUT) + inner;
-    const T* ip = in + ib;
-    T* op = out + ob;
-    T y[DOUT];
-    constexpr bool VIN = NIN == 1 && !EX && (DIN * sizeof(T)) % 16 == 0;
-    constexpr bool VOUT = (DOUT * sizeof(T)) % 16 == 0;
-    if constexpr (NIN + (EX ? 1 : 0) == 1) {
-      T x[DIN];
-      bool loaded = false;
-      if constexpr (VIN) {
-        // a line along x is contiguous: 16-byte accesses avoid the bank conflicts of threads reading
-        // DIN-value lines at a DIN-value stride
-        if (n0 == 1 && (reinterpret_cast<uintptr_t>(ip) & 15) == 0) {
-          vec_load<T, DIN>(ip, x);
-          loaded = true;
-        }
-      }
-      if (!loaded) {
+      vec_store<T, K>(p, x);
+  } else if constexpr (sizeof(T) == 4 && K % 2 == 0) {
 #pragma unroll
-        for (int i = 0; i < DIN; ++i) x[i] = ip[i * n0];
-      }
-      line_apply<T, DIN, DOUT, SYM>(E, x, y);
-    } else {
-      constexpr int NA = NIN + (EX ? 1 : 0);
-      T x[NA][DIN];
-#pragma unroll
-      for (int a = 0; a < NA; ++a) {
-        const T* p = EX && a == NIN ? extra + ib : ip + (size_t)a * ks;
-#pragma unroll
-        for (int i = 0; i < DIN; ++i) x[a][i] = p[i * n0];
-      }
-      line_apply_sum<T, NA, DIN, DOUT, SYM>(E, x, y);
-    }
-    if constexpr (VOUT) {
-      if (n0 == 1 && (reinterpret_cast<uintptr_t>(op) & 15) == 0) {
-        vec_store<T, DOUT>(op, y);
-        continue;
+    for (int i = 0; i < K; i += 2) {
+      if constexpr (LD) {
+        const float2 v = *reinterpret_cast<const float2*>(p + i);
+        x[i] = v.x;
+        x[i + 1] = v.y;
+      } else {
+        *reinterpret_cast<float2*>(p + i) = make_float2(x[i], x[i + 1]);
       }
     }
+  } else {
 #pragma unroll
-    for (int q = 0; q < DOUT; ++q) op[q * n0] = y[q];
+    for (int i = 0; i < K; ++i) {
+      if constexpr (LD)
+        x[i] = p[i];
+      else
+        p[i] = x[i];
+    }
   }
 }
-// FP64: one function per shape, not inlined (the code of an integer line is long; the axes share it)
+
+// FP64 line by line (what a chain cannot take, and stored geometry's last sweeps): line l = (outer, inner) with
+// inner < n0 starts at outer n0 DIN + inner.  One function per shape, not inlined (the code of an integer line is
+// long; the axes share it).  OG: OG consecutive outers form a block, blocks IBS apart.
 template <int DIN, int DOUT, int SYM, int NIN, bool EX, int OG, int IBS, int OBS>
 __device__ __noinline__ void lines_fp64(const double* in, int ks, const double* extra, double* out, EoFp64 E, int nlines,
                                         int n0, uint32_t magic) {
-  lines_body<double, DIN, DOUT, SYM, NIN, EX, OG, IBS, OBS>(in, ks, extra, out, E, nlines, n0, magic, threadIdx.x,
-                                                            blockDim.x);
-}
-template <typename T, int N0, int DIN, int DOUT, int SYM, int NIN = 1, bool EX = false, int OG = 0, int IBS = 0,
-          int OBS = 0>
-__device__ __forceinline__ void lines(const T* in, T* out, Eo<T> E, int nouter, int ks = 0, const T* extra = nullptr) {
-  constexpr uint32_t magic = N0 > 1 ? (uint32_t)((0x100000000ull + N0 - 1) / N0) : 0u;  // l / N0 for l N0 < 2^32
-  if constexpr (sizeof(T) == 8)
-    lines_fp64<DIN, DOUT, SYM, NIN, EX, OG, IBS, OBS>(in, ks, extra, out, E, nouter * N0, N0, magic);
-  else
-    lines_body<T, DIN, DOUT, SYM, NIN, EX, OG, IBS, OBS>(in, ks, extra, out, E, nouter * N0, N0, magic, threadIdx.x,
-                                                         blockDim.x);
+  DGCNS_SHARED(in);
+  DGCNS_SHARED(out);
+  DGCNS_SHARED(E.f);
+  DGCNS_SHARED(E.p);
+#pragma unroll 1
+  for (int l = threadIdx.x; l < nlines; l += blockDim.x) {
+    const int outer = n0 > 1 ? (int)__umulhi((uint32_t)l, magic) : l;
+    const int inner = l - outer * n0;
+    const int ib = (OG > 0 ? (outer / (OG > 0 ? OG : 1)) * IBS + (outer % (OG > 0 ? OG : 1)) * n0 * DIN : outer * n0 * DIN) + inner;
+    const int ob = (OBS > 0 ? outer * OBS : outer * n0 * DOUT) + inner;
+    constexpr int NA = NIN + (EX ? 1 : 0);
+    double x[NA][DIN], y[DOUT];
+#pragma unroll
+    for (int a = 0; a < NA; ++a) {
+      const double* p = EX && a == NIN ? extra + ib : in + ib + (size_t)a * ks;
+#pragma unroll
+      for (int i = 0; i < DIN; ++i) x[a][i] = p[i * n0];
+    }
+    line_apply_sum<double, NA, DIN, DOUT, SYM>(E, x, y);
+#pragma unroll
+    for (int q = 0; q < DOUT; ++q) out[ob + q * n0] = y[q];
+  }
 }
 
-// V_d <- D~_d V_d + the shares of the two faces of direction d, in place.  V: [nb][5][N^3]; F: the cells' face
+template <typename T, int AX, int D0, int D1, int D2, int DOUT, int SYM, int IPS = D0 * D1,
+          int OPS = (AX == 0 ? DOUT * D1 : (AX == 1 ? D0 * DOUT : D0 * D1)), int NIN = 1, bool EX = false, int IBS = 0,
+          int OBS = 0>
+__device__ __forceinline__ void sw(const T* in, T* out, Eo<T> E, int nblk, int ks = 0, const T* extra = nullptr) {
+  constexpr int DIN = AX == 0 ? D0 : (AX == 1 ? D1 : D2);
+  constexpr int n0 = AX == 0 ? 1 : (AX == 1 ? D0 : D0 * D1);  // values below the axis
+  constexpr int per = AX == 0 ? D1 * D2 : (AX == 1 ? D2 : 1);  // groups of n0 lines per block
+  if constexpr (sizeof(T) == 8) {
+    constexpr uint32_t magic = n0 > 1 ? (uint32_t)((0x100000000ull + n0 - 1) / n0) : 0u;  // l / n0 for l n0 < 2^32
+    lines_fp64<DIN, DOUT, SYM, NIN, EX, (IBS > 0 ? per : 0), IBS, OBS>(in, ks, extra, out, E, nblk * per * n0, n0, magic);
+  } else {
+    constexpr int NA = NIN + (EX ? 1 : 0);
+    constexpr int ist = AX == 0 ? 1 : (AX == 1 ? D0 : IPS), ost = AX == 0 ? 1 : (AX == 1 ? D0 : OPS);
+    // lines along x: row l of plane l / D1; along y: neighbour `inner` of plane g; along z: of block g
+    constexpr int igs = AX == 1 ? IPS : D2 * IPS, ogs = AX == 1 ? OPS : (OBS > 0 ? OBS : DOUT * OPS);
+    for (int l = threadIdx.x; l < nblk * per * n0; l += blockDim.x) {
+      const int g = l / n0, inner = l - g * n0;
+      int ib, ob;
+      if constexpr (AX == 0) {
+        ib = l * D0 + l / D1 * (IPS - D0 * D1);
+        ob = l * DOUT + l / D1 * (OPS - DOUT * D1);
+      } else {
+        ib = (IBS > 0 ? g / per * IBS + g % per * IPS : g * igs) + inner;
+        ob = g * ogs + inner;
+      }
+      T x[NA][DIN], y[DOUT];
+#pragma unroll
+      for (int a = 0; a < NA; ++a) {
+        const T* p = EX && a == NIN ? extra + ib : in + ib + (size_t)a * ks;
+        if constexpr (AX == 0) {
+          line_io<T, DIN, true>(const_cast<T*>(p), x[a]);
+        } else {
+#pragma unroll
+          for (int i = 0; i < DIN; ++i) x[a][i] = p[i * ist];
+        }
+      }
+      line_apply_sum<T, NA, DIN, DOUT, SYM>(E, x, y);
+      if constexpr (AX == 0) {
+        line_io<T, DOUT, false>(out + ob, y);
+      } else {
+#pragma unroll
+        for (int q = 0; q < DOUT; ++q) out[ob + q * ost] = y[q];
+      }
+    }
+  }
+}
+
+// V_d <- D~_d V_d + the shares of the two faces of direction d, in place.  V: [nb][5][N][N, N]; F: the cells' face
 // shares [nb][6][2][5][N^2] (global).  The line's operator takes D_0, L_0, the N values, -L_1, D_1: with the sign
 // of L_1 it is antisymmetric under reflection like D~ itself.
 template <typename T, int N, int D>
 __device__ __forceinline__ void lift_body(T* V, const T* __restrict__ F, Eo<T> E, int nb, bool vol) {
-  constexpr int N2 = N * N, N3 = N2 * N, st = D == 0 ? 1 : (D == 1 ? N : N2);
+  constexpr int N2 = N * N, PS = plane_stride<T>(N, N), st = D == 0 ? 1 : (D == 1 ? N : PS);
   for (int l = threadIdx.x; l < nb * 5 * N2; l += blockDim.x) {
-    const int ec = l / N2, j = l - ec * N2, e = ec / 5, c = ec - 5 * e;
+    const int ec = l / N2, j = l - ec * N2, e = ec / 5, c = ec - 5 * e, j1 = j % N, j2 = j / N;
     const T* f0 = F + (size_t)e * fbuf_per_cell<N>() + (2 * D * 2 * 5 + c) * N2 + j;
     const T* f1 = f0 + 2 * 5 * N2;
     T x[N + 4], y[N];
@@ -149,16 +209,29 @@ __device__ __forceinline__ void lift_body(T* V, const T* __restrict__ F, Eo<T> E
     x[1] = f0[0];
     x[N + 2] = -f1[0];
     x[N + 3] = f1[5 * N2];
-    T* v = V + ec * N3 + face_node<N>(D, 0, j % N, j / N);
+    T* v = V + ec * N * PS + (D == 0 ? j1 * N + j2 * PS : (D == 1 ? j1 + j2 * PS : j1 + N * j2));
+    if constexpr (D == 0) {
+      line_io<T, N, true>(v, y);
+    } else {
 #pragma unroll
-    for (int i = 0; i < N; ++i) x[2 + i] = vol ? v[i * st] : T(0);
+      for (int i = 0; i < N; ++i) y[i] = v[i * st];
+    }
+#pragma unroll
+    for (int i = 0; i < N; ++i) x[2 + i] = vol ? y[i] : T(0);
     line_apply<T, N + 4, N, -1>(E, x, y);
+    if constexpr (D == 0) {
+      line_io<T, N, false>(v, y);
+    } else {
 #pragma unroll
-    for (int i = 0; i < N; ++i) v[i * st] = y[i];
+      for (int i = 0; i < N; ++i) v[i * st] = y[i];
+    }
   }
 }
 template <int N>
 __device__ __noinline__ void lift_fp64(double* V, const double* F, EoFp64 E, int nb, bool vol, int n3) {
+  DGCNS_SHARED(V);
+  DGCNS_SHARED(E.f);
+  DGCNS_SHARED(E.p);
   // the three directions one after the other, V_d n3 values apart
   lift_body<double, N, 0>(V, F, E, nb, vol);
   lift_body<double, N, 1>(V + n3, F, E, nb, vol);
@@ -168,26 +241,27 @@ __device__ __noinline__ void lift_fp64(double* V, const double* F, EoFp64 E, int
 // ---------------------------------------------------------------------------
 // Point fluxes
 // ---------------------------------------------------------------------------
-// Convective flux through a face with unit normal n (any normal, or n = sgn e_D when AFF), LLF:
-// f = ({{F_c}} + lambda/2 [[U]]) . n.  Components in physical order.
+// Convective flux w F_c . n of one side of a face and its wave speed (LLF); n any unit normal, or e_D when AFF (w then
+// carries the sign).  Components in physical order.
 template <typename T, int D, bool AFF>
-__device__ __forceinline__ void llf_side(const T u[5], const T n[3], T sgn, const PhysT<T>& ph, T f[5], T& lam) {
+__device__ __forceinline__ void llf_side(const T u[5], const T n[3], T w, const PhysT<T>& ph, T f[5], T& lam) {
   const T rinv = rcp_of(ph.rho_r + u[0]);
   const T m2 = u[1] * u[1] + u[2] * u[2] + u[3] * u[3];
-  const T dp = ph.gm1 * (u[4] - T(0.5) * rinv * m2);
-  lam = sqrt_of(m2) * rinv + sqrt_of(fabs(ph.gamma * (ph.p_r + dp) * rinv));
-  const T mn = AFF ? sgn * u[1 + D] : u[1] * n[0] + u[2] * n[1] + u[3] * n[2];
+  const T dp = ph.gm1 * u[4] - (ph.hgm1 * rinv) * m2;
+  lam = sqrt_of(m2) * rinv + sqrt_of(fabs((ph.g_pr + ph.gamma * dp) * rinv));
+  const T mn = w * (AFF ? u[1 + D] : u[1] * n[0] + u[2] * n[1] + u[3] * n[2]);
   const T vn = mn * rinv;
   f[0] = mn;
   f[1] = u[1] * vn;
   f[2] = u[2] * vn;
   f[3] = u[3] * vn;
   if (AFF) {
-    f[1 + D] += sgn * dp;
+    f[1 + D] += w * dp;
   } else {
-    f[1] += dp * n[0];
-    f[2] += dp * n[1];
-    f[3] += dp * n[2];
+    const T wp = w * dp;
+    f[1] += wp * n[0];
+    f[2] += wp * n[1];
+    f[3] += wp * n[2];
   }
   f[4] = (ph.H_r + u[4] + dp) * vn;
 }
@@ -208,50 +282,47 @@ __device__ __forceinline__ SideState<T> side_state(const T u[5], const PhysT<T>&
 }
 
 // Normal viscous flux F_v(U, G) e_D on an axis-aligned face: only the normal derivatives and, of the
-// tangential ones, those of rho, m_D and the tangential momentum along its own direction enter.
-// gd: normal derivatives (physical order); r1, d1, a1: d/dx_t1 of rho, m_D, m_t1; r2, d2, a2: d/dx_t2 of
-// rho, m_D, m_t2.  f: components (m_D, m_t1, m_t2, rho E).
+// tangential ones, those of rho, m_D and the tangential momentum along its own direction enter.  All derivatives are
+// reference ones (times hinv).  gd: along the normal (physical order); r1, d1, a1: along t1 of rho, m_D, m_t1; r2, d2,
+// a2: along t2 of rho, m_D, m_t2.  f: components (m_D, m_t1, m_t2, rho E).
 template <typename T, int D>
 __device__ __forceinline__ void visc_normal(const SideState<T>& s, const T gd[5], T r1, T d1, T a1, T r2, T d2, T a2,
-                                            const PhysT<T>& ph, T f[4]) {
+                                            const KConst<T>& kc, T f[4]) {
   constexpr int t1 = D == 0 ? 1 : 0, t2 = D == 2 ? 1 : 2;
-  const T ad = (gd[1 + D] - s.v[D] * gd[0]) * s.rinv;
-  const T at1 = (gd[1 + t1] - s.v[t1] * gd[0]) * s.rinv;
-  const T at2 = (gd[1 + t2] - s.v[t2] * gd[0]) * s.rinv;
-  const T b1 = (d1 - s.v[D] * r1) * s.rinv;
-  const T b2 = (d2 - s.v[D] * r2) * s.rinv;
-  const T cc = ((a1 - s.v[t1] * r1) + (a2 - s.v[t2] * r2)) * s.rinv;
-  f[0] = ph.mu * (T(4) / T(3) * ad - T(2) / T(3) * cc);
-  f[1] = ph.mu * (at1 + b1);
-  f[2] = ph.mu * (at2 + b2);
-  const T q = (gd[4] - s.E * gd[0]) * s.rinv - (s.v[D] * ad + s.v[t1] * at1 + s.v[t2] * at2);
-  f[3] = f[0] * s.v[D] + f[1] * s.v[t1] + f[2] * s.v[t2] + ph.lam_cv * q;
+  const T rd = kc.hinv[D] * s.rinv, ra = kc.hinv[t1] * s.rinv, rb = kc.hinv[t2] * s.rinv;
+  const T ad = (gd[1 + D] - s.v[D] * gd[0]) * rd;
+  const T at1 = (gd[1 + t1] - s.v[t1] * gd[0]) * rd;
+  const T at2 = (gd[1 + t2] - s.v[t2] * gd[0]) * rd;
+  const T cc = (a1 - s.v[t1] * r1) * ra + (a2 - s.v[t2] * r2) * rb;
+  f[0] = kc.mu43 * ad - kc.mu23 * cc;
+  f[1] = kc.mu * (at1 + (d1 - s.v[D] * r1) * ra);
+  f[2] = kc.mu * (at2 + (d2 - s.v[D] * r2) * rb);
+  const T q = (gd[4] - s.E * gd[0]) * rd - (s.v[D] * ad + s.v[t1] * at1 + s.v[t2] * at2);
+  f[3] = f[0] * s.v[D] + f[1] * s.v[t1] + f[2] * s.v[t2] + kc.lam_cv * q;
 }
 
-// F_v(U, j (x) e_D) on an axis-aligned face: normal column fd (m_D, m_t1, m_t2, rho E) and the nonzero entries
-// (m_D, m_t, rho E) of the tangential columns.
+// Integrands of +1/2 (grad V, F_v(U, j (x) e_D)) on an axis-aligned face over the cell's |J|: normal column
+// fd (m_D, m_t1, m_t2, rho E) and the nonzero entries (m_D, m_t, rho E) of the tangential columns, with all
+// constant factors (mu/2, 1/h of both directions) in kc.mus and kc.lams.
 template <typename T, int D>
-__device__ __forceinline__ void visc_jump(const SideState<T>& s, const T j[5], const PhysT<T>& ph, T fd[4], T f1[3],
+__device__ __forceinline__ void visc_jump(const SideState<T>& s, const T j[5], const KConst<T>& kc, T fd[4], T f1[3],
                                           T f2[3]) {
   constexpr int t1 = D == 0 ? 1 : 0, t2 = D == 2 ? 1 : 2;
-  const T mr = ph.mu * s.rinv;
-  const T gd = mr * (j[1 + D] - s.v[D] * j[0]);
-  const T g1 = mr * (j[1 + t1] - s.v[t1] * j[0]);
-  const T g2 = mr * (j[1 + t2] - s.v[t2] * j[0]);
-  const T h = T(-2) / T(3) * gd;
-  fd[0] = T(4) / T(3) * gd;
-  fd[1] = g1;
-  fd[2] = g2;
-  // lambda/c_v ((j_E - E j_0)/rho - v . g/mu), g/mu = (j_m - v j_0)/rho
-  const T v2 = s.v[0] * s.v[0] + s.v[1] * s.v[1] + s.v[2] * s.v[2];
-  const T q = j[4] - s.E * j[0] - (s.v[0] * j[1] + s.v[1] * j[2] + s.v[2] * j[3] - v2 * j[0]);
-  fd[3] = fd[0] * s.v[D] + g1 * s.v[t1] + g2 * s.v[t2] + (ph.lam_cv * s.rinv) * q;
-  f1[0] = g1;
-  f1[1] = h;
-  f1[2] = g1 * s.v[D] + h * s.v[t1];
-  f2[0] = g2;
-  f2[1] = h;
-  f2[2] = g2 * s.v[D] + h * s.v[t2];
+  const T gd = j[1 + D] - s.v[D] * j[0];
+  const T g1 = j[1 + t1] - s.v[t1] * j[0];
+  const T g2 = j[1 + t2] - s.v[t2] * j[0];
+  const T rd = kc.mus[D][D] * s.rinv, ra = kc.mus[D][t1] * s.rinv, rb = kc.mus[D][t2] * s.rinv;
+  fd[0] = (kc.mus43[D] * s.rinv) * gd;
+  fd[1] = rd * g1;
+  fd[2] = rd * g2;
+  const T vg = s.v[D] * gd + s.v[t1] * g1 + s.v[t2] * g2;
+  fd[3] = fd[0] * s.v[D] + fd[1] * s.v[t1] + fd[2] * s.v[t2] + (kc.lams[D] * s.rinv) * (j[4] - s.E * j[0] - vg);
+  f1[0] = ra * g1;
+  f1[1] = -(kc.mus23[D][t1] * s.rinv) * gd;
+  f1[2] = f1[0] * s.v[D] + f1[1] * s.v[t1];
+  f2[0] = rb * g2;
+  f2[1] = -(kc.mus23[D][t2] * s.rinv) * gd;
+  f2[2] = f2[0] * s.v[D] + f2[1] * s.v[t2];
 }
 
 // F_v(U, G) n for a general unit normal; rows of f: momenta and energy.
@@ -287,12 +358,15 @@ __device__ __forceinline__ JumpFlux<T> visc_jump_any(const SideState<T>& s, cons
                                                      const PhysT<T>& ph) {
   JumpFlux<T> r;
   const T mr = ph.mu * s.rinv;
+  T vg = T(0);
 #pragma unroll
-  for (int i = 0; i < 3; ++i) r.g[i] = mr * (j[1 + i] - s.v[i] * j[0]);
+  for (int i = 0; i < 3; ++i) {
+    const T g = j[1 + i] - s.v[i] * j[0];
+    vg += s.v[i] * g;
+    r.g[i] = mr * g;
+  }
   r.h = T(-2) / T(3) * (r.g[0] * n[0] + r.g[1] * n[1] + r.g[2] * n[2]);
-  const T v2 = s.v[0] * s.v[0] + s.v[1] * s.v[1] + s.v[2] * s.v[2];
-  r.q = (ph.lam_cv * s.rinv) *
-        (j[4] - s.E * j[0] - (s.v[0] * j[1] + s.v[1] * j[2] + s.v[2] * j[3] - v2 * j[0]));
+  r.q = (ph.lam_cv * s.rinv) * (j[4] - s.E * j[0] - vg);
   return r;
 }
 template <typename T>
@@ -313,22 +387,26 @@ __device__ __forceinline__ void jump_row(const JumpFlux<T>& r, const SideState<T
 // Shared memory per cell: the three convective flux arrays [3][5][QC^3] (their space also holds the nodal
 // state, the interpolation temporaries, the projected residual and M^-1's temporaries) and the viscous
 // point arrays [3][5][N^3] (gradients, then fluxes) with the values U_g [5][N^3].
-template <int N, int QC>
+template <typename T, int N, int QC>
 struct CollSizes {
   static constexpr int N2 = N * N, N3 = N2 * N, PC = QC * QC * QC;
-  static constexpr int F = PC > N3 ? PC : N3;
-  static constexpr int PER_CELL = 15 * F + 20 * N3;
+  // plane strides of the point and node arrays, and of the (QC x, N y) planes; block sizes
+  static constexpr int PN = plane_stride<T>(N, N), PQ = plane_stride<T>(QC, QC), P1 = plane_stride<T>(QC, N);
+  static constexpr int BN = N * PN, BQ = QC * PQ;
+  static constexpr int F0 = BQ > BN ? BQ : BN, F1 = N * P1 > F0 ? N * P1 : F0;
+  static constexpr int F = (F1 + 3) & ~3;
+  static constexpr int PER_CELL = 15 * F + 20 * BN;
 };
 template <typename T, int N, int QC, int QV, int CB>
 constexpr size_t coll_cell_smem() {
-  return ((size_t)table_elems<T, N, QC, QV>() + (size_t)CB * CollSizes<N, QC>::PER_CELL) * sizeof(T) + 64;
+  return ((size_t)table_elems<T, N, QC, QV>() + (size_t)CB * CollSizes<T, N, QC>::PER_CELL) * sizeof(T) + 192;
 }
 
 // Cells per CTA and threads.
 template <typename T, int N, int QC, int QV>
 constexpr int coll_cells() {
   int cb = 2;
-  while (cb > 1 && ((size_t)table_elems<T, N, QC, QV>() + (size_t)cb * CollSizes<N, QC>::PER_CELL) * sizeof(T) > 74 * 1024)
+  while (cb > 1 && ((size_t)table_elems<T, N, QC, QV>() + (size_t)cb * CollSizes<T, N, QC>::PER_CELL) * sizeof(T) > 74 * 1024)
     --cb;
   return cb;
 }
@@ -341,28 +419,30 @@ constexpr int coll_threads() {
   constexpr size_t smem = coll_cell_smem<T, N, QC, QV, coll_cells<T, N, QC, QV>()>();
   return sizeof(T) == 8 ? (smem > 64 * 1024 ? 192 : 128) : (smem > 40 * 1024 ? 256 : 128);
 }
-template <typename T, int N, int QC, int QV>
+template <typename T, int N, int QC, int QV, int CB>
 constexpr int coll_ctas() {  // resident CTAs that the registers have to allow
-  const int b = (int)(227 * 1024 / coll_cell_smem<T, N, QC, QV, coll_cells<T, N, QC, QV>()>());
+  const int b = (int)(227 * 1024 / coll_cell_smem<T, N, QC, QV, CB>());
   return b < 1 ? 1 : (b > 4 ? 4 : b);
 }
 
 // kp.out_mode: 0 writes F(U), 1 L(U), 2 the stage update (as dg_op_kernel).
 template <typename T, int N, int QC, int QV, int CB, int GEO>
-__global__ void __launch_bounds__(coll_threads<T, N, QC, QV>(), coll_ctas<T, N, QC, QV>())
+__global__ void __launch_bounds__(coll_threads<T, N, QC, QV>(), coll_ctas<T, N, QC, QV, CB>())
     dg_coll_cell_kernel(const KParams kp, const double* __restrict__ U,
                                                                          T* Rout, T* dU, double* Uout) {
   static_assert(QV == N && GEO != GEO_FLY, "collocation form");
-  using S = CollSizes<N, QC>;
-  constexpr int N2 = S::N2, N3 = S::N3, PC = S::PC, NTH = coll_threads<T, N, QC, QV>();
+  using S = CollSizes<T, N, QC>;
+  constexpr int N2 = S::N2, N3 = S::N3, PC = S::PC, PN = S::PN, PQ = S::PQ, P1 = S::P1, BN = S::BN, BQ = S::BQ;
+  constexpr int QC2 = QC * QC, NTH = coll_threads<T, N, QC, QV>();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   T* stab = reinterpret_cast<T*>(smem_raw);
   T* F0 = stab + table_elems<T, N, QC, QV>();
   T* F1 = F0 + CB * 5 * S::F;
   T* F2 = F1 + CB * 5 * S::F;
-  T* V = F2 + CB * 5 * S::F;  // [3][CB][5][N^3]
-  T* Ug = V + 3 * CB * 5 * N3;
-  constexpr int VS = CB * 5 * N3;
+  T* V = F2 + CB * 5 * S::F;  // [3][CB][5][N][PN]
+  constexpr int VS = CB * 5 * BN;
+  T* Ug = V + 3 * VS;
+  auto pad = [](int i) { return i / N2 * PN + i % N2; };  // value i of node arrays
   const int e0 = blockIdx.x * CB;
   const int nb = min(CB, kp.Nc - e0);
   const Tab<T> tb = load_tables<T, N, QC, QV>(static_cast<const T*>(kp.tables), stab);
@@ -371,35 +451,108 @@ __global__ void __launch_bounds__(coll_threads<T, N, QC, QV>(), coll_ctas<T, N, 
   const size_t base = (size_t)e0 * 5 * N3;
   const int nvals = nb * 5 * N3, nbl = nb * 5;
   constexpr int PER = (CB * 5 * N3 + NTH - 1) / NTH;
+  constexpr bool FX = sizeof(T) == 8;  // integer chains
   const T* Ud = static_cast<const T*>(kp.Udev);
-  if (Ud)
-    batched_pass<PER>(threadIdx.x, NTH, nvals, [&](int i) { return Ud[base + i]; }, [&](int i, T v) { F0[i] = v; });
-  else
-    batched_pass<PER>(threadIdx.x, NTH, nvals, [&](int i) { return U[base + i]; }, [&](int i, double v) {
-      F0[i] = dev_value<T>(kp, v, (i / N3) % 5);
-    });
-  __syncthreads();
+  const T* FBc = static_cast<const T*>(kp.fbuf) + (size_t)e0 * fbuf_per_cell<N>();
   const bool conv = kp.conv != 0, visc = kp.visc != 0;
   const bool force = kp.has_bf && kp.out_mode != 0;
+  // FP64: per-component maxima of the state [0], the convective flux [5], the viscous flux and the face shares [10];
+  // divergence of the convective
+  // flux [15] and the first S^-1 sweep's result [20]
+  uint32_t* ex = reinterpret_cast<uint32_t*>(Ug + VS);
+  bool fixA = false, fixB = false, fixR = false;  // chains: values, convective flux, residual and M^-1
+  if constexpr (FX) {
+    constexpr int PV = (CB * N3 + NTH - 1) / NTH;
+    double x[5][PV];
+#pragma unroll
+    for (int c = 0; c < 5; ++c)
+#pragma unroll
+      for (int k = 0; k < PV; ++k) {
+        const int i = k * NTH + threadIdx.x, e = i / N3;
+        x[c][k] = i < nb * N3 ? U[base + (size_t)e * 4 * N3 + c * N3 + i] : 0.0;
+      }
+    if (threadIdx.x < 25) ex[threadIdx.x] = 0;
+    __syncthreads();
+#pragma unroll
+    for (int c = 0; c < 5; ++c) {
+      uint32_t m = 0, f = 0;
+#pragma unroll
+      for (int k = 0; k < PV; ++k) {
+        if ((c == 0 || c == 4) && k * NTH + (int)threadIdx.x < nb * N3) x[c][k] -= c == 0 ? kp.rho_ref : kp.rhoE_ref;
+        m = max(m, fx_mag(x[c][k]));
+      }
+      block_max(ex + c, m);
+      // the shares of the batch, also brought nearer for the lift sweeps
+      for (int i = threadIdx.x; i < nb * 12 * N2; i += NTH)
+        f = max(f, reinterpret_cast<const uint32_t*>(FBc + (i / N2 * 5 + c) * N2 + i % N2)[1] & 0x7fffffffu);
+      block_max(ex + 10 + c, f);
+    }
+    __syncthreads();
+    fixA = block_ok<5>(ex);
+#pragma unroll
+    for (int c = 0; c < 5; ++c) {
+      const int E = fx_exp(ex[c]);
+#pragma unroll
+      for (int k = 0; k < PV; ++k) {
+        const int i = k * NTH + threadIdx.x, e = i / N3;
+        if (i < nb * N3) F0[e * 4 * N3 + c * N3 + i] = fixA ? __longlong_as_double(fx_of(x[c][k], E)) : x[c][k];
+      }
+    }
+  } else if (Ud) {
+    batched_pass<PER>(threadIdx.x, NTH, nvals, [&](int i) { return Ud[base + i]; }, [&](int i, T v) { F0[pad(i)] = v; });
+  } else {
+    batched_pass<PER>(threadIdx.x, NTH, nvals, [&](int i) { return U[base + i]; }, [&](int i, double v) {
+      F0[pad(i)] = dev_value<T>(kp, v, (i / N3) % 5);
+    });
+  }
+  __syncthreads();
   // 1-3. values at the convective and at the viscous points
-  if (conv) lines<T, 1, N, QC, 1>(F0, F1, tb.eSc, nbl * N2);
-  lines<T, 1, N, N, 1>(F0, V, tb.eSm, nbl * N2);
+  int gS = 0;  // exponent of U_g over the state's (chains)
+  if (FX && fixA) {
+    if constexpr (FX) {
+      const int gC = chain_gain(tb.eSc);
+      gS = chain_gain(tb.eSm);
+      if (conv) chain<1, N, QC, 1, FROM_INT, TO_INT>(F0, F1, tb.eSc, nbl * N2, 1, ex, 0);
+      chain<1, N, N, 1, FROM_INT, TO_INT>(F0, V, tb.eSm, nbl * N2, 1, ex, 0);
+      __syncthreads();
+      if (conv) chain<QC, N, QC, 1, FROM_INT, TO_INT>(F1, F2, tb.eSc, nbl * N, 1, ex, 0);
+      chain<N, N, N, 1, FROM_INT, TO_INT>(V, V + VS, tb.eSm, nbl * N, 1, ex, 0);
+      __syncthreads();
+      if (conv) chain<QC * QC, N, QC, 1, FROM_INT, TO_DOUBLE>(F2, F0, tb.eSc, nbl, QC * QC, ex, 2 * gC);
+      chain<N2, N, N, 1, FROM_INT, TO_INT>(V + VS, Ug, tb.eSm, nbl, 1, ex, 0);
+      gS *= 3;
+    }
+  } else {
+    if (conv) sw<T, 0, N, N, N, QC, 1, PN, P1>(F0, F1, tb.eSc, nbl);
+    sw<T, 0, N, N, N, N, 1, PN, PN>(F0, V, tb.eSm, nbl);
+    __syncthreads();
+    if (conv) sw<T, 1, QC, N, N, QC, 1, P1, PQ>(F1, F2, tb.eSc, nbl);
+    sw<T, 1, N, N, N, N, 1, PN, PN>(V, V + VS, tb.eSm, nbl);
+    __syncthreads();
+    if (conv) sw<T, 2, QC, QC, N, QC, 1, PQ, PQ>(F2, F0, tb.eSc, nbl);
+    sw<T, 2, N, N, N, N, 1, PN, PN>(V + VS, Ug, tb.eSm, nbl);
+  }
   __syncthreads();
-  if (conv) lines<T, QC, N, QC, 1>(F1, F2, tb.eSc, nbl * N);
-  lines<T, N, N, N, 1>(V, V + VS, tb.eSm, nbl * N);
-  __syncthreads();
-  if (conv) lines<T, QC * QC, N, QC, 1>(F2, F0, tb.eSc, nbl);
-  lines<T, N2, N, N, 1>(V + VS, Ug, tb.eSm, nbl);
-  __syncthreads();
+  auto ug = [&](int i, int c) -> T {
+    if constexpr (FX) {
+      if (fixA) return fx_store(__double_as_longlong(Ug[i]), fx_exp(ex[c]) + gS + 3);
+    }
+    return Ug[i];
+  };
+  uint32_t mag[5] = {0, 0, 0, 0, 0};
+  auto see = [&](int c, T v) {
+    if constexpr (FX) mag[c] = max(mag[c], fx_mag(v));
+    return v;
+  };
   // 4. convective flux (point arithmetic); reference gradients at the viscous points (sweeps)
   if (conv) {
     for (int idx = threadIdx.x; idx < nb * PC; idx += NTH) {
-      const int e = idx / PC, p = idx - e * PC, o = e * 5 * PC + p;
+      const int e = idx / PC, p = idx - e * PC, o = e * 5 * BQ + p / QC2 * PQ + p % QC2;
       T u[5];
 #pragma unroll
-      for (int c = 0; c < 5; ++c) u[c] = F0[o + c * PC];
+      for (int c = 0; c < 5; ++c) u[c] = F0[o + c * BQ];
       const T rinv = rcp_of(ph.rho_r + u[0]);
-      const T dp = pressure_dev(u, rinv, ph.gm1);
+      const T dp = ph.gm1 * u[4] - (ph.hgm1 * rinv) * (u[1] * u[1] + u[2] * u[2] + u[3] * u[3]);
       const T Hr = (ph.H_r + u[4] + dp) * rinv;
       T* Fd[3] = {F0, F1, F2};
       if (GEO == GEO_AFFINE) {
@@ -408,10 +561,11 @@ __global__ void __launch_bounds__(coll_threads<T, N, QC, QV>(), coll_ctas<T, N, 
           const T m = kc.hinv[j] * u[1 + j];
           const T a = m * rinv;
           T* f = Fd[j] + o;
-          f[0] = m;
+          f[0] = see(0, m);
 #pragma unroll
-          for (int i = 0; i < 3; ++i) f[(1 + i) * PC] = i == j ? u[1 + i] * a + kc.hinv[j] * dp : u[1 + i] * a;
-          f[4 * PC] = Hr * m;
+          for (int i = 0; i < 3; ++i)
+            f[(1 + i) * BQ] = see(1 + i, i == j ? u[1 + i] * a + kc.hinv[j] * dp : u[1 + i] * a);
+          f[4 * BQ] = see(4, Hr * m);
         }
       } else {
         const T* g = static_cast<const T*>(kp.gcc) + (size_t)(e0 + e) * 10 * PC + p;
@@ -422,140 +576,212 @@ __global__ void __launch_bounds__(coll_threads<T, N, QC, QV>(), coll_ctas<T, N, 
           const T j0 = dj * g[(3 * b) * PC], j1 = dj * g[(3 * b + 1) * PC], j2 = dj * g[(3 * b + 2) * PC];
           const T m = j0 * u[1] + j1 * u[2] + j2 * u[3];
           T* f = Fd[b] + o;
-          f[0] = m;
-          f[PC] = m * v[0] + dp * j0;
-          f[2 * PC] = m * v[1] + dp * j1;
-          f[3 * PC] = m * v[2] + dp * j2;
-          f[4 * PC] = Hr * m;
+          f[0] = see(0, m);
+          f[BQ] = see(1, m * v[0] + dp * j0);
+          f[2 * BQ] = see(2, m * v[1] + dp * j1);
+          f[3 * BQ] = see(3, m * v[2] + dp * j2);
+          f[4 * BQ] = see(4, Hr * m);
         }
       }
     }
   }
-  if (visc) {
-    lines<T, 1, N, N, -1>(Ug, V, tb.eDv, nbl * N2);
-    lines<T, N, N, N, -1>(Ug, V + VS, tb.eDv, nbl * N);
-    lines<T, N2, N, N, -1>(Ug, V + 2 * VS, tb.eDv, nbl);
+  if constexpr (FX) {
+    if (conv) {
+#pragma unroll
+      for (int c = 0; c < 5; ++c) {
+        block_max(ex + 5 + c, mag[c]);
+        mag[c] = 0;
+      }
+    }
+    if (visc && fixA) {
+      chain<1, N, N, -1, FROM_INT, TO_DOUBLE>(Ug, V, tb.eDv, nbl * N2, N2, ex, gS);
+      chain<N, N, N, -1, FROM_INT, TO_DOUBLE>(Ug, V + VS, tb.eDv, nbl * N, N2, ex, gS);
+      chain<N2, N, N, -1, FROM_INT, TO_DOUBLE>(Ug, V + 2 * VS, tb.eDv, nbl, N2, ex, gS);
+    }
+  }
+  if (visc && !fixA) {
+    sw<T, 0, N, N, N, N, -1, PN, PN>(Ug, V, tb.eDv, nbl);
+    sw<T, 1, N, N, N, N, -1, PN, PN>(Ug, V + VS, tb.eDv, nbl);
+    sw<T, 2, N, N, N, N, -1, PN, PN>(Ug, V + 2 * VS, tb.eDv, nbl);
   }
   __syncthreads();
   // 5. viscous flux with the sign of -F (point arithmetic); D~ of the convective flux, in place (sweeps)
   if (visc) {
     for (int idx = threadIdx.x; idx < nb * N3; idx += NTH) {
-      const int e = idx / N3, p = idx - e * N3, o = e * 5 * N3 + p;
-      T u[5], G[5][3];
+      const int e = idx / N3, p = idx - e * N3, o = e * 5 * BN + pad(p);
+      T u[5];
       T* v0 = V + o;
 #pragma unroll
-      for (int c = 0; c < 5; ++c) u[c] = Ug[o + c * N3];
-      T Jd[9];
+      for (int c = 0; c < 5; ++c) u[c] = ug(o + c * BN, c);
+      const SideState<T> s = side_state(u, ph);
       if (GEO == GEO_AFFINE) {
+        // reference derivatives; 1/h_j enters with 1/rho and with the flux constants
+        T gu[3][3], ge[3];
 #pragma unroll
-        for (int c = 0; c < 5; ++c)
+        for (int j = 0; j < 3; ++j) {
+          const T* g = v0 + j * VS;
+          const T r = kc.hinv[j] * s.rinv, g0 = g[0];
 #pragma unroll
-          for (int j = 0; j < 3; ++j) G[c][j] = kc.hinv[j] * v0[j * VS + c * N3];
+          for (int i = 0; i < 3; ++i) gu[i][j] = (g[(1 + i) * BN] - s.v[i] * g0) * r;
+          ge[j] = (g[4 * BN] - s.E * g0) * r - (s.v[0] * gu[0][j] + s.v[1] * gu[1][j] + s.v[2] * gu[2][j]);
+        }
+        const T div = T(2) / T(3) * (gu[0][0] + gu[1][1] + gu[2][2]);
+        const T s01 = gu[0][1] + gu[1][0], s02 = gu[0][2] + gu[2][0], s12 = gu[1][2] + gu[2][1];
+        const T S[3][3] = {{T(2) * gu[0][0] - div, s01, s02}, {s01, T(2) * gu[1][1] - div, s12},
+                           {s02, s12, T(2) * gu[2][2] - div}};
+#pragma unroll
+        for (int b = 0; b < 3; ++b) {
+          T* f = v0 + b * VS;
+          const T w = -kc.muh[b];
+          const T t0 = w * S[b][0], t1 = w * S[b][1], t2 = w * S[b][2];
+          f[0] = T(0);
+          f[BN] = see(1, t0);
+          f[2 * BN] = see(2, t1);
+          f[3 * BN] = see(3, t2);
+          f[4 * BN] = see(4, t0 * s.v[0] + t1 * s.v[1] + t2 * s.v[2] - kc.lamh[b] * ge[b]);
+        }
       } else {
+        T Jd[9], G[5][3];
         const T* g = static_cast<const T*>(kp.gcv) + (size_t)(e0 + e) * 10 * N3 + p;
 #pragma unroll
         for (int m = 0; m < 9; ++m) Jd[m] = g[m * N3];
 #pragma unroll
         for (int c = 0; c < 5; ++c) {
-          const T g0 = v0[c * N3], g1 = v0[VS + c * N3], g2 = v0[2 * VS + c * N3];
+          const T g0 = v0[c * BN], g1 = v0[VS + c * BN], g2 = v0[2 * VS + c * BN];
 #pragma unroll
           for (int a = 0; a < 3; ++a) G[c][a] = Jd[a] * g0 + Jd[3 + a] * g1 + Jd[6 + a] * g2;
         }
         const T dj = -g[9 * N3];
 #pragma unroll
         for (int m = 0; m < 9; ++m) Jd[m] *= dj;
-      }
-      const SideState<T> s = side_state(u, ph);
-      T gu[3][3];
+        T gu[3][3];
 #pragma unroll
-      for (int i = 0; i < 3; ++i)
+        for (int i = 0; i < 3; ++i)
 #pragma unroll
-        for (int j = 0; j < 3; ++j) gu[i][j] = (G[1 + i][j] - s.v[i] * G[0][j]) * s.rinv;
-      const T div = T(2) / T(3) * (gu[0][0] + gu[1][1] + gu[2][2]);
-      T t[3][3];
+          for (int j = 0; j < 3; ++j) gu[i][j] = (G[1 + i][j] - s.v[i] * G[0][j]) * s.rinv;
+        const T div = T(2) / T(3) * (gu[0][0] + gu[1][1] + gu[2][2]);
+        T t[3][3];
 #pragma unroll
-      for (int i = 0; i < 3; ++i) {
-        t[i][i] = ph.mu * (T(2) * gu[i][i] - div);
+        for (int i = 0; i < 3; ++i) {
+          t[i][i] = ph.mu * (T(2) * gu[i][i] - div);
 #pragma unroll
-        for (int j = i + 1; j < 3; ++j) t[i][j] = t[j][i] = ph.mu * (gu[i][j] + gu[j][i]);
-      }
-      T q[3];
+          for (int j = i + 1; j < 3; ++j) t[i][j] = t[j][i] = ph.mu * (gu[i][j] + gu[j][i]);
+        }
+        T q[3];
 #pragma unroll
-      for (int j = 0; j < 3; ++j)
-        q[j] = t[0][j] * s.v[0] + t[1][j] * s.v[1] + t[2][j] * s.v[2] +
-               ph.lam_cv * ((G[4][j] - s.E * G[0][j]) * s.rinv -
-                            (s.v[0] * gu[0][j] + s.v[1] * gu[1][j] + s.v[2] * gu[2][j]));
+        for (int j = 0; j < 3; ++j)
+          q[j] = t[0][j] * s.v[0] + t[1][j] * s.v[1] + t[2][j] * s.v[2] +
+                 ph.lam_cv * ((G[4][j] - s.E * G[0][j]) * s.rinv -
+                              (s.v[0] * gu[0][j] + s.v[1] * gu[1][j] + s.v[2] * gu[2][j]));
 #pragma unroll
-      for (int b = 0; b < 3; ++b) {
-        T* f = v0 + b * VS;
-        f[0] = T(0);
-        if (GEO == GEO_AFFINE) {
-          const T w = -kc.hinv[b];
-#pragma unroll
-          for (int i = 0; i < 3; ++i) f[(1 + i) * N3] = w * t[i][b];
-          f[4 * N3] = w * q[b];
-        } else {
+        for (int b = 0; b < 3; ++b) {
+          T* f = v0 + b * VS;
           const T j0 = Jd[3 * b], j1 = Jd[3 * b + 1], j2 = Jd[3 * b + 2];
+          f[0] = T(0);
 #pragma unroll
-          for (int i = 0; i < 3; ++i) f[(1 + i) * N3] = j0 * t[i][0] + j1 * t[i][1] + j2 * t[i][2];
-          f[4 * N3] = j0 * q[0] + j1 * q[1] + j2 * q[2];
+          for (int i = 0; i < 3; ++i) f[(1 + i) * BN] = see(1 + i, j0 * t[i][0] + j1 * t[i][1] + j2 * t[i][2]);
+          f[4 * BN] = see(4, j0 * q[0] + j1 * q[1] + j2 * q[2]);
         }
       }
     }
   }
-  if (conv) {
-    lines<T, 1, QC, QC, -1>(F0, F0, tb.eDcW, nbl * QC * QC);
-    lines<T, QC, QC, QC, -1>(F1, F1, tb.eDcW, nbl * QC);
-    lines<T, QC * QC, QC, QC, -1>(F2, F2, tb.eDcW, nbl);
+  if constexpr (FX) {
+    if (visc) {
+#pragma unroll
+      for (int c = 1; c < 5; ++c) block_max(ex + 10 + c, mag[c]);
+    }
+    fixB = conv && fixA && block_ok<5>(ex + 5);
+    if (fixB) {
+      chain<1, QC, QC, -1, FROM_DOUBLE, TO_INT>(F0, F0, tb.eDcW, nbl * QC * QC, QC * QC, ex + 5, 0, 2);
+      chain<QC, QC, QC, -1, FROM_DOUBLE, TO_INT>(F1, F1, tb.eDcW, nbl * QC, QC * QC, ex + 5, 0, 2);
+      chain<QC * QC, QC, QC, -1, FROM_DOUBLE, TO_INT>(F2, F2, tb.eDcW, nbl, QC * QC, ex + 5, 0, 2);
+    }
+  }
+  if (conv && !fixB) {
+    sw<T, 0, QC, QC, QC, QC, -1, PQ, PQ>(F0, F0, tb.eDcW, nbl);
+    sw<T, 1, QC, QC, QC, QC, -1, PQ, PQ>(F1, F1, tb.eDcW, nbl);
+    sw<T, 2, QC, QC, QC, QC, -1, PQ, PQ>(F2, F2, tb.eDcW, nbl);
   }
   __syncthreads();
   // 6-8. projection of the summed convective parts onto the l_g; D~ and face shares of the viscous arrays
-  const T* FBc = static_cast<const T*>(kp.fbuf) + (size_t)e0 * fbuf_per_cell<N>();
-  if (conv) lines<T, QC * QC, QC, N, 1, 3, false, 0, 0, PC>(F0, F0, tb.ePc, nbl, CB * 5 * S::F);
-  if constexpr (sizeof(T) == 8) {
-    lift_fp64<N>(V, FBc, tb.eLift, nb, visc, VS);
+  int gF = 0;  // exponent after the lift over the viscous fluxes' and shares'
+  if constexpr (FX) {
+    fixR = fixB && GEO == GEO_AFFINE && !force && kp.out_mode != 0 && block_ok<5>(ex + 10);
+    if (fixB) {
+      gF = chain_gain(tb.eLift, 2);
+      chain<QC * QC, QC, N, 1, FROM_SUM, TO_DOUBLE, 0, 0, PC>(F0, F0, tb.ePc, nbl, QC * QC, ex + 5, chain_gain(tb.eDcW, 2), 0,
+                                                              CB * 5 * S::F, 5, ex + 15);
+    }
+    if (fixR)
+      chain_lift<N>(V, FBc, tb.eLift, nb, visc, VS, ex + 10);
+    else
+      lift_fp64<N>(V, FBc, tb.eLift, nb, visc, VS);
   } else {
     lift_body<T, N, 0>(V, FBc, tb.eLift, nb, visc);
     lift_body<T, N, 1>(V + VS, FBc, tb.eLift, nb, visc);
     lift_body<T, N, 2>(V + 2 * VS, FBc, tb.eLift, nb, visc);
   }
+  if (conv && !fixB) sw<T, 2, QC, QC, QC, N, 1, PQ, PQ, 3, false, 0, BQ>(F0, F0, tb.ePc, nbl, CB * 5 * S::F);
   __syncthreads();
-  if (conv) {
-    lines<T, QC, QC, N, 1, 1, false, N, PC>(F0, F1, tb.ePc, nbl * N);
-    __syncthreads();
-    lines<T, 1, QC, N, 1>(F1, F2, tb.ePc, nbl * N2);
-  } else {
-    for (int i = threadIdx.x; i < nvals; i += NTH) F2[i] = T(0);
+  if constexpr (FX) {
+    if (fixB) {
+      // (ex + 15 was valid if the fluxes' maxima were: the sums only shrink them)
+      chain<QC, QC, N, 1, FROM_DOUBLE, TO_INT, N, PC>(F0, F1, tb.ePc, nbl * N, N * QC, ex + 15, 0);
+      __syncthreads();
+      chain<1, QC, N, 1, FROM_INT, TO_DOUBLE>(F1, F2, tb.ePc, nbl * N2, N2, ex + 15, chain_gain(tb.ePc));
+    }
   }
+  if (conv && !fixB) {
+    sw<T, 1, QC, QC, N, N, 1, PQ, P1, 1, false, BQ>(F0, F1, tb.ePc, nbl);
+    __syncthreads();
+    sw<T, 0, QC, N, N, N, 1, P1, PN>(F1, F2, tb.ePc, nbl);
+  }
+  if (!conv)
+    for (int i = threadIdx.x; i < nbl * BN; i += NTH) F2[i] = T(0);
   __syncthreads();
   // 9-11. M^-1 in the l_g basis is a scaling by 1/|J| (affine: in the flux scales); S^-1 back to the nodes
   T* sr = F2;
-  if (GEO == GEO_AFFINE && !force && kp.out_mode != 0) {
-    lines<T, 1, N, N, 1, 3, true>(V, F1, tb.eSmi, nbl * N2, VS, F2);
+  if constexpr (FX) {
+    if (fixR) chain_sum<N>(V, VS, F2, F1, tb.eSmi, nbl * N2, ex + 10, gF, ex + 15, 2 * chain_gain(tb.ePc), ex + 20);
+  }
+  if (fixR) {
+  } else if (GEO == GEO_AFFINE && !force && kp.out_mode != 0) {
+    sw<T, 0, N, N, N, N, 1, PN, PN, 3, true>(V, F1, tb.eSmi, nbl, VS, F2);
   } else {
     for (int i = threadIdx.x; i < nvals; i += NTH) {
       const int p = i % N3, e = i / (5 * N3), c = (i / N3) % 5;
-      T r = F2[i] + (V[i] + (V[VS + i] + V[2 * VS + i]));
+      const int ip = pad(i);
+      T r = F2[ip] + (V[ip] + (V[VS + ip] + V[2 * VS + ip]));
       if (kp.out_mode == 0) {
         const T w = tb.wm[p % N] * tb.wm[(p / N) % N] * tb.wm[p / N2];
         r *= GEO == GEO_AFFINE ? -w * kc.detJ : -w;
       } else {
         if (GEO == GEO_STORED) r *= rcp_of(static_cast<const T*>(kp.gm)[(size_t)(e0 + e) * N3 + p]);
         if (force && c > 0) {
-          const T* ug = Ug + e * 5 * N3 + p;
+          const int g = e * 5 * BN + pad(p);
           r += c < 4 ? kc.bf[c - 1]
-                     : (kc.bf[0] * ug[N3] + kc.bf[1] * ug[2 * N3] + kc.bf[2] * ug[3 * N3]) * rcp_of(ph.rho_r + ug[0]);
+                     : (kc.bf[0] * ug(g + BN, 1) + kc.bf[1] * ug(g + 2 * BN, 2) + kc.bf[2] * ug(g + 3 * BN, 3)) *
+                           rcp_of(ph.rho_r + ug(g, 0));
         }
       }
-      F0[i] = r;
+      F0[ip] = r;
     }
     __syncthreads();
-    lines<T, 1, N, N, 1>(F0, F1, kp.out_mode == 0 ? tb.eSvT : tb.eSmi, nbl * N2);
+    sw<T, 0, N, N, N, N, 1, PN, PN>(F0, F1, kp.out_mode == 0 ? tb.eSvT : tb.eSmi, nbl);
   }
   __syncthreads();
-  lines<T, N, N, N, 1>(F1, F0, kp.out_mode == 0 ? tb.eSvT : tb.eSmi, nbl * N);
-  __syncthreads();
-  lines<T, N2, N, N, 1>(F0, sr, kp.out_mode == 0 ? tb.eSvT : tb.eSmi, nbl);
+  if constexpr (FX) {
+    if (fixR) {
+      chain<N, N, N, 1, FROM_DOUBLE, TO_INT>(F1, F0, tb.eSmi, nbl * N, N2, ex + 20, 0);
+      __syncthreads();
+      chain<N2, N, N, 1, FROM_INT, TO_DOUBLE>(F0, sr, tb.eSmi, nbl, N2, ex + 20, chain_gain(tb.eSmi));
+    }
+  }
+  if (!fixR) {
+    sw<T, 1, N, N, N, N, 1, PN, PN>(F1, F0, kp.out_mode == 0 ? tb.eSvT : tb.eSmi, nbl);
+    __syncthreads();
+    sw<T, 2, N, N, N, N, 1, PN, N2>(F0, sr, kp.out_mode == 0 ? tb.eSvT : tb.eSmi, nbl);
+  }
   __syncthreads();
   if (kp.out_mode == 2)
     stage_update<PER, N3>(kp, U, dU, Uout, sr, base, nvals, threadIdx.x, NTH);
@@ -587,7 +813,7 @@ struct CollFaceSizes {
 template <typename T, int N, int QC, int QV, int FB_>
 constexpr size_t coll_face_smem() {
   return ((size_t)table_elems<T, N, QC, QV>() + (size_t)FB_ * (CollFaceSizes<N, QC>::PER_FACE + 1)) * sizeof(T) +
-         3 * FB_ * sizeof(int) + 64;
+         (3 * FB_ + 20) * sizeof(int) + 64;
 }
 template <typename T, int N, int QC, int QV>
 constexpr int coll_faces() {
@@ -596,23 +822,23 @@ constexpr int coll_faces() {
     --fb;
   return fb;
 }
-template <typename T>
+// (FP32 at k = 4, 5: 256 threads for the larger faces, 1.10 -> 0.89 ms at 40^3, k = 5)
+template <typename T, int N>
 constexpr int coll_face_threads() {
-  return 128;
+  return sizeof(T) == 4 && N >= 5 ? 256 : 128;
 }
 
 template <typename T, int N, int QC, int QV, int FB_, int D, int GEO>
 __device__ __forceinline__ void coll_face_terms(const double* __restrict__ U, const T* __restrict__ Ud, const int* eo,
                                                 const int* en, const int* oc, const T* tau_f, T* sm, const Tab<T>& tb,
-                                                const KParams& kp, const PhysT<T>& ph, int nb, int s, T* __restrict__ FBuf) {
+                                                const KParams& kp, const PhysT<T>& ph, int nb, int s, T* __restrict__ FBuf,
+                                                uint32_t* ex) {
   using Z = CollFaceSizes<N, QC>;
-  constexpr int N2 = N * N, N3 = N2 * N, QC2 = QC * QC, NTH = coll_face_threads<T>();
+  constexpr int N2 = N * N, N3 = N2 * N, QC2 = QC * QC, NTH = coll_face_threads<T, N>();
   constexpr int t1 = D == 0 ? 1 : 0, t2 = D == 2 ? 1 : 2;
   constexpr bool AFF = GEO == GEO_AFFINE;
   const KConst<T>& kc = kconst<T>(kp);
   const int f = 2 * D + s, fo = 2 * D + (1 - s);
-  const T sgn = s ? T(1) : T(-1);
-  const int idm = s ? N - 1 : 0, idp = s ? 0 : N - 1;
   const T* dlm = s ? tb.dl1 : tb.dl0;
   const T* dlp = s ? tb.dl0 : tb.dl1;
   const int nf = nb * N2, nl = 5 * nf;  // values per slot and per array
@@ -621,7 +847,16 @@ __device__ __forceinline__ void coll_face_terms(const double* __restrict__ U, co
   T* C0 = TT + FB_ * Z::TT;
   T* C1 = C0 + FB_ * Z::C0;        // [m, p][5][nb][QC2]; later the convective share [5][nb][N2]
   const bool conv = kp.conv != 0, visc = kp.visc != 0;
+  constexpr bool FX = sizeof(T) == 8;  // integer chains
+  constexpr int NTT = AFF ? 3 : 5;     // tested components of a tangential direction
+  // FP64: per-slot maxima of the traces [0], the normal derivatives [5], the convective flux [10] and the tangential
+  // gradient tests [15]
+  auto see = [&](uint32_t& m, T v) {
+    if constexpr (FX) m = max(m, fx_mag(v));
+    return v;
+  };
   // traces along the normal lines, from global memory
+  uint32_t mL[5] = {0, 0, 0, 0, 0}, mD[5] = {0, 0, 0, 0, 0};
   for (int idx = threadIdx.x; idx < nl; idx += NTH) {
     const int sl = idx / nf, r = idx - sl * nf, e = r / N2, j = r - e * N2;
     const int c = slot_comp<D>(sl);
@@ -660,29 +895,81 @@ __device__ __forceinline__ void coll_face_terms(const double* __restrict__ U, co
         b[i] = eq < 0 ? T(0) : dev_value<T>(kp, un[i], c);
       }
     }
-    T dm = T(0), dp = T(0), vm = T(0), vp = T(0);
+    T dm, dp;
+    if constexpr (FX) {
+      T y[2], z[2];
+      line_apply<T, N, 2, -1>(tb.eDl, a, y);
+      line_apply<T, N, 2, -1>(tb.eDl, b, z);
+      dm = s ? y[1] : y[0];
+      dp = s ? z[0] : z[1];
+    } else {
+      dm = dp = T(0);
 #pragma unroll
-    for (int i = 0; i < N; ++i) {
-      dm += dlm[i] * a[i];
-      dp += dlp[i] * b[i];
-      if (i == idm) vm = a[i];
-      if (i == idp) vp = b[i];
+      for (int i = 0; i < N; ++i) {
+        dm += dlm[i] * a[i];
+        dp += dlp[i] * b[i];
+      }
     }
+    const T vm = s ? a[N - 1] : a[0], vp = s ? b[0] : b[N - 1];
     VV[idx] = vm;
     VV[nl + idx] = vp;
     VV[2 * nl + idx] = dm;
     VV[3 * nl + idx] = dp;
+    if constexpr (FX) {
+      const uint32_t ml = max(fx_mag(vm), fx_mag(vp)), md = max(fx_mag(dm), fx_mag(dp));
+#pragma unroll
+      for (int q = 0; q < 5; ++q)
+        if (q == sl) {
+          mL[q] = max(mL[q], ml);
+          mD[q] = max(mD[q], md);
+        }
+    }
+  }
+  if constexpr (FX) {
+#pragma unroll
+    for (int q = 0; q < 5; ++q) {
+      block_max(ex + q, mL[q]);
+      block_max(ex + 5 + q, mD[q]);
+    }
   }
   __syncthreads();
-  if (conv) lines<T, 1, N, QC, 1>(VV, C0, tb.eSc, 2 * 5 * nb * N);
-  if (visc) lines<T, 1, N, N, 1>(VV, TT, tb.eSm, 4 * 5 * nb * N);
+  bool fixA = false;
+  int gS = 0;
+  if constexpr (FX) {
+    fixA = block_ok<10>(ex);
+    if (fixA) {
+      gS = chain_gain(tb.eSm);
+      if (conv) chain<1, N, QC, 1, FROM_DOUBLE, TO_INT>(VV, C0, tb.eSc, 2 * 5 * nb * N, nb * N, ex, 0);
+      if (visc) {
+        chain<1, N, N, 1, FROM_DOUBLE, TO_INT>(VV, TT, tb.eSm, 2 * 5 * nb * N, nb * N, ex, 0);
+        chain<1, N, N, 1, FROM_DOUBLE, TO_INT>(VV + 2 * nl, TT + 2 * nl, tb.eSm, 2 * 5 * nb * N, nb * N, ex + 5, 0);
+      }
+    }
+  }
+  if (!fixA) {
+    if (conv) sw<T, 0, N, N, 1, QC, 1>(VV, C0, tb.eSc, 10 * nb);
+    if (visc) sw<T, 0, N, N, 1, N, 1>(VV, TT, tb.eSm, 20 * nb);
+  }
   __syncthreads();
-  if (conv) lines<T, QC, N, QC, 1>(C0, C1, tb.eSc, 2 * 5 * nb);
-  if (visc) lines<T, N, N, N, 1>(TT, VV, tb.eSm, 4 * 5 * nb);
+  if constexpr (FX) {
+    if (fixA) {
+      if (conv) chain<QC, N, QC, 1, FROM_INT, TO_DOUBLE>(C0, C1, tb.eSc, 2 * 5 * nb, nb * QC, ex, chain_gain(tb.eSc));
+      if (visc) {
+        chain<N, N, N, 1, FROM_INT, TO_INT>(TT, VV, tb.eSm, 2 * 5 * nb, 1, ex, 0);
+        chain<N, N, N, 1, FROM_INT, TO_DOUBLE>(TT + 2 * nl, VV + 2 * nl, tb.eSm, 2 * 5 * nb, nb * N, ex + 5, gS);
+      }
+      gS *= 2;
+    }
+  }
+  if (!fixA) {
+    if (conv) sw<T, 1, QC, N, 1, QC, 1>(C0, C1, tb.eSc, 10 * nb);
+    if (visc) sw<T, 1, N, N, 1, N, 1>(TT, VV, tb.eSm, 20 * nb);
+  }
   __syncthreads();
   // convective flux (point arithmetic); tangential derivatives (sweeps)
   if (conv) {
     const int nc = nb * QC2;
+    uint32_t mC[5] = {0, 0, 0, 0, 0};
     for (int idx = threadIdx.x; idx < nc; idx += NTH) {
       const int e = idx / QC2, p = idx - e * QC2;
       T um[5], up[5], fm[5], fp[5], n[3] = {T(0), T(0), T(0)}, w;
@@ -702,39 +989,68 @@ __device__ __forceinline__ void coll_face_terms(const double* __restrict__ U, co
         w = T(-0.5) * g[12 * QC2];
       }
       T lm, lp;
-      llf_side<T, D, AFF>(um, n, sgn, ph, fm, lm);
-      llf_side<T, D, AFF>(up, n, sgn, ph, fp, lp);
-      const T lam = lm > lp ? lm : lp;
+      const T ws = AFF && !s ? -w : w;
+      llf_side<T, D, AFF>(um, n, ws, ph, fm, lm);
+      llf_side<T, D, AFF>(up, n, ws, ph, fp, lp);
+      const T lam = w * (lm > lp ? lm : lp);
 #pragma unroll
       for (int q = 0; q < 5; ++q) {
         const int c = slot_comp<D>(q);
-        C1[q * nc + idx] = w * (fm[c] + fp[c] + lam * (um[c] - up[c]));
+        C1[q * nc + idx] = see(mC[q], fm[c] + fp[c] + lam * (um[c] - up[c]));
+      }
+    }
+    if constexpr (FX) {
+#pragma unroll
+      for (int q = 0; q < 5; ++q) block_max(ex + 10 + q, mC[q]);
+    }
+  }
+  if constexpr (FX) {
+    if (visc && fixA) {
+#pragma unroll
+      for (int sd = 0; sd < 2; ++sd) {
+        const int o = sd * nl;
+        if (AFF) {
+          chain<1, N, N, -1, FROM_INT, TO_DOUBLE>(VV + o, TT + o, tb.eDv, 3 * nb * N, nb * N, ex, gS, 0, 0, 3);
+          chain<N, N, N, -1, FROM_INT, TO_DOUBLE>(VV + o + nf, TT + 2 * nl + o, tb.eDv, 3 * nb, nb * N, ex + 1, gS, 0, 0, 3);
+        } else {
+          chain<1, N, N, -1, FROM_INT, TO_DOUBLE>(VV + o, TT + o, tb.eDv, 5 * nb * N, nb * N, ex, gS);
+          chain<N, N, N, -1, FROM_INT, TO_DOUBLE>(VV + o, TT + 2 * nl + o, tb.eDv, 5 * nb, nb * N, ex, gS);
+        }
       }
     }
   }
-  if (visc) {
+  if (visc && !fixA) {
     if (AFF) {
 #pragma unroll
       for (int sd = 0; sd < 2; ++sd) {
-        lines<T, 1, N, N, -1>(VV + sd * nl, TT + sd * nl, tb.eDv, 3 * nb * N);
-        lines<T, N, N, N, -1>(VV + sd * nl + nf, TT + (2 + sd) * nl, tb.eDv, 3 * nb);
+        sw<T, 0, N, N, 1, N, -1>(VV + sd * nl, TT + sd * nl, tb.eDv, 3 * nb);
+        sw<T, 1, N, N, 1, N, -1>(VV + sd * nl + nf, TT + (2 + sd) * nl, tb.eDv, 3 * nb);
       }
     } else {
-      lines<T, 1, N, N, -1>(VV, TT, tb.eDv, 2 * 5 * nb * N);
-      lines<T, N, N, N, -1>(VV, TT + 2 * nl, tb.eDv, 2 * 5 * nb);
+      sw<T, 0, N, N, 1, N, -1>(VV, TT, tb.eDv, 10 * nb);
+      sw<T, 1, N, N, 1, N, -1>(VV, TT + 2 * nl, tb.eDv, 10 * nb);
     }
   }
   __syncthreads();
   // viscous fluxes (point arithmetic); projection of the convective flux (sweeps).  Shares are of -F.
   if (visc) {
+    uint32_t mT[5] = {0, 0, 0, 0, 0};
     for (int idx = threadIdx.x; idx < nf; idx += NTH) {
       const int e = idx / N2, p = idx - e * N2;
       const bool wall = en[e] < 0;
       T um[5], up[5], jmp[5];
 #pragma unroll
       for (int q = 0; q < 5; ++q) {
-        um[slot_comp<D>(q)] = VV[q * nf + idx];
-        up[slot_comp<D>(q)] = VV[nl + q * nf + idx];
+        T a = VV[q * nf + idx], b = VV[nl + q * nf + idx];
+        if constexpr (FX) {
+          if (fixA) {
+            const int X = fx_exp(ex[q]) + gS + 3;
+            a = fx_store(__double_as_longlong(a), X);
+            b = fx_store(__double_as_longlong(b), X);
+          }
+        }
+        um[slot_comp<D>(q)] = a;
+        up[slot_comp<D>(q)] = b;
       }
       if (wall) wall_ghost(um, ph, up);
       const SideState<T> sm_ = side_state(um, ph), sp_ = side_state(up, ph);
@@ -743,7 +1059,7 @@ __device__ __forceinline__ void coll_face_terms(const double* __restrict__ U, co
       for (int c = 0; c < 5; ++c) jmp[c] = um[c] - up[c];
       T fm[4], fp[4];
       if (AFF) {
-        const T hd = kc.hinv[D], h1 = kc.hinv[t1], h2 = kc.hinv[t2];
+        const T hd = kc.hinv[D];
         T* T1m = TT + idx;
         T* T1p = T1m + nl;
         T* T2m = T1p + nl;
@@ -751,21 +1067,16 @@ __device__ __forceinline__ void coll_face_terms(const double* __restrict__ U, co
         T gm[5], gp[5];
 #pragma unroll
         for (int q = 0; q < 5; ++q) {
-          gm[slot_comp<D>(q)] = hd * VV[2 * nl + q * nf + idx];
-          gp[slot_comp<D>(q)] = hd * VV[3 * nl + q * nf + idx];
+          gm[slot_comp<D>(q)] = VV[2 * nl + q * nf + idx];
+          gp[slot_comp<D>(q)] = VV[3 * nl + q * nf + idx];
         }
-        visc_normal<T, D>(sm_, gm, h1 * T1m[nf], h1 * T1m[2 * nf], h1 * T1m[0], h2 * T2m[0], h2 * T2m[nf],
-                          h2 * T2m[2 * nf], ph, fm);
-        if (wall) {
-          // grad U+ = grad U-, at the ghost state
-          visc_normal<T, D>(sp_, gm, h1 * T1m[nf], h1 * T1m[2 * nf], h1 * T1m[0], h2 * T2m[0], h2 * T2m[nf],
-                            h2 * T2m[2 * nf], ph, fp);
-        } else {
-          visc_normal<T, D>(sp_, gp, h1 * T1p[nf], h1 * T1p[2 * nf], h1 * T1p[0], h2 * T2p[0], h2 * T2p[nf],
-                            h2 * T2p[2 * nf], ph, fp);
-        }
+        visc_normal<T, D>(sm_, gm, T1m[nf], T1m[2 * nf], T1m[0], T2m[0], T2m[nf], T2m[2 * nf], kc, fm);
+        if (wall)  // grad U+ = grad U-, at the ghost state
+          visc_normal<T, D>(sp_, gm, T1m[nf], T1m[2 * nf], T1m[0], T2m[0], T2m[nf], T2m[2 * nf], kc, fp);
+        else
+          visc_normal<T, D>(sp_, gp, T1p[nf], T1p[2 * nf], T1p[0], T2p[0], T2p[nf], T2p[2 * nf], kc, fp);
         // value share (own side): (V, Q*.n), Q*.n = {{F_v}}.n - tau [[U]]; the other side's is the negative
-        const T wv = T(0.5) * sgn * hd, wt = hd * tau;
+        const T wv = s ? T(0.5) * hd : T(-0.5) * hd, wt = hd * tau;
         const int fs[5] = {1, -1, 0, 2, 3};  // slot -> entry of fm
 #pragma unroll
         for (int q = 0; q < 5; ++q) {
@@ -773,29 +1084,32 @@ __device__ __forceinline__ void coll_face_terms(const double* __restrict__ U, co
           VV[q * nf + idx] = fs[q] < 0 ? t : t + wv * (fm[fs[q] < 0 ? 0 : fs[q]] + fp[fs[q] < 0 ? 0 : fs[q]]);
         }
         // +1/2 (grad V, F_v(U, [[U]])), [[U]] = sgn jmp (x) e_D
-        const T hw = T(0.5) * sgn * hd;
-        T a[4], b1[3], b2[3];
-        visc_jump<T, D>(sm_, jmp, ph, a, b1, b2);
-        VV[2 * nl + idx] = hw * hd * a[1];
-        VV[2 * nl + nf + idx] = T(0);
-        VV[2 * nl + 2 * nf + idx] = hw * hd * a[0];
-        VV[2 * nl + 3 * nf + idx] = hw * hd * a[2];
-        VV[2 * nl + 4 * nf + idx] = hw * hd * a[3];
+        if (!s) {
 #pragma unroll
-        for (int i = 0; i < 3; ++i) {
-          T1m[i * nf] = hw * h1 * b1[i];
-          T2m[i * nf] = hw * h2 * b2[i];
+          for (int c = 0; c < 5; ++c) jmp[c] = -jmp[c];
         }
-        if (!wall) visc_jump<T, D>(sp_, jmp, ph, a, b1, b2);
-        VV[3 * nl + idx] = hw * hd * a[1];
-        VV[3 * nl + nf + idx] = T(0);
-        VV[3 * nl + 2 * nf + idx] = hw * hd * a[0];
-        VV[3 * nl + 3 * nf + idx] = hw * hd * a[2];
-        VV[3 * nl + 4 * nf + idx] = hw * hd * a[3];
+        T a[4], b1[3], b2[3];
+        visc_jump<T, D>(sm_, jmp, kc, a, b1, b2);
+        VV[2 * nl + idx] = a[1];
+        VV[2 * nl + nf + idx] = T(0);
+        VV[2 * nl + 2 * nf + idx] = a[0];
+        VV[2 * nl + 3 * nf + idx] = a[2];
+        VV[2 * nl + 4 * nf + idx] = a[3];
 #pragma unroll
         for (int i = 0; i < 3; ++i) {
-          T1p[i * nf] = hw * h1 * b1[i];
-          T2p[i * nf] = hw * h2 * b2[i];
+          T1m[i * nf] = see(mT[i], b1[i]);
+          T2m[i * nf] = see(mT[i], b2[i]);
+        }
+        if (!wall) visc_jump<T, D>(sp_, jmp, kc, a, b1, b2);
+        VV[3 * nl + idx] = a[1];
+        VV[3 * nl + nf + idx] = T(0);
+        VV[3 * nl + 2 * nf + idx] = a[0];
+        VV[3 * nl + 3 * nf + idx] = a[2];
+        VV[3 * nl + 4 * nf + idx] = a[3];
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+          T1p[i * nf] = see(mT[i], b1[i]);
+          T2p[i * nf] = see(mT[i], b2[i]);
         }
       } else {
         const T* g = static_cast<const T*>(kp.gfv) + ((size_t)eo[e] * 6 + f) * 13 * N2 + p;
@@ -851,29 +1165,54 @@ __device__ __forceinline__ void coll_face_terms(const double* __restrict__ U, co
 #pragma unroll
             for (int q = 0; q < 5; ++q) {
               const int c = slot_comp<D>(q);
-              dst[b][q * nf] = c == 0 ? T(0) : r[c == 0 ? 0 : c - 1];
+              const T v = c == 0 ? T(0) : r[c == 0 ? 0 : c - 1];
+              dst[b][q * nf] = b < 2 ? see(mT[q], v) : v;
             }
           }
         }
       }
     }
+    if constexpr (FX) {
+#pragma unroll
+      for (int q = 0; q < NTT; ++q) block_max(ex + 15 + q, mT[q]);
+    }
   }
-  if (conv) lines<T, QC, QC, N, 1>(C1, C0, tb.ePc, 5 * nb);
+  bool fixB = false, fixT = false;
+  if constexpr (FX) {
+    fixB = conv && block_ok<5>(ex + 10);
+    if (fixB) chain<QC, QC, N, 1, FROM_DOUBLE, TO_INT>(C1, C0, tb.ePc, 5 * nb, nb * QC, ex + 10, 0);
+  }
+  if (conv && !fixB) sw<T, 1, QC, QC, 1, N, 1>(C1, C0, tb.ePc, 5 * nb);
   __syncthreads();
   // tangential gradient tests, in place; the convective share
-  if (visc) {
+  int gT = 0;
+  if constexpr (FX) {
+    fixT = visc && block_ok<NTT>(ex + 15);
+    if (fixT) {
+      gT = chain_gain(tb.eDvW, 1);
+#pragma unroll
+      for (int sd = 0; sd < 2; ++sd) {
+        double* t1a = TT + sd * nl;
+        double* t2a = TT + (2 + sd) * nl;
+        chain<1, N, N, -1, FROM_DOUBLE, TO_INT>(t1a, t1a, tb.eDvW, NTT * nb * N, nb * N, ex + 15, 0, 1, 0, NTT);
+        chain<N, N, N, -1, FROM_DOUBLE, TO_INT>(t2a, t2a, tb.eDvW, NTT * nb, nb * N, ex + 15, 0, 1, 0, NTT);
+      }
+    }
+    if (fixB) chain<1, QC, N, 1, FROM_INT, TO_DOUBLE>(C0, C1, tb.ePc, 5 * nb * N, nb * N, ex + 10, chain_gain(tb.ePc));
+  }
+  if (visc && !fixT) {
     if (AFF) {
 #pragma unroll
       for (int sd = 0; sd < 2; ++sd) {
-        lines<T, 1, N, N, -1>(TT + sd * nl, TT + sd * nl, tb.eDvW, 3 * nb * N);
-        lines<T, N, N, N, -1>(TT + (2 + sd) * nl, TT + (2 + sd) * nl, tb.eDvW, 3 * nb);
+        sw<T, 0, N, N, 1, N, -1>(TT + sd * nl, TT + sd * nl, tb.eDvW, 3 * nb);
+        sw<T, 1, N, N, 1, N, -1>(TT + (2 + sd) * nl, TT + (2 + sd) * nl, tb.eDvW, 3 * nb);
       }
     } else {
-      lines<T, 1, N, N, -1>(TT, TT, tb.eDvW, 2 * 5 * nb * N);
-      lines<T, N, N, N, -1>(TT + 2 * nl, TT + 2 * nl, tb.eDvW, 2 * 5 * nb);
+      sw<T, 0, N, N, 1, N, -1>(TT, TT, tb.eDvW, 10 * nb);
+      sw<T, 1, N, N, 1, N, -1>(TT + 2 * nl, TT + 2 * nl, tb.eDvW, 10 * nb);
     }
   }
-  if (conv) lines<T, 1, QC, N, 1>(C0, C1, tb.ePc, 5 * nb * N);
+  if (conv && !fixB) sw<T, 0, QC, N, 1, N, 1>(C0, C1, tb.ePc, 5 * nb);
   __syncthreads();
   // shares of the own and the other cell
   for (int idx = threadIdx.x; idx < nl; idx += NTH) {
@@ -885,10 +1224,32 @@ __device__ __forceinline__ void coll_face_terms(const double* __restrict__ U, co
       lp = -lm;
       dm = VV[2 * nl + idx];
       dp = VV[3 * nl + idx];
-      if (AFF) {
-        // tested entries: along t1 (m_D, m_t1, rho E), along t2 (m_D, m_t2, rho E)
-        const int k1 = sl == 2 ? 0 : (sl == 0 ? 1 : (sl == 4 ? 2 : -1));
-        const int k2 = sl == 2 ? 0 : (sl == 3 ? 1 : (sl == 4 ? 2 : -1));
+      // tested entries of an axis-aligned face: along t1 (m_D, m_t1, rho E), along t2 (m_D, m_t2, rho E)
+      const int k1 = !AFF ? sl : (sl == 2 ? 0 : (sl == 0 ? 1 : (sl == 4 ? 2 : -1)));
+      const int k2 = !AFF ? sl : (sl == 2 ? 0 : (sl == 3 ? 1 : (sl == 4 ? 2 : -1)));
+      bool done = false;
+      if constexpr (FX) {
+        if (fixT) {
+          const int k = k1 < 0 ? k2 : k1;
+          if (k >= 0) {
+            const int64_t* t = reinterpret_cast<const int64_t*>(TT) + r;
+            int64_t a = 0, b = 0;
+            if (k1 >= 0) {
+              a = t[k1 * nf];
+              b = t[nl + k1 * nf];
+            }
+            if (k2 >= 0) {
+              a += t[2 * nl + k2 * nf];
+              b += t[3 * nl + k2 * nf];
+            }
+            const int X = fx_exp(ex[15 + k]) + gT + 3;
+            lm += fx_store(a, X);
+            lp += fx_store(b, X);
+          }
+          done = true;
+        }
+      }
+      if (!done) {
         if (k1 >= 0) {
           lm += TT[k1 * nf + r];
           lp += TT[nl + k1 * nf + r];
@@ -897,9 +1258,6 @@ __device__ __forceinline__ void coll_face_terms(const double* __restrict__ U, co
           lm += TT[2 * nl + k2 * nf + r];
           lp += TT[3 * nl + k2 * nf + r];
         }
-      } else {
-        lm += TT[idx] + TT[2 * nl + idx];
-        lp += TT[nl + idx] + TT[3 * nl + idx];
       }
     }
     if (conv) {
@@ -932,7 +1290,7 @@ __device__ __forceinline__ void coll_face_terms(const double* __restrict__ U, co
 
 // blockIdx.y = direction; blocks as dg_face_kernel.
 template <typename T, int N, int QC, int QV, int FB_, int GEO>
-__global__ void __launch_bounds__(coll_face_threads<T>()) dg_coll_face_kernel(const KParams kp,
+__global__ void __launch_bounds__(coll_face_threads<T, N>()) dg_coll_face_kernel(const KParams kp,
                                                                               const double* __restrict__ U,
                                                                               T* __restrict__ FBuf) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -942,6 +1300,8 @@ __global__ void __launch_bounds__(coll_face_threads<T>()) dg_coll_face_kernel(co
   int* eo = reinterpret_cast<int*>(tau_f + FB_);
   int* en = eo + FB_;
   int* oc = en + FB_;
+  uint32_t* ex = reinterpret_cast<uint32_t*>(oc + FB_);
+  if (threadIdx.x < 20) ex[threadIdx.x] = 0;
   const int d = blockIdx.y;
   int s, nb;
   if (!face_batch<FB_>(kp, d, s, nb, eo, en, oc, tau_f)) return;
@@ -951,11 +1311,11 @@ __global__ void __launch_bounds__(coll_face_threads<T>()) dg_coll_face_kernel(co
   const T* Ud = static_cast<const T*>(kp.Udev);
   const int* ocp = kp.flist ? oc : nullptr;
   if (d == 0)
-    coll_face_terms<T, N, QC, QV, FB_, 0, GEO>(U, Ud, eo, en, ocp, tau_f, sm, tb, kp, ph, nb, s, FBuf);
+    coll_face_terms<T, N, QC, QV, FB_, 0, GEO>(U, Ud, eo, en, ocp, tau_f, sm, tb, kp, ph, nb, s, FBuf, ex);
   else if (d == 1)
-    coll_face_terms<T, N, QC, QV, FB_, 1, GEO>(U, Ud, eo, en, ocp, tau_f, sm, tb, kp, ph, nb, s, FBuf);
+    coll_face_terms<T, N, QC, QV, FB_, 1, GEO>(U, Ud, eo, en, ocp, tau_f, sm, tb, kp, ph, nb, s, FBuf, ex);
   else
-    coll_face_terms<T, N, QC, QV, FB_, 2, GEO>(U, Ud, eo, en, ocp, tau_f, sm, tb, kp, ph, nb, s, FBuf);
+    coll_face_terms<T, N, QC, QV, FB_, 2, GEO>(U, Ud, eo, en, ocp, tau_f, sm, tb, kp, ph, nb, s, FBuf, ex);
 }
 
 // Where the collocation kernels are used.
@@ -964,28 +1324,48 @@ constexpr bool coll_ok() {
   return QV == N && coll_rule(N, QV) && GEO != GEO_FLY && coll_cell_smem<T, N, QC, QV, 1>() <= 227 * 1024;
 }
 
-template <typename T, int N, int QC, int QV, int GEO>
-int launch_coll_cell(const KParams& kp, const double* U, void* Rout, void* dU, double* Uout, cudaStream_t st) {
-  constexpr int CB = coll_cells<T, N, QC, QV>();
+// Small meshes: where the usual batches would not give every SM its resident CTAs, half the cells (a third of the
+// faces) per CTA with as many threads, so that the phases of a CTA get shorter.
+constexpr int kSMs = 152;
+
+template <typename T, int N, int QC, int QV, int CB, int GEO>
+int launch_coll_cell_cb(const KParams& kp, const double* U, void* Rout, void* dU, double* Uout, cudaStream_t st) {
   constexpr size_t smem = coll_cell_smem<T, N, QC, QV, CB>();
   static_assert(smem <= 227 * 1024, "cell kernel shared memory");
   auto k = dg_coll_cell_kernel<T, N, QC, QV, CB, GEO>;
   static bool attr[kMaxDevices] = {};
   if (smem_attr_once(k, smem, attr)) return -1;
-  k<<<(kp.Nc + CB - 1) / CB, coll_threads<T, N, QC, QV>(), smem, st>>>(kp, U, static_cast<T*>(Rout), static_cast<T*>(dU), Uout);
+  k<<<(kp.Nc + CB - 1) / CB, coll_threads<T, N, QC, QV>(), smem, st>>>(kp, U, static_cast<T*>(Rout), static_cast<T*>(dU),
+                                                                       Uout);
   return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
-
 template <typename T, int N, int QC, int QV, int GEO>
-int launch_coll_faces(const KParams& kp, const double* U, void* FB, cudaStream_t st) {
-  constexpr int FB_ = coll_faces<T, N, QC, QV>();
+int launch_coll_cell(const KParams& kp, const double* U, void* Rout, void* dU, double* Uout, cudaStream_t st) {
+  constexpr int CB = coll_cells<T, N, QC, QV>();
+  if constexpr (CB > 1) {
+    if (kp.Nc <= CB * kSMs * coll_ctas<T, N, QC, QV, CB>())
+      return launch_coll_cell_cb<T, N, QC, QV, 1, GEO>(kp, U, Rout, dU, Uout, st);
+  }
+  return launch_coll_cell_cb<T, N, QC, QV, CB, GEO>(kp, U, Rout, dU, Uout, st);
+}
+
+template <typename T, int N, int QC, int QV, int FB_, int GEO>
+int launch_coll_faces_fb(const KParams& kp, const double* U, void* FB, cudaStream_t st) {
   constexpr size_t smem = coll_face_smem<T, N, QC, QV, FB_>();
   static_assert(smem <= 227 * 1024, "face kernel shared memory");
   auto k = dg_coll_face_kernel<T, N, QC, QV, FB_, GEO>;
   static bool attr[kMaxDevices] = {};
   if (smem_attr_once(k, smem, attr)) return -1;
-  k<<<dim3(face_blocks(kp, FB_), 3), coll_face_threads<T>(), smem, st>>>(kp, U, static_cast<T*>(FB));
+  k<<<dim3(face_blocks(kp, FB_), 3), coll_face_threads<T, N>(), smem, st>>>(kp, U, static_cast<T*>(FB));
   return cudaGetLastError() == cudaSuccess ? 0 : -1;
+}
+template <typename T, int N, int QC, int QV, int GEO>
+int launch_coll_faces(const KParams& kp, const double* U, void* FB, cudaStream_t st) {
+  constexpr int FB_ = coll_faces<T, N, QC, QV>(), FS = FB_ / 2;
+  if constexpr (FS >= 1) {
+    if (3 * (kp.Nc / FB_) <= 4 * kSMs) return launch_coll_faces_fb<T, N, QC, QV, FS, GEO>(kp, U, FB, st);
+  }
+  return launch_coll_faces_fb<T, N, QC, QV, FB_, GEO>(kp, U, FB, st);
 }
 
 }  // namespace dgcns

@@ -18,7 +18,9 @@ namespace dgcns {
 enum EoOp { EO_SC, EO_SCT, EO_DC, EO_DCT, EO_SV, EO_SVT, EO_DV, EO_DVT, EO_SMI, EO_SMIT, EO_SM, EO_DM,
             // collocation form: W^-1 D^T W at the convective and the viscous points, the projection
             // l_g(x_q) w_q / w_g of the convective points, and W^-1 D^T W extended by the face shares
-            EO_DCW, EO_DVW, EO_PC, EO_LIFT, EO_NOPS };
+            EO_DCW, EO_DVW, EO_PC, EO_LIFT,
+            EO_DL,  // (l_i'(0), l_i'(1)): derivatives at both ends of a nodal line
+            EO_NOPS };
 
 constexpr int eo_size(int dout, int din) { return ((dout + 1) / 2) * (din / 2) * 2 + (dout + 1) / 2; }
 
@@ -28,7 +30,7 @@ struct TableLayout {
   int wc, wv, wm;   // 1D Gauss weights on [0,1]
   int dl0, dl1;     // dl0[i] = l_i'(0), dl1[i] = l_i'(1)
   int total;
-  // FP64 form only, after the `total` doubles: the even-odd operators as scaled integers ({t, 0} and one
+  // FP64 form only, after the `total` doubles: the even-odd operators as scaled integers ({t, SH} and one
   // {high, low} pair per entry, dg_fixed.cuh), 8 bytes each
   int fx[EO_NOPS];
   int total64;
@@ -44,7 +46,7 @@ struct EoDims {
 };
 constexpr EoDims eo_dims(int k, int N, int QC, int QV) {
   const int dims[EO_NOPS][2] = {{QC, N}, {N, QC}, {QC, QC}, {QC, QC}, {QV, N}, {N, QV}, {QV, QV}, {QV, QV},
-                                {N, N},  {N, N},  {N, N},   {N, N},   {QC, QC}, {N, N}, {N, QC},  {N, N + 4}};
+                                {N, N},  {N, N},  {N, N},   {N, N},   {QC, QC}, {N, N}, {N, QC},  {N, N + 4}, {2, N}};
   if (k >= EO_DCW && !coll_rule(N, QV)) return EoDims{0, 0};
   return EoDims{dims[k][0], dims[k][1]};
 }
@@ -83,6 +85,10 @@ struct KConst {
   T rho_r, rhoE_r, p_r, H_r; // reference state, its pressure and rhoE_r + p_r
   T cvTw2;                   // 2 c_v T_wall
   T bf[3];                   // body force
+  T hgm1, g_pr, mu43, mu23;  // (gamma - 1) / 2, gamma p_r, 4/3 and 2/3 of mu
+  T muh[3], lamh[3];         // mu / h_d, lambda / (c_v h_d)
+  // face terms along direction d: mu / (2 h_d h_e) and 4/3, 2/3 of it, lambda / (2 c_v h_d^2)
+  T mus[3][3], mus43[3], mus23[3][3], lams[3];
 };
 
 // Per-launch parameters (passed by value).
@@ -155,6 +161,21 @@ void fill_kconst(const KParams& kp, KConst<T>& c) {
   c.p_r = T((kp.gamma - 1.0) * kp.rhoE_ref);
   c.H_r = T(kp.gamma * kp.rhoE_ref);
   c.cvTw2 = T(2.0 * kp.cv * kp.Tw);
+  c.mu43 = T(4.0 / 3.0 * kp.mu);
+  c.mu23 = T(2.0 / 3.0 * kp.mu);
+  c.hgm1 = T(0.5 * (kp.gamma - 1.0));
+  c.g_pr = T(kp.gamma * (kp.gamma - 1.0) * kp.rhoE_ref);
+  for (int d = 0; d < 3; ++d) {
+    c.muh[d] = T(kp.mu / kp.h[d]);
+    c.lamh[d] = T(kp.lam / kp.cv / kp.h[d]);
+    for (int e = 0; e < 3; ++e) {
+      const double m = 0.5 * kp.mu / (kp.h[d] * kp.h[e]);
+      c.mus[d][e] = T(m);
+      c.mus23[d][e] = T(2.0 / 3.0 * m);
+      if (d == e) c.mus43[d] = T(4.0 / 3.0 * m);
+    }
+    c.lams[d] = T(0.5 * kp.lam / kp.cv / (kp.h[d] * kp.h[d]));
+  }
 }
 
 constexpr int GEO_AFFINE = 0, GEO_STORED = 1, GEO_FLY = 2;

@@ -213,7 +213,7 @@ __device__ __forceinline__ void face_task_body(const KParams& kp, float* __restr
   constexpr int N2 = N * N, N3 = N * N * N, PC = S::PC, PV = S::PV;
   constexpr int d = DIR, t1 = DIR == 0 ? 1 : 0, t2 = DIR == 2 ? 1 : 2;
   const KConst<float>& kc = kconst<float>(kp);
-  const float hinv_d = kc.hinv[d], hinv_1 = kc.hinv[t1], hinv_2 = kc.hinv[t2];
+  const float hinv_d = kc.hinv[d];
   const float sgn = s ? 1.f : -1.f;
   const float* __restrict__ Ud = static_cast<const float*>(kp.Udev);
 
@@ -266,11 +266,12 @@ __device__ __forceinline__ void face_task_body(const KParams& kp, float* __restr
       }
       const float nd[3] = {0.f, 0.f, 0.f};
       float fm[5], fp[5], lm, lp;
-      llf_side<float, DIR, true>(um, nd, sgn, ph, fm, lm);
-      llf_side<float, DIR, true>(up, nd, sgn, ph, fp, lp);
-      const float lam = lm > lp ? lm : lp, w = -0.5f * hinv_d;
+      const float w = -0.5f * hinv_d;
+      llf_side<float, DIR, true>(um, nd, sgn * w, ph, fm, lm);
+      llf_side<float, DIR, true>(up, nd, sgn * w, ph, fp, lp);
+      const float lam = w * (lm > lp ? lm : lp);
 #pragma unroll
-      for (int c = 0; c < 5; ++c) fb[c * PC + p] = w * (fm[c] + fp[c] + lam * (um[c] - up[c]));
+      for (int c = 0; c < 5; ++c) fb[c * PC + p] = fm[c] + fp[c] + lam * (um[c] - up[c]);
     }
   }
 
@@ -294,9 +295,9 @@ __device__ __forceinline__ void face_task_body(const KParams& kp, float* __restr
       auto normal = [&](const SideState<float>& st, const float* v, float f[4]) {
         const float *g1 = v + PV, *g2 = v + 2 * PV;
 #pragma unroll
-        for (int c = 0; c < 5; ++c) gd[c] = hinv_d * v[c * S::VS + 3 * PV];
-        visc_normal<float, DIR>(st, gd, hinv_1 * g1[0], hinv_1 * g1[(1 + d) * S::VS], hinv_1 * g1[(1 + t1) * S::VS],
-                                hinv_2 * g2[0], hinv_2 * g2[(1 + d) * S::VS], hinv_2 * g2[(1 + t2) * S::VS], ph, f);
+        for (int c = 0; c < 5; ++c) gd[c] = v[c * S::VS + 3 * PV];
+        visc_normal<float, DIR>(st, gd, g1[0], g1[(1 + d) * S::VS], g1[(1 + t1) * S::VS], g2[0], g2[(1 + d) * S::VS],
+                                g2[(1 + t2) * S::VS], kc, f);
       };
       normal(sm, vm, fm);
       normal(sp, wall ? vm : vp, fp);  // wall: grad U+ = grad U-, at the ghost state
@@ -311,28 +312,30 @@ __device__ __forceinline__ void face_task_body(const KParams& kp, float* __restr
       v[1 + t1] += wv * (fm[1] + fp[1]);
       v[1 + t2] += wv * (fm[2] + fp[2]);
       v[4] += wv * (fm[3] + fp[3]);
-      const float hd = wv * hinv_d, h1 = wv * hinv_1, h2 = wv * hinv_2;
+      // [[U]] = sgn jmp (x) e_d
+#pragma unroll
+      for (int c = 0; c < 5; ++c) jmp[c] *= sgn;
       auto tests = [&](const SideState<float>& st, float* q, float sg) {
         float a[4], b1[3], b2[3];
-        visc_jump<float, DIR>(st, jmp, ph, a, b1, b2);
+        visc_jump<float, DIR>(st, jmp, kc, a, b1, b2);
 #pragma unroll
         for (int c = 0; c < 5; ++c) q[c * S::VS] = sg * v[c];
         float* q1 = q + PV;
         q1[0] = q1[(1 + t2) * S::VS] = 0.f;
-        q1[(1 + d) * S::VS] = h1 * b1[0];
-        q1[(1 + t1) * S::VS] = h1 * b1[1];
-        q1[4 * S::VS] = h1 * b1[2];
+        q1[(1 + d) * S::VS] = b1[0];
+        q1[(1 + t1) * S::VS] = b1[1];
+        q1[4 * S::VS] = b1[2];
         float* q2 = q + 2 * PV;
         q2[0] = q2[(1 + t1) * S::VS] = 0.f;
-        q2[(1 + d) * S::VS] = h2 * b2[0];
-        q2[(1 + t2) * S::VS] = h2 * b2[1];
-        q2[4 * S::VS] = h2 * b2[2];
+        q2[(1 + d) * S::VS] = b2[0];
+        q2[(1 + t2) * S::VS] = b2[1];
+        q2[4 * S::VS] = b2[2];
         float* q3 = q + 3 * PV;
         q3[0] = 0.f;
-        q3[(1 + d) * S::VS] = hd * a[0];
-        q3[(1 + t1) * S::VS] = hd * a[1];
-        q3[(1 + t2) * S::VS] = hd * a[2];
-        q3[4 * S::VS] = hd * a[3];
+        q3[(1 + d) * S::VS] = a[0];
+        q3[(1 + t1) * S::VS] = a[1];
+        q3[(1 + t2) * S::VS] = a[2];
+        q3[4 * S::VS] = a[3];
       };
       tests(sm, vm, 1.f);
       if (!wall) tests(sp, vp, -1.f);
@@ -415,9 +418,8 @@ constexpr bool task_faces_ok() {
   return N == 4 && coll_rule(N, QV);
 }
 
-template <int N, int QC, int QV>
-int launch_task_faces(const KParams& kp, void* FB, cudaStream_t st) {
-  constexpr int FPB = 12, NTH = 128;
+template <int N, int QC, int QV, int FPB, int NTH>
+int launch_task_faces_fpb(const KParams& kp, void* FB, cudaStream_t st) {
   constexpr size_t smem = task_face_smem_bytes<N, QC, QV, FPB>();
   static_assert(smem <= 227 * 1024, "task face kernel shared memory");
   auto k = dg_face_task_kernel<N, QC, QV, FPB, NTH>;
@@ -425,6 +427,13 @@ int launch_task_faces(const KParams& kp, void* FB, cudaStream_t st) {
   if (smem_attr_once(k, smem, attr)) return -1;
   k<<<dim3(face_blocks(kp, FPB), 3), NTH, smem, st>>>(kp, static_cast<float*>(FB));
   return cudaGetLastError() == cudaSuccess ? 0 : -1;
+}
+// 12 faces and 128 threads per CTA (120 trace and test tasks); on meshes that would not fill the chip with those,
+// 3 faces and one warp.
+template <int N, int QC, int QV>
+int launch_task_faces(const KParams& kp, void* FB, cudaStream_t st) {
+  if (3 * (kp.Nc / 12) <= 4 * kSMs) return launch_task_faces_fpb<N, QC, QV, 3, 32>(kp, FB, st);
+  return launch_task_faces_fpb<N, QC, QV, 12, 128>(kp, FB, st);
 }
 
 }  // namespace dgcns

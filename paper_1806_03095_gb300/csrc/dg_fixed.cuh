@@ -107,6 +107,14 @@ __host__ __device__ __forceinline__ void fx_split(int64_t v, int32_t& h, int32_t
   h = (int32_t)((uint32_t)((uint64_t)v >> 32) + ((uint32_t)(uint64_t)v >> 31));
 }
 
+// What a function that is not inlined cannot see: its pointer is to shared memory (generic loads took 5 % of the
+// face kernel's time).
+#ifdef __CUDA_ARCH__
+#define DGCNS_SHARED(p) __builtin_assume(__isShared(p))
+#else
+#define DGCNS_SHARED(p)
+#endif
+
 struct FxAcc {
   int64_t hh, m;
   __host__ __device__ __forceinline__ void zero() {
@@ -124,18 +132,14 @@ struct FxAcc {
   }
 };
 
-// One line through an operator in even-odd form.  f: {t, 0}, then the even part A [OH][IH], the odd part
-// B [OH][IH] and the middle column C [OH] as {high, low} halves of round(entry 2^t), t the largest scale
-// with (row sum) 2^t <= 2^61.  |sum and difference| of two inputs < 2^62, so the high products add up to
-// less than 2^60; the cross products are folded into them after every two terms (2 (2^61 + 2^60) and the
-// middle column's share stay below 2^63).
-template <int NA, int DIN, int DOUT, int SYM>
-__host__ __device__ __forceinline__ bool fx_line(const int2* __restrict__ f, const double (&x)[NA][DIN],
-                                                 double (&y)[DOUT]) {
+// One line through an operator in even-odd form, integers in, raw sums out (units 2^(64 - t) of the input's).
+// f: {t, SH}, then the even part A [OH][IH], the odd part B [OH][IH] and the middle column C [OH] as {high, low}
+// halves of round(entry 2^t), t the largest scale with (row sum of a half) 2^t <= 2^61.  |sum and difference|
+// of two inputs < 2^62, so the high products add up to less than 2^60; the cross products are folded into them
+// after every two terms (2 (2^61 + 2^60) and the middle column's share stay below 2^63).
+template <int DIN, int DOUT, int SYM>
+__host__ __device__ __forceinline__ void fx_core(const int2* __restrict__ f, const int64_t (&F)[DIN], int64_t (&y)[DOUT]) {
   constexpr int IH = DIN / 2, OH = (DOUT + 1) / 2;
-  int64_t F[DIN];
-  int E;
-  if (!fx_load<NA, DIN>(x, F, E)) return false;
   int32_t eh[IH > 0 ? IH : 1], el[IH > 0 ? IH : 1], oh[IH > 0 ? IH : 1], ol[IH > 0 ? IH : 1], mh = 0, ml = 0;
 #pragma unroll
   for (int i = 0; i < IH; ++i) {
@@ -143,7 +147,6 @@ __host__ __device__ __forceinline__ bool fx_line(const int2* __restrict__ f, con
     fx_split(F[i] - F[DIN - 1 - i], oh[i], ol[i]);
   }
   if (DIN & 1) fx_split(F[IH], mh, ml);
-  const int X = E + 75 - fx_shift<NA>() - f[0].x;
   const int2* __restrict__ A = f + 1;
   const int2* __restrict__ B = A + OH * IH;
   const int2* __restrict__ C = B + OH * IH;
@@ -165,14 +168,43 @@ __host__ __device__ __forceinline__ bool fx_line(const int2* __restrict__ f, con
       }
     }
     if (centre) {
-      y[q] = fx_store(SYM > 0 ? e.hh : o.hh, X);
+      y[q] = SYM > 0 ? e.hh : o.hh;
     } else {
-      y[q] = fx_store(e.hh + o.hh, X);
-      y[DOUT - 1 - q] = fx_store(SYM > 0 ? e.hh - o.hh : o.hh - e.hh, X);
+      y[q] = e.hh + o.hh;
+      y[DOUT - 1 - q] = SYM > 0 ? e.hh - o.hh : o.hh - e.hh;
     }
   }
+}
+
+// The same from and to doubles, with the line's own exponent.
+template <int NA, int DIN, int DOUT, int SYM>
+__host__ __device__ __forceinline__ bool fx_line(const int2* __restrict__ f, const double (&x)[NA][DIN],
+                                                 double (&y)[DOUT]) {
+  int64_t F[DIN], Y[DOUT];
+  int E;
+  if (!fx_load<NA, DIN>(x, F, E)) return false;
+  fx_core<DIN, DOUT, SYM>(f, F, Y);
+  const int X = E + 75 - fx_shift<NA>() - f[0].x;
+#pragma unroll
+  for (int q = 0; q < DOUT; ++q) y[q] = fx_store(Y[q], X);
   return true;
 }
+
+// One value as an integer relative to a block's largest exponent E: x = F 2^(E - 1083), |F| < 2^61.
+__device__ __forceinline__ int64_t fx_of(double x, int E) {
+  const uint32_t h = (uint32_t)__double2hiint(x), l = (uint32_t)__double2loint(x);
+  int s = E - (int)((h >> 20) & 0x7ffu);
+  s = s < 63 ? s : 63;
+  const uint64_t v = ((((uint64_t)((h & 0xfffffu) | 0x100000u) << 32) | l) << 8) >> s;
+  return (int32_t)h < 0 ? -(int64_t)v : (int64_t)v;
+}
+// What a value adds to its block's maximum, and the exponent of a block from it (a block of zeros takes the lowest,
+// so that a sum with another block keeps that block's).
+__device__ __forceinline__ uint32_t fx_mag(double x) {
+  return ((uint32_t)__double2hiint(x) & 0x7fffffffu) | (__double2loint(x) != 0 ? 1u : 0u);
+}
+__device__ __forceinline__ int fx_exp(uint32_t m) { return m ? (int)(m >> 20) : 300; }
+__device__ __forceinline__ bool fx_exp_ok(uint32_t m) { return m == 0 || (m >> 20) - 300u <= 1400u; }
 
 // ---------------------------------------------------------------------------
 // float <-> double on the integer units, bit for bit the hardware conversions (which run on the FP64 pipe, two

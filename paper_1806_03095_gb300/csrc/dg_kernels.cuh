@@ -85,7 +85,7 @@ using Eo = typename EoOf<T>::type;
 template <typename T>
 struct Tab {
   Eo<T> eSc, eScT, eDc, eDcT, eSv, eSvT, eDv, eDvT, eSmi, eSmiT, eSm, eDm;
-  Eo<T> eDcW, eDvW, ePc, eLift;  // collocation form (dg_coll.cuh)
+  Eo<T> eDcW, eDvW, ePc, eLift, eDl;  // collocation form (dg_coll.cuh)
   const T *wc, *wv, *wm, *dl0, *dl1;
 };
 
@@ -137,7 +137,7 @@ __device__ __forceinline__ Tab<T> load_tables(const T* __restrict__ g, T* s) {
   t.eSc = op(EO_SC); t.eScT = op(EO_SCT); t.eDc = op(EO_DC); t.eDcT = op(EO_DCT);
   t.eSv = op(EO_SV); t.eSvT = op(EO_SVT); t.eDv = op(EO_DV); t.eDvT = op(EO_DVT);
   t.eSmi = op(EO_SMI); t.eSmiT = op(EO_SMIT); t.eSm = op(EO_SM); t.eDm = op(EO_DM);
-  t.eDcW = op(EO_DCW); t.eDvW = op(EO_DVW); t.ePc = op(EO_PC); t.eLift = op(EO_LIFT);
+  t.eDcW = op(EO_DCW); t.eDvW = op(EO_DVW); t.ePc = op(EO_PC); t.eLift = op(EO_LIFT); t.eDl = op(EO_DL);
   s -= first;
   t.wc = s + L.wc; t.wv = s + L.wv; t.wm = s + L.wm; t.dl0 = s + L.dl0; t.dl1 = s + L.dl1;
   return t;
@@ -246,6 +246,8 @@ __device__ __forceinline__ void line_apply(Eo<T> E, const T (&x)[DIN], T (&y)[DO
 template <int DIN, int DOUT, int SYM, bool ACC>
 __device__ __noinline__ void fx_sweep(const double* in, double* out, EoFp64 E, int nlines, int n0, uint32_t magic,
                                       int rank, int stride) {
+  DGCNS_SHARED(E.f);
+  DGCNS_SHARED(E.p);
 #pragma unroll 1
   for (int l = rank; l < nlines; l += stride) {
     const int outer = n0 > 1 ? (int)__umulhi((uint32_t)l, magic) : l;
@@ -378,6 +380,7 @@ struct PhysT {
   T gamma, gm1, mu, lam_cv;  // lam_cv = lambda / c_v
   T rho_r, rhoE_r, p_r, H_r; // reference density, energy, pressure, rhoE_r + p_r
   T cvTw2;                   // 2 c_v T_wall
+  T hgm1, g_pr;              // (gamma - 1) / 2, gamma p_r
 };
 
 // pressure deviation p - p_r = (gamma-1)(d(rho E) - |m|^2/(2 rho))
@@ -450,6 +453,8 @@ __device__ __forceinline__ PhysT<T> make_phys(const KParams& kp) {
   ph.p_r = c.p_r;
   ph.H_r = c.H_r;
   ph.cvTw2 = c.cvTw2;
+  ph.hgm1 = c.hgm1;
+  ph.g_pr = c.g_pr;
   return ph;
 }
 

@@ -50,21 +50,20 @@ constexpr int op_threads() {
 }
 
 // Deviation state U - U_ref in FP32 (elementwise pre-pass of the mixed form): 12 bytes a value, so it should run
-// at the memory's rate (conversions by integer operations: 0.34 -> 0.21 ms at 64^3, k = 3).  A CTA converts tiles of kDevCells consecutive cells, four values per thread and
+// at the memory's rate (conversions by integer operations: 0.34 -> 0.21 ms at 64^3, k = 3).  A CTA converts tiles of `cells` consecutive cells (a multiple of 4), four values per thread and
 // access (a tile is a multiple of 16 bytes in both types for every N); the component comes from 32-bit
 // arithmetic within the tile.
-constexpr int kDevCells = 4;  // (16 left half the chip idle at 8^3)
 __device__ __forceinline__ float dev_int(const KParams& kp, double u, int c) {
   if (c == 0 || c == 4) u -= c == 0 ? kp.rho_ref : kp.rhoE_ref;
   return f32_of<float>(u);
 }
 template <int N, bool VEC>
 __global__ void __launch_bounds__(256) dg_dev_kernel(const KParams kp, const double* __restrict__ U,
-                                                     float* __restrict__ D) {
+                                                     float* __restrict__ D, int cells) {
   constexpr int N3 = N * N * N, W = VEC ? 4 : 1;
-  for (int t = blockIdx.x; t * kDevCells < kp.Nc; t += gridDim.x) {
-    const size_t base = (size_t)t * kDevCells * 5 * N3;
-    const int nv = min(kDevCells, kp.Nc - t * kDevCells) * 5 * N3;
+  for (int t = blockIdx.x; t * cells < kp.Nc; t += gridDim.x) {
+    const size_t base = (size_t)t * cells * 5 * N3;
+    const int nv = min(cells, kp.Nc - t * cells) * 5 * N3;
 #pragma unroll 2
     for (int i = threadIdx.x * W; i < nv; i += 256 * W) {
       if (VEC && i + 3 < nv) {
@@ -1048,11 +1047,12 @@ int diag_launch(const KParams& kp, const double* U, const void* LU, double* part
 
 template <int N>
 int dev_launch(const KParams& kp, const double* U, void* D, cudaStream_t st) {
-  const int tiles = (kp.Nc + kDevCells - 1) / kDevCells, grid = tiles < 152 * 16 ? tiles : 152 * 16;
+  const int cells = kp.Nc >= 16 * 152 * 4 ? 16 : 4;  // (tiles of 16 leave half the chip idle at 8^3; of 4, 20 % slower at 64^3)
+  const int tiles = (kp.Nc + cells - 1) / cells, grid = tiles < 152 * 16 ? tiles : 152 * 16;
   if (((reinterpret_cast<uintptr_t>(U) | reinterpret_cast<uintptr_t>(D)) & 15) == 0)
-    dg_dev_kernel<N, true><<<grid, 256, 0, st>>>(kp, U, static_cast<float*>(D));
+    dg_dev_kernel<N, true><<<grid, 256, 0, st>>>(kp, U, static_cast<float*>(D), cells);
   else
-    dg_dev_kernel<N, false><<<grid, 256, 0, st>>>(kp, U, static_cast<float*>(D));
+    dg_dev_kernel<N, false><<<grid, 256, 0, st>>>(kp, U, static_cast<float*>(D), cells);
   return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 

@@ -181,7 +181,7 @@ void put_eo(std::vector<double>& t, int off, const std::vector<double>& O, int d
 }
 
 // The even-odd operator at t + off (oh x ih halves, as put_eo leaves it) as integers at t + fx, for fx_line:
-// {t, 0}, then {high, low} of round(entry 2^t) with the largest t for which (row sum) 2^t <= 2^61.
+// {t, SH}, then {high, low} of round(entry 2^t) with the largest t for which (row sum of a half) 2^t <= 2^61.
 void put_fixed(std::vector<double>& t, int off, int fx, int dout, int din) {
   const int oh = (dout + 1) / 2, ih = din / 2;
   const double *A = &t[off], *B = A + oh * ih, *C = B + oh * ih;
@@ -200,7 +200,18 @@ void put_fixed(std::vector<double>& t, int off, int fx, int dout, int din) {
     const int32_t v[2] = {a, b};
     std::memcpy(&t[at], v, sizeof v);
   };
-  put(fx, 61 - sc, 0);
+  // a sweep from integers below 2^61 to integers below 2^61 shifts its sums by SH: (operator norm) 2^(t - 64 + SH) <= 1
+  double norm = 0.0;
+  for (int q = 0; q < oh; ++q) {
+    double r = std::fabs(C[q]);
+    for (int i = 0; i < ih; ++i) {
+      r += std::fabs(A[q * ih + i] + B[q * ih + i]) + std::fabs(A[q * ih + i] - B[q * ih + i]);
+    }
+    norm = std::max(norm, r);
+  }
+  int sn = 0;
+  std::frexp(norm, &sn);  // norm < 2^sn
+  put(fx, 61 - sc, 64 - (61 - sc) - sn);
   for (int i = 0; i < eo_size(dout, din); ++i) {
     int32_t h, l;
     fx_split((int64_t)std::llrint(std::ldexp(A[i], 61 - sc)), h, l);
@@ -285,6 +296,8 @@ std::vector<double> build_tables(int k, int QC, int QV) {
       r[N + 3] = D[N + g] / wm[g];
     }
     put_eo(t, L.eo[EO_LIFT], F, N, N + 4);
+    lagrange(nodes, std::vector<double>{0.0, 1.0}, V, D);
+    put_eo(t, L.eo[EO_DL], D, 2, N);
   }
   for (int q = 0; q < EO_NOPS; ++q) {
     const EoDims d = eo_dims(q, N, QC, QV);
