@@ -111,7 +111,12 @@ __device__ void adj_cell_terms(const T* su, const T* sy, T* sg, T* ar, const Tab
         ub[c] = T(0);
         const T y0 = B1[o + c * P], y1 = B2[o + c * P], y2 = B3[o + c * P];
 #pragma unroll
-        for (int a = 0; a < 3; ++a) Fb[a][c] = jw * (Ji[a] * y0 + Ji[3 + a] * y1 + Ji[6 + a] * y2);
+        for (int a = 0; a < 3; ++a) {
+          if (GEO == GEO_AFFINE)
+            Fb[a][c] = (jw * Ji[4 * a]) * (a == 0 ? y0 : (a == 1 ? y1 : y2));
+          else
+            Fb[a][c] = jw * (Ji[a] * y0 + Ji[3 + a] * y1 + Ji[6 + a] * y2);
+        }
       }
       conv_flux_vjp(u, Fb, ph, ub);
 #pragma unroll
@@ -169,8 +174,13 @@ __device__ void adj_cell_terms(const T* su, const T* sy, T* sg, T* ar, const Tab
         const T y0 = B1[o + c * P], y1 = B2[o + c * P], y2 = B3[o + c * P];
 #pragma unroll
         for (int a = 0; a < 3; ++a) {
-          G[c][a] = Ji[a] * g0 + Ji[3 + a] * g1 + Ji[6 + a] * g2;
-          Fb[c][a] = jw * (Ji[a] * y0 + Ji[3 + a] * y1 + Ji[6 + a] * y2);
+          if (GEO == GEO_AFFINE) {
+            G[c][a] = Ji[4 * a] * (a == 0 ? g0 : (a == 1 ? g1 : g2));
+            Fb[c][a] = (jw * Ji[4 * a]) * (a == 0 ? y0 : (a == 1 ? y1 : y2));
+          } else {
+            G[c][a] = Ji[a] * g0 + Ji[3 + a] * g1 + Ji[6 + a] * g2;
+            Fb[c][a] = jw * (Ji[a] * y0 + Ji[3 + a] * y1 + Ji[6 + a] * y2);
+          }
           Gb[c][a] = T(0);
         }
       }
@@ -178,9 +188,15 @@ __device__ void adj_cell_terms(const T* su, const T* sy, T* sg, T* ar, const Tab
 #pragma unroll
       for (int c = 0; c < 5; ++c) {
         A0[o + c * P] = ub[c];
-        A1[o + c * P] = Ji[0] * Gb[c][0] + Ji[1] * Gb[c][1] + Ji[2] * Gb[c][2];
-        A2[o + c * P] = Ji[3] * Gb[c][0] + Ji[4] * Gb[c][1] + Ji[5] * Gb[c][2];
-        A3[o + c * P] = Ji[6] * Gb[c][0] + Ji[7] * Gb[c][1] + Ji[8] * Gb[c][2];
+        if (GEO == GEO_AFFINE) {
+          A1[o + c * P] = Ji[0] * Gb[c][0];
+          A2[o + c * P] = Ji[4] * Gb[c][1];
+          A3[o + c * P] = Ji[8] * Gb[c][2];
+        } else {
+          A1[o + c * P] = Ji[0] * Gb[c][0] + Ji[1] * Gb[c][1] + Ji[2] * Gb[c][2];
+          A2[o + c * P] = Ji[3] * Gb[c][0] + Ji[4] * Gb[c][1] + Ji[5] * Gb[c][2];
+          A3[o + c * P] = Ji[6] * Gb[c][0] + Ji[7] * Gb[c][1] + Ji[8] * Gb[c][2];
+        }
       }
     }
     __syncthreads();

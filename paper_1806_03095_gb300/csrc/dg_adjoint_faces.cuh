@@ -18,40 +18,41 @@ namespace dgcns {
 // SIPG face point, both sides: adjoint of val^- (and of val^+ = -val^-) through yvd = Y^- - Y^+,
 // of the own gradient term through ybm (reference derivatives of Y^- at the point) and, unless at a
 // wall, of the other side's gradient term through ybp.  Accumulates umb, Gmb, upb, Gpb.
-template <typename T>
+template <typename T, int DIR, bool AFF>
 __device__ __forceinline__ void sipg_pair_vjp(const T um[5], const T Gm[5][3], const T up[5], const T Gp[5][3],
-                                              const T n[3], const T Jm[9], const T Jp[9], T w, T tau,
+                                              const T n[3], const T Jm[9], const T Jp[9], T w, T ws, T tau,
                                               const T yvd[5], const T ybm[3][5], const T ybp[3][5], bool wall,
                                               const PhysT<T>& ph, T umb[5], T Gmb[5][3], T upb[5], T Gpb[5][3]) {
-  T jmpb[5], Jg[5][3], Jgb[5][3], Fb[5][3];
+  T jmp[5], jmpb[5], Fb[5][3], b[5];
+  const T hw = T(-0.5) * ws;
+  auto grad = [&](const T J[9], const T yb[3][5]) {  // adjoint of F_v(u, [[U]])
+    const T h0 = hw * J[0], h1 = hw * J[4], h2 = hw * J[8];
 #pragma unroll
-  for (int c = 0; c < 5; ++c) {
-    const T jmp = um[c] - up[c];
-    jmpb[c] = w * tau * yvd[c];
+    for (int c = 1; c < 5; ++c) {
+      if (AFF) {
+        Fb[c][0] = h0 * yb[0][c];
+        Fb[c][1] = h1 * yb[1][c];
+        Fb[c][2] = h2 * yb[2][c];
+      } else {
 #pragma unroll
-    for (int a = 0; a < 3; ++a) {
-      Jg[c][a] = jmp * n[a];
-      Jgb[c][a] = T(0);
-      Fb[c][a] = T(-0.5) * w * (Jm[a] * ybm[0][c] + Jm[3 + a] * ybm[1][c] + Jm[6 + a] * ybm[2][c]);
+        for (int a = 0; a < 3; ++a) Fb[c][a] = hw * (J[a] * yb[0][c] + J[3 + a] * yb[1][c] + J[6 + a] * yb[2][c]);
+      }
     }
-  }
-  visc_flux_vjp(um, Jg, Fb, ph, umb, Jgb);
-  if (!wall) {
-#pragma unroll
-    for (int c = 0; c < 5; ++c)
-#pragma unroll
-      for (int a = 0; a < 3; ++a)
-        Fb[c][a] = T(-0.5) * w * (Jp[a] * ybp[0][c] + Jp[3 + a] * ybp[1][c] + Jp[6 + a] * ybp[2][c]);
-    visc_flux_vjp(up, Jg, Fb, ph, upb, Jgb);
-  }
+  };
 #pragma unroll
   for (int c = 0; c < 5; ++c) {
-    jmpb[c] += Jgb[c][0] * n[0] + Jgb[c][1] * n[1] + Jgb[c][2] * n[2];
-#pragma unroll
-    for (int a = 0; a < 3; ++a) Fb[c][a] = T(-0.5) * w * yvd[c] * n[a];
+    jmp[c] = um[c] - up[c];
+    jmpb[c] = w * tau * yvd[c];
+    b[c] = hw * yvd[c];
   }
-  visc_flux_vjp(um, Gm, Fb, ph, umb, Gmb);
-  visc_flux_vjp(up, Gp, Fb, ph, upb, Gpb);
+  grad(Jm, ybm);
+  visc_jump_vjp<T, DIR, AFF>(um, jmp, n, Fb, ph, umb, jmpb);
+  if (!wall) {
+    grad(Jp, ybp);
+    visc_jump_vjp<T, DIR, AFF>(up, jmp, n, Fb, ph, upb, jmpb);
+  }
+  visc_normal_vjp<T, DIR, AFF>(um, Gm, n, b, ph, umb, Gmb);
+  visc_normal_vjp<T, DIR, AFF>(up, Gp, n, b, ph, upb, Gpb);
 #pragma unroll
   for (int c = 0; c < 5; ++c) {
     umb[c] += jmpb[c];
@@ -178,7 +179,7 @@ __device__ void adj_face_pair_terms(const double* __restrict__ U, const T* __res
         upb[c] = T(0);
       }
       if (wall) wall_ghost(um, ph, up);
-      llf_vjp(um, up, nv, w, yd, ph, umb, upb);
+      llf_pair_vjp<T, d, GEO == GEO_AFFINE>(um, up, nv, w, GEO == GEO_AFFINE && !s ? -w : w, yd, ph, umb, upb);
       if (wall) {
         wall_ghost_vjp(um, upb, ph, umb);
 #pragma unroll
@@ -249,8 +250,13 @@ __device__ void adj_face_pair_terms(const double* __restrict__ U, const T* __res
         }
 #pragma unroll
         for (int a = 0; a < 3; ++a) {
-          Gm[c][a] = Jm[a] * gm[0] + Jm[3 + a] * gm[1] + Jm[6 + a] * gm[2];
-          Gp[c][a] = Jp[a] * gp[0] + Jp[3 + a] * gp[1] + Jp[6 + a] * gp[2];
+          if (GEO == GEO_AFFINE) {
+            Gm[c][a] = Jm[4 * a] * gm[a];
+            Gp[c][a] = Jm[4 * a] * gp[a];
+          } else {
+            Gm[c][a] = Jm[a] * gm[0] + Jm[3 + a] * gm[1] + Jm[6 + a] * gm[2];
+            Gp[c][a] = Jp[a] * gp[0] + Jp[3 + a] * gp[1] + Jp[6 + a] * gp[2];
+          }
         }
       }
       if (wall) {
@@ -267,7 +273,8 @@ __device__ void adj_face_pair_terms(const double* __restrict__ U, const T* __res
 #pragma unroll
         for (int a = 0; a < 3; ++a) Gmb[c][a] = Gpb[c][a] = T(0);
       }
-      sipg_pair_vjp(um, Gm, up, Gp, nv, Jm, Jp, w, tau, yvd, ybm, ybp, wall, ph, umb, Gmb, upb, Gpb);
+      sipg_pair_vjp<T, d, GEO == GEO_AFFINE>(um, Gm, up, Gp, nv, Jm, Jp, w, GEO == GEO_AFFINE && !s ? -w : w, tau, yvd,
+                                             ybm, ybp, wall, ph, umb, Gmb, upb, Gpb);
       if (wall) {
         wall_ghost_vjp(um, upb, ph, umb);
 #pragma unroll
@@ -286,8 +293,13 @@ __device__ void adj_face_pair_terms(const double* __restrict__ U, const T* __res
         PT(4)[o + c * P] = upb[c];
 #pragma unroll
         for (int b = 0; b < 3; ++b) {
-          PT(slot[b])[o + c * P] = Jm[3 * b] * Gmb[c][0] + Jm[3 * b + 1] * Gmb[c][1] + Jm[3 * b + 2] * Gmb[c][2];
-          PT(4 + slot[b])[o + c * P] = Jp[3 * b] * Gpb[c][0] + Jp[3 * b + 1] * Gpb[c][1] + Jp[3 * b + 2] * Gpb[c][2];
+          if (GEO == GEO_AFFINE) {
+            PT(slot[b])[o + c * P] = Jm[4 * b] * Gmb[c][b];
+            PT(4 + slot[b])[o + c * P] = Jm[4 * b] * Gpb[c][b];
+          } else {
+            PT(slot[b])[o + c * P] = Jm[3 * b] * Gmb[c][0] + Jm[3 * b + 1] * Gmb[c][1] + Jm[3 * b + 2] * Gmb[c][2];
+            PT(4 + slot[b])[o + c * P] = Jp[3 * b] * Gpb[c][0] + Jp[3 * b + 1] * Gpb[c][1] + Jp[3 * b + 2] * Gpb[c][2];
+          }
         }
       }
     }

@@ -364,6 +364,33 @@ __device__ __forceinline__ void sweep(const T* __restrict__ in, T* __restrict__ 
 }
 
 // ---------------------------------------------------------------------------
+// Reciprocal and square root of the point fluxes.  FP64: the hardware's seed (about 2^-20) and one
+// third-order step, r (1 + e + e^2) with e = 1 - x r (Householder's iteration; the error is e^3 and one
+// rounding): 3 FP64 instructions where the division measured 8 on GB300.  Outside the seed's range (zero,
+// denormal, huge, infinite, NaN) the division itself.
+// ---------------------------------------------------------------------------
+__device__ __forceinline__ float rcp_of(float x) { return 1.f / x; }
+__device__ __forceinline__ double rcp_of(double x) {
+  const uint32_t h = (uint32_t)__double2hiint(x) & 0x7fffffffu;
+  if (h - 0x01000000u > 0x7d000000u) return 1.0 / x;
+  double r;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
+  const double e = fma(-x, r, 1.0);
+  return fma(r, fma(e, e, e), r);
+}
+// sqrt(a), a >= 0: h = a y with y the seed of 1/sqrt(a), e = 1 - h y, h (1 + e/2 + 3 e^2/8).
+__device__ __forceinline__ float sqrt_of(float a) { return sqrtf(a); }
+__device__ __forceinline__ double sqrt_of(double a) {
+  const uint32_t t = (uint32_t)__double2hiint(a);
+  if (t - 0x01000000u > 0x7d000000u) return sqrt(a);
+  double y;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(a));
+  const double h = a * y;
+  const double e = fma(-h, y, 1.0);
+  return fma(h, fma(e, 0.375, 0.5) * e, h);
+}
+
+// ---------------------------------------------------------------------------
 // Pointwise physics (Eq. CompressibleNavierStokesFluxes).  F[c][j], c the
 // conserved component, j the physical direction.
 // ---------------------------------------------------------------------------
