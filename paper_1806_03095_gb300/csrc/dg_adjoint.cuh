@@ -42,6 +42,19 @@ constexpr int adj_cells_per_cta() {
   return cb < 1 ? 1 : (cb > 4 ? 4 : cb);
 }
 
+// Threads of the adjoint kernels: their working sets leave two CTAs per SM, so that 128 threads are only 8 warps an SM.
+// FP32, TGV 24^3, k = 4: cell kernel 0.44 -> 0.34 ms with 256 threads; face kernel 0.60 -> 0.43 ms with 192 threads and
+// 4 faces (256 threads and 6 faces 0.46).  FP64 is not helped: its cell kernel runs the same with 256 (2.80 ms), its
+// face kernel holds 184 registers and is slower with any other number than 128.
+template <typename T, bool PAIR>
+constexpr int adj_cell_threads() {
+  return PAIR && sizeof(T) == 4 ? 256 : NT;
+}
+template <typename T>
+constexpr int adj_face_threads() {
+  return sizeof(T) == 4 ? 192 : NT;
+}
+
 template <typename T, int N, int QC, int QV, int CB, bool PAIR>
 constexpr size_t adj_smem_bytes() {
   return (table_elems<T, N, QC, QV>() + (size_t)CB * adj_cell_elems<N, QC, QV, PAIR>() + CB) * sizeof(T) +
@@ -510,7 +523,7 @@ __device__ void adj_face_terms(const T* su, const T* sy, const T* snu, const T* 
 // G = -(dF/dU)^T Y; out_mode 2: lam_U += dt * (-(dF/dU)^T Y) (RK stage adjoint).
 // ---------------------------------------------------------------------------
 template <typename T, int N, int QC, int QV, int CB, int GEO, bool PAIR>
-__global__ void __launch_bounds__(NT) dg_adj_kernel(const KParams kp, const double* __restrict__ U,
+__global__ void __launch_bounds__(adj_cell_threads<T, PAIR>()) dg_adj_kernel(const KParams kp, const double* __restrict__ U,
                                                     const T* __restrict__ Y, T* __restrict__ G,
                                                     double* __restrict__ lamU) {
   using S = AdjSizes<N, QC, QV>;
@@ -539,8 +552,8 @@ __global__ void __launch_bounds__(NT) dg_adj_kernel(const KParams kp, const doub
       double u;
       T y;
     };
-    constexpr int PER = (CB * 5 * N3 + NT - 1) / NT;
-    batched_pass<PER>(threadIdx.x, NT, nvals, [&](int i) { return UY{U[base + i], Y[base + i]}; }, [&](int i, UY v) {
+    constexpr int NTH = adj_cell_threads<T, PAIR>(), PER = (CB * 5 * N3 + NTH - 1) / NTH;
+    batched_pass<PER>(threadIdx.x, NTH, nvals, [&](int i) { return UY{U[base + i], Y[base + i]}; }, [&](int i, UY v) {
       su[i] = dev_value<T>(kp, v.u, (i / N3) % 5);
       sy[i] = v.y;
       sg[i] = T(0);
@@ -620,7 +633,7 @@ int adj_launch_geo(const KParams& kp, const double* U, const void* Y, void* G, d
   static bool attr[kMaxDevices] = {};
   if (smem_attr_once(k, smem, attr)) return -1;
   const int grid = (kp.Nc + CB - 1) / CB;
-  k<<<grid, NT, smem, st>>>(kp, U, static_cast<const T*>(Y), static_cast<T*>(G), lamU);
+  k<<<grid, adj_cell_threads<T, PAIR>(), smem, st>>>(kp, U, static_cast<const T*>(Y), static_cast<T*>(G), lamU);
   return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 

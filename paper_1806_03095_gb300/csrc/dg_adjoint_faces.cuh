@@ -335,12 +335,13 @@ __device__ void adj_face_pair_terms(const double* __restrict__ U, const T* __res
   }
 }
 
-// Faces per CTA of the adjoint face kernel (<= 8, ~112 KB of shared memory).
+// Faces per CTA of the adjoint face kernel (FP32 <= 4, FP64 <= 8, ~112 KB of shared memory).
 template <typename T, int N, int QC, int QV>
 constexpr int adj_faces_per_cta() {
   constexpr int per_face = AdjPairSizes<N, QC, QV>::PER_FACE * (int)sizeof(T) + 16;
   constexpr int cb = (112 * 1024 - table_elems<T, N, QC, QV>() * (int)sizeof(T)) / per_face;
-  return cb < 1 ? 1 : (cb > 8 ? 8 : cb);
+  constexpr int cap = sizeof(T) == 4 ? 4 : 8;
+  return cb < 1 ? 1 : (cb > cap ? cap : cb);
 }
 
 template <typename T, int N, int QC, int QV, int CB>
@@ -351,7 +352,7 @@ constexpr size_t adj_face_smem_bytes() {
 
 // Grid as the forward face kernel: blockIdx.y = d; upper faces of every cell, then lower walls.
 template <typename T, int N, int QC, int QV, int CB, int GEO>
-__global__ void __launch_bounds__(NT) dg_adj_face_kernel(const KParams kp, const double* __restrict__ U,
+__global__ void __launch_bounds__(adj_face_threads<T>()) dg_adj_face_kernel(const KParams kp, const double* __restrict__ U,
                                                          const T* __restrict__ Y, T* __restrict__ FB) {
   using S = AdjPairSizes<N, QC, QV>;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -434,7 +435,7 @@ int launch_adj_faces(const KParams& kp, const double* U, const void* Y, void* FB
     if (nbk > extra) extra = nbk;
   }
   const dim3 grid((kp.Nc + CB - 1) / CB + extra, 3);
-  k<<<grid, NT, smem, st>>>(kp, U, static_cast<const T*>(Y), static_cast<T*>(FB));
+  k<<<grid, adj_face_threads<T>(), smem, st>>>(kp, U, static_cast<const T*>(Y), static_cast<T*>(FB));
   return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 
