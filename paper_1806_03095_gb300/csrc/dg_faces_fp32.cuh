@@ -252,8 +252,11 @@ __device__ __forceinline__ void face_task_body(const KParams& kp, float* __restr
 
   // 2. convective points: LLF integrand of the own side (the other side's is its negative)
   if (kp.conv) {
-    for (int task = threadIdx.x; task < nb * PC; task += NTH) {
-      const int b = task / PC, p = task - PC * b;
+    // one face per warp and pass: the points of two faces on one warp would share banks
+    static_assert(PC <= 32, "points of a face in one warp");
+    for (int b = threadIdx.x / 32; b < nb; b += NTH / 32) {
+      const int p = threadIdx.x % 32;
+      if (p >= PC) continue;
       float* fb = sface + b * S::PER_FACE;
       float um[5], up[5];
 #pragma unroll
@@ -277,8 +280,10 @@ __device__ __forceinline__ void face_task_body(const KParams& kp, float* __restr
 
   // viscous points: value share (V, Q*.n) and the +1/2 (grad V, F_v(U, [[U]] (x) n)) integrands of both sides
   if (kp.visc) {
-    for (int task = threadIdx.x; task < nb * PV; task += NTH) {
-      const int b = task / PV, p = task - PV * b;
+    // two faces per warp, b and b + 2: their blocks start 16 banks apart (neighbours only 8)
+    for (int task = threadIdx.x; task < ((nb + 3) & ~3) * PV; task += NTH) {
+      const int bt = task / PV, p = task - PV * bt, b = (bt & ~3) | (bt & 1) << 1 | (bt >> 1 & 1);
+      if (b >= nb) continue;
       const bool wall = en[b] < 0;
       float* vm = sface + b * S::PER_FACE + S::CIN + p;
       float* vp = vm + 5 * S::VS;
