@@ -421,6 +421,7 @@ __global__ void __launch_bounds__(coll_threads<T, N, QC, QV>(), coll_ctas<T, N, 
   const Tab<T> tb = load_tables<T, N, QC, QV>(static_cast<const T*>(kp.tables), stab);
   const PhysT<T> ph = make_phys<T>(kp);
   const KConst<T>& kc = kconst<T>(kp);
+  wait_for_predecessor();
   const size_t base = (size_t)e0 * 5 * N3;
   const int nvals = nb * 5 * N3, nbl = nb * 5;
   constexpr int PER = (CB * 5 * N3 + NTH - 1) / NTH;
@@ -1277,9 +1278,10 @@ __global__ void __launch_bounds__(coll_face_threads<T, N>()) dg_coll_face_kernel
   if (threadIdx.x < 20) ex[threadIdx.x] = 0;
   const int d = blockIdx.y;
   int s, nb;
-  if (!face_batch<FB_>(kp, d, s, nb, eo, en, oc, tau_f)) return;
   const Tab<T> tb = load_tables<T, N, QC, QV>(static_cast<const T*>(kp.tables), stab);
   const PhysT<T> ph = make_phys<T>(kp);
+  wait_for_predecessor();
+  if (!face_batch<FB_>(kp, d, s, nb, eo, en, oc, tau_f)) return;
   __syncthreads();
   const T* Ud = static_cast<const T*>(kp.Udev);
   const int* ocp = kp.flist ? oc : nullptr;
@@ -1308,9 +1310,8 @@ int launch_coll_cell_cb(const KParams& kp, const double* U, void* Rout, void* dU
   auto k = dg_coll_cell_kernel<T, N, QC, QV, CB, GEO>;
   static bool attr[kMaxDevices] = {};
   if (smem_attr_once(k, smem, attr)) return -1;
-  k<<<(kp.Nc + CB - 1) / CB, coll_threads<T, N, QC, QV>(), smem, st>>>(kp, U, static_cast<T*>(Rout), static_cast<T*>(dU),
-                                                                       Uout);
-  return cudaGetLastError() == cudaSuccess ? 0 : -1;
+  return launch_after(k, dim3((kp.Nc + CB - 1) / CB), coll_threads<T, N, QC, QV>(), smem, st, kp, U, static_cast<T*>(Rout),
+                      static_cast<T*>(dU), Uout);
 }
 template <typename T, int N, int QC, int QV, int GEO>
 int launch_coll_cell(const KParams& kp, const double* U, void* Rout, void* dU, double* Uout, cudaStream_t st) {
@@ -1329,8 +1330,7 @@ int launch_coll_faces_fb(const KParams& kp, const double* U, void* FB, cudaStrea
   auto k = dg_coll_face_kernel<T, N, QC, QV, FB_, GEO>;
   static bool attr[kMaxDevices] = {};
   if (smem_attr_once(k, smem, attr)) return -1;
-  k<<<dim3(face_blocks(kp, FB_), 3), coll_face_threads<T, N>(), smem, st>>>(kp, U, static_cast<T*>(FB));
-  return cudaGetLastError() == cudaSuccess ? 0 : -1;
+  return launch_after(k, dim3(face_blocks(kp, FB_), 3), coll_face_threads<T, N>(), smem, st, kp, U, static_cast<T*>(FB));
 }
 template <typename T, int N, int QC, int QV, int GEO>
 int launch_coll_faces(const KParams& kp, const double* U, void* FB, cudaStream_t st) {

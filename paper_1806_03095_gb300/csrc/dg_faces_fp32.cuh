@@ -403,9 +403,10 @@ __global__ void __launch_bounds__(NTH) dg_face_task_kernel(const KParams kp, flo
   int* en = eo + FPB;
   const int d = blockIdx.y;
   int s, nb;
-  if (!face_batch<FPB>(kp, d, s, nb, eo, en, en, stau)) return;  // (no orientation codes: structured meshes only)
   const Tab<float> tb = load_tables<float, N, QC, QV>(static_cast<const float*>(kp.tables), stab);
   const PhysT<float> ph = make_phys<float>(kp);
+  wait_for_predecessor();
+  if (!face_batch<FPB>(kp, d, s, nb, eo, en, en, stau)) return;  // (no orientation codes: structured meshes only)
   __syncthreads();
 
   if (d == 0)
@@ -430,8 +431,7 @@ int launch_task_faces_fpb(const KParams& kp, void* FB, cudaStream_t st) {
   auto k = dg_face_task_kernel<N, QC, QV, FPB, NTH>;
   static bool attr[kMaxDevices] = {};
   if (smem_attr_once(k, smem, attr)) return -1;
-  k<<<dim3(face_blocks(kp, FPB), 3), NTH, smem, st>>>(kp, static_cast<float*>(FB));
-  return cudaGetLastError() == cudaSuccess ? 0 : -1;
+  return launch_after(k, dim3(face_blocks(kp, FPB), 3), NTH, smem, st, kp, static_cast<float*>(FB));
 }
 // 12 faces and 128 threads per CTA (120 trace and test tasks); on meshes that would not fill the chip with those,
 // 3 faces and one warp.

@@ -61,6 +61,7 @@ template <int N, bool VEC>
 __global__ void __launch_bounds__(256) dg_dev_kernel(const KParams kp, const double* __restrict__ U,
                                                      float* __restrict__ D, int cells) {
   constexpr int N3 = N * N * N, W = VEC ? 4 : 1;
+  wait_for_predecessor();
   for (int t = blockIdx.x; t * cells < kp.Nc; t += gridDim.x) {
     const size_t base = (size_t)t * cells * 5 * N3;
     const int nv = min(cells, kp.Nc - t * cells) * 5 * N3;
@@ -1050,10 +1051,8 @@ int dev_launch(const KParams& kp, const double* U, void* D, cudaStream_t st) {
   const int cells = kp.Nc >= 16 * 152 * 4 ? 16 : 4;  // (tiles of 16 leave half the chip idle at 8^3; of 4, 20 % slower at 64^3)
   const int tiles = (kp.Nc + cells - 1) / cells, grid = tiles < 152 * 16 ? tiles : 152 * 16;
   if (((reinterpret_cast<uintptr_t>(U) | reinterpret_cast<uintptr_t>(D)) & 15) == 0)
-    dg_dev_kernel<N, true><<<grid, 256, 0, st>>>(kp, U, static_cast<float*>(D), cells);
-  else
-    dg_dev_kernel<N, false><<<grid, 256, 0, st>>>(kp, U, static_cast<float*>(D), cells);
-  return cudaGetLastError() == cudaSuccess ? 0 : -1;
+    return launch_after(dg_dev_kernel<N, true>, dim3(grid), 256, 0, st, kp, U, static_cast<float*>(D), cells);
+  return launch_after(dg_dev_kernel<N, false>, dim3(grid), 256, 0, st, kp, U, static_cast<float*>(D), cells);
 }
 
 // ---------------------------------------------------------------------------
