@@ -21,7 +21,12 @@ __all__ = ["DGCNS", "DGCNSError", "FP64", "MIXED", "KERNEL_SPLIT", "KERNEL_FUSED
 
 
 def _ptr(t):
-    return ctypes.c_void_p(t.data_ptr()) if t is not None else ctypes.c_void_p(0)
+    return t.data_ptr() if t is not None else None
+
+
+# the raw handle of torch's current stream, without a Stream object per call (a call on a small mesh takes the GPU
+# about as long as the binding's own work)
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
 
 
 def cuda_device(device=None):
@@ -79,7 +84,9 @@ class DGCNS:
 
     # -- helpers --------------------------------------------------------------------
     def _stream(self):
-        return ctypes.c_void_p(torch.cuda.current_stream(self.device).cuda_stream)
+        if _raw_stream is not None:
+            return _raw_stream(self.device.index)
+        return torch.cuda.current_stream(self.device).cuda_stream
 
     def _check(self, rc):
         if rc != 0:
@@ -91,7 +98,7 @@ class DGCNS:
     def _state(self, t, name, dtype=torch.float64):
         if not isinstance(t, torch.Tensor) or t.device != self.device or t.dtype != dtype:
             raise TypeError("%s must be a %s tensor on %s" % (name, dtype, self.device))
-        if tuple(t.shape) != self.shape or not t.is_contiguous():
+        if t.shape != self.shape or not t.is_contiguous():
             raise ValueError("%s must be contiguous with shape %s" % (name, self.shape))
         return t
 
