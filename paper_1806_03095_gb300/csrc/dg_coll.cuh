@@ -17,12 +17,15 @@
 // (dg_fixed.cuh), so a phase that holds both sweeps and point fluxes keeps both pipes busy.  On axis-aligned
 // faces the point fluxes form only the normal flux column and the nonzero entries of the jump term.
 //
-// Measured per launch, against the kernels that test with the LGL basis (face / cell + stage kernel):
-// FP64 TGV 64^3, k = 3: 24.6 -> 13.4 / 21.2 -> 14.9 ms; 40^3, k = 5: 14.9 -> 10.9 / 25.7 -> 15.2 ms;
-// FP32 40^3, k = 5: 1.36 -> 1.12 / 2.51 -> 1.30 ms; channel 32^3, k = 3: 0.36 -> 0.29 / 0.36 -> 0.26 ms;
-// FP32 64^3, k = 3, cell + stage: 2.14 (register-resident tasks, one cell per CTA) -> 1.60 ms.
-// Bound by: FP64 faces the FP64 pipe (64 % busy, 6,450 instructions a face); FP64 cells latency and
-// instruction fetch (ALU 46 %, FP64 34 %, issue 43 %).
+// Measured per launch (face / cell + stage kernel), against the kernels that test with the LGL basis and contract in
+// FP64, and with the integer sweeps of both (dg_fixed.cuh):
+// FP64 TGV 64^3, k = 3: 30.5 -> 24.6 -> 11.8 / 32.5 -> 21.2 -> 10.8 ms; 40^3, k = 5: 20.4 -> 14.9 -> 9.3 /
+// 35.8 -> 25.7 -> 13.0 ms; FP64 channel 32^3, k = 3 (stored geometry), with and without the chains of the M^-1 sweeps:
+// cell 1.96 -> 1.78 ms.
+// FP32 40^3, k = 5: 1.36 -> 0.88 / 2.51 -> 1.21 ms; channel 32^3, k = 3: 0.36 -> 0.24 / 0.36 -> 0.24 ms;
+// FP32 64^3, k = 3, cell + stage: 2.14 (register-resident tasks, one cell per CTA) -> 1.39 ms.
+// Bound by: FP64 faces the FP64 pipe in the point phases (60 % busy overall) and latency; FP64 cells latency (ALU and
+// FP64 pipes about 40 % each, four CTAs per SM); FP32 shared-memory wavefronts (82 %) and issue (61 %).
 #pragma once
 #include "dg_chain.cuh"
 #include "dg_faces.cuh"
@@ -384,9 +387,9 @@ constexpr int coll_cells() {
   return cb;
 }
 // Threads: 128, and more where only two (FP64) or four (FP32) large cells fit an SM.  Measured: FP64 k = 3, 2 cells
-// and 128 threads 14.9 ms per stage at 64^3 (192 threads 17.4, one cell 17.9 to 23.6); FP64 k = 5, 40^3, 192 threads
-// 15.2 ms (128: 18.5, 256: 27.0, their registers no longer hold the point fluxes); FP32 k = 5, 256 threads 1.30 ms
-// (128: 1.67, 192: 1.34); FP32 k = 3 stored, 32^3, 2 cells and 128 threads 0.264 ms (256: 0.326; one cell 0.277).
+// and 128 threads 14.9 ms per stage at 64^3 (192 threads 17.4, one cell 17.9 to 23.6), before the chains, now 10.8;
+// FP64 k = 5, 40^3, 192 threads 15.2 ms (128: 18.5, 256: 27.0, their registers no longer hold the point fluxes), now
+// 13.0; FP32 k = 5, 256 threads 1.30 ms (128: 1.67, 192: 1.34), now 1.21; FP32 k = 3 stored, 32^3, 2 cells and 128 threads 0.264 ms (256: 0.326; one cell 0.277).
 template <typename T, int N, int QC, int QV>
 constexpr int coll_threads() {
   constexpr size_t smem = coll_cell_smem<T, N, QC, QV, coll_cells<T, N, QC, QV>()>();
@@ -434,7 +437,7 @@ __global__ void __launch_bounds__(coll_threads<T, N, QC, QV>(), coll_ctas<T, N, 
   // divergence of the convective
   // flux [15] and the first S^-1 sweep's result [20]
   uint32_t* ex = reinterpret_cast<uint32_t*>(Ug + VS);
-  bool fixA = false, fixB = false, fixR = false;  // chains: values, convective flux, residual and M^-1
+  bool fixA = false, fixB = false, fixL = false, fixR = false;  // chains: values, convective flux, lift, residual and M^-1
   if constexpr (FX) {
     constexpr int PV = (CB * N3 + NTH - 1) / NTH;
     double x[5][PV];
@@ -662,7 +665,10 @@ __global__ void __launch_bounds__(coll_threads<T, N, QC, QV>(), coll_ctas<T, N, 
   if constexpr (FX) {
     if (visc) {
 #pragma unroll
-      for (int c = 1; c < 5; ++c) block_max(ex + 10 + c, mag[c]);
+      for (int c = 1; c < 5; ++c) {
+        block_max(ex + 10 + c, mag[c]);
+        mag[c] = 0;
+      }
     }
     fixB = conv && fixA && block_ok<5>(ex + 5);
     if (fixB) {
@@ -680,13 +686,15 @@ __global__ void __launch_bounds__(coll_threads<T, N, QC, QV>(), coll_ctas<T, N, 
   // 6-8. projection of the summed convective parts onto the l_g; D~ and face shares of the viscous arrays
   int gF = 0;  // exponent after the lift over the viscous fluxes' and shares'
   if constexpr (FX) {
-    fixR = fixB && GEO == GEO_AFFINE && !force && kp.out_mode != 0 && block_ok<5>(ex + 10);
+    fixL = block_ok<5>(ex + 10);
+    fixR = fixB && fixL && GEO == GEO_AFFINE && !force && kp.out_mode != 0;
+    gF = chain_gain(tb.eLift, 2);
+    fixL = fixL && (fixR || GEO == GEO_STORED || force || kp.out_mode == 0);  // (else the summed S^-1 sweep takes doubles)
     if (fixB) {
-      gF = chain_gain(tb.eLift, 2);
       chain<QC * QC, QC, N, 1, FROM_SUM, TO_DOUBLE, 0, 0, PC>(F0, F0, tb.ePc, nbl, QC * QC, ex + 5, chain_gain(tb.eDcW, 2), 0,
                                                               CB * 5 * S::F, 5, ex + 15);
     }
-    if (fixR)
+    if (fixL)
       chain_lift<N>(V, FBc, tb.eLift, nb, visc, VS, ex + 10);
     else
       lift_fp64<N>(V, FBc, tb.eLift, nb, visc, VS);
@@ -715,6 +723,8 @@ __global__ void __launch_bounds__(coll_threads<T, N, QC, QV>(), coll_ctas<T, N, 
   __syncthreads();
   // 9-11. M^-1 in the l_g basis is a scaling by 1/|J| (affine: in the flux scales); S^-1 back to the nodes
   T* sr = F2;
+  const Eo<T> eBack = kp.out_mode == 0 ? tb.eSvT : tb.eSmi;
+  int back = 0;  // the chain back to the nodes starts from the pass below
   if constexpr (FX) {
     if (fixR) chain_sum<N>(V, VS, F2, F1, tb.eSmi, nbl * N2, ex + 10, gF, ex + 15, 2 * chain_gain(tb.ePc), ex + 20);
   }
@@ -725,7 +735,13 @@ __global__ void __launch_bounds__(coll_threads<T, N, QC, QV>(), coll_ctas<T, N, 
     for (int i = threadIdx.x; i < nvals; i += NTH) {
       const int p = i % N3, e = i / (5 * N3), c = (i / N3) % 5;
       const int ip = pad(i);
-      T r = F2[ip] + (V[ip] + (V[VS + ip] + V[2 * VS + ip]));
+      T r;
+      if (FX && fixL) {
+        const int64_t* v = reinterpret_cast<const int64_t*>(V) + ip;
+        r = F2[ip] + T(fx_store(v[0] + v[VS] + v[2 * VS], fx_exp(ex[10 + c]) + gF + 3));
+      } else {
+        r = F2[ip] + (V[ip] + (V[VS + ip] + V[2 * VS + ip]));
+      }
       if (kp.out_mode == 0) {
         const T w = tb.wm[p % N] * tb.wm[(p / N) % N] * tb.wm[p / N2];
         r *= GEO == GEO_AFFINE ? -w * kc.detJ : -w;
@@ -739,22 +755,40 @@ __global__ void __launch_bounds__(coll_threads<T, N, QC, QV>(), coll_ctas<T, N, 
         }
       }
       F0[ip] = r;
+      if constexpr (FX) {
+#pragma unroll
+        for (int q = 0; q < 5; ++q) mag[q] = max(mag[q], c == q ? fx_mag(r) : 0u);
+      }
+    }
+    if constexpr (FX) {
+      __syncwarp();
+#pragma unroll
+      for (int q = 0; q < 5; ++q) block_max(ex + 20 + q, mag[q]);
     }
     __syncthreads();
-    sw<T, 0, N, N, N, N, 1, PN, PN>(F0, F1, kp.out_mode == 0 ? tb.eSvT : tb.eSmi, nbl);
+    if constexpr (FX) {
+      fixR = block_ok<5>(ex + 20);
+      if (fixR) chain<1, N, N, 1, FROM_DOUBLE, TO_INT>(F0, F1, eBack, nbl * N2, N2, ex + 20, 0);
+      back = 1;
+    }
+    if (!fixR) sw<T, 0, N, N, N, N, 1, PN, PN>(F0, F1, eBack, nbl);
   }
   __syncthreads();
   if constexpr (FX) {
-    if (fixR) {
+    if (fixR && back) {
+      chain<N, N, N, 1, FROM_INT, TO_INT>(F1, F0, eBack, nbl * N, 1, ex, 0);
+      __syncthreads();
+      chain<N2, N, N, 1, FROM_INT, TO_DOUBLE>(F0, sr, eBack, nbl, N2, ex + 20, 2 * chain_gain(eBack));
+    } else if (fixR) {
       chain<N, N, N, 1, FROM_DOUBLE, TO_INT>(F1, F0, tb.eSmi, nbl * N, N2, ex + 20, 0);
       __syncthreads();
       chain<N2, N, N, 1, FROM_INT, TO_DOUBLE>(F0, sr, tb.eSmi, nbl, N2, ex + 20, chain_gain(tb.eSmi));
     }
   }
   if (!fixR) {
-    sw<T, 1, N, N, N, N, 1, PN, PN>(F1, F0, kp.out_mode == 0 ? tb.eSvT : tb.eSmi, nbl);
+    sw<T, 1, N, N, N, N, 1, PN, PN>(F1, F0, eBack, nbl);
     __syncthreads();
-    sw<T, 2, N, N, N, N, 1, PN, N2>(F0, sr, kp.out_mode == 0 ? tb.eSvT : tb.eSmi, nbl);
+    sw<T, 2, N, N, N, N, 1, PN, N2>(F0, sr, eBack, nbl);
   }
   __syncthreads();
   if (kp.out_mode == 2)

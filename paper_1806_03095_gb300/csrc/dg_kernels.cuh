@@ -45,7 +45,7 @@ struct WarpGroup {
 // be set up while its predecessor on the stream finishes; it loads its 1D tables (constant since dg_cns_create) and
 // then waits, before it touches any array, until the predecessor has finished and its writes are visible.  Every
 // thread of such a kernel passes wait_for_predecessor, so completion is transitive along the stream.  The predecessor
-// gives no early signal: its exit is the signal.  (TGV 8^3, k = 3: mixed L(U), three launches, 24.6 -> 18.7 us, FP64
+// gives no early signal: its exit is the signal.  (TGV 8^3, k = 3: mixed L(U), three launches, 24.6 -> 19.7 us, FP64
 // steps 85.6 -> 80.7 us per stage; with a signal at the start of each kernel the successor's blocks filled the SMs
 // unevenly and L(U) took 28 us.)
 __device__ __forceinline__ void wait_for_predecessor() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
