@@ -973,8 +973,8 @@ int op_dispatch_geo(int mode, const KParams& kp, const double* U, const void* Ri
         // FP32 at k = 3: every block in registers (16-byte aligned arrays, no body force)
         const auto al = [](const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; };
         if (!kp.has_bf && al(Rin) && al(Rout) && al(dU) && al(U) && al(Uout)) {
-          if (kp.out_mode == 2) return launch_mass_reg<N, QC, QV, true>(kp, Rin, Rout, dU, U, Uout, st);
-          return launch_mass_reg<N, QC, QV, false>(kp, Rin, Rout, dU, U, Uout, st);
+          if (kp.out_mode == 2) return launch_mass_stage<N, QC, QV>(kp, Rin, dU, U, Uout, st);
+          return launch_mass_stream<N, QC, QV>(kp, Rin, Rout, st);
         }
       }
       if constexpr (mass_tma_ok<T, N>() && GEO != GEO_FLY && mass_tma_bytes<T, N, QC, QV, true>(1) <= 227 * 1024) {

@@ -249,15 +249,15 @@ int launch_mass_tma(const KParams& kp, const void* Rin, void* Rout, void* dU, co
 
 // ---------------------------------------------------------------------------
 // M^{-1} of FP32 data at k = 3 (affine): one (cell, component) block of N^3 = 64 values per thread, the six
-// 1D sweeps and the scaling in registers (S^-T along x, y, z; 1 / (|J| w); S^-1 along x, y, z).  A CTA
-// takes 128 consecutive blocks (one contiguous range): coalesced 16-byte loads into shared memory rows
-// padded to N^3 + 4 floats (so the 16-byte row reads of 8 neighbouring threads meet distinct banks),
-// the per-thread sweeps, and coalesced 16-byte stores; with STAGE the 2N update (and the next deviation
-// state when kp.devOut is set) runs in that store pass.  No shared-memory traffic inside the sweeps, so
-// the kernel is bound by HBM.  out_mode 0: Rout = M^-1 Rin; 1: Rout = -M^-1 Rin; STAGE: L = -M^-1 Rin.
-// Rin may alias Rout and U may alias Uout (a CTA reads its whole range before it writes).
+// 1D sweeps and the scaling in registers (S^-T along x, y, z; 1 / (|J| w); S^-1 along x, y, z), so that no
+// shared-memory traffic lies inside the sweeps and the kernels are bound by HBM.  Blocks pass through shared-memory
+// rows padded to N^3 + 4 floats (so the 16-byte row reads of 8 neighbouring threads meet distinct banks), with
+// coalesced 16-byte copies on the other side.  Two kernels: M^-1 alone streams tiles per warp; with the stage update
+// (and the next deviation state when kp.devOut is set) a CTA takes 64 consecutive blocks and updates in its store
+// pass.  out_mode 0: Rout = M^-1 Rin; 1: Rout = -M^-1 Rin; stage: L = -M^-1 Rin.  Rin may alias Rout and U may alias
+// Uout (a tile is read before it is written).
 // ---------------------------------------------------------------------------
-constexpr int kMassRegThreads = 128;
+constexpr int kMassRegThreads = 64;
 
 template <int N>
 __device__ __forceinline__ void mass_block_regs(float (&x)[N * N * N], const Tab<float>& tb, float sg_detJinv) {
@@ -322,10 +322,72 @@ __device__ __forceinline__ void mass_block_regs(float (&x)[N * N * N], const Tab
   }
 }
 
-template <int N, int QC, int QV, bool STAGE>
-__global__ void __launch_bounds__(kMassRegThreads) dg_mass_reg_kernel(const KParams kp, const double* U,
-                                                                      const float* Rin, float* Rout, float* dU,
-                                                                      double* Uout) {
+// M^-1 alone: every warp streams tiles of 32 blocks on its own, the copy of its next tile (cp.async) in flight while it
+// sweeps the current one, one block per lane, in rows padded to N^3 + 4 floats (no bank conflicts).  Bound by HBM: 64^3,
+// k = 3, 671 MB, 121 us (5.5 TB/s; 100 us at the rate of a copy).  The kernel that loads, sweeps and stores a CTA's
+// blocks in turn took 153 us (96 registers, 5 CTAs of 128 threads per SM) and 135 us as 11 CTAs of 64 threads.  The 12
+// warps per SM are what 168 registers allow; as 1, 4 or 12 warps per CTA, or 8 warps with two tiles ahead, 119 to 123
+// us; 6 warps with three tiles ahead 131 us.
+constexpr int kMassStreamWarps = 2, kMassStreamCtas = 6, kMassStreamStages = 2;
+template <int N, int QC, int QV>
+__global__ void __launch_bounds__(32 * kMassStreamWarps, kMassStreamCtas)
+    dg_mass_stream_kernel(const KParams kp, const float* Rin, float* Rout) {
+  constexpr int N3 = N * N * N, V4 = N3 / 4, RS = N3 + 4, NS = kMassStreamStages;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  float* stab = reinterpret_cast<float*>(smem_raw);
+  const int w = threadIdx.x / 32, lane = threadIdx.x % 32;
+  float* buf = stab + ((table_elems<float, N, QC, QV>() + 3) & ~3) + w * NS * 32 * RS;
+  const Tab<float> tb = load_tables<float, N, QC, QV>(static_cast<const float*>(kp.tables), stab);
+  const long long nblocks = (long long)kp.Nc * 5, ntiles = (nblocks + 31) / 32;
+  const long long first = (long long)blockIdx.x * kMassStreamWarps + w, step = (long long)gridDim.x * kMassStreamWarps;
+  const float sg = (kp.out_mode != 0 ? -1.f : 1.f) / kconst<float>(kp).detJ;
+  auto fetch = [&](long long t, float* b) {  // always one commit group, empty past the end
+    if (t < ntiles) {
+      const float4* src = reinterpret_cast<const float4*>(Rin + (size_t)t * 32 * N3);
+      const int nv = (int)min((long long)32, nblocks - t * 32) * V4;
+#pragma unroll
+      for (int j = 0; j < V4; ++j) {
+        const int f = j * 32 + lane;
+        if (f < nv)
+          asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_addr(b + f / V4 * RS + f % V4 * 4)),
+                       "l"(src + f)
+                       : "memory");
+      }
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+#pragma unroll
+  for (int q = 0; q < NS - 1; ++q) fetch(first + q * step, buf + q * 32 * RS);
+  __syncthreads();  // the tables
+  int cur = 0;
+  for (long long t = first; t < ntiles; t += step, cur = cur + 1 == NS ? 0 : cur + 1) {
+    float* b = buf + cur * 32 * RS;
+    fetch(t + (NS - 1) * step, buf + (cur == 0 ? NS - 1 : cur - 1) * 32 * RS);
+    asm volatile("cp.async.wait_group %0;" ::"n"(NS - 1) : "memory");
+    __syncwarp();
+    const int nb = (int)min((long long)32, nblocks - t * 32);
+    if (lane < nb) {
+      float x[N3];
+      float* row = b + lane * RS;
+      vec_load<float, N3>(row, x);
+      mass_block_regs<N>(x, tb, sg);
+      vec_store<float, N3>(row, x);
+    }
+    __syncwarp();
+    float4* dst = reinterpret_cast<float4*>(Rout + (size_t)t * 32 * N3);
+#pragma unroll
+    for (int j = 0; j < V4; ++j) {
+      const int f = j * 32 + lane;
+      if (f < nb * V4) dst[f] = *reinterpret_cast<const float4*>(b + f / V4 * RS + f % V4 * 4);
+    }
+    __syncwarp();
+  }
+}
+
+// M^-1 and the stage update.
+template <int N, int QC, int QV>
+__global__ void __launch_bounds__(kMassRegThreads, 8) dg_mass_reg_kernel(const KParams kp, const double* U,
+                                                                      const float* Rin, float* dU, double* Uout) {
   constexpr int N3 = N * N * N, V4 = N3 / 4, RS = N3 + 4, NB = kMassRegThreads;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   float* stab = reinterpret_cast<float*>(smem_raw);
@@ -345,17 +407,10 @@ __global__ void __launch_bounds__(kMassRegThreads) dg_mass_reg_kernel(const KPar
     float x[N3];
     float* row = sb + threadIdx.x * RS;
     vec_load<float, N3>(row, x);
-    const float sg = (STAGE || kp.out_mode != 0) ? -1.f : 1.f;
-    mass_block_regs<N>(x, tb, sg / kconst<float>(kp).detJ);
+    mass_block_regs<N>(x, tb, -1.f / kconst<float>(kp).detJ);
     vec_store<float, N3>(row, x);
   }
   __syncthreads();
-  if (!STAGE) {
-    float4* dst = reinterpret_cast<float4*>(Rout + base);
-    for (int f = threadIdx.x; f < nb * V4; f += kMassRegThreads)
-      dst[f] = reinterpret_cast<const float4*>(sb + (f / V4) * RS)[f % V4];
-    return;
-  }
   const float A = kp.A32, dt = kp.dt32;
   const double B = kp.B;
   const bool readD = kp.A != 0.0;
@@ -408,19 +463,32 @@ constexpr bool mass_reg_ok() {
   return N == 4;
 }
 
-template <int N, int QC, int QV, bool STAGE>
-int launch_mass_reg(const KParams& kp, const void* Rin, void* Rout, void* dU, const double* U, double* Uout,
-                    cudaStream_t st) {
+template <int N, int QC, int QV>
+int launch_mass_stage(const KParams& kp, const void* Rin, void* dU, const double* U, double* Uout, cudaStream_t st) {
   constexpr size_t smem =
       ((size_t)((table_elems<float, N, QC, QV>() + 3) & ~3) + (size_t)kMassRegThreads * (N * N * N + 4)) * sizeof(float) + 64;
   static_assert(smem <= 227 * 1024, "register mass kernel shared memory");
-  auto k = dg_mass_reg_kernel<N, QC, QV, STAGE>;
+  auto k = dg_mass_reg_kernel<N, QC, QV>;
   static bool attr[kMaxDevices] = {};
   if (smem_attr_once(k, smem, attr)) return -1;
   const long long nblocks = (long long)kp.Nc * 5;
   const int grid = (int)((nblocks + kMassRegThreads - 1) / kMassRegThreads);
-  k<<<grid, kMassRegThreads, smem, st>>>(kp, U, static_cast<const float*>(Rin), static_cast<float*>(Rout),
-                                         static_cast<float*>(dU), Uout);
+  k<<<grid, kMassRegThreads, smem, st>>>(kp, U, static_cast<const float*>(Rin), static_cast<float*>(dU), Uout);
+  return cudaGetLastError() == cudaSuccess ? 0 : -1;
+}
+
+template <int N, int QC, int QV>
+int launch_mass_stream(const KParams& kp, const void* Rin, void* Rout, cudaStream_t st) {
+  constexpr size_t smem = ((size_t)((table_elems<float, N, QC, QV>() + 3) & ~3) +
+                           (size_t)kMassStreamWarps * kMassStreamStages * 32 * (N * N * N + 4)) * sizeof(float) + 64;
+  static_assert(smem + 1024 <= 227 * 1024 / kMassStreamCtas, "resident CTAs");
+  auto k = dg_mass_stream_kernel<N, QC, QV>;
+  static bool attr[kMaxDevices] = {};
+  if (smem_attr_once(k, smem, attr)) return -1;
+  const long long tiles = ((long long)kp.Nc * 5 + 31) / 32, ctas = (tiles + kMassStreamWarps - 1) / kMassStreamWarps;
+  constexpr int kResident = 152 * kMassStreamCtas;
+  k<<<(int)(ctas < kResident ? ctas : kResident), 32 * kMassStreamWarps, smem, st>>>(kp, static_cast<const float*>(Rin),
+                                                                                static_cast<float*>(Rout));
   return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 }  // namespace dgcns

@@ -63,3 +63,29 @@ def test_non_finite_values_stay_in_their_block(bad):
     keep = torch.ones(g.shape[:2], dtype=torch.bool)
     keep[7, 2] = False
     assert torch.equal(out[keep], clean[keep])
+
+
+@pytest.mark.parametrize("in_place", [False, True])
+@pytest.mark.parametrize("cells", [(2, 2, 2), (3, 2, 5), (23, 23, 23)])
+def test_inverse_mass_of_fp32_residuals(cells, in_place):
+    """Fewer blocks than a tile of 32 per warp, a ragged last tile, and more tiles than resident warps."""
+    n, k = 4, 3
+    g = api.DGCNS(cells, (-math.pi,) * 3, (math.pi,) * 3, (1, 1, 1), k, 5, 4, precision=api.MIXED)
+    r = (torch.rand(g.shape, generator=torch.Generator().manual_seed(5)) * 2 - 1).float()
+    rg = r.cuda()
+    out = g.inverse_mass(rg, rg) if in_place else g.inverse_mass(rg)
+    if not in_place:
+        assert torch.equal(rg.cpu(), r)
+    Si, w = _one(k)
+    W = 1.0 / (np.einsum("z,y,x->zyx", w, w, w) * np.prod([2 * math.pi / c for c in cells]))
+    b = a = r.double().numpy().reshape(-1, 5, n, n, n)
+    for ax in (2, 3, 4):
+        b = np.moveaxis(np.tensordot(Si.T, b, (1, ax)), 0, ax)
+    b = b * W
+    for ax in (2, 3, 4):
+        b = np.moveaxis(np.tensordot(Si, b, (1, ax)), 0, ax)
+    # six sweeps and the scaling, each with its rounded table at most 8 2^-24 of its largest input times its row sum
+    amp = np.abs(Si.T).sum(1).max() ** 3 * W.max() * np.abs(Si).sum(1).max() ** 3
+    tol = 7 * 8 * 2.0 ** -24 * amp * np.abs(a).reshape(a.shape[0], 5, -1).max(-1)
+    err = np.abs(out.cpu().double().numpy().reshape(b.shape) - b).reshape(a.shape[0], 5, -1).max(-1)
+    assert (err <= tol).all(), float((err / tol).max())
