@@ -1271,7 +1271,7 @@ __global__ void __launch_bounds__(WPC * 32) dg_face_warp_kernel(const KParams kp
 template <typename T, int N, int QC, int QV, int GEO>
 int launch_faces(const KParams& kp, const double* U, void* FB, cudaStream_t st) {
   if constexpr (use_coll<T, N, QC, QV, GEO>()) {
-    // FP32 affine at k = 3: the register-resident kernel (1.39 ms against 1.63 ms per launch at 64^3, measured)
+    // FP32 affine at k = 3: the register-resident kernel (1.13 ms against 1.46 ms per launch at 64^3, measured)
     if constexpr (sizeof(T) == 4 && GEO == GEO_AFFINE && task_faces_ok<N, QC, QV>()) {
       if (kp.Udev != nullptr && kp.flist == nullptr && (reinterpret_cast<uintptr_t>(kp.Udev) & 15) == 0)
         return launch_task_faces<N, QC, QV>(kp, FB, st);

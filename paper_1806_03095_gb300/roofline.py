@@ -3,7 +3,10 @@
 Counts mirror the kernels' structure: every 1D sweep line with DIN inputs and
 DOUT outputs costs 2*DIN*DOUT flops (one FMA = 2 flops), pointwise work uses
 per-point operation counts of the flux routines (a division or square root
-counts as one flop).  Bytes are the algorithmic HBM traffic of one launch
+counts as one flop).  The counts are those of testing with the nodal basis; the
+collocation form (q_visc = k+1) cancels six cell and eight face sweeps, and the
+FP64 kernels contract in integer arithmetic, so a rate above the FP64 FMA peak
+is possible.  Bytes are the algorithmic HBM traffic of one launch
 (each array read or written once).
 """
 
