@@ -39,14 +39,14 @@ FP32_PEAK_TFLOPS = 73.5  # measured FP32 FMA throughput, same probe
 # (kind, precision 0/1, N, QC, QV) -> (bytes per cell, sources digest, profile summary under profiles/).
 # The roofline reports traffic = bytes per cell x cells only while the sources still have that digest.
 TRAFFIC = {
-    ("faces", 0, 4, 5, 4): (15115.6, "cc826ba75499d748a67d4103685ebe4090f2818998df31d1db553338e0ad948a",
-                            "profiles/face_centric_fp64_tgv64_k3_launches.md"),
-    ("cell_stage", 0, 4, 5, 4): (17651.0, "cc826ba75499d748a67d4103685ebe4090f2818998df31d1db553338e0ad948a",
-                                 "profiles/face_centric_fp64_tgv64_k3_launches.md"),
-    ("faces", 1, 4, 5, 4): (7333.7, "cc826ba75499d748a67d4103685ebe4090f2818998df31d1db553338e0ad948a",
-                            "profiles/dg_face_task_kernel_mixed_tgv48_k3.md"),
-    ("cell_stage", 1, 4, 5, 4): (13743.6, "cc826ba75499d748a67d4103685ebe4090f2818998df31d1db553338e0ad948a",
-                                 "profiles/dg_cell_task_kernel_mixed_tgv48_k3.md"),
+    ("faces", 0, 4, 5, 4): (15079.6, "7b418df6514491a66e56887a02c9aeca47a856f9f6f22fffa02619783930d26d",
+                            "profiles/collocation_kernels_tgv48_k3.md"),
+    ("cell_stage", 0, 4, 5, 4): (17673.7, "7b418df6514491a66e56887a02c9aeca47a856f9f6f22fffa02619783930d26d",
+                                 "profiles/collocation_kernels_tgv48_k3.md"),
+    ("faces", 1, 4, 5, 4): (7332.0, "7b418df6514491a66e56887a02c9aeca47a856f9f6f22fffa02619783930d26d",
+                            "profiles/collocation_kernels_tgv48_k3.md"),
+    ("cell_stage", 1, 4, 5, 4): (13750.6, "7b418df6514491a66e56887a02c9aeca47a856f9f6f22fffa02619783930d26d",
+                                 "profiles/collocation_kernels_tgv48_k3.md"),
 }
 
 
