@@ -50,9 +50,9 @@ constexpr int op_threads() {
 }
 
 // Deviation state U - U_ref in FP32 (elementwise pre-pass of the mixed form): 12 bytes a value, so it should run
-// at the memory's rate (conversions by integer operations: 0.34 -> 0.21 ms at 64^3, k = 3).  A CTA converts tiles of `cells` consecutive cells (a multiple of 4), four values per thread and
-// access (a tile is a multiple of 16 bytes in both types for every N); the component comes from 32-bit
-// arithmetic within the tile.
+// at the memory's rate (conversions by integer operations: 0.34 -> 0.21 ms at 64^3, k = 3).  A CTA converts tiles of
+// `cells` consecutive cells (a multiple of 4), four values per thread and access (a tile is a multiple of 16 bytes in
+// both types for every N); the component comes from 32-bit arithmetic within the tile.
 __device__ __forceinline__ float dev_int(const KParams& kp, double u, int c) {
   if (c == 0 || c == 4) u -= c == 0 ? kp.rho_ref : kp.rhoE_ref;
   return f32_of<float>(u);
@@ -793,9 +793,16 @@ constexpr int warp_slice_elems() {
   return (e + 7) & ~7;
 }
 
+// Elements before the first slice.  The face kernel of the split organisation keeps the room of all 1D tables, though
+// it copies only the weights: without it the kernel is slower (2.59 ms against 2.44 ms at 48^3, k = 3).
+template <typename T, int N, int QC, int QV, bool CELL, bool FACE>
+constexpr int warp_table_elems() {
+  return FACE && !CELL ? make_layout(N, QC, QV).total : table_elems<T, N, QC, QV>();
+}
+
 template <typename T, int N, int QC, int QV, int WPC, bool CELL, bool FACE, bool MASS, int GEO>
 constexpr size_t warp_smem_bytes() {
-  return ((size_t)table_elems<T, N, QC, QV>() +
+  return ((size_t)warp_table_elems<T, N, QC, QV, CELL, FACE>() +
           (size_t)WPC * warp_slice_elems<T, N, QC, QV, CELL, FACE, MASS, GEO>()) * sizeof(T) + 64;
 }
 
@@ -814,7 +821,7 @@ __global__ void __launch_bounds__(WPC * 32) dg_op_warp_kernel(const KParams kp, 
   const int e0 = blockIdx.x * WPC + w;
   if (e0 >= kp.Nc) return;  // only warp barriers below
   const WarpGroup grp;
-  T* su = stab + table_elems<T, N, QC, QV>() + w * SL;
+  T* su = stab + warp_table_elems<T, N, QC, QV, CELL, FACE>() + w * SL;
   T* sr = su + 5 * N3;
   T* sn = sr + 5 * N3;
   T* ar = sn + (FACE ? 5 * N3 : 0);
