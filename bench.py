@@ -59,7 +59,7 @@ def kernel_digest():
         if name.endswith((".cuh", ".h")) or name == "dg_inst.cu":
             h.update(name.encode())
             h.update(open(os.path.join(build.CSRC, name), "rb").read())
-    h.update(" ".join(build.ARCH + build.FLAGS).encode())
+    h.update(" ".join(build.ARCH + [f for f in build.FLAGS if not os.path.isabs(f)]).encode())  # (no include paths)
     return h.hexdigest()
 
 
