@@ -39,13 +39,13 @@ FP32_PEAK_TFLOPS = 73.5  # measured FP32 FMA throughput, same probe
 # (kind, precision 0/1, N, QC, QV) -> (bytes per cell, sources digest, profile summary under profiles/).
 # The roofline reports traffic = bytes per cell x cells only while the sources still have that digest.
 TRAFFIC = {
-    ("faces", 0, 4, 5, 4): (15079.6, "7b418df6514491a66e56887a02c9aeca47a856f9f6f22fffa02619783930d26d",
+    ("faces", 0, 4, 5, 4): (15098.0, "fe3a2cccb0f35e22aeca52de0a8521be427c037633c16de9050e65b32e1c6b39",
                             "profiles/collocation_kernels_tgv48_k3.md"),
-    ("cell_stage", 0, 4, 5, 4): (17673.7, "7b418df6514491a66e56887a02c9aeca47a856f9f6f22fffa02619783930d26d",
+    ("cell_stage", 0, 4, 5, 4): (17644.5, "fe3a2cccb0f35e22aeca52de0a8521be427c037633c16de9050e65b32e1c6b39",
                                  "profiles/collocation_kernels_tgv48_k3.md"),
-    ("faces", 1, 4, 5, 4): (7332.0, "7b418df6514491a66e56887a02c9aeca47a856f9f6f22fffa02619783930d26d",
+    ("faces", 1, 4, 5, 4): (7331.9, "fe3a2cccb0f35e22aeca52de0a8521be427c037633c16de9050e65b32e1c6b39",
                             "profiles/collocation_kernels_tgv48_k3.md"),
-    ("cell_stage", 1, 4, 5, 4): (13750.6, "7b418df6514491a66e56887a02c9aeca47a856f9f6f22fffa02619783930d26d",
+    ("cell_stage", 1, 4, 5, 4): (13723.3, "fe3a2cccb0f35e22aeca52de0a8521be427c037633c16de9050e65b32e1c6b39",
                                  "profiles/collocation_kernels_tgv48_k3.md"),
 }
 
