@@ -167,7 +167,7 @@ __device__ __noinline__ void chain_sum(const double* V, int ks, const double* P,
 
 // V_d <- D~_d V_d + the face shares of direction d (lift_body), doubles in, integers out, block exponents ex.
 template <int N, int D>
-__device__ __forceinline__ void chain_lift_dir(double* V, const double* __restrict__ F, EoFp64 E, int nb, bool vol,
+__device__ __forceinline__ void chain_lift_dir(double* V, const double* F, EoFp64 E, int nb, bool vol,
                                                const uint32_t* ex) {
   constexpr int N2 = N * N, N3 = N2 * N, st = D == 0 ? 1 : (D == 1 ? N : N2);
   const int sh = E.f[0].y - 2;

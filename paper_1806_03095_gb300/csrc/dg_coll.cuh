@@ -174,7 +174,7 @@ __device__ __forceinline__ void sw(const T* in, T* out, Eo<T> E, int nblk, int k
 // shares [nb][6][2][5][N^2] (global).  The line's operator takes D_0, L_0, the N values, -L_1, D_1: with the sign
 // of L_1 it is antisymmetric under reflection like D~ itself.
 template <typename T, int N, int D>
-__device__ __forceinline__ void lift_body(T* V, const T* __restrict__ F, Eo<T> E, int nb, bool vol) {
+__device__ __forceinline__ void lift_body(T* V, const T* F, Eo<T> E, int nb, bool vol) {
   constexpr int N2 = N * N, PS = plane_stride<T>(N, N), st = D == 0 ? 1 : (D == 1 ? N : PS);
   for (int l = threadIdx.x; l < nb * 5 * N2; l += blockDim.x) {
     const int ec = l / N2, j = l - ec * N2, e = ec / 5, c = ec - 5 * e, j1 = j % N, j2 = j / N;
@@ -404,7 +404,7 @@ constexpr int coll_ctas() {  // resident CTAs that the registers have to allow
 // kp.out_mode: 0 writes F(U), 1 L(U), 2 the stage update (as dg_op_kernel).
 template <typename T, int N, int QC, int QV, int CB, int GEO>
 __global__ void __launch_bounds__(coll_threads<T, N, QC, QV>(), coll_ctas<T, N, QC, QV, CB>())
-    dg_coll_cell_kernel(const KParams kp, const double* __restrict__ U,
+    dg_coll_cell_kernel(const KParams kp, const double* U,
                                                                          T* Rout, T* dU, double* Uout) {
   static_assert(QV == N && GEO != GEO_FLY, "collocation form");
   using S = CollSizes<T, N, QC>;
@@ -837,9 +837,9 @@ constexpr int coll_face_threads() {
 }
 
 template <typename T, int N, int QC, int QV, int FB_, int D, int GEO>
-__device__ __forceinline__ void coll_face_terms(const double* __restrict__ U, const T* __restrict__ Ud, const int* eo,
+__device__ __forceinline__ void coll_face_terms(const double* U, const T* Ud, const int* eo,
                                                 const int* en, const int* oc, const T* tau_f, T* sm, const Tab<T>& tb,
-                                                const KParams& kp, const PhysT<T>& ph, int nb, int s, T* __restrict__ FBuf,
+                                                const KParams& kp, const PhysT<T>& ph, int nb, int s, T* FBuf,
                                                 uint32_t* ex) {
   using Z = CollFaceSizes<N, QC>;
   constexpr int N2 = N * N, N3 = N2 * N, QC2 = QC * QC, NTH = coll_face_threads<T, N>();
@@ -1299,8 +1299,7 @@ __device__ __forceinline__ void coll_face_terms(const double* __restrict__ U, co
 // blockIdx.y = direction; blocks as dg_face_kernel.
 template <typename T, int N, int QC, int QV, int FB_, int GEO>
 __global__ void __launch_bounds__(coll_face_threads<T, N>()) dg_coll_face_kernel(const KParams kp,
-                                                                              const double* __restrict__ U,
-                                                                              T* __restrict__ FBuf) {
+                                                                              const double* U, T* FBuf) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   T* stab = reinterpret_cast<T*>(smem_raw);
   T* sm = stab + table_elems<T, N, QC, QV>();

@@ -130,7 +130,7 @@ __device__ __forceinline__ void eo_dir1(const float* __restrict__ E, const float
 // (j1 along the first tangent, fastest) of one component block src [N^3] of a cell, the face at layer
 // id (0 or N-1) along direction DIR; the block is read as its N^2 x-lines.
 template <int N, int DIR>
-__device__ __forceinline__ void face_traces(const float* __restrict__ src, const float* __restrict__ dl, int id,
+__device__ __forceinline__ void face_traces(const float* src, const float* __restrict__ dl, int id,
                                             float (&L)[N * N], float (&D)[N * N]) {
   const bool last = id != 0;
 #pragma unroll
@@ -206,7 +206,7 @@ constexpr size_t task_face_smem_bytes() {
 // Phases 1-4 of the task kernel for faces normal to direction DIR (compile-time, so that the small
 // per-point arrays indexed by direction stay in registers).
 template <int N, int QC, int QV, int FPB, int NTH, int DIR>
-__device__ __forceinline__ void face_task_body(const KParams& kp, float* __restrict__ FB, const Tab<float>& tb,
+__device__ __forceinline__ void face_task_body(const KParams& kp, float* FB, const Tab<float>& tb,
                                                const PhysT<float>& ph, float* sface, const float* stau, const int* eo,
                                                const int* en, int nb, int s) {
   using S = TaskFaceSizes<N, QC, QV>;
@@ -215,7 +215,7 @@ __device__ __forceinline__ void face_task_body(const KParams& kp, float* __restr
   const KConst<float>& kc = kconst<float>(kp);
   const float hinv_d = kc.hinv[d];
   const float sgn = s ? 1.f : -1.f;
-  const float* __restrict__ Ud = static_cast<const float*>(kp.Udev);
+  const float* Ud = static_cast<const float*>(kp.Udev);
 
   // 1. trace tasks (face b, side sd: 0 own / 1 other, component c)
   for (int task = threadIdx.x; task < nb * 10; task += NTH) {
@@ -224,7 +224,7 @@ __device__ __forceinline__ void face_task_body(const KParams& kp, float* __restr
     if (cell < 0) continue;  // wall: the ghost state is formed at the points
     const int id = (sd ? 1 - s : s) ? N - 1 : 0;  // the face's layer index along d in this cell
     const float* dl = (sd ? 1 - s : s) ? tb.dl1 : tb.dl0;
-    const float* __restrict__ src = Ud + ((size_t)cell * 5 + c) * N3;
+    const float* src = Ud + ((size_t)cell * 5 + c) * N3;
     float L[N2], D[N2];
     face_traces<N, DIR>(src, dl, id, L, D);
     float* fb = sface + b * S::PER_FACE;
@@ -393,7 +393,7 @@ __device__ __forceinline__ void face_task_body(const KParams& kp, float* __restr
 }
 
 template <int N, int QC, int QV, int FPB, int NTH>
-__global__ void __launch_bounds__(NTH) dg_face_task_kernel(const KParams kp, float* __restrict__ FB) {
+__global__ void __launch_bounds__(NTH) dg_face_task_kernel(const KParams kp, float* FB) {
   using S = TaskFaceSizes<N, QC, QV>;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   float* stab = reinterpret_cast<float*>(smem_raw);

@@ -48,6 +48,9 @@ struct WarpGroup {
 // gives no early signal: its exit is the signal.  (TGV 8^3, k = 3: mixed L(U), three launches, 24.6 -> 19.7 us, FP64
 // steps 85.6 -> 80.7 us per stage; with a signal at the start of each kernel the successor's blocks filled the SMs
 // unevenly and L(U) took 28 us.)
+// An array that a predecessor may write (state, deviation state, face shares, increment) is not a __restrict__ pointer
+// in such a kernel: `const __restrict__` would promise constant data from the kernel's start, which is now before the
+// wait, and allow loads that the wait does not order.
 __device__ __forceinline__ void wait_for_predecessor() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 template <class... P, class... A>

@@ -58,8 +58,7 @@ __device__ __forceinline__ float dev_int(const KParams& kp, double u, int c) {
   return f32_of<float>(u);
 }
 template <int N, bool VEC>
-__global__ void __launch_bounds__(256) dg_dev_kernel(const KParams kp, const double* __restrict__ U,
-                                                     float* __restrict__ D, int cells) {
+__global__ void __launch_bounds__(256) dg_dev_kernel(const KParams kp, const double* U, float* D, int cells) {
   constexpr int N3 = N * N * N, W = VEC ? 4 : 1;
   wait_for_predecessor();
   for (int t = blockIdx.x; t * cells < kp.Nc; t += gridDim.x) {
