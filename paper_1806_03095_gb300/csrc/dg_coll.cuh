@@ -375,7 +375,8 @@ struct CollSizes {
 };
 template <typename T, int N, int QC, int QV, int CB>
 constexpr size_t coll_cell_smem() {
-  return ((size_t)table_elems<T, N, QC, QV>() + (size_t)CB * CollSizes<T, N, QC>::PER_CELL) * sizeof(T) + 192;
+  return ((size_t)table_elems<T, N, QC, QV>() + (size_t)CB * CollSizes<T, N, QC>::PER_CELL) * sizeof(T) +
+         (sizeof(T) == 8 ? 25 * CB * sizeof(uint32_t) : 0) + 64;
 }
 
 // Cells per CTA and threads.
@@ -433,46 +434,56 @@ __global__ void __launch_bounds__(coll_threads<T, N, QC, QV>(), coll_ctas<T, N, 
   const T* FBc = static_cast<const T*>(kp.fbuf) + (size_t)e0 * fbuf_per_cell<N>();
   const bool conv = kp.conv != 0, visc = kp.visc != 0;
   const bool force = kp.has_bf && kp.out_mode != 0;
-  // FP64: per-component maxima of the state [0], the convective flux [5], the viscous flux and the face shares [10];
-  // divergence of the convective
-  // flux [15] and the first S^-1 sweep's result [20]
-  uint32_t* ex = reinterpret_cast<uint32_t*>(Ug + VS);
+  // FP64: maxima of the blocks (cell, component): of the state, of the convective flux, of the viscous flux and the face
+  // shares, of the divergence of the convective flux, of the first S^-1 sweep's result
+  uint32_t* exU = reinterpret_cast<uint32_t*>(Ug + VS);
+  uint32_t *exC = exU + 5 * CB, *exV = exC + 5 * CB, *exP = exV + 5 * CB, *exR = exP + 5 * CB;
+  // FP64: the point phases give each cell its own warps, so that a thread's maxima belong to one cell
+  constexpr int NTE = FX ? NTH / CB : NTH;
+  static_assert(!FX || NTE % 32 == 0, "whole warps per cell");
+  const int pe = FX ? threadIdx.x / NTE : 0, pt = FX ? threadIdx.x % NTE : threadIdx.x;
   bool fixA = false, fixB = false, fixL = false, fixR = false;  // chains: values, convective flux, lift, residual and M^-1
   if constexpr (FX) {
-    constexpr int PV = (CB * N3 + NTH - 1) / NTH;
+    constexpr int PV = (N3 + NTE - 1) / NTE;
+    const bool own = pe < nb;
     double x[5][PV];
 #pragma unroll
     for (int c = 0; c < 5; ++c)
 #pragma unroll
       for (int k = 0; k < PV; ++k) {
-        const int i = k * NTH + threadIdx.x, e = i / N3;
-        x[c][k] = i < nb * N3 ? U[base + (size_t)e * 4 * N3 + c * N3 + i] : 0.0;
+        const int i = k * NTE + pt;
+        x[c][k] = own && i < N3 ? U[base + (pe * 5 + c) * N3 + i] : 0.0;
       }
-    if (threadIdx.x < 25) ex[threadIdx.x] = 0;
+    if (threadIdx.x < 25 * CB) exU[threadIdx.x] = 0;
     __syncthreads();
+    uint32_t m[5], f[5];
 #pragma unroll
     for (int c = 0; c < 5; ++c) {
-      uint32_t m = 0, f = 0;
+      m[c] = f[c] = 0;
 #pragma unroll
       for (int k = 0; k < PV; ++k) {
-        if ((c == 0 || c == 4) && k * NTH + (int)threadIdx.x < nb * N3) x[c][k] -= c == 0 ? kp.rho_ref : kp.rhoE_ref;
-        m = max(m, fx_mag(x[c][k]));
+        if ((c == 0 || c == 4) && own && k * NTE + pt < N3) x[c][k] -= c == 0 ? kp.rho_ref : kp.rhoE_ref;
+        m[c] = max(m[c], fx_mag(x[c][k]));
       }
-      block_max(ex + c, m);
       // the shares of the batch, also brought nearer for the lift sweeps
-      for (int i = threadIdx.x; i < nb * 12 * N2; i += NTH)
-        f = max(f, reinterpret_cast<const uint32_t*>(FBc + (i / N2 * 5 + c) * N2 + i % N2)[1] & 0x7fffffffu);
-      block_max(ex + 10 + c, f);
+      for (int i = pt; own && i < 12 * N2; i += NTE)
+        f[c] = max(f[c], reinterpret_cast<const uint32_t*>(FBc + pe * fbuf_per_cell<N>() + (i / N2 * 5 + c) * N2 + i % N2)[1] &
+                             0x7fffffffu);
+    }
+    if (own) {
+      block_max<32>(exU + pe * 5, 1, 0, m);
+      block_max<32>(exV + pe * 5, 1, 0, f);
     }
     __syncthreads();
-    fixA = block_ok<5>(ex);
+    fixA = blocks_ok(exU, 5 * CB);
 #pragma unroll
     for (int c = 0; c < 5; ++c) {
-      const int E = fx_exp(ex[c]);
+      const int E = fx_exp(exU[pe * 5 + c]);
 #pragma unroll
       for (int k = 0; k < PV; ++k) {
-        const int i = k * NTH + threadIdx.x, e = i / N3;
-        if (i < nb * N3) F0[e * 4 * N3 + c * N3 + i] = fixA ? __longlong_as_double(fx_of(x[c][k], E)) : x[c][k];
+        const int i = k * NTE + pt;
+        if (own && i < N3)
+          F0[(pe * 5 + c) * N3 + i] = fixA ? __longlong_as_double(fx_of(x[c][k], E)) : x[c][k];
       }
     }
   } else if (Ud) {
@@ -489,14 +500,14 @@ __global__ void __launch_bounds__(coll_threads<T, N, QC, QV>(), coll_ctas<T, N, 
     if constexpr (FX) {
       const int gC = chain_gain(tb.eSc);
       gS = chain_gain(tb.eSm);
-      if (conv) chain<1, N, QC, 1, FROM_INT, TO_INT>(F0, F1, tb.eSc, nbl * N2, 1, ex, 0);
-      chain<1, N, N, 1, FROM_INT, TO_INT>(F0, V, tb.eSm, nbl * N2, 1, ex, 0);
+      if (conv) chain<1, N, QC, 1, FROM_INT, TO_INT, N2>(F0, F1, tb.eSc, nbl * N2, exU, 0);
+      chain<1, N, N, 1, FROM_INT, TO_INT, N2>(F0, V, tb.eSm, nbl * N2, exU, 0);
       __syncthreads();
-      if (conv) chain<QC, N, QC, 1, FROM_INT, TO_INT>(F1, F2, tb.eSc, nbl * N, 1, ex, 0);
-      chain<N, N, N, 1, FROM_INT, TO_INT>(V, V + VS, tb.eSm, nbl * N, 1, ex, 0);
+      if (conv) chain<QC, N, QC, 1, FROM_INT, TO_INT, QC * N>(F1, F2, tb.eSc, nbl * N, exU, 0);
+      chain<N, N, N, 1, FROM_INT, TO_INT, N2>(V, V + VS, tb.eSm, nbl * N, exU, 0);
       __syncthreads();
-      if (conv) chain<QC * QC, N, QC, 1, FROM_INT, TO_DOUBLE>(F2, F0, tb.eSc, nbl, QC * QC, ex, 2 * gC);
-      chain<N2, N, N, 1, FROM_INT, TO_INT>(V + VS, Ug, tb.eSm, nbl, 1, ex, 0);
+      if (conv) chain<QC * QC, N, QC, 1, FROM_INT, TO_DOUBLE, QC2>(F2, F0, tb.eSc, nbl, exU, 2 * gC);
+      chain<N2, N, N, 1, FROM_INT, TO_INT, N2>(V + VS, Ug, tb.eSm, nbl, exU, 0);
       gS *= 3;
     }
   } else {
@@ -510,9 +521,9 @@ __global__ void __launch_bounds__(coll_threads<T, N, QC, QV>(), coll_ctas<T, N, 
     sw<T, 2, N, N, N, N, 1, PN, PN>(V + VS, Ug, tb.eSm, nbl);
   }
   __syncthreads();
-  auto ug = [&](int i, int c) -> T {
+  auto ug = [&](int i, int b) -> T {  // value i of U_g, in block b
     if constexpr (FX) {
-      if (fixA) return fx_store(__double_as_longlong(Ug[i]), fx_exp(ex[c]) + gS + 3);
+      if (fixA) return fx_store(__double_as_longlong(Ug[i]), fx_exp(exU[b]) + gS + 3);
     }
     return Ug[i];
   };
@@ -523,8 +534,8 @@ __global__ void __launch_bounds__(coll_threads<T, N, QC, QV>(), coll_ctas<T, N, 
   };
   // 4. convective flux (point arithmetic); reference gradients at the viscous points (sweeps)
   if (conv) {
-    for (int idx = threadIdx.x; idx < nb * PC; idx += NTH) {
-      const int e = idx / PC, p = idx - e * PC, o = e * 5 * BQ + p / QC2 * PQ + p % QC2;
+    for (int idx = pt; idx < (FX ? (pe < nb ? PC : 0) : nb * PC); idx += NTE) {
+      const int e = FX ? pe : idx / PC, p = FX ? idx : idx - e * PC, o = e * 5 * BQ + p / QC2 * PQ + p % QC2;
       T u[5];
 #pragma unroll
       for (int c = 0; c < 5; ++c) u[c] = F0[o + c * BQ];
@@ -564,16 +575,14 @@ __global__ void __launch_bounds__(coll_threads<T, N, QC, QV>(), coll_ctas<T, N, 
   }
   if constexpr (FX) {
     if (conv) {
+      if (pe < nb) block_max<32>(exC + pe * 5, 1, 0, mag);
 #pragma unroll
-      for (int c = 0; c < 5; ++c) {
-        block_max(ex + 5 + c, mag[c]);
-        mag[c] = 0;
-      }
+      for (int c = 0; c < 5; ++c) mag[c] = 0;
     }
     if (visc && fixA) {
-      chain<1, N, N, -1, FROM_INT, TO_DOUBLE>(Ug, V, tb.eDv, nbl * N2, N2, ex, gS);
-      chain<N, N, N, -1, FROM_INT, TO_DOUBLE>(Ug, V + VS, tb.eDv, nbl * N, N2, ex, gS);
-      chain<N2, N, N, -1, FROM_INT, TO_DOUBLE>(Ug, V + 2 * VS, tb.eDv, nbl, N2, ex, gS);
+      chain<1, N, N, -1, FROM_INT, TO_DOUBLE, N2>(Ug, V, tb.eDv, nbl * N2, exU, gS);
+      chain<N, N, N, -1, FROM_INT, TO_DOUBLE, N2>(Ug, V + VS, tb.eDv, nbl * N, exU, gS);
+      chain<N2, N, N, -1, FROM_INT, TO_DOUBLE, N2>(Ug, V + 2 * VS, tb.eDv, nbl, exU, gS);
     }
   }
   if (visc && !fixA) {
@@ -584,12 +593,12 @@ __global__ void __launch_bounds__(coll_threads<T, N, QC, QV>(), coll_ctas<T, N, 
   __syncthreads();
   // 5. viscous flux with the sign of -F (point arithmetic); D~ of the convective flux, in place (sweeps)
   if (visc) {
-    for (int idx = threadIdx.x; idx < nb * N3; idx += NTH) {
-      const int e = idx / N3, p = idx - e * N3, o = e * 5 * BN + pad(p);
+    for (int idx = pt; idx < (FX ? (pe < nb ? N3 : 0) : nb * N3); idx += NTE) {
+      const int e = FX ? pe : idx / N3, p = FX ? idx : idx - e * N3, o = e * 5 * BN + pad(p);
       T u[5];
       T* v0 = V + o;
 #pragma unroll
-      for (int c = 0; c < 5; ++c) u[c] = ug(o + c * BN, c);
+      for (int c = 0; c < 5; ++c) u[c] = ug(o + c * BN, e * 5 + c);
       const SideState<T> s = side_state(u, ph);
       if (GEO == GEO_AFFINE) {
         // reference derivatives; 1/h_j enters with 1/rho and with the flux constants
@@ -663,18 +672,12 @@ __global__ void __launch_bounds__(coll_threads<T, N, QC, QV>(), coll_ctas<T, N, 
     }
   }
   if constexpr (FX) {
-    if (visc) {
-#pragma unroll
-      for (int c = 1; c < 5; ++c) {
-        block_max(ex + 10 + c, mag[c]);
-        mag[c] = 0;
-      }
-    }
-    fixB = conv && fixA && block_ok<5>(ex + 5);
+    if (visc && pe < nb) block_max<32>(exV + pe * 5, 1, 0, mag);
+    fixB = conv && fixA && blocks_ok(exC, 5 * CB);
     if (fixB) {
-      chain<1, QC, QC, -1, FROM_DOUBLE, TO_INT>(F0, F0, tb.eDcW, nbl * QC * QC, QC * QC, ex + 5, 0, 2);
-      chain<QC, QC, QC, -1, FROM_DOUBLE, TO_INT>(F1, F1, tb.eDcW, nbl * QC, QC * QC, ex + 5, 0, 2);
-      chain<QC * QC, QC, QC, -1, FROM_DOUBLE, TO_INT>(F2, F2, tb.eDcW, nbl, QC * QC, ex + 5, 0, 2);
+      chain<1, QC, QC, -1, FROM_DOUBLE, TO_INT, QC2>(F0, F0, tb.eDcW, nbl * QC * QC, exC, 0, 2);
+      chain<QC, QC, QC, -1, FROM_DOUBLE, TO_INT, QC2>(F1, F1, tb.eDcW, nbl * QC, exC, 0, 2);
+      chain<QC * QC, QC, QC, -1, FROM_DOUBLE, TO_INT, QC2>(F2, F2, tb.eDcW, nbl, exC, 0, 2);
     }
   }
   if (conv && !fixB) {
@@ -686,16 +689,16 @@ __global__ void __launch_bounds__(coll_threads<T, N, QC, QV>(), coll_ctas<T, N, 
   // 6-8. projection of the summed convective parts onto the l_g; D~ and face shares of the viscous arrays
   int gF = 0;  // exponent after the lift over the viscous fluxes' and shares'
   if constexpr (FX) {
-    fixL = block_ok<5>(ex + 10);
+    fixL = blocks_ok(exV, 5 * CB);
     fixR = fixB && fixL && GEO == GEO_AFFINE && !force && kp.out_mode != 0;
     gF = chain_gain(tb.eLift, 2);
     fixL = fixL && (fixR || GEO == GEO_STORED || force || kp.out_mode == 0);  // (else the summed S^-1 sweep takes doubles)
     if (fixB) {
-      chain<QC * QC, QC, N, 1, FROM_SUM, TO_DOUBLE, 0, 0, PC>(F0, F0, tb.ePc, nbl, QC * QC, ex + 5, chain_gain(tb.eDcW, 2), 0,
-                                                              CB * 5 * S::F, 5, ex + 15);
+      chain<QC * QC, QC, N, 1, FROM_SUM, TO_DOUBLE, QC2, 0, 0, PC>(F0, F0, tb.ePc, nbl, exC, chain_gain(tb.eDcW, 2), 0,
+                                                                   CB * 5 * S::F, 1 << 30, exP);
     }
     if (fixL)
-      chain_lift<N>(V, FBc, tb.eLift, nb, visc, VS, ex + 10);
+      chain_lift<N>(V, FBc, tb.eLift, nb, visc, VS, exV);
     else
       lift_fp64<N>(V, FBc, tb.eLift, nb, visc, VS);
   } else {
@@ -707,10 +710,12 @@ __global__ void __launch_bounds__(coll_threads<T, N, QC, QV>(), coll_ctas<T, N, 
   __syncthreads();
   if constexpr (FX) {
     if (fixB) {
-      // (ex + 15 was valid if the fluxes' maxima were: the sums only shrink them)
-      chain<QC, QC, N, 1, FROM_DOUBLE, TO_INT, N, PC>(F0, F1, tb.ePc, nbl * N, N * QC, ex + 15, 0);
+      // exP and exR need no check of their own: the fluxes lie in 2^-723..2^677 (fx_exp_ok), D~, P and S^-1 raise that by
+      // less than 2^20, and a sum that cancels keeps at least one of its 61 bits or is zero, so that each of the three
+      // results loses at most 64 bits: all exponents stay within the normal range (biased 100 to 1720)
+      chain<QC, QC, N, 1, FROM_DOUBLE, TO_INT, N * QC, N, PC>(F0, F1, tb.ePc, nbl * N, exP, 0);
       __syncthreads();
-      chain<1, QC, N, 1, FROM_INT, TO_DOUBLE>(F1, F2, tb.ePc, nbl * N2, N2, ex + 15, chain_gain(tb.ePc));
+      chain<1, QC, N, 1, FROM_INT, TO_DOUBLE, N2>(F1, F2, tb.ePc, nbl * N2, exP, chain_gain(tb.ePc));
     }
   }
   if (conv && !fixB) {
@@ -726,49 +731,45 @@ __global__ void __launch_bounds__(coll_threads<T, N, QC, QV>(), coll_ctas<T, N, 
   const Eo<T> eBack = kp.out_mode == 0 ? tb.eSvT : tb.eSmi;
   int back = 0;  // the chain back to the nodes starts from the pass below
   if constexpr (FX) {
-    if (fixR) chain_sum<N>(V, VS, F2, F1, tb.eSmi, nbl * N2, ex + 10, gF, ex + 15, 2 * chain_gain(tb.ePc), ex + 20);
+    if (fixR) chain_sum<N>(V, VS, F2, F1, tb.eSmi, nbl * N2, exV, gF, exP, 2 * chain_gain(tb.ePc), exR);
   }
   if (fixR) {
   } else if (GEO == GEO_AFFINE && !force && kp.out_mode != 0) {
     sw<T, 0, N, N, N, N, 1, PN, PN, 3, true>(V, F1, tb.eSmi, nbl, VS, F2);
   } else {
-    for (int i = threadIdx.x; i < nvals; i += NTH) {
-      const int p = i % N3, e = i / (5 * N3), c = (i / N3) % 5;
-      const int ip = pad(i);
-      T r;
-      if (FX && fixL) {
-        const int64_t* v = reinterpret_cast<const int64_t*>(V) + ip;
-        r = F2[ip] + T(fx_store(v[0] + v[VS] + v[2 * VS], fx_exp(ex[10 + c]) + gF + 3));
-      } else {
-        r = F2[ip] + (V[ip] + (V[VS + ip] + V[2 * VS + ip]));
-      }
-      if (kp.out_mode == 0) {
-        const T w = tb.wm[p % N] * tb.wm[(p / N) % N] * tb.wm[p / N2];
-        r *= GEO == GEO_AFFINE ? -w * kc.detJ : -w;
-      } else {
-        if (GEO == GEO_STORED) r *= rcp_of(static_cast<const T*>(kp.gm)[(size_t)(e0 + e) * N3 + p]);
-        if (force && c > 0) {
-          const int g = e * 5 * BN + pad(p);
-          r += c < 4 ? kc.bf[c - 1]
-                     : (kc.bf[0] * ug(g + BN, 1) + kc.bf[1] * ug(g + 2 * BN, 2) + kc.bf[2] * ug(g + 3 * BN, 3)) *
-                           rcp_of(ph.rho_r + ug(g, 0));
+    for (int i = threadIdx.x; (FX ? i & ~31 : i) < nvals; i += NTH) {  // (FP64: whole warps, for the maxima)
+      uint32_t m[1] = {0};
+      if (!FX || i < nvals) {
+        const int p = i % N3, e = i / (5 * N3), c = (i / N3) % 5;
+        const int ip = pad(i);
+        T r;
+        if (FX && fixL) {
+          const int64_t* v = reinterpret_cast<const int64_t*>(V) + ip;
+          r = F2[ip] + T(fx_store(v[0] + v[VS] + v[2 * VS], fx_exp(exV[i / N3]) + gF + 3));
+        } else {
+          r = F2[ip] + (V[ip] + (V[VS + ip] + V[2 * VS + ip]));
         }
+        if (kp.out_mode == 0) {
+          const T w = tb.wm[p % N] * tb.wm[(p / N) % N] * tb.wm[p / N2];
+          r *= GEO == GEO_AFFINE ? -w * kc.detJ : -w;
+        } else {
+          if (GEO == GEO_STORED) r *= rcp_of(static_cast<const T*>(kp.gm)[(size_t)(e0 + e) * N3 + p]);
+          if (force && c > 0) {
+            const int g = e * 5 * BN + pad(p), b = e * 5;
+            r += c < 4 ? kc.bf[c - 1]
+                       : (kc.bf[0] * ug(g + BN, b + 1) + kc.bf[1] * ug(g + 2 * BN, b + 2) + kc.bf[2] * ug(g + 3 * BN, b + 3)) *
+                             rcp_of(ph.rho_r + ug(g, b));
+          }
+        }
+        F0[ip] = r;
+        if constexpr (FX) m[0] = fx_mag(r);
       }
-      F0[ip] = r;
-      if constexpr (FX) {
-#pragma unroll
-        for (int q = 0; q < 5; ++q) mag[q] = max(mag[q], c == q ? fx_mag(r) : 0u);
-      }
-    }
-    if constexpr (FX) {
-      __syncwarp();
-#pragma unroll
-      for (int q = 0; q < 5; ++q) block_max(ex + 20 + q, mag[q]);
+      if constexpr (FX) block_max<N3>(exR, 0, min(i, nvals - 1) / N3, m);
     }
     __syncthreads();
     if constexpr (FX) {
-      fixR = block_ok<5>(ex + 20);
-      if (fixR) chain<1, N, N, 1, FROM_DOUBLE, TO_INT>(F0, F1, eBack, nbl * N2, N2, ex + 20, 0);
+      fixR = blocks_ok(exR, 5 * CB);
+      if (fixR) chain<1, N, N, 1, FROM_DOUBLE, TO_INT, N2>(F0, F1, eBack, nbl * N2, exR, 0);
       back = 1;
     }
     if (!fixR) sw<T, 0, N, N, N, N, 1, PN, PN>(F0, F1, eBack, nbl);
@@ -776,13 +777,13 @@ __global__ void __launch_bounds__(coll_threads<T, N, QC, QV>(), coll_ctas<T, N, 
   __syncthreads();
   if constexpr (FX) {
     if (fixR && back) {
-      chain<N, N, N, 1, FROM_INT, TO_INT>(F1, F0, eBack, nbl * N, 1, ex, 0);
+      chain<N, N, N, 1, FROM_INT, TO_INT, N2>(F1, F0, eBack, nbl * N, exR, 0);
       __syncthreads();
-      chain<N2, N, N, 1, FROM_INT, TO_DOUBLE>(F0, sr, eBack, nbl, N2, ex + 20, 2 * chain_gain(eBack));
+      chain<N2, N, N, 1, FROM_INT, TO_DOUBLE, N2>(F0, sr, eBack, nbl, exR, 2 * chain_gain(eBack));
     } else if (fixR) {
-      chain<N, N, N, 1, FROM_DOUBLE, TO_INT>(F1, F0, tb.eSmi, nbl * N, N2, ex + 20, 0);
+      chain<N, N, N, 1, FROM_DOUBLE, TO_INT, N2>(F1, F0, tb.eSmi, nbl * N, exR, 0);
       __syncthreads();
-      chain<N2, N, N, 1, FROM_INT, TO_DOUBLE>(F0, sr, tb.eSmi, nbl, N2, ex + 20, chain_gain(tb.eSmi));
+      chain<N2, N, N, 1, FROM_INT, TO_DOUBLE, N2>(F0, sr, tb.eSmi, nbl, exR, chain_gain(tb.eSmi));
     }
   }
   if (!fixR) {
@@ -818,16 +819,16 @@ struct CollFaceSizes {
   static constexpr int C1 = 2 * 5 * QC2;
   static constexpr int PER_FACE = VV + TT + C0 + C1;
 };
-template <typename T, int N, int QC, int QV, int FB_>
-constexpr size_t coll_face_smem() {
-  return ((size_t)table_elems<T, N, QC, QV>() + (size_t)FB_ * (CollFaceSizes<N, QC>::PER_FACE + 1)) * sizeof(T) +
-         (3 * FB_ + 20) * sizeof(int) + 64;
+template <typename T, int N, int QC, int QV>
+constexpr size_t coll_face_smem(int fb) {
+  return ((size_t)table_elems<T, N, QC, QV>() + (size_t)fb * (CollFaceSizes<N, QC>::PER_FACE + 1)) * sizeof(T) +
+         (3 + (sizeof(T) == 8 ? 20 : 0)) * fb * sizeof(int) + 64;
 }
+// Faces per CTA: up to 8, as long as four CTAs fit an SM (56 KB each).
 template <typename T, int N, int QC, int QV>
 constexpr int coll_faces() {
   int fb = 8;
-  while (fb > 1 && ((size_t)table_elems<T, N, QC, QV>() + (size_t)fb * CollFaceSizes<N, QC>::PER_FACE) * sizeof(T) > 56 * 1024)
-    --fb;
+  while (fb > 1 && coll_face_smem<T, N, QC, QV>(fb) > 56 * 1024) --fb;
   return fb;
 }
 // (FP32 at k = 4, 5: 256 threads for the larger faces, 1.10 -> 0.89 ms at 40^3, k = 5)
@@ -857,15 +858,16 @@ __device__ __forceinline__ void coll_face_terms(const double* U, const T* Ud, co
   const bool conv = kp.conv != 0, visc = kp.visc != 0;
   constexpr bool FX = sizeof(T) == 8;  // integer chains
   constexpr int NTT = AFF ? 3 : 5;     // tested components of a tangential direction
-  // FP64: per-slot maxima of the traces [0], the normal derivatives [5], the convective flux [10] and the tangential
-  // gradient tests [15]
+  // FP64: maxima of the blocks (slot, face), both sides together: of the traces, of the normal derivatives, of the
+  // convective flux and of the tangential gradient tests
+  uint32_t *exL = ex, *exD = exL + 5 * FB_, *exC = exD + 5 * FB_, *exT = exC + 5 * FB_;
   auto see = [&](uint32_t& m, T v) {
     if constexpr (FX) m = max(m, fx_mag(v));
     return v;
   };
   // traces along the normal lines, from global memory
-  uint32_t mL[5] = {0, 0, 0, 0, 0}, mD[5] = {0, 0, 0, 0, 0};
-  for (int idx = threadIdx.x; idx < nl; idx += NTH) {
+  for (int idx0 = threadIdx.x; (FX ? idx0 & ~31 : idx0) < nl; idx0 += NTH) {  // (FP64: whole warps, for the maxima)
+    const int idx = FX ? min(idx0, nl - 1) : idx0;
     const int sl = idx / nf, r = idx - sl * nf, e = r / N2, j = r - e * N2;
     const int c = slot_comp<D>(sl);
     const int q0 = face_node<N>(D, 0, j % N, j / N);
@@ -919,38 +921,28 @@ __device__ __forceinline__ void coll_face_terms(const double* U, const T* Ud, co
       }
     }
     const T vm = s ? a[N - 1] : a[0], vp = s ? b[0] : b[N - 1];
-    VV[idx] = vm;
-    VV[nl + idx] = vp;
-    VV[2 * nl + idx] = dm;
-    VV[3 * nl + idx] = dp;
-    if constexpr (FX) {
-      const uint32_t ml = max(fx_mag(vm), fx_mag(vp)), md = max(fx_mag(dm), fx_mag(dp));
-#pragma unroll
-      for (int q = 0; q < 5; ++q)
-        if (q == sl) {
-          mL[q] = max(mL[q], ml);
-          mD[q] = max(mD[q], md);
-        }
+    if (!FX || idx0 < nl) {
+      VV[idx] = vm;
+      VV[nl + idx] = vp;
+      VV[2 * nl + idx] = dm;
+      VV[3 * nl + idx] = dp;
     }
-  }
-  if constexpr (FX) {
-#pragma unroll
-    for (int q = 0; q < 5; ++q) {
-      block_max(ex + q, mL[q]);
-      block_max(ex + 5 + q, mD[q]);
+    if constexpr (FX) {
+      const uint32_t m[2] = {max(fx_mag(vm), fx_mag(vp)), max(fx_mag(dm), fx_mag(dp))};
+      block_max<N2>(exL, 5 * FB_, idx / N2, m);
     }
   }
   __syncthreads();
   bool fixA = false;
   int gS = 0;
   if constexpr (FX) {
-    fixA = block_ok<10>(ex);
+    fixA = blocks_ok(exL, 10 * FB_);
     if (fixA) {
       gS = chain_gain(tb.eSm);
-      if (conv) chain<1, N, QC, 1, FROM_DOUBLE, TO_INT>(VV, C0, tb.eSc, 2 * 5 * nb * N, nb * N, ex, 0);
+      if (conv) chain<1, N, QC, 1, FROM_DOUBLE, TO_INT, N>(VV, C0, tb.eSc, 2 * 5 * nb * N, exL, 0, 0, 0, 5 * nb);
       if (visc) {
-        chain<1, N, N, 1, FROM_DOUBLE, TO_INT>(VV, TT, tb.eSm, 2 * 5 * nb * N, nb * N, ex, 0);
-        chain<1, N, N, 1, FROM_DOUBLE, TO_INT>(VV + 2 * nl, TT + 2 * nl, tb.eSm, 2 * 5 * nb * N, nb * N, ex + 5, 0);
+        chain<1, N, N, 1, FROM_DOUBLE, TO_INT, N>(VV, TT, tb.eSm, 2 * 5 * nb * N, exL, 0, 0, 0, 5 * nb);
+        chain<1, N, N, 1, FROM_DOUBLE, TO_INT, N>(VV + 2 * nl, TT + 2 * nl, tb.eSm, 2 * 5 * nb * N, exD, 0, 0, 0, 5 * nb);
       }
     }
   }
@@ -961,10 +953,10 @@ __device__ __forceinline__ void coll_face_terms(const double* U, const T* Ud, co
   __syncthreads();
   if constexpr (FX) {
     if (fixA) {
-      if (conv) chain<QC, N, QC, 1, FROM_INT, TO_DOUBLE>(C0, C1, tb.eSc, 2 * 5 * nb, nb * QC, ex, chain_gain(tb.eSc));
+      if (conv) chain<QC, N, QC, 1, FROM_INT, TO_DOUBLE, QC>(C0, C1, tb.eSc, 2 * 5 * nb, exL, chain_gain(tb.eSc), 0, 0, 5 * nb);
       if (visc) {
-        chain<N, N, N, 1, FROM_INT, TO_INT>(TT, VV, tb.eSm, 2 * 5 * nb, 1, ex, 0);
-        chain<N, N, N, 1, FROM_INT, TO_DOUBLE>(TT + 2 * nl, VV + 2 * nl, tb.eSm, 2 * 5 * nb, nb * N, ex + 5, gS);
+        chain<N, N, N, 1, FROM_INT, TO_INT, N>(TT, VV, tb.eSm, 2 * 5 * nb, exL, 0);
+        chain<N, N, N, 1, FROM_INT, TO_DOUBLE, N>(TT + 2 * nl, VV + 2 * nl, tb.eSm, 2 * 5 * nb, exD, gS, 0, 0, 5 * nb);
       }
       gS *= 2;
     }
@@ -977,39 +969,38 @@ __device__ __forceinline__ void coll_face_terms(const double* U, const T* Ud, co
   // convective flux (point arithmetic); tangential derivatives (sweeps)
   if (conv) {
     const int nc = nb * QC2;
-    uint32_t mC[5] = {0, 0, 0, 0, 0};
-    for (int idx = threadIdx.x; idx < nc; idx += NTH) {
-      const int e = idx / QC2, p = idx - e * QC2;
-      T um[5], up[5], fm[5], fp[5], n[3] = {T(0), T(0), T(0)}, w;
+    for (int idx = threadIdx.x; (FX ? idx & ~31 : idx) < nc; idx += NTH) {
+      uint32_t mC[5] = {0, 0, 0, 0, 0};
+      if (!FX || idx < nc) {
+        const int e = idx / QC2, p = idx - e * QC2;
+        T um[5], up[5], fm[5], fp[5], n[3] = {T(0), T(0), T(0)}, w;
 #pragma unroll
-      for (int q = 0; q < 5; ++q) {
-        um[slot_comp<D>(q)] = C1[q * nc + idx];
-        up[slot_comp<D>(q)] = C1[(5 + q) * nc + idx];
-      }
-      if (en[e] < 0) wall_ghost(um, ph, up);
-      if (AFF) {
-        w = T(-0.5) * kc.hinv[D];
-      } else {
-        const T* g = static_cast<const T*>(kp.gfc) + ((size_t)eo[e] * 6 + f) * 13 * QC2 + p;
-        n[0] = g[9 * QC2];
-        n[1] = g[10 * QC2];
-        n[2] = g[11 * QC2];
-        w = T(-0.5) * g[12 * QC2];
-      }
-      T lm, lp;
-      const T ws = AFF && !s ? -w : w;
-      llf_side<T, D, AFF>(um, n, ws, ph, fm, lm);
-      llf_side<T, D, AFF>(up, n, ws, ph, fp, lp);
-      const T lam = w * (lm > lp ? lm : lp);
+        for (int q = 0; q < 5; ++q) {
+          um[slot_comp<D>(q)] = C1[q * nc + idx];
+          up[slot_comp<D>(q)] = C1[(5 + q) * nc + idx];
+        }
+        if (en[e] < 0) wall_ghost(um, ph, up);
+        if (AFF) {
+          w = T(-0.5) * kc.hinv[D];
+        } else {
+          const T* g = static_cast<const T*>(kp.gfc) + ((size_t)eo[e] * 6 + f) * 13 * QC2 + p;
+          n[0] = g[9 * QC2];
+          n[1] = g[10 * QC2];
+          n[2] = g[11 * QC2];
+          w = T(-0.5) * g[12 * QC2];
+        }
+        T lm, lp;
+        const T ws = AFF && !s ? -w : w;
+        llf_side<T, D, AFF>(um, n, ws, ph, fm, lm);
+        llf_side<T, D, AFF>(up, n, ws, ph, fp, lp);
+        const T lam = w * (lm > lp ? lm : lp);
 #pragma unroll
-      for (int q = 0; q < 5; ++q) {
-        const int c = slot_comp<D>(q);
-        C1[q * nc + idx] = see(mC[q], fm[c] + fp[c] + lam * (um[c] - up[c]));
+        for (int q = 0; q < 5; ++q) {
+          const int c = slot_comp<D>(q);
+          C1[q * nc + idx] = see(mC[q], fm[c] + fp[c] + lam * (um[c] - up[c]));
+        }
       }
-    }
-    if constexpr (FX) {
-#pragma unroll
-      for (int q = 0; q < 5; ++q) block_max(ex + 10 + q, mC[q]);
+      if constexpr (FX) block_max<QC2>(exC, nb, min(idx, nc - 1) / QC2, mC);
     }
   }
   if constexpr (FX) {
@@ -1018,11 +1009,11 @@ __device__ __forceinline__ void coll_face_terms(const double* U, const T* Ud, co
       for (int sd = 0; sd < 2; ++sd) {
         const int o = sd * nl;
         if (AFF) {
-          chain<1, N, N, -1, FROM_INT, TO_DOUBLE>(VV + o, TT + o, tb.eDv, 3 * nb * N, nb * N, ex, gS, 0, 0, 3);
-          chain<N, N, N, -1, FROM_INT, TO_DOUBLE>(VV + o + nf, TT + 2 * nl + o, tb.eDv, 3 * nb, nb * N, ex + 1, gS, 0, 0, 3);
+          chain<1, N, N, -1, FROM_INT, TO_DOUBLE, N>(VV + o, TT + o, tb.eDv, 3 * nb * N, exL, gS);
+          chain<N, N, N, -1, FROM_INT, TO_DOUBLE, N>(VV + o + nf, TT + 2 * nl + o, tb.eDv, 3 * nb, exL + nb, gS);
         } else {
-          chain<1, N, N, -1, FROM_INT, TO_DOUBLE>(VV + o, TT + o, tb.eDv, 5 * nb * N, nb * N, ex, gS);
-          chain<N, N, N, -1, FROM_INT, TO_DOUBLE>(VV + o, TT + 2 * nl + o, tb.eDv, 5 * nb, nb * N, ex, gS);
+          chain<1, N, N, -1, FROM_INT, TO_DOUBLE, N>(VV + o, TT + o, tb.eDv, 5 * nb * N, exL, gS);
+          chain<N, N, N, -1, FROM_INT, TO_DOUBLE, N>(VV + o, TT + 2 * nl + o, tb.eDv, 5 * nb, exL, gS);
         }
       }
     }
@@ -1042,171 +1033,170 @@ __device__ __forceinline__ void coll_face_terms(const double* U, const T* Ud, co
   __syncthreads();
   // viscous fluxes (point arithmetic); projection of the convective flux (sweeps).  Shares are of -F.
   if (visc) {
-    uint32_t mT[5] = {0, 0, 0, 0, 0};
-    for (int idx = threadIdx.x; idx < nf; idx += NTH) {
-      const int e = idx / N2, p = idx - e * N2;
-      const bool wall = en[e] < 0;
-      T um[5], up[5], jmp[5];
+    for (int idx = threadIdx.x; (FX ? idx & ~31 : idx) < nf; idx += NTH) {
+      uint32_t mT[NTT] = {};
+      if (!FX || idx < nf) {
+        const int e = idx / N2, p = idx - e * N2;
+        const bool wall = en[e] < 0;
+        T um[5], up[5], jmp[5];
 #pragma unroll
-      for (int q = 0; q < 5; ++q) {
-        T a = VV[q * nf + idx], b = VV[nl + q * nf + idx];
-        if constexpr (FX) {
-          if (fixA) {
-            const int X = fx_exp(ex[q]) + gS + 3;
-            a = fx_store(__double_as_longlong(a), X);
-            b = fx_store(__double_as_longlong(b), X);
+        for (int q = 0; q < 5; ++q) {
+          T a = VV[q * nf + idx], b = VV[nl + q * nf + idx];
+          if constexpr (FX) {
+            if (fixA) {
+              const int X = fx_exp(exL[q * nb + e]) + gS + 3;
+              a = fx_store(__double_as_longlong(a), X);
+              b = fx_store(__double_as_longlong(b), X);
+            }
           }
+          um[slot_comp<D>(q)] = a;
+          up[slot_comp<D>(q)] = b;
         }
-        um[slot_comp<D>(q)] = a;
-        up[slot_comp<D>(q)] = b;
-      }
-      if (wall) wall_ghost(um, ph, up);
-      const SideState<T> sm_ = side_state(um, ph), sp_ = side_state(up, ph);
-      const T tau = tau_f[e];
+        if (wall) wall_ghost(um, ph, up);
+        const SideState<T> sm_ = side_state(um, ph), sp_ = side_state(up, ph);
+        const T tau = tau_f[e];
 #pragma unroll
-      for (int c = 0; c < 5; ++c) jmp[c] = um[c] - up[c];
-      T fm[4], fp[4];
-      if (AFF) {
-        const T hd = kc.hinv[D];
-        T* T1m = TT + idx;
-        T* T1p = T1m + nl;
-        T* T2m = T1p + nl;
-        T* T2p = T2m + nl;
-        T gm[5], gp[5];
-#pragma unroll
-        for (int q = 0; q < 5; ++q) {
-          gm[slot_comp<D>(q)] = VV[2 * nl + q * nf + idx];
-          gp[slot_comp<D>(q)] = VV[3 * nl + q * nf + idx];
-        }
-        visc_normal<T, D>(sm_, gm, T1m[nf], T1m[2 * nf], T1m[0], T2m[0], T2m[nf], T2m[2 * nf], kc, fm);
-        if (wall)  // grad U+ = grad U-, at the ghost state
-          visc_normal<T, D>(sp_, gm, T1m[nf], T1m[2 * nf], T1m[0], T2m[0], T2m[nf], T2m[2 * nf], kc, fp);
-        else
-          visc_normal<T, D>(sp_, gp, T1p[nf], T1p[2 * nf], T1p[0], T2p[0], T2p[nf], T2p[2 * nf], kc, fp);
-        // value share (own side): (V, Q*.n), Q*.n = {{F_v}}.n - tau [[U]]; the other side's is the negative
-        const T wv = s ? T(0.5) * hd : T(-0.5) * hd, wt = hd * tau;
-        const int fs[5] = {1, -1, 0, 2, 3};  // slot -> entry of fm
-#pragma unroll
-        for (int q = 0; q < 5; ++q) {
-          const T t = -wt * jmp[slot_comp<D>(q)];
-          VV[q * nf + idx] = fs[q] < 0 ? t : t + wv * (fm[fs[q] < 0 ? 0 : fs[q]] + fp[fs[q] < 0 ? 0 : fs[q]]);
-        }
-        // +1/2 (grad V, F_v(U, [[U]])), [[U]] = sgn jmp (x) e_D
-        if (!s) {
-#pragma unroll
-          for (int c = 0; c < 5; ++c) jmp[c] = -jmp[c];
-        }
-        T a[4], b1[3], b2[3];
-        visc_jump<T, D>(sm_, jmp, kc, a, b1, b2);
-        VV[2 * nl + idx] = a[1];
-        VV[2 * nl + nf + idx] = T(0);
-        VV[2 * nl + 2 * nf + idx] = a[0];
-        VV[2 * nl + 3 * nf + idx] = a[2];
-        VV[2 * nl + 4 * nf + idx] = a[3];
-#pragma unroll
-        for (int i = 0; i < 3; ++i) {
-          T1m[i * nf] = see(mT[i], b1[i]);
-          T2m[i * nf] = see(mT[i], b2[i]);
-        }
-        if (!wall) visc_jump<T, D>(sp_, jmp, kc, a, b1, b2);
-        VV[3 * nl + idx] = a[1];
-        VV[3 * nl + nf + idx] = T(0);
-        VV[3 * nl + 2 * nf + idx] = a[0];
-        VV[3 * nl + 3 * nf + idx] = a[2];
-        VV[3 * nl + 4 * nf + idx] = a[3];
-#pragma unroll
-        for (int i = 0; i < 3; ++i) {
-          T1p[i * nf] = see(mT[i], b1[i]);
-          T2p[i * nf] = see(mT[i], b2[i]);
-        }
-      } else {
-        const T* g = static_cast<const T*>(kp.gfv) + ((size_t)eo[e] * 6 + f) * 13 * N2 + p;
-        T Jm[9], Jp[9], n[3];
-#pragma unroll
-        for (int m = 0; m < 9; ++m) Jm[m] = g[m * N2];
-        n[0] = g[9 * N2];
-        n[1] = g[10 * N2];
-        n[2] = g[11 * N2];
-        const T dA = g[12 * N2];
-        if (!wall && oc) {
-          frame_face_jinv<T, N>(static_cast<const T*>(kp.gfv), en[e], oc[e], D, s, p, Jp);
-        } else {
-          const T* gp = wall ? g : static_cast<const T*>(kp.gfv) + ((size_t)en[e] * 6 + fo) * 13 * N2 + p;
-#pragma unroll
-          for (int m = 0; m < 9; ++m) Jp[m] = gp[m * N2];
-        }
-        T G[5][3];
-#pragma unroll
-        for (int q = 0; q < 5; ++q) {
-          const T a1 = TT[q * nf + idx], a2 = TT[2 * nl + q * nf + idx], ad = VV[2 * nl + q * nf + idx];
-#pragma unroll
-          for (int a = 0; a < 3; ++a) G[slot_comp<D>(q)][a] = Jm[3 * t1 + a] * a1 + Jm[3 * t2 + a] * a2 + Jm[3 * D + a] * ad;
-        }
-        visc_normal_any(sm_, G, n, ph, fm);
-        if (!wall) {
+        for (int c = 0; c < 5; ++c) jmp[c] = um[c] - up[c];
+        T fm[4], fp[4];
+        if (AFF) {
+          const T hd = kc.hinv[D];
+          T* T1m = TT + idx;
+          T* T1p = T1m + nl;
+          T* T2m = T1p + nl;
+          T* T2p = T2m + nl;
+          T gm[5], gp[5];
 #pragma unroll
           for (int q = 0; q < 5; ++q) {
-            const T a1 = TT[nl + q * nf + idx], a2 = TT[3 * nl + q * nf + idx], ad = VV[3 * nl + q * nf + idx];
-#pragma unroll
-            for (int a = 0; a < 3; ++a) G[slot_comp<D>(q)][a] = Jp[3 * t1 + a] * a1 + Jp[3 * t2 + a] * a2 + Jp[3 * D + a] * ad;
+            gm[slot_comp<D>(q)] = VV[2 * nl + q * nf + idx];
+            gp[slot_comp<D>(q)] = VV[3 * nl + q * nf + idx];
           }
-        }
-        visc_normal_any(sp_, G, n, ph, fp);
-        const T hw = T(0.5) * dA, wt = dA * tau;
+          visc_normal<T, D>(sm_, gm, T1m[nf], T1m[2 * nf], T1m[0], T2m[0], T2m[nf], T2m[2 * nf], kc, fm);
+          if (wall)  // grad U+ = grad U-, at the ghost state
+            visc_normal<T, D>(sp_, gm, T1m[nf], T1m[2 * nf], T1m[0], T2m[0], T2m[nf], T2m[2 * nf], kc, fp);
+          else
+            visc_normal<T, D>(sp_, gp, T1p[nf], T1p[2 * nf], T1p[0], T2p[0], T2p[nf], T2p[2 * nf], kc, fp);
+          // value share (own side): (V, Q*.n), Q*.n = {{F_v}}.n - tau [[U]]; the other side's is the negative
+          const T wv = s ? T(0.5) * hd : T(-0.5) * hd, wt = hd * tau;
+          const int fs[5] = {1, -1, 0, 2, 3};  // slot -> entry of fm
 #pragma unroll
-        for (int q = 0; q < 5; ++q) {
-          const int c = slot_comp<D>(q);
-          const T t = -wt * jmp[c];
-          VV[q * nf + idx] = c == 0 ? t : t + hw * (fm[c == 0 ? 0 : c - 1] + fp[c == 0 ? 0 : c - 1]);
-        }
+          for (int q = 0; q < 5; ++q) {
+            const T t = -wt * jmp[slot_comp<D>(q)];
+            VV[q * nf + idx] = fs[q] < 0 ? t : t + wv * (fm[fs[q] < 0 ? 0 : fs[q]] + fp[fs[q] < 0 ? 0 : fs[q]]);
+          }
+          // +1/2 (grad V, F_v(U, [[U]])), [[U]] = sgn jmp (x) e_D
+          if (!s) {
 #pragma unroll
-        for (int sd = 0; sd < 2; ++sd) {
-          const SideState<T>& ss = sd ? sp_ : sm_;
-          const T* J = sd ? Jp : Jm;
-          const JumpFlux<T> jf = visc_jump_any(ss, jmp, n, ph);
-          T* dst[3] = {TT + sd * nl + idx, TT + (2 + sd) * nl + idx, VV + (2 + sd) * nl + idx};
-          const int row[3] = {t1, t2, D};
+            for (int c = 0; c < 5; ++c) jmp[c] = -jmp[c];
+          }
+          T a[4], b1[3], b2[3];
+          visc_jump<T, D>(sm_, jmp, kc, a, b1, b2);
+          VV[2 * nl + idx] = a[1];
+          VV[2 * nl + nf + idx] = T(0);
+          VV[2 * nl + 2 * nf + idx] = a[0];
+          VV[2 * nl + 3 * nf + idx] = a[2];
+          VV[2 * nl + 4 * nf + idx] = a[3];
 #pragma unroll
-          for (int b = 0; b < 3; ++b) {
-            T r[4];
-            jump_row(jf, ss, n, J + 3 * row[b], hw, r);
+          for (int i = 0; i < 3; ++i) {
+            T1m[i * nf] = see(mT[i], b1[i]);
+            T2m[i * nf] = see(mT[i], b2[i]);
+          }
+          if (!wall) visc_jump<T, D>(sp_, jmp, kc, a, b1, b2);
+          VV[3 * nl + idx] = a[1];
+          VV[3 * nl + nf + idx] = T(0);
+          VV[3 * nl + 2 * nf + idx] = a[0];
+          VV[3 * nl + 3 * nf + idx] = a[2];
+          VV[3 * nl + 4 * nf + idx] = a[3];
+#pragma unroll
+          for (int i = 0; i < 3; ++i) {
+            T1p[i * nf] = see(mT[i], b1[i]);
+            T2p[i * nf] = see(mT[i], b2[i]);
+          }
+        } else {
+          const T* g = static_cast<const T*>(kp.gfv) + ((size_t)eo[e] * 6 + f) * 13 * N2 + p;
+          T Jm[9], Jp[9], n[3];
+#pragma unroll
+          for (int m = 0; m < 9; ++m) Jm[m] = g[m * N2];
+          n[0] = g[9 * N2];
+          n[1] = g[10 * N2];
+          n[2] = g[11 * N2];
+          const T dA = g[12 * N2];
+          if (!wall && oc) {
+            frame_face_jinv<T, N>(static_cast<const T*>(kp.gfv), en[e], oc[e], D, s, p, Jp);
+          } else {
+            const T* gp = wall ? g : static_cast<const T*>(kp.gfv) + ((size_t)en[e] * 6 + fo) * 13 * N2 + p;
+#pragma unroll
+            for (int m = 0; m < 9; ++m) Jp[m] = gp[m * N2];
+          }
+          T G[5][3];
+#pragma unroll
+          for (int q = 0; q < 5; ++q) {
+            const T a1 = TT[q * nf + idx], a2 = TT[2 * nl + q * nf + idx], ad = VV[2 * nl + q * nf + idx];
+#pragma unroll
+            for (int a = 0; a < 3; ++a) G[slot_comp<D>(q)][a] = Jm[3 * t1 + a] * a1 + Jm[3 * t2 + a] * a2 + Jm[3 * D + a] * ad;
+          }
+          visc_normal_any(sm_, G, n, ph, fm);
+          if (!wall) {
 #pragma unroll
             for (int q = 0; q < 5; ++q) {
-              const int c = slot_comp<D>(q);
-              const T v = c == 0 ? T(0) : r[c == 0 ? 0 : c - 1];
-              dst[b][q * nf] = b < 2 ? see(mT[q], v) : v;
+              const T a1 = TT[nl + q * nf + idx], a2 = TT[3 * nl + q * nf + idx], ad = VV[3 * nl + q * nf + idx];
+#pragma unroll
+              for (int a = 0; a < 3; ++a) G[slot_comp<D>(q)][a] = Jp[3 * t1 + a] * a1 + Jp[3 * t2 + a] * a2 + Jp[3 * D + a] * ad;
+            }
+          }
+          visc_normal_any(sp_, G, n, ph, fp);
+          const T hw = T(0.5) * dA, wt = dA * tau;
+#pragma unroll
+          for (int q = 0; q < 5; ++q) {
+            const int c = slot_comp<D>(q);
+            const T t = -wt * jmp[c];
+            VV[q * nf + idx] = c == 0 ? t : t + hw * (fm[c == 0 ? 0 : c - 1] + fp[c == 0 ? 0 : c - 1]);
+          }
+#pragma unroll
+          for (int sd = 0; sd < 2; ++sd) {
+            const SideState<T>& ss = sd ? sp_ : sm_;
+            const T* J = sd ? Jp : Jm;
+            const JumpFlux<T> jf = visc_jump_any(ss, jmp, n, ph);
+            T* dst[3] = {TT + sd * nl + idx, TT + (2 + sd) * nl + idx, VV + (2 + sd) * nl + idx};
+            const int row[3] = {t1, t2, D};
+#pragma unroll
+            for (int b = 0; b < 3; ++b) {
+              T r[4];
+              jump_row(jf, ss, n, J + 3 * row[b], hw, r);
+#pragma unroll
+              for (int q = 0; q < 5; ++q) {
+                const int c = slot_comp<D>(q);
+                const T v = c == 0 ? T(0) : r[c == 0 ? 0 : c - 1];
+                dst[b][q * nf] = b < 2 ? see(mT[q], v) : v;
+              }
             }
           }
         }
       }
-    }
-    if constexpr (FX) {
-#pragma unroll
-      for (int q = 0; q < NTT; ++q) block_max(ex + 15 + q, mT[q]);
+      if constexpr (FX) block_max<N2>(exT, nb, min(idx, nf - 1) / N2, mT);
     }
   }
   bool fixB = false, fixT = false;
   if constexpr (FX) {
-    fixB = conv && block_ok<5>(ex + 10);
-    if (fixB) chain<QC, QC, N, 1, FROM_DOUBLE, TO_INT>(C1, C0, tb.ePc, 5 * nb, nb * QC, ex + 10, 0);
+    fixB = conv && blocks_ok(exC, 5 * nb);
+    if (fixB) chain<QC, QC, N, 1, FROM_DOUBLE, TO_INT, QC>(C1, C0, tb.ePc, 5 * nb, exC, 0);
   }
   if (conv && !fixB) sw<T, 1, QC, QC, 1, N, 1>(C1, C0, tb.ePc, 5 * nb);
   __syncthreads();
   // tangential gradient tests, in place; the convective share
   int gT = 0;
   if constexpr (FX) {
-    fixT = visc && block_ok<NTT>(ex + 15);
+    fixT = visc && blocks_ok(exT, NTT * nb);
     if (fixT) {
       gT = chain_gain(tb.eDvW, 1);
 #pragma unroll
       for (int sd = 0; sd < 2; ++sd) {
         double* t1a = TT + sd * nl;
         double* t2a = TT + (2 + sd) * nl;
-        chain<1, N, N, -1, FROM_DOUBLE, TO_INT>(t1a, t1a, tb.eDvW, NTT * nb * N, nb * N, ex + 15, 0, 1, 0, NTT);
-        chain<N, N, N, -1, FROM_DOUBLE, TO_INT>(t2a, t2a, tb.eDvW, NTT * nb, nb * N, ex + 15, 0, 1, 0, NTT);
+        chain<1, N, N, -1, FROM_DOUBLE, TO_INT, N>(t1a, t1a, tb.eDvW, NTT * nb * N, exT, 0, 1);
+        chain<N, N, N, -1, FROM_DOUBLE, TO_INT, N>(t2a, t2a, tb.eDvW, NTT * nb, exT, 0, 1);
       }
     }
-    if (fixB) chain<1, QC, N, 1, FROM_INT, TO_DOUBLE>(C0, C1, tb.ePc, 5 * nb * N, nb * N, ex + 10, chain_gain(tb.ePc));
+    if (fixB) chain<1, QC, N, 1, FROM_INT, TO_DOUBLE, N>(C0, C1, tb.ePc, 5 * nb * N, exC, chain_gain(tb.ePc));
   }
   if (visc && !fixT) {
     if (AFF) {
@@ -1250,7 +1240,7 @@ __device__ __forceinline__ void coll_face_terms(const double* U, const T* Ud, co
               a += t[2 * nl + k2 * nf];
               b += t[3 * nl + k2 * nf];
             }
-            const int X = fx_exp(ex[15 + k]) + gT + 3;
+            const int X = fx_exp(exT[k * nb + e]) + gT + 3;
             lm += fx_store(a, X);
             lp += fx_store(b, X);
           }
@@ -1308,7 +1298,7 @@ __global__ void __launch_bounds__(coll_face_threads<T, N>()) dg_coll_face_kernel
   int* en = eo + FB_;
   int* oc = en + FB_;
   uint32_t* ex = reinterpret_cast<uint32_t*>(oc + FB_);
-  if (threadIdx.x < 20) ex[threadIdx.x] = 0;
+  for (int i = threadIdx.x; sizeof(T) == 8 && i < 20 * FB_; i += blockDim.x) ex[i] = 0;
   const int d = blockIdx.y;
   int s, nb;
   const Tab<T> tb = load_tables<T, N, QC, QV>(static_cast<const T*>(kp.tables), stab);
@@ -1358,7 +1348,7 @@ int launch_coll_cell(const KParams& kp, const double* U, void* Rout, void* dU, d
 
 template <typename T, int N, int QC, int QV, int FB_, int GEO>
 int launch_coll_faces_fb(const KParams& kp, const double* U, void* FB, cudaStream_t st) {
-  constexpr size_t smem = coll_face_smem<T, N, QC, QV, FB_>();
+  constexpr size_t smem = coll_face_smem<T, N, QC, QV>(FB_);
   static_assert(smem <= 227 * 1024, "face kernel shared memory");
   auto k = dg_coll_face_kernel<T, N, QC, QV, FB_, GEO>;
   static bool attr[kMaxDevices] = {};
