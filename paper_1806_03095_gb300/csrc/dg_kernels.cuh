@@ -391,10 +391,11 @@ __device__ __forceinline__ void sweep(const T* __restrict__ in, T* __restrict__ 
 }
 
 // ---------------------------------------------------------------------------
-// Reciprocal and square root of the point fluxes.  FP64: the hardware's seed (about 2^-20) and one
-// third-order step, r (1 + e + e^2) with e = 1 - x r (Householder's iteration; the error is e^3 and one
-// rounding): 3 FP64 instructions where the division measured 8 on GB300.  Outside the seed's range (zero,
-// denormal, huge, infinite, NaN) the division itself.
+// Reciprocal and square root of the point fluxes.  FP64: the hardware's seed (relative error 2^-20 at most) and one
+// third-order step; outside the seed's range (zero, denormal, huge, infinite, negative, NaN) the division and the square
+// root themselves.
+// Reciprocal: Householder's iteration r (1 + e + e^2), e = 1 - x r: 3 FP64 instructions where the division measured 8 on
+// GB300; within 1/2 + 2^-7 ulp (the truncated e^3 and the last rounding).
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ float rcp_of(float x) { return 1.f / x; }
 __device__ __forceinline__ double rcp_of(double x) {
@@ -405,7 +406,10 @@ __device__ __forceinline__ double rcp_of(double x) {
   const double e = fma(-x, r, 1.0);
   return fma(r, fma(e, e, e), r);
 }
-// sqrt(a), a >= 0: h = a y with y the seed of 1/sqrt(a), e = 1 - h y, h (1 + e/2 + 3 e^2/8).
+// Square root: y the seed of 1/sqrt(a), h = a y, e = 1 - h y, and the residual r = a - h^2, which one fused multiply-add
+// forms exactly up to its own rounding.  sqrt(a) - h = r / (sqrt(a) + h) = r y (1/2 + 3 e/8 + 5 e^2/16 + ...) (the binomial
+// series of (1 - e)^(1/2) = h / sqrt(a), and r y = h e); the terms from e^2 on are dropped.  h's rounding is in r, so the
+// result is within 1/2 + 2^-5.5 ulp: 6 FP64 instructions (adding h (e/2 + 3 e^2/8) to h takes 5 and errs 3/4 ulp).
 __device__ __forceinline__ float sqrt_of(float a) { return sqrtf(a); }
 __device__ __forceinline__ double sqrt_of(double a) {
   const uint32_t t = (uint32_t)__double2hiint(a);
@@ -413,8 +417,8 @@ __device__ __forceinline__ double sqrt_of(double a) {
   double y;
   asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(a));
   const double h = a * y;
-  const double e = fma(-h, y, 1.0);
-  return fma(h, fma(e, 0.375, 0.5) * e, h);
+  const double e = fma(-h, y, 1.0), r = fma(-h, h, a);
+  return fma(r * y, fma(e, 0.375, 0.5), h);
 }
 
 // ---------------------------------------------------------------------------
