@@ -329,7 +329,11 @@ __device__ __forceinline__ void sweep(const T* __restrict__ in, T* __restrict__ 
   constexpr int O2 = AX == 2 ? DOUT : D2;
   constexpr int ISZ = D0 * D1 * D2, OSZ = O0 * O1 * O2;
   constexpr int NL = ISZ / DIN;
-  if constexpr (sizeof(T) == 8) {
+  // FP64 lines of two values (k = 1) are too short for a call: inlined, and on the planes of the element-centric faces,
+  // whose code is the longest, in FP64.  20^3 cells, split, cell / face / M^-1 kernel: all in FP64 75 / 430 / 43 us, all by
+  // fx_sweep 92 / 449 / 47, all integer and inlined 45 / 752 / 31, this rule 45 / 432 / 31.
+  constexpr bool two = sizeof(T) == 8 && DIN * DOUT <= 4;
+  if constexpr (sizeof(T) == 8 && !two) {
     constexpr int n0 = AX == 0 ? 1 : (AX == 1 ? D0 : D0 * D1);
     constexpr uint32_t magic = n0 > 1 ? (uint32_t)((0x100000000ull + n0 - 1) / n0) : 0u;
     fx_sweep<DIN, DOUT, SYM, ACC>(in, out, E, nblk * NL, n0, magic, grp.rank(), grp.size());
@@ -369,7 +373,10 @@ __device__ __forceinline__ void sweep(const T* __restrict__ in, T* __restrict__ 
       for (int i = 0; i < DIN; ++i) x[i] = ip[i * IST];
     }
     T y[DOUT];
-    line_apply<T, DIN, DOUT, SYM>(Ep, x, y);
+    if constexpr (two && D2 == 1)
+      eo_apply<T, DIN, DOUT, SYM>(Ep.p, x, y);
+    else
+      line_apply<T, DIN, DOUT, SYM>(Ep, x, y);
     if (VOUT && (reinterpret_cast<uintptr_t>(op) & 15) == 0) {
       if (ACC) {
         T z[DOUT];
