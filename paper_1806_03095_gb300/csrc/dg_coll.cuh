@@ -1322,46 +1322,54 @@ constexpr bool coll_ok() {
   return QV == N && coll_rule(N, QV) && GEO != GEO_FLY && coll_cell_smem<T, N, QC, QV, 1>() <= 227 * 1024;
 }
 
-// Small meshes: where the usual batches would not give every SM its resident CTAs, half the cells (a third of the
-// faces) per CTA with as many threads, so that the phases of a CTA get shorter.
-constexpr int kSMs = 152;
-
+// Small meshes: half the cells or faces per CTA with as many threads, so that the phases of a CTA get shorter, as long as
+// all those CTAs are resident at once; beyond that the second, partly empty wave costs more than the shorter phases give
+// (FP64 L(U), half batches -> this rule: k = 3 9^3 cells 121 -> 105 us, k = 1 10^3 67 -> 45 us; FP32 k = 5 10^3 54 -> 42 us).
 template <typename T, int N, int QC, int QV, int CB, int GEO>
-int launch_coll_cell_cb(const KParams& kp, const double* U, void* Rout, void* dU, double* Uout, cudaStream_t st) {
+int launch_coll_cell_cb(const KParams& kp, bool only_one_wave, const double* U, void* Rout, void* dU, double* Uout,
+                        cudaStream_t st) {
   constexpr size_t smem = coll_cell_smem<T, N, QC, QV, CB>();
   static_assert(smem <= 227 * 1024, "cell kernel shared memory");
   auto k = dg_coll_cell_kernel<T, N, QC, QV, CB, GEO>;
+  constexpr int threads = coll_threads<T, N, QC, QV>();
   static bool attr[kMaxDevices] = {};
+  static int per_sm[kMaxDevices] = {};
   if (smem_attr_once(k, smem, attr)) return -1;
-  return launch_after(k, dim3((kp.Nc + CB - 1) / CB), coll_threads<T, N, QC, QV>(), smem, st, kp, U, static_cast<T*>(Rout),
-                      static_cast<T*>(dU), Uout);
+  const int ctas = (kp.Nc + CB - 1) / CB;
+  if (only_one_wave && !one_wave(k, threads, smem, ctas, per_sm)) return 1;
+  return launch_after(k, dim3(ctas), threads, smem, st, kp, U, static_cast<T*>(Rout), static_cast<T*>(dU), Uout);
 }
 template <typename T, int N, int QC, int QV, int GEO>
 int launch_coll_cell(const KParams& kp, const double* U, void* Rout, void* dU, double* Uout, cudaStream_t st) {
   constexpr int CB = coll_cells<T, N, QC, QV>();
   if constexpr (CB > 1) {
-    if (kp.Nc <= CB * kSMs * coll_ctas<T, N, QC, QV, CB>())
-      return launch_coll_cell_cb<T, N, QC, QV, 1, GEO>(kp, U, Rout, dU, Uout, st);
+    const int r = launch_coll_cell_cb<T, N, QC, QV, CB / 2, GEO>(kp, true, U, Rout, dU, Uout, st);
+    if (r <= 0) return r;
   }
-  return launch_coll_cell_cb<T, N, QC, QV, CB, GEO>(kp, U, Rout, dU, Uout, st);
+  return launch_coll_cell_cb<T, N, QC, QV, CB, GEO>(kp, false, U, Rout, dU, Uout, st);
 }
 
 template <typename T, int N, int QC, int QV, int FB_, int GEO>
-int launch_coll_faces_fb(const KParams& kp, const double* U, void* FB, cudaStream_t st) {
+int launch_coll_faces_fb(const KParams& kp, bool only_one_wave, const double* U, void* FB, cudaStream_t st) {
   constexpr size_t smem = coll_face_smem<T, N, QC, QV>(FB_);
   static_assert(smem <= 227 * 1024, "face kernel shared memory");
   auto k = dg_coll_face_kernel<T, N, QC, QV, FB_, GEO>;
+  constexpr int threads = coll_face_threads<T, N>();
   static bool attr[kMaxDevices] = {};
+  static int per_sm[kMaxDevices] = {};
   if (smem_attr_once(k, smem, attr)) return -1;
-  return launch_after(k, dim3(face_blocks(kp, FB_), 3), coll_face_threads<T, N>(), smem, st, kp, U, static_cast<T*>(FB));
+  const int blocks = face_blocks(kp, FB_);
+  if (only_one_wave && !one_wave(k, threads, smem, 3ll * blocks, per_sm)) return 1;
+  return launch_after(k, dim3(blocks, 3), threads, smem, st, kp, U, static_cast<T*>(FB));
 }
 template <typename T, int N, int QC, int QV, int GEO>
 int launch_coll_faces(const KParams& kp, const double* U, void* FB, cudaStream_t st) {
-  constexpr int FB_ = coll_faces<T, N, QC, QV>(), FS = FB_ / 2;
-  if constexpr (FS >= 1) {
-    if (3 * (kp.Nc / FB_) <= 4 * kSMs) return launch_coll_faces_fb<T, N, QC, QV, FS, GEO>(kp, U, FB, st);
+  constexpr int FB_ = coll_faces<T, N, QC, QV>();
+  if constexpr (FB_ > 1) {
+    const int r = launch_coll_faces_fb<T, N, QC, QV, FB_ / 2, GEO>(kp, true, U, FB, st);
+    if (r <= 0) return r;
   }
-  return launch_coll_faces_fb<T, N, QC, QV, FB_, GEO>(kp, U, FB, st);
+  return launch_coll_faces_fb<T, N, QC, QV, FB_, GEO>(kp, false, U, FB, st);
 }
 
 }  // namespace dgcns

@@ -230,4 +230,23 @@ inline int smem_attr_once(K kernel, size_t smem, bool* done) {
   return 0;
 }
 
+// Whether `ctas` CTAs of a kernel (its smem_attr_once done) are all resident at a time on GB300's 152 SMs; the count per
+// SM is asked once per (kernel, device) and kept in the launcher's static per_sm[] (0: not asked yet).
+constexpr int kSMs = 152;
+template <class K>
+inline bool one_wave(K kernel, int threads, size_t smem, long long ctas, int* per_sm) {
+  int dev = 0, n = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return false;
+  const bool keep = dev >= 0 && dev < kMaxDevices;
+  if (keep) n = per_sm[dev];
+  if (n == 0) {
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kernel, threads, smem) != cudaSuccess) {
+      cudaGetLastError();
+      return false;
+    }
+    if (keep) per_sm[dev] = n;
+  }
+  return ctas <= (long long)n * kSMs;
+}
+
 }  // namespace dgcns

@@ -425,20 +425,22 @@ constexpr bool task_faces_ok() {
 }
 
 template <int N, int QC, int QV, int FPB, int NTH>
-int launch_task_faces_fpb(const KParams& kp, void* FB, cudaStream_t st) {
+int launch_task_faces_fpb(const KParams& kp, bool only_one_wave, void* FB, cudaStream_t st) {
   constexpr size_t smem = task_face_smem_bytes<N, QC, QV, FPB>();
   static_assert(smem <= 227 * 1024, "task face kernel shared memory");
   auto k = dg_face_task_kernel<N, QC, QV, FPB, NTH>;
   static bool attr[kMaxDevices] = {};
+  static int per_sm[kMaxDevices] = {};
   if (smem_attr_once(k, smem, attr)) return -1;
-  return launch_after(k, dim3(face_blocks(kp, FPB), 3), NTH, smem, st, kp, static_cast<float*>(FB));
+  const int blocks = face_blocks(kp, FPB);
+  if (only_one_wave && !one_wave(k, NTH, smem, 3ll * blocks, per_sm)) return 1;
+  return launch_after(k, dim3(blocks, 3), NTH, smem, st, kp, static_cast<float*>(FB));
 }
-// 12 faces and 128 threads per CTA (120 trace and test tasks); on meshes that would not fill the chip with those,
-// 3 faces and one warp.
+// 12 faces and 128 threads per CTA (120 trace and test tasks); on small meshes, as in dg_coll.cuh, 3 faces and one warp.
 template <int N, int QC, int QV>
 int launch_task_faces(const KParams& kp, void* FB, cudaStream_t st) {
-  if (3 * (kp.Nc / 12) <= 4 * kSMs) return launch_task_faces_fpb<N, QC, QV, 3, 32>(kp, FB, st);
-  return launch_task_faces_fpb<N, QC, QV, 12, 128>(kp, FB, st);
+  const int r = launch_task_faces_fpb<N, QC, QV, 3, 32>(kp, true, FB, st);
+  return r <= 0 ? r : launch_task_faces_fpb<N, QC, QV, 12, 128>(kp, false, FB, st);
 }
 
 }  // namespace dgcns
