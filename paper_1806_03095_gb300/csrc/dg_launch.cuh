@@ -1279,10 +1279,12 @@ int launch_faces(const KParams& kp, const double* U, void* FB, cudaStream_t st) 
   if constexpr (use_coll<T, N, QC, QV, GEO>()) {
     // FP32 affine at k = 3: the register-resident kernel (1.13 ms against 1.46 ms per launch at 64^3, measured)
     if constexpr (sizeof(T) == 4 && GEO == GEO_AFFINE && task_faces_ok<N, QC, QV>()) {
-      if (kp.Udev != nullptr && kp.flist == nullptr && (reinterpret_cast<uintptr_t>(kp.Udev) & 15) == 0)
-        return launch_task_faces<N, QC, QV>(kp, FB, st);
+      // (a mixed evaluation starts with the deviation state, in a buffer of its own; face lists come with stored geometry)
+      if (kp.Udev == nullptr || kp.flist != nullptr) return -2;
+      return launch_task_faces<N, QC, QV>(kp, FB, st);
+    } else {
+      return launch_coll_faces<T, N, QC, QV, GEO>(kp, U, FB, st);
     }
-    return launch_coll_faces<T, N, QC, QV, GEO>(kp, U, FB, st);
   } else if constexpr (sizeof(T) == 4) {
     constexpr int WPC = 8;
     constexpr size_t smem = face_warp_smem_bytes<T, N, QC, QV, WPC, GEO>();
