@@ -218,14 +218,18 @@ __host__ __device__ __forceinline__ T stage_dt(const KParams& kp) {
 }
 
 // Dynamic shared-memory attribute of a kernel: a per-device setting, made once per (kernel, device) on
-// the current device.  done[] is the kernel's own flag array (a static of its launcher).
+// the current device.  done[] is the kernel's own flag array (a static of its launcher); carveout: the preferred share
+// of the SM's memory for shared memory (percent), -1 leaves it to the driver.
 constexpr int kMaxDevices = 64;
 template <class K>
-inline int smem_attr_once(K kernel, size_t smem, bool* done) {
+inline int smem_attr_once(K kernel, size_t smem, bool* done, int carveout = -1) {
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return -1;
   if (dev >= 0 && dev < kMaxDevices && done[dev]) return 0;
   if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return -1;
+  if (carveout >= 0 &&
+      cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, carveout) != cudaSuccess)
+    return -1;
   if (dev >= 0 && dev < kMaxDevices) done[dev] = true;
   return 0;
 }

@@ -792,16 +792,9 @@ constexpr int warp_slice_elems() {
   return (e + 7) & ~7;
 }
 
-// Elements before the first slice.  The face kernel of the split organisation keeps the room of all 1D tables, though
-// it copies only the weights: without it the kernel is slower (2.59 ms against 2.44 ms at 48^3, k = 3).
-template <typename T, int N, int QC, int QV, bool CELL, bool FACE>
-constexpr int warp_table_elems() {
-  return FACE && !CELL ? make_layout(N, QC, QV).total : table_elems<T, N, QC, QV>();
-}
-
 template <typename T, int N, int QC, int QV, int WPC, bool CELL, bool FACE, bool MASS, int GEO>
 constexpr size_t warp_smem_bytes() {
-  return ((size_t)warp_table_elems<T, N, QC, QV, CELL, FACE>() +
+  return ((size_t)table_elems<T, N, QC, QV>() +
           (size_t)WPC * warp_slice_elems<T, N, QC, QV, CELL, FACE, MASS, GEO>()) * sizeof(T) + 64;
 }
 
@@ -820,7 +813,7 @@ __global__ void __launch_bounds__(WPC * 32) dg_op_warp_kernel(const KParams kp, 
   const int e0 = blockIdx.x * WPC + w;
   if (e0 >= kp.Nc) return;  // only warp barriers below
   const WarpGroup grp;
-  T* su = stab + warp_table_elems<T, N, QC, QV, CELL, FACE>() + w * SL;
+  T* su = stab + table_elems<T, N, QC, QV>() + w * SL;
   T* sr = su + 5 * N3;
   T* sn = sr + 5 * N3;
   T* ar = sn + (FACE ? 5 * N3 : 0);
@@ -935,7 +928,10 @@ int launch_op_warp(const KParams& kp, const double* U, const void* Rin, void* Ro
   if (smem > 227 * 1024) return -2;
   auto k = dg_op_warp_kernel<T, N, QC, QV, WPC, CELL, FACE, MASS, GEO>;
   static bool attr[kMaxDevices] = {};
-  if (smem_attr_once(k, smem, attr)) return -1;
+  // Element-centric faces run faster with all of the SM's memory as shared memory than with the smallest partition that
+  // holds their resident CTAs, which the driver takes: 48^3, k = 3, split face kernel 2.59 -> 2.45 ms (six CTAs, which
+  // fit 196 KB too; L1 hits 21 -> 12 %), fused with geometry on the fly 9.9 -> 8.5 ms, other fused kernels unchanged.
+  if (smem_attr_once(k, smem, attr, FACE ? cudaSharedmemCarveoutMaxShared : -1)) return -1;
   const int grid = (kp.Nc + WPC - 1) / WPC;
   k<<<grid, WPC * 32, smem, st>>>(kp, U, static_cast<const T*>(Rin), static_cast<T*>(Rout), static_cast<T*>(dU),
                                     Uout);
