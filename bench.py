@@ -30,7 +30,11 @@ sys.path.insert(0, ROOT)
 
 METRIC = "GDoF/s per RK stage"
 UNIT = "GDoF/s"
-FP64_PEAK_TFLOPS = 1.2   # measured FP64 FMA throughput of this machine's GB300 (FMA-chain probe, 152 SMs)
+FP64_FMA_TFLOPS = 1.2    # measured FP64 FMA throughput of GB300 (FMA-chain probe, 152 SMs)
+# The FP64 kernels contract in integer arithmetic beside the FP64 pipe: 14 widening integer multiply-adds per SM and cycle
+# (throughput probe), three to a product, next to 1.6 FP64 ones: 6.3 multiply-adds, 3.2 times the FP64 pipe's own, before
+# the conversions between the two.
+FP64_PEAK_TFLOPS = 3.2 * FP64_FMA_TFLOPS
 FP32_PEAK_TFLOPS = 73.5  # measured FP32 FMA throughput, same probe
 
 
@@ -335,11 +339,9 @@ def roofline_entry(ktimes, cfg, prec, peaks):
     traffic, traffic_src = traffic_per_launch(dom, prec, N, QC, QV, Nc)
     return {"bound": "alu", "achieved": round(ach, 4), "peak": peak, "unit": "TFLOP/s", "frac": round(ach / peak, 4),
             "traffic": traffic, "traffic_source": traffic_src,
-            # flops count every 1D line as a dense product; the FP64 kernels do those lines in integer arithmetic, on
-            # other units than the FMA probe's, so that frac can exceed 1
-            "peak_source": "measured %s FMA probe (no %s entry in MEASURED_PEAKS.json)%s"
-            % ("FP32" if prec else "FP64", "FP32" if prec else "FP64",
-               "" if prec else "; FP64 contractions run on the integer units"),
+            "peak_source": "measured FP32 FMA probe (no FP32 entry in MEASURED_PEAKS.json)" if prec else
+            "measured FP64 FMA probe (%.1f TFLOP/s) and integer multiply-add probe together: FP64 contractions run on the "
+            "integer units (no FP64 entry in MEASURED_PEAKS.json)" % FP64_FMA_TFLOPS,
             "kernel": KERNEL_NAMES.get(dom, dom), "avg_launch_ms": round(kms / n, 4), "flops_per_launch": fl,
             "hbm": {"achieved": round(by / t / 1e9, 2), "peak": hbm_peak, "unit": "GB/s",
                     "frac": round(by / t / 1e9 / hbm_peak, 5), "bytes_per_launch": by},
