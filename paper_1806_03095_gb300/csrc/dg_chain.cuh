@@ -24,11 +24,12 @@ namespace dgcns {
 __device__ __forceinline__ int chain_gain(EoFp64 E, int room = 0) { return 64 - E.f[0].x - E.f[0].y + room; }
 
 // Maxima of blocks: slot[q stride + i] takes the largest m[q] over the lanes of block i (0 where a lane has none).
-// Whole warps call; blocks are runs of consecutive lanes, LEN lanes long (the first and last may be shorter): one
-// reduction per run and value, by atomics of the lanes themselves where the runs are short.
+// By atomics of the lanes, or, where blocks are runs of LEN > 16 consecutive lanes (the first and last may be shorter),
+// one reduction per run and value; whole warps call.  Measured at 48^3, k = 3: cell kernel 4.0 ms (atomics of all lanes
+// 4.5, reductions also for its runs of 16 4.05), face kernel 4.53 ms with atomics (reductions 4.86).
 template <int LEN, int K>
 __device__ __forceinline__ void block_max(uint32_t* slot, int stride, int i, const uint32_t (&m)[K]) {
-  if constexpr (LEN < 8) {
+  if constexpr (LEN <= 16) {
 #pragma unroll
     for (int q = 0; q < K; ++q)
       if (m[q]) atomicMax(slot + q * stride + i, m[q]);

@@ -446,6 +446,7 @@ __global__ void __launch_bounds__(coll_threads<T, N, QC, QV>(), coll_ctas<T, N, 
   if constexpr (FX) {
     constexpr int PV = (N3 + NTE - 1) / NTE;
     const bool own = pe < nb;
+    const T* sh = FBc + (own ? pe : 0) * fbuf_per_cell<N>();
     double x[5][PV];
 #pragma unroll
     for (int c = 0; c < 5; ++c)
@@ -466,9 +467,12 @@ __global__ void __launch_bounds__(coll_threads<T, N, QC, QV>(), coll_ctas<T, N, 
         m[c] = max(m[c], fx_mag(x[c][k]));
       }
       // the shares of the batch, also brought nearer for the lift sweeps
-      for (int i = pt; own && i < 12 * N2; i += NTE)
-        f[c] = max(f[c], reinterpret_cast<const uint32_t*>(FBc + pe * fbuf_per_cell<N>() + (i / N2 * 5 + c) * N2 + i % N2)[1] &
-                             0x7fffffffu);
+#pragma unroll
+      for (int k = 0; k < (12 * N2 + NTE - 1) / NTE; ++k) {
+        // (past the end the cell's last share again, so that no load waits for a condition)
+        const int i = min(k * NTE + pt, 12 * N2 - 1);
+        f[c] = max(f[c], reinterpret_cast<const uint32_t*>(sh + (i / N2 * 5 + c) * N2 + i % N2)[1] & 0x7fffffffu);
+      }
     }
     if (own) {
       block_max<32>(exU + pe * 5, 1, 0, m);
@@ -836,6 +840,12 @@ template <typename T, int N>
 constexpr int coll_face_threads() {
   return sizeof(T) == 4 && N >= 5 ? 256 : 128;
 }
+// Resident CTAs that the registers have to allow: FP64 four, with general metrics three (168 registers; without the bound
+// they are two and the kernel a third slower); FP32 0, no bound.
+template <typename T, int GEO>
+constexpr int coll_face_ctas() {
+  return sizeof(T) == 4 ? 0 : (GEO == GEO_AFFINE ? 4 : 3);
+}
 
 template <typename T, int N, int QC, int QV, int FB_, int D, int GEO>
 __device__ __forceinline__ void coll_face_terms(const double* U, const T* Ud, const int* eo,
@@ -859,15 +869,16 @@ __device__ __forceinline__ void coll_face_terms(const double* U, const T* Ud, co
   constexpr bool FX = sizeof(T) == 8;  // integer chains
   constexpr int NTT = AFF ? 3 : 5;     // tested components of a tangential direction
   // FP64: maxima of the blocks (slot, face), both sides together: of the traces, of the normal derivatives, of the
-  // convective flux and of the tangential gradient tests
+  // convective flux and of the tangential gradient tests (on an axis-aligned face m_t1 along t1 and m_t2 along t2 share
+  // a block: both are -2/3 mu g_D / rho times 1/h_t1 or 1/h_t2, so the smaller is cut by the aspect ratio of two faces of the cell, less
+  // than the rounding of its own row's derivatives across that aspect ratio)
   uint32_t *exL = ex, *exD = exL + 5 * FB_, *exC = exD + 5 * FB_, *exT = exC + 5 * FB_;
   auto see = [&](uint32_t& m, T v) {
     if constexpr (FX) m = max(m, fx_mag(v));
     return v;
   };
   // traces along the normal lines, from global memory
-  for (int idx0 = threadIdx.x; (FX ? idx0 & ~31 : idx0) < nl; idx0 += NTH) {  // (FP64: whole warps, for the maxima)
-    const int idx = FX ? min(idx0, nl - 1) : idx0;
+  for (int idx = threadIdx.x; idx < nl; idx += NTH) {
     const int sl = idx / nf, r = idx - sl * nf, e = r / N2, j = r - e * N2;
     const int c = slot_comp<D>(sl);
     const int q0 = face_node<N>(D, 0, j % N, j / N);
@@ -921,15 +932,13 @@ __device__ __forceinline__ void coll_face_terms(const double* U, const T* Ud, co
       }
     }
     const T vm = s ? a[N - 1] : a[0], vp = s ? b[0] : b[N - 1];
-    if (!FX || idx0 < nl) {
-      VV[idx] = vm;
-      VV[nl + idx] = vp;
-      VV[2 * nl + idx] = dm;
-      VV[3 * nl + idx] = dp;
-    }
+    VV[idx] = vm;
+    VV[nl + idx] = vp;
+    VV[2 * nl + idx] = dm;
+    VV[3 * nl + idx] = dp;
     if constexpr (FX) {
       const uint32_t m[2] = {max(fx_mag(vm), fx_mag(vp)), max(fx_mag(dm), fx_mag(dp))};
-      block_max<N2>(exL, 5 * FB_, idx / N2, m);
+      block_max<1>(exL, 5 * FB_, idx / N2, m);
     }
   }
   __syncthreads();
@@ -969,38 +978,36 @@ __device__ __forceinline__ void coll_face_terms(const double* U, const T* Ud, co
   // convective flux (point arithmetic); tangential derivatives (sweeps)
   if (conv) {
     const int nc = nb * QC2;
-    for (int idx = threadIdx.x; (FX ? idx & ~31 : idx) < nc; idx += NTH) {
+    for (int idx = threadIdx.x; idx < nc; idx += NTH) {
       uint32_t mC[5] = {0, 0, 0, 0, 0};
-      if (!FX || idx < nc) {
-        const int e = idx / QC2, p = idx - e * QC2;
-        T um[5], up[5], fm[5], fp[5], n[3] = {T(0), T(0), T(0)}, w;
+      const int e = idx / QC2, p = idx - e * QC2;
+      T um[5], up[5], fm[5], fp[5], n[3] = {T(0), T(0), T(0)}, w;
 #pragma unroll
-        for (int q = 0; q < 5; ++q) {
-          um[slot_comp<D>(q)] = C1[q * nc + idx];
-          up[slot_comp<D>(q)] = C1[(5 + q) * nc + idx];
-        }
-        if (en[e] < 0) wall_ghost(um, ph, up);
-        if (AFF) {
-          w = T(-0.5) * kc.hinv[D];
-        } else {
-          const T* g = static_cast<const T*>(kp.gfc) + ((size_t)eo[e] * 6 + f) * 13 * QC2 + p;
-          n[0] = g[9 * QC2];
-          n[1] = g[10 * QC2];
-          n[2] = g[11 * QC2];
-          w = T(-0.5) * g[12 * QC2];
-        }
-        T lm, lp;
-        const T ws = AFF && !s ? -w : w;
-        llf_side<T, D, AFF>(um, n, ws, ph, fm, lm);
-        llf_side<T, D, AFF>(up, n, ws, ph, fp, lp);
-        const T lam = w * (lm > lp ? lm : lp);
-#pragma unroll
-        for (int q = 0; q < 5; ++q) {
-          const int c = slot_comp<D>(q);
-          C1[q * nc + idx] = see(mC[q], fm[c] + fp[c] + lam * (um[c] - up[c]));
-        }
+      for (int q = 0; q < 5; ++q) {
+        um[slot_comp<D>(q)] = C1[q * nc + idx];
+        up[slot_comp<D>(q)] = C1[(5 + q) * nc + idx];
       }
-      if constexpr (FX) block_max<QC2>(exC, nb, min(idx, nc - 1) / QC2, mC);
+      if (en[e] < 0) wall_ghost(um, ph, up);
+      if (AFF) {
+        w = T(-0.5) * kc.hinv[D];
+      } else {
+        const T* g = static_cast<const T*>(kp.gfc) + ((size_t)eo[e] * 6 + f) * 13 * QC2 + p;
+        n[0] = g[9 * QC2];
+        n[1] = g[10 * QC2];
+        n[2] = g[11 * QC2];
+        w = T(-0.5) * g[12 * QC2];
+      }
+      T lm, lp;
+      const T ws = AFF && !s ? -w : w;
+      llf_side<T, D, AFF>(um, n, ws, ph, fm, lm);
+      llf_side<T, D, AFF>(up, n, ws, ph, fp, lp);
+      const T lam = w * (lm > lp ? lm : lp);
+#pragma unroll
+      for (int q = 0; q < 5; ++q) {
+        const int c = slot_comp<D>(q);
+        C1[q * nc + idx] = see(mC[q], fm[c] + fp[c] + lam * (um[c] - up[c]));
+      }
+      if constexpr (FX) block_max<1>(exC, nb, e, mC);
     }
   }
   if constexpr (FX) {
@@ -1033,146 +1040,144 @@ __device__ __forceinline__ void coll_face_terms(const double* U, const T* Ud, co
   __syncthreads();
   // viscous fluxes (point arithmetic); projection of the convective flux (sweeps).  Shares are of -F.
   if (visc) {
-    for (int idx = threadIdx.x; (FX ? idx & ~31 : idx) < nf; idx += NTH) {
+    for (int idx = threadIdx.x; idx < nf; idx += NTH) {
       uint32_t mT[NTT] = {};
-      if (!FX || idx < nf) {
-        const int e = idx / N2, p = idx - e * N2;
-        const bool wall = en[e] < 0;
-        T um[5], up[5], jmp[5];
+      const int e = idx / N2, p = idx - e * N2;
+      const bool wall = en[e] < 0;
+      T um[5], up[5], jmp[5];
+#pragma unroll
+      for (int q = 0; q < 5; ++q) {
+        T a = VV[q * nf + idx], b = VV[nl + q * nf + idx];
+        if constexpr (FX) {
+          if (fixA) {
+            const int X = fx_exp(exL[q * nb + e]) + gS + 3;
+            a = fx_store(__double_as_longlong(a), X);
+            b = fx_store(__double_as_longlong(b), X);
+          }
+        }
+        um[slot_comp<D>(q)] = a;
+        up[slot_comp<D>(q)] = b;
+      }
+      if (wall) wall_ghost(um, ph, up);
+      const SideState<T> sm_ = side_state(um, ph), sp_ = side_state(up, ph);
+      const T tau = tau_f[e];
+#pragma unroll
+      for (int c = 0; c < 5; ++c) jmp[c] = um[c] - up[c];
+      T fm[4], fp[4];
+      if (AFF) {
+        const T hd = kc.hinv[D];
+        T* T1m = TT + idx;
+        T* T1p = T1m + nl;
+        T* T2m = T1p + nl;
+        T* T2p = T2m + nl;
+        T gm[5], gp[5];
 #pragma unroll
         for (int q = 0; q < 5; ++q) {
-          T a = VV[q * nf + idx], b = VV[nl + q * nf + idx];
-          if constexpr (FX) {
-            if (fixA) {
-              const int X = fx_exp(exL[q * nb + e]) + gS + 3;
-              a = fx_store(__double_as_longlong(a), X);
-              b = fx_store(__double_as_longlong(b), X);
-            }
-          }
-          um[slot_comp<D>(q)] = a;
-          up[slot_comp<D>(q)] = b;
+          gm[slot_comp<D>(q)] = VV[2 * nl + q * nf + idx];
+          gp[slot_comp<D>(q)] = VV[3 * nl + q * nf + idx];
         }
-        if (wall) wall_ghost(um, ph, up);
-        const SideState<T> sm_ = side_state(um, ph), sp_ = side_state(up, ph);
-        const T tau = tau_f[e];
+        visc_normal<T, D>(sm_, gm, T1m[nf], T1m[2 * nf], T1m[0], T2m[0], T2m[nf], T2m[2 * nf], kc, fm);
+        if (wall)  // grad U+ = grad U-, at the ghost state
+          visc_normal<T, D>(sp_, gm, T1m[nf], T1m[2 * nf], T1m[0], T2m[0], T2m[nf], T2m[2 * nf], kc, fp);
+        else
+          visc_normal<T, D>(sp_, gp, T1p[nf], T1p[2 * nf], T1p[0], T2p[0], T2p[nf], T2p[2 * nf], kc, fp);
+        // value share (own side): (V, Q*.n), Q*.n = {{F_v}}.n - tau [[U]]; the other side's is the negative
+        const T wv = s ? T(0.5) * hd : T(-0.5) * hd, wt = hd * tau;
+        const int fs[5] = {1, -1, 0, 2, 3};  // slot -> entry of fm
 #pragma unroll
-        for (int c = 0; c < 5; ++c) jmp[c] = um[c] - up[c];
-        T fm[4], fp[4];
-        if (AFF) {
-          const T hd = kc.hinv[D];
-          T* T1m = TT + idx;
-          T* T1p = T1m + nl;
-          T* T2m = T1p + nl;
-          T* T2p = T2m + nl;
-          T gm[5], gp[5];
+        for (int q = 0; q < 5; ++q) {
+          const T t = -wt * jmp[slot_comp<D>(q)];
+          VV[q * nf + idx] = fs[q] < 0 ? t : t + wv * (fm[fs[q] < 0 ? 0 : fs[q]] + fp[fs[q] < 0 ? 0 : fs[q]]);
+        }
+        // +1/2 (grad V, F_v(U, [[U]])), [[U]] = sgn jmp (x) e_D
+        if (!s) {
 #pragma unroll
-          for (int q = 0; q < 5; ++q) {
-            gm[slot_comp<D>(q)] = VV[2 * nl + q * nf + idx];
-            gp[slot_comp<D>(q)] = VV[3 * nl + q * nf + idx];
-          }
-          visc_normal<T, D>(sm_, gm, T1m[nf], T1m[2 * nf], T1m[0], T2m[0], T2m[nf], T2m[2 * nf], kc, fm);
-          if (wall)  // grad U+ = grad U-, at the ghost state
-            visc_normal<T, D>(sp_, gm, T1m[nf], T1m[2 * nf], T1m[0], T2m[0], T2m[nf], T2m[2 * nf], kc, fp);
-          else
-            visc_normal<T, D>(sp_, gp, T1p[nf], T1p[2 * nf], T1p[0], T2p[0], T2p[nf], T2p[2 * nf], kc, fp);
-          // value share (own side): (V, Q*.n), Q*.n = {{F_v}}.n - tau [[U]]; the other side's is the negative
-          const T wv = s ? T(0.5) * hd : T(-0.5) * hd, wt = hd * tau;
-          const int fs[5] = {1, -1, 0, 2, 3};  // slot -> entry of fm
+          for (int c = 0; c < 5; ++c) jmp[c] = -jmp[c];
+        }
+        T a[4], b1[3], b2[3];
+        visc_jump<T, D>(sm_, jmp, kc, a, b1, b2);
+        VV[2 * nl + idx] = a[1];
+        VV[2 * nl + nf + idx] = T(0);
+        VV[2 * nl + 2 * nf + idx] = a[0];
+        VV[2 * nl + 3 * nf + idx] = a[2];
+        VV[2 * nl + 4 * nf + idx] = a[3];
 #pragma unroll
-          for (int q = 0; q < 5; ++q) {
-            const T t = -wt * jmp[slot_comp<D>(q)];
-            VV[q * nf + idx] = fs[q] < 0 ? t : t + wv * (fm[fs[q] < 0 ? 0 : fs[q]] + fp[fs[q] < 0 ? 0 : fs[q]]);
-          }
-          // +1/2 (grad V, F_v(U, [[U]])), [[U]] = sgn jmp (x) e_D
-          if (!s) {
+        for (int i = 0; i < 3; ++i) {
+          T1m[i * nf] = see(mT[i], b1[i]);
+          T2m[i * nf] = see(mT[i], b2[i]);
+        }
+        if (!wall) visc_jump<T, D>(sp_, jmp, kc, a, b1, b2);
+        VV[3 * nl + idx] = a[1];
+        VV[3 * nl + nf + idx] = T(0);
+        VV[3 * nl + 2 * nf + idx] = a[0];
+        VV[3 * nl + 3 * nf + idx] = a[2];
+        VV[3 * nl + 4 * nf + idx] = a[3];
 #pragma unroll
-            for (int c = 0; c < 5; ++c) jmp[c] = -jmp[c];
-          }
-          T a[4], b1[3], b2[3];
-          visc_jump<T, D>(sm_, jmp, kc, a, b1, b2);
-          VV[2 * nl + idx] = a[1];
-          VV[2 * nl + nf + idx] = T(0);
-          VV[2 * nl + 2 * nf + idx] = a[0];
-          VV[2 * nl + 3 * nf + idx] = a[2];
-          VV[2 * nl + 4 * nf + idx] = a[3];
+        for (int i = 0; i < 3; ++i) {
+          T1p[i * nf] = see(mT[i], b1[i]);
+          T2p[i * nf] = see(mT[i], b2[i]);
+        }
+      } else {
+        const T* g = static_cast<const T*>(kp.gfv) + ((size_t)eo[e] * 6 + f) * 13 * N2 + p;
+        T Jm[9], Jp[9], n[3];
 #pragma unroll
-          for (int i = 0; i < 3; ++i) {
-            T1m[i * nf] = see(mT[i], b1[i]);
-            T2m[i * nf] = see(mT[i], b2[i]);
-          }
-          if (!wall) visc_jump<T, D>(sp_, jmp, kc, a, b1, b2);
-          VV[3 * nl + idx] = a[1];
-          VV[3 * nl + nf + idx] = T(0);
-          VV[3 * nl + 2 * nf + idx] = a[0];
-          VV[3 * nl + 3 * nf + idx] = a[2];
-          VV[3 * nl + 4 * nf + idx] = a[3];
-#pragma unroll
-          for (int i = 0; i < 3; ++i) {
-            T1p[i * nf] = see(mT[i], b1[i]);
-            T2p[i * nf] = see(mT[i], b2[i]);
-          }
+        for (int m = 0; m < 9; ++m) Jm[m] = g[m * N2];
+        n[0] = g[9 * N2];
+        n[1] = g[10 * N2];
+        n[2] = g[11 * N2];
+        const T dA = g[12 * N2];
+        if (!wall && oc) {
+          frame_face_jinv<T, N>(static_cast<const T*>(kp.gfv), en[e], oc[e], D, s, p, Jp);
         } else {
-          const T* g = static_cast<const T*>(kp.gfv) + ((size_t)eo[e] * 6 + f) * 13 * N2 + p;
-          T Jm[9], Jp[9], n[3];
+          const T* gp = wall ? g : static_cast<const T*>(kp.gfv) + ((size_t)en[e] * 6 + fo) * 13 * N2 + p;
 #pragma unroll
-          for (int m = 0; m < 9; ++m) Jm[m] = g[m * N2];
-          n[0] = g[9 * N2];
-          n[1] = g[10 * N2];
-          n[2] = g[11 * N2];
-          const T dA = g[12 * N2];
-          if (!wall && oc) {
-            frame_face_jinv<T, N>(static_cast<const T*>(kp.gfv), en[e], oc[e], D, s, p, Jp);
-          } else {
-            const T* gp = wall ? g : static_cast<const T*>(kp.gfv) + ((size_t)en[e] * 6 + fo) * 13 * N2 + p;
+          for (int m = 0; m < 9; ++m) Jp[m] = gp[m * N2];
+        }
+        T G[5][3];
 #pragma unroll
-            for (int m = 0; m < 9; ++m) Jp[m] = gp[m * N2];
-          }
-          T G[5][3];
+        for (int q = 0; q < 5; ++q) {
+          const T a1 = TT[q * nf + idx], a2 = TT[2 * nl + q * nf + idx], ad = VV[2 * nl + q * nf + idx];
+#pragma unroll
+          for (int a = 0; a < 3; ++a) G[slot_comp<D>(q)][a] = Jm[3 * t1 + a] * a1 + Jm[3 * t2 + a] * a2 + Jm[3 * D + a] * ad;
+        }
+        visc_normal_any(sm_, G, n, ph, fm);
+        if (!wall) {
 #pragma unroll
           for (int q = 0; q < 5; ++q) {
-            const T a1 = TT[q * nf + idx], a2 = TT[2 * nl + q * nf + idx], ad = VV[2 * nl + q * nf + idx];
+            const T a1 = TT[nl + q * nf + idx], a2 = TT[3 * nl + q * nf + idx], ad = VV[3 * nl + q * nf + idx];
 #pragma unroll
-            for (int a = 0; a < 3; ++a) G[slot_comp<D>(q)][a] = Jm[3 * t1 + a] * a1 + Jm[3 * t2 + a] * a2 + Jm[3 * D + a] * ad;
+            for (int a = 0; a < 3; ++a) G[slot_comp<D>(q)][a] = Jp[3 * t1 + a] * a1 + Jp[3 * t2 + a] * a2 + Jp[3 * D + a] * ad;
           }
-          visc_normal_any(sm_, G, n, ph, fm);
-          if (!wall) {
+        }
+        visc_normal_any(sp_, G, n, ph, fp);
+        const T hw = T(0.5) * dA, wt = dA * tau;
+#pragma unroll
+        for (int q = 0; q < 5; ++q) {
+          const int c = slot_comp<D>(q);
+          const T t = -wt * jmp[c];
+          VV[q * nf + idx] = c == 0 ? t : t + hw * (fm[c == 0 ? 0 : c - 1] + fp[c == 0 ? 0 : c - 1]);
+        }
+#pragma unroll
+        for (int sd = 0; sd < 2; ++sd) {
+          const SideState<T>& ss = sd ? sp_ : sm_;
+          const T* J = sd ? Jp : Jm;
+          const JumpFlux<T> jf = visc_jump_any(ss, jmp, n, ph);
+          T* dst[3] = {TT + sd * nl + idx, TT + (2 + sd) * nl + idx, VV + (2 + sd) * nl + idx};
+          const int row[3] = {t1, t2, D};
+#pragma unroll
+          for (int b = 0; b < 3; ++b) {
+            T r[4];
+            jump_row(jf, ss, n, J + 3 * row[b], hw, r);
 #pragma unroll
             for (int q = 0; q < 5; ++q) {
-              const T a1 = TT[nl + q * nf + idx], a2 = TT[3 * nl + q * nf + idx], ad = VV[3 * nl + q * nf + idx];
-#pragma unroll
-              for (int a = 0; a < 3; ++a) G[slot_comp<D>(q)][a] = Jp[3 * t1 + a] * a1 + Jp[3 * t2 + a] * a2 + Jp[3 * D + a] * ad;
-            }
-          }
-          visc_normal_any(sp_, G, n, ph, fp);
-          const T hw = T(0.5) * dA, wt = dA * tau;
-#pragma unroll
-          for (int q = 0; q < 5; ++q) {
-            const int c = slot_comp<D>(q);
-            const T t = -wt * jmp[c];
-            VV[q * nf + idx] = c == 0 ? t : t + hw * (fm[c == 0 ? 0 : c - 1] + fp[c == 0 ? 0 : c - 1]);
-          }
-#pragma unroll
-          for (int sd = 0; sd < 2; ++sd) {
-            const SideState<T>& ss = sd ? sp_ : sm_;
-            const T* J = sd ? Jp : Jm;
-            const JumpFlux<T> jf = visc_jump_any(ss, jmp, n, ph);
-            T* dst[3] = {TT + sd * nl + idx, TT + (2 + sd) * nl + idx, VV + (2 + sd) * nl + idx};
-            const int row[3] = {t1, t2, D};
-#pragma unroll
-            for (int b = 0; b < 3; ++b) {
-              T r[4];
-              jump_row(jf, ss, n, J + 3 * row[b], hw, r);
-#pragma unroll
-              for (int q = 0; q < 5; ++q) {
-                const int c = slot_comp<D>(q);
-                const T v = c == 0 ? T(0) : r[c == 0 ? 0 : c - 1];
-                dst[b][q * nf] = b < 2 ? see(mT[q], v) : v;
-              }
+              const int c = slot_comp<D>(q);
+              const T v = c == 0 ? T(0) : r[c == 0 ? 0 : c - 1];
+              dst[b][q * nf] = b < 2 ? see(mT[q], v) : v;
             }
           }
         }
       }
-      if constexpr (FX) block_max<N2>(exT, nb, min(idx, nf - 1) / N2, mT);
+      if constexpr (FX) block_max<1>(exT, nb, e, mT);
     }
   }
   bool fixB = false, fixT = false;
@@ -1288,7 +1293,7 @@ __device__ __forceinline__ void coll_face_terms(const double* U, const T* Ud, co
 
 // blockIdx.y = direction; blocks as dg_face_kernel.
 template <typename T, int N, int QC, int QV, int FB_, int GEO>
-__global__ void __launch_bounds__(coll_face_threads<T, N>()) dg_coll_face_kernel(const KParams kp,
+__global__ void __launch_bounds__(coll_face_threads<T, N>(), coll_face_ctas<T, GEO>()) dg_coll_face_kernel(const KParams kp,
                                                                               const double* U, T* FBuf) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   T* stab = reinterpret_cast<T*>(smem_raw);
