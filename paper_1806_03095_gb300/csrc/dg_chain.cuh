@@ -13,8 +13,8 @@
 // total residual) the values fall far below that bound, so the next sweep first shifts each line up to the full
 // width (RENORM) and ends in doubles, and a new chain starts from their maxima.  (Without this the error of L(U)
 // at 40^3, k = 5 grew from 1.1e-14 to 5.5e-13.)  A chain ends with one rounding to 53 bits.
-// A batch whose exponents leave fx_exp_ok's range (NaN, infinities, denormals, extreme scales) takes the
-// line-by-line sweeps.
+// A CTA that holds an exponent outside fx_exp_ok's range (NaN, infinities, denormals, extreme scales) takes the
+// line-by-line sweeps for all its cells or faces, whose last bits may then differ.
 #pragma once
 #include "dg_kernels.cuh"
 
@@ -67,10 +67,10 @@ __device__ __forceinline__ int fx_renorm(int64_t (&F)[D]) {
   return s;
 }
 
-// Lines as lines_fp64; blocks of LPB lines (PER = LPB / n0 outer indices each), a block's exponent fx_exp(ex[b]) + add for integer inputs (value
-// F 2^(exponent - 1083)) and without add for doubles; from block `nex` on the exponents repeat (a face's two sides).
-// Integer outputs keep `room` bits free.  FROM_SUM: the input is the sum of three integer arrays ks apart, renormalised,
-// and the maxima of the outputs' blocks go to omax.
+// Lines as lines_fp64, in blocks of LPB lines (PER = LPB / n0 outer indices each).  A block's exponent is fx_exp(ex[b]) +
+// add for integer inputs (value F 2^(exponent - 1083)) and without add for doubles; from block `nex` on the exponents
+// repeat (a face's two sides).  Integer outputs keep `room` bits free.  FROM_SUM: the input is the sum of three integer
+// arrays ks apart, renormalised, and the maxima of the outputs' blocks go to omax.
 template <int DIN, int DOUT, int SYM, int IN, int OUT, int LPB, int PER, int OG, int IBS, int OBS>
 __device__ __forceinline__ void chain_fp64(const double* in, int ks, double* out, EoFp64 E, int nlines, int n0,
                                         uint32_t magic, int nex, const uint32_t* ex, int add, int room, uint32_t* omax) {

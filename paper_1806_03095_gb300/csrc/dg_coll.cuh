@@ -19,13 +19,13 @@
 //
 // Measured per launch (face / cell + stage kernel), against the kernels that test with the LGL basis and contract in
 // FP64, and with the integer sweeps of both (dg_fixed.cuh):
-// FP64 TGV 64^3, k = 3: 30.5 -> 24.6 -> 11.8 / 32.5 -> 21.2 -> 10.8 ms; 40^3, k = 5: 20.4 -> 14.9 -> 9.3 /
-// 35.8 -> 25.7 -> 13.0 ms; FP64 channel 32^3, k = 3 (stored geometry), with and without the chains of the M^-1 sweeps:
-// cell 1.96 -> 1.78 ms.
-// FP32 40^3, k = 5: 1.36 -> 0.88 / 2.51 -> 1.21 ms; channel 32^3, k = 3: 0.36 -> 0.24 / 0.36 -> 0.24 ms;
+// FP64 TGV 64^3, k = 3: 30.5 -> 24.6 -> 10.8 / 32.5 -> 21.2 -> 9.3 ms; 40^3, k = 5: 20.4 -> 14.9 -> 9.1 /
+// 35.8 -> 25.7 -> 12.1 ms; FP64 channel 32^3, k = 3 (stored geometry): cell 1.65 ms (1.96 without the chains of the M^-1
+// sweeps, before the share scan's loads were issued together).
+// FP32 40^3, k = 5: 1.36 -> 0.88 / 2.51 -> 1.23 ms; channel 32^3, k = 3: 0.36 -> 0.24 / 0.36 -> 0.24 ms;
 // FP32 64^3, k = 3, cell + stage: 2.14 (register-resident tasks, one cell per CTA) -> 1.39 ms.
-// Bound by: FP64 faces the FP64 pipe in the point phases (60 % busy overall) and latency; FP64 cells latency (ALU and
-// FP64 pipes about 40 % each, four CTAs per SM); FP32 shared-memory wavefronts (82 %) and issue (61 %).
+// Bound by: FP64 faces the FP64 pipe in the point phases (63 % busy overall) and latency; FP64 cells latency (FP64 pipe
+// 49 %, ALU 42 %, four CTAs per SM); FP32 shared-memory wavefronts (89 %) and issue (62 %).
 #pragma once
 #include "dg_chain.cuh"
 #include "dg_faces.cuh"
@@ -388,9 +388,10 @@ constexpr int coll_cells() {
   return cb;
 }
 // Threads: 128, and more where only two (FP64) or four (FP32) large cells fit an SM.  Measured: FP64 k = 3, 2 cells
-// and 128 threads 14.9 ms per stage at 64^3 (192 threads 17.4, one cell 17.9 to 23.6), before the chains, now 10.8;
+// and 128 threads 14.9 ms per stage at 64^3 (192 threads 17.4, one cell 17.9 to 23.6), before the chains, now 9.3;
 // FP64 k = 5, 40^3, 192 threads 15.2 ms (128: 18.5, 256: 27.0, their registers no longer hold the point fluxes), now
-// 13.0; FP32 k = 5, 256 threads 1.30 ms (128: 1.67, 192: 1.34), now 1.21; FP32 k = 3 stored, 32^3, 2 cells and 128 threads 0.264 ms (256: 0.326; one cell 0.277).
+// 12.1; FP32 k = 5, 256 threads 1.30 ms (128: 1.67, 192: 1.34), now 1.23; FP32 k = 3 stored, 32^3, 2 cells and 128
+// threads 0.264 ms (256: 0.326; one cell 0.277).
 template <typename T, int N, int QC, int QV>
 constexpr int coll_threads() {
   constexpr size_t smem = coll_cell_smem<T, N, QC, QV, coll_cells<T, N, QC, QV>()>();
@@ -869,9 +870,9 @@ __device__ __forceinline__ void coll_face_terms(const double* U, const T* Ud, co
   constexpr bool FX = sizeof(T) == 8;  // integer chains
   constexpr int NTT = AFF ? 3 : 5;     // tested components of a tangential direction
   // FP64: maxima of the blocks (slot, face), both sides together: of the traces, of the normal derivatives, of the
-  // convective flux and of the tangential gradient tests (on an axis-aligned face m_t1 along t1 and m_t2 along t2 share
-  // a block: both are -2/3 mu g_D / rho times 1/h_t1 or 1/h_t2, so the smaller is cut by the aspect ratio of two faces of the cell, less
-  // than the rounding of its own row's derivatives across that aspect ratio)
+  // convective flux and of the tangential gradient tests.  (On an axis-aligned face m_t1 along t1 and m_t2 along t2 share
+  // a block: both are -2/3 mu g_D / rho, times 1/h_t1 and 1/h_t2, so that the smaller loses the bits of that aspect ratio,
+  // of 61; its row's own second derivatives lose twice as many to rounding, of 53.)
   uint32_t *exL = ex, *exD = exL + 5 * FB_, *exC = exD + 5 * FB_, *exT = exC + 5 * FB_;
   auto see = [&](uint32_t& m, T v) {
     if constexpr (FX) m = max(m, fx_mag(v));
@@ -1321,7 +1322,8 @@ __global__ void __launch_bounds__(coll_face_threads<T, N>(), coll_face_ctas<T, G
     coll_face_terms<T, N, QC, QV, FB_, 2, GEO>(U, Ud, eo, en, ocp, tau_f, sm, tb, kp, ph, nb, s, FBuf, ex);
 }
 
-// Where the collocation kernels are used.
+// Where the collocation kernels exist; the face-centric organisation then runs them (face and cell kernel share the face
+// buffer's basis, so both follow this rule).
 template <typename T, int N, int QC, int QV, int GEO>
 constexpr bool coll_ok() {
   return QV == N && coll_rule(N, QV) && GEO != GEO_FLY && coll_cell_smem<T, N, QC, QV, 1>() <= 227 * 1024;
@@ -1329,7 +1331,8 @@ constexpr bool coll_ok() {
 
 // Small meshes: half the cells or faces per CTA with as many threads, so that the phases of a CTA get shorter, as long as
 // all those CTAs are resident at once; beyond that the second, partly empty wave costs more than the shorter phases give
-// (FP64 L(U), half batches -> this rule: k = 3 9^3 cells 121 -> 105 us, k = 1 10^3 67 -> 45 us; FP32 k = 5 10^3 54 -> 42 us).
+// (L(U), half batches up to twice that size -> this rule: FP64 k = 3 9^3 cells 121 -> 105 us, k = 1 10^3 67 -> 45 us; FP32
+// k = 5 10^3 54 -> 42 us).
 template <typename T, int N, int QC, int QV, int CB, int GEO>
 int launch_coll_cell_cb(const KParams& kp, bool only_one_wave, const double* U, void* Rout, void* dU, double* Uout,
                         cudaStream_t st) {

@@ -949,13 +949,6 @@ int launch_op_any(const KParams& kp, const double* U, const void* Rin, void* Rou
   }
 }
 
-// The face-centric organisation runs the collocation kernels wherever they exist.  Face and cell kernel share the
-// face buffer's basis, so both follow this rule.
-template <typename T, int N, int QC, int QV, int GEO>
-constexpr bool use_coll() {
-  return coll_ok<T, N, QC, QV, GEO>();
-}
-
 template <typename T, int N, int QC, int QV, int GEO>
 int op_dispatch_geo(int mode, const KParams& kp, const double* U, const void* Rin, void* Rout, void* dU,
                     double* Uout, cudaStream_t st) {
@@ -963,7 +956,7 @@ int op_dispatch_geo(int mode, const KParams& kp, const double* U, const void* Ri
   // (only while a warp's slice stays small: at k = 5 a cell needs ~49 KB, which would leave 4 warps per SM)
   constexpr bool WARP =
       sizeof(T) == 4 && warp_slice_elems<T, N, QC, QV, true, true, true, GEO>() * sizeof(T) <= 20 * 1024;
-  if constexpr (use_coll<T, N, QC, QV, GEO>()) {
+  if constexpr (coll_ok<T, N, QC, QV, GEO>()) {
     if ((mode == OP_CELL || mode == (OP_CELL | OP_MASS)) && kp.fbuf != nullptr)
       return launch_coll_cell<T, N, QC, QV, GEO>(kp, U, Rout, dU, Uout, st);
   }
@@ -991,7 +984,7 @@ int op_dispatch_geo(int mode, const KParams& kp, const double* U, const void* Ri
     case OP_CELL | OP_FACE:
       return launch_op_any<T, N, QC, QV, GEO, WARP, true, true, false>(kp, U, Rin, Rout, dU, Uout, st);
     case OP_CELL | OP_MASS:
-      if constexpr (Feat<N, QC, QV>::faces && !use_coll<T, N, QC, QV, GEO>())
+      if constexpr (Feat<N, QC, QV>::faces && !coll_ok<T, N, QC, QV, GEO>())
         return launch_op_any<T, N, QC, QV, GEO, WARP, true, false, true>(kp, U, Rin, Rout, dU, Uout, st);
       return -2;
     case OP_CELL | OP_FACE | OP_MASS:
@@ -1272,7 +1265,7 @@ __global__ void __launch_bounds__(WPC * 32) dg_face_warp_kernel(const KParams kp
 
 template <typename T, int N, int QC, int QV, int GEO>
 int launch_faces(const KParams& kp, const double* U, void* FB, cudaStream_t st) {
-  if constexpr (use_coll<T, N, QC, QV, GEO>()) {
+  if constexpr (coll_ok<T, N, QC, QV, GEO>()) {
     // FP32 affine at k = 3: the register-resident kernel (1.13 ms against 1.46 ms per launch at 64^3, measured)
     if constexpr (sizeof(T) == 4 && GEO == GEO_AFFINE && task_faces_ok<N, QC, QV>()) {
       // (a mixed evaluation starts with the deviation state, in a buffer of its own; face lists come with stored geometry)
