@@ -43,13 +43,13 @@ FP32_PEAK_TFLOPS = 73.5  # measured FP32 FMA throughput, same probe
 # (kind, precision 0/1, N, QC, QV) -> (bytes per cell, sources digest, profile summary under profiles/).
 # The roofline reports traffic = bytes per cell x cells only while the sources still have that digest.
 TRAFFIC = {
-    ("faces", 0, 4, 5, 4): (15098.0, "fe3a2cccb0f35e22aeca52de0a8521be427c037633c16de9050e65b32e1c6b39",
+    ("faces", 0, 4, 5, 4): (15081.2, "da45aa28975853a610de66295900c4a05da6c5b6b0ee4748b16c59d4da821c44",
                             "profiles/collocation_kernels_tgv48_k3.md"),
-    ("cell_stage", 0, 4, 5, 4): (17644.5, "fe3a2cccb0f35e22aeca52de0a8521be427c037633c16de9050e65b32e1c6b39",
+    ("cell_stage", 0, 4, 5, 4): (17670.6, "da45aa28975853a610de66295900c4a05da6c5b6b0ee4748b16c59d4da821c44",
                                  "profiles/collocation_kernels_tgv48_k3.md"),
-    ("faces", 1, 4, 5, 4): (7331.9, "fe3a2cccb0f35e22aeca52de0a8521be427c037633c16de9050e65b32e1c6b39",
+    ("faces", 1, 4, 5, 4): (7331.2, "da45aa28975853a610de66295900c4a05da6c5b6b0ee4748b16c59d4da821c44",
                             "profiles/collocation_kernels_tgv48_k3.md"),
-    ("cell_stage", 1, 4, 5, 4): (13723.3, "fe3a2cccb0f35e22aeca52de0a8521be427c037633c16de9050e65b32e1c6b39",
+    ("cell_stage", 1, 4, 5, 4): (13751.4, "da45aa28975853a610de66295900c4a05da6c5b6b0ee4748b16c59d4da821c44",
                                  "profiles/collocation_kernels_tgv48_k3.md"),
 }
 
